@@ -101,6 +101,8 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+// A value that is the same in all lanes, said so to the compiler (all 32 lanes call).
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -142,6 +144,26 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
   return mbar_wait_slow(bar, parity, w, code);
 }
 
+// The same for a whole warp in uniform control flow: every lane polls, the vote decides.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtx& w, int code) {
+  unsigned long long t0 = 0;
+  uint32_t spins = 0;
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    if ((++spins & 31u) == 0) {
+      bool give_up = *w.abort_flag != 0;
+      const unsigned long long now = global_ns();
+      if (t0 == 0) t0 = now;
+      if (!give_up && now - t0 > w.limit_ns) {
+        *w.abort_flag = 1;
+        if (w.status) atomicCAS(w.status, 0, code);
+        give_up = true;
+      }
+      if (__any_sync(0xffffffffu, give_up)) return false;
+    }
+  }
+  return true;
+}
+
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
                                             int c0, int c1, int c2, int c3) {
   asm volatile(
@@ -163,8 +185,20 @@ __device__ __forceinline__ void tma_store_wait_read() {
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+// The MMA-issuing warps run in uniform control flow: all 32 lanes execute the loop, the waits and the
+// address arithmetic, and a predicate (`issue`, set on one lane by elect.sync) picks the lane that issues.
+// With a branch on the lane index instead, every tcgen05.mma takes ~50 cycles to issue whatever its size
+// (a group of 8: 400 cycles against 101-136 in this form, one CTA per SM, with or without 16 busy warps
+// beside it), which held the tensor pipe below its rate of one 128 x 128 x 16 product per 64 cycles.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void tc_commit(uint32_t bar, uint32_t issue) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}" ::"r"(bar), "r"(issue) : "memory");
 }
 __device__ __forceinline__ void tc_wait_ld() { __syncwarp(); asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_st() { __syncwarp(); asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -180,21 +214,21 @@ constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
 
 // D[tmem] (+)= A[smem] * B[smem]
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc,
-                                       uint32_t accumulate) {
+                                       uint32_t accumulate, uint32_t issue) {
   asm volatile(
-      "{\n.reg .pred p;\n.reg .b64 da, db;\nsetp.ne.b32 p, %4, 0;\n"
+      "{\n.reg .pred p, q;\n.reg .b64 da, db;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %6, 0;\n"
       "mov.b64 da, {%1, %5};\nmov.b64 db, {%2, %5};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi) : "memory");
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi), "r"(issue) : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem]
 __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc,
-                                       uint32_t accumulate) {
+                                       uint32_t accumulate, uint32_t issue) {
   asm volatile(
-      "{\n.reg .pred p;\n.reg .b64 db;\nsetp.ne.b32 p, %4, 0;\n"
+      "{\n.reg .pred p, q;\n.reg .b64 db;\nsetp.ne.b32 p, %4, 0;\nsetp.ne.b32 q, %6, 0;\n"
       "mov.b64 db, {%2, %5};\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n}"
-      ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi) : "memory");
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n}"
+      ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(accumulate), "r"(kDescHi), "r"(issue) : "memory");
 }
 
 // 32 consecutive fp32 columns of this thread's TMEM lane.
@@ -416,7 +450,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   static_assert(416 + 2 * kRing * kRingInts * 4 <= 896, "ring does not fit");
   static_assert(NK <= 4 && NV <= 4, "barrier slots");
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = uniform((int)(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
   const WaitCtx wctx{s_abort, args.status, args.wait_limit_ns};
 
@@ -454,7 +488,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem_base = *s_tmem_base;
+  const uint32_t tmem_base = (uint32_t)uniform((int)*s_tmem_base);
   // Everything above is set-up that touches no tensor: with a programmatic dependent launch it runs
   // while the kernel before this one (rotation / cache scatter) is still finishing.
   pdl_wait();
@@ -510,15 +544,16 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (!ok) break;
           ++it_n;
         }
-      } else if (warp < 2 && lane == 0) {
+      } else if (warp < 2) {
         // -------------------------------------------------------------- MMA issuer of slot t
-        // One issuing thread per slot (warps 0 and 1 sit on different schedulers), plain blocking
+        // One issuing warp per slot (warps 0 and 1 sit on different schedulers), plain blocking
         // waits. S_t has two 64-column buffers, tile k of the slot's stream uses buffer k & 1, and
         // P(k) is written over S(k). The issue order  S(k+1), then P(k) V(k)  lets the tensor pipe
         // compute the next scores while the softmax threads work on tile k, and P(k) V(k) while they
         // work on tile k+1; the pipe runs one thread's MMAs in order, so S(k+2) cannot overwrite
         // P(k) before P(k) V(k) has read it.
         const int t = warp;
+        const uint32_t issue = elect_one();
         constexpr uint32_t idesc_qk = instr_desc(BN, false);
         constexpr uint32_t idesc_pv = instr_desc(D, true);
         const uint32_t a_lo = desc_lo(s_q, 0) + (uint32_t)t * (Cfg::kQBytes >> 4);
@@ -539,7 +574,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // S(kq) = Q_t K(kq)^T into buffer kq & 1
         auto issue_qk = [&](const uint32_t kq, const bool last_of_item) -> bool {
           const uint32_t b = kq & 1u;
-          if (!mbar_wait(b_k_full + 8 * b, (kq >> 1) & 1u, wctx, kWaitKFull)) return false;
+          if (!mbar_wait_warp(b_k_full + 8 * b, (kq >> 1) & 1u, wctx, kWaitKFull)) return false;
           tc_fence_after();
           const uint32_t d = tm_s + 64u * b;
           const uint32_t kb = k_lo + b * (Cfg::kKVBytes >> 4);
@@ -547,11 +582,11 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int kk = 0; kk < D / 16; ++kk) {
             constexpr uint32_t kChunkQ = (BM * 128) >> 4, kChunkK = (BN * 128) >> 4;
             mma_ss(d, a_lo + (uint32_t)(kk >> 2) * kChunkQ + (uint32_t)(kk & 3) * 2,
-                   kb + (uint32_t)(kk >> 2) * kChunkK + (uint32_t)(kk & 3) * 2, idesc_qk, kk > 0 ? 1u : 0u);
+                   kb + (uint32_t)(kk >> 2) * kChunkK + (uint32_t)(kk & 3) * 2, idesc_qk, kk > 0 ? 1u : 0u, issue);
           }
-          tc_commit(b_k_empty + 8 * b);
-          tc_commit(b_s_full + 8 * b);
-          if (last_of_item) tc_commit(b_q_empty);     // last read of Q_t in this item
+          tc_commit(b_k_empty + 8 * b, issue);
+          tc_commit(b_s_full + 8 * b, issue);
+          if (last_of_item) tc_commit(b_q_empty, issue);     // last read of Q_t in this item
           return true;
         };
         // The slot's tiles form one stream across items: while the softmax threads work on tile k,
@@ -559,48 +594,48 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // next item (its Q was loaded as soon as this item's last scores had been issued).
         int w = -1, n = 0, j = 0;
         {
-          if (!mbar_wait(b_item_full, 0u, wctx, kWaitItemFull)) ok = false;
+          if (!mbar_wait_warp(b_item_full, 0u, wctx, kWaitItemFull)) ok = false;
           if (ok) {
             const volatile int* e = s_ring + (t * (int)kRing) * kRingInts;
-            w = e[0]; n = e[3];
-            mbar_arrive(b_item_empty);
+            w = uniform(e[0]); n = uniform(e[3]);
+            if (issue) mbar_arrive(b_item_empty);
           }
         }
-        if (ok && w >= 0) ok = mbar_wait(bar_q_ready, 0u, wctx, kWaitQFull) && issue_qk(kc, n == 1);
+        if (ok && w >= 0) ok = mbar_wait_warp(bar_q_ready, 0u, wctx, kWaitQFull) && issue_qk(kc, n == 1);
         while (ok && w >= 0) {
           const bool last_tile = (j + 1 == n);
           int w_next = w, n_next = n;
           bool have = true, last_flag = (j + 2 == n);
           // With one tile per item the next item's scores would be issued before the previous item's
           // epilogue has read O_t; the softmax threads must not get that far ahead of it.
-          if (j == 0 && last_tile && !(ok = mbar_wait(b_o_empty, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
+          if (j == 0 && last_tile && !(ok = mbar_wait_warp(b_o_empty, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
           if (last_tile) {
             const uint32_t item = it_n + 1u, ring = item % kRing;
-            if (!(ok = mbar_wait(b_item_full + 8 * ring, (item / kRing) & 1u, wctx, kWaitItemFull))) break;
+            if (!(ok = mbar_wait_warp(b_item_full + 8 * ring, (item / kRing) & 1u, wctx, kWaitItemFull))) break;
             const volatile int* e = s_ring + (t * (int)kRing + (int)ring) * kRingInts;
-            w_next = e[0]; n_next = e[3];
-            mbar_arrive(b_item_empty + 8 * ring);
+            w_next = uniform(e[0]); n_next = uniform(e[3]);
+            if (issue) mbar_arrive(b_item_empty + 8 * ring);
             have = w_next >= 0;
             last_flag = n_next == 1;
-            if (have && !(ok = mbar_wait(bar_q_ready, item & 1u, wctx, kWaitQFull))) break;
+            if (have && !(ok = mbar_wait_warp(bar_q_ready, item & 1u, wctx, kWaitQFull))) break;
           }
           if (have && !(ok = issue_qk(kc + 1, last_flag))) break;
           // the previous item's epilogue must have read O_t before it is overwritten
-          if (j == 0 && !last_tile && !(ok = mbar_wait(b_o_empty, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
+          if (j == 0 && !last_tile && !(ok = mbar_wait_warp(b_o_empty, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
           const uint32_t b = kc & 1u, parity = (kc >> 1) & 1u;
-          if (!(ok = mbar_wait(b_p_full + 8 * b, parity, wctx, kWaitP))) break;
-          if (!(ok = mbar_wait(b_v_full + 8 * b, parity, wctx, kWaitVFull))) break;
+          if (!(ok = mbar_wait_warp(b_p_full + 8 * b, parity, wctx, kWaitP))) break;
+          if (!(ok = mbar_wait_warp(b_v_full + 8 * b, parity, wctx, kWaitVFull))) break;
           tc_fence_after();            // O_t (+)= P(k) V(k)
           const uint32_t a = tm_s + 64u * b;
           const uint32_t vb = v_lo + b * (Cfg::kKVBytes >> 4);
-          mma_ts(tm_o, a, vb, idesc_pv, j == 0 ? 0u : 1u);
+          mma_ts(tm_o, a, vb, idesc_pv, j == 0 ? 0u : 1u, issue);
 #pragma unroll
           for (int kk = 1; kk < BN / 16; ++kk)
-            mma_ts(tm_o, a + kk * 8, vb + (uint32_t)kk * ((16 * 128) >> 4), idesc_pv, 1u);
-          tc_commit(b_v_empty + 8 * b);
+            mma_ts(tm_o, a + kk * 8, vb + (uint32_t)kk * ((16 * 128) >> 4), idesc_pv, 1u, issue);
+          tc_commit(b_v_empty + 8 * b, issue);
           ++kc;
           if (last_tile) {
-            tc_commit(b_o_full);
+            tc_commit(b_o_full, issue);
             ++it_n;
             w = w_next; n = n_next; j = 0;
           } else {
@@ -672,21 +707,22 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         ++it_n;
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
       // ---------------------------------------------------------------- MMA issuer
-      // Kept lean on purpose: one thread feeds the tensor pipe, so every scalar instruction
-      // between two tcgen05.mma counts. Descriptor low words are precomputed; inside a group of
+      // Kept lean on purpose: one warp feeds the tensor pipe, so every instruction between two
+      // tcgen05.mma counts. Descriptor low words are precomputed; inside a group of
       // MMAs only compile-time constants are added.
       constexpr uint32_t idesc_qk = instr_desc(BN, false);
       constexpr uint32_t idesc_pv = instr_desc(D, true);
       const uint32_t q_lo0 = desc_lo(s_q, 0), k_lo0 = desc_lo(s_k, 0), v_lo0 = desc_lo(s_v, BN * 128);
+      const uint32_t issue = elect_one();
       uint32_t it_n = 0, kc0 = 0, vc0 = 0, tc0 = 0, tc1 = 0;
       int n = 0, je0 = 0, jb1 = 0, je1 = 0;
       bool ok = true;
       // S_t = Q_t K_j^T; the K stage is released after the last slot that reads it
       auto issue_qk = [&](const int t, const int j) -> bool {
         const uint32_t kc = kc0 + (uint32_t)j, s = kc % NK;
-        if (!mbar_wait(bar_k_full + 8 * s, (kc / NK) & 1u, wctx, kWaitKFull)) return false;
+        if (!mbar_wait_warp(bar_k_full + 8 * s, (kc / NK) & 1u, wctx, kWaitKFull)) return false;
         tc_fence_after();
         const uint32_t d = tmem_base + Cfg::kTmemS + 128u * t;
         const uint32_t a_lo = q_lo0 + (uint32_t)t * (Cfg::kQBytes >> 4);
@@ -695,12 +731,12 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         for (int kk = 0; kk < D / 16; ++kk) {
           constexpr uint32_t kChunkQ = (BM * 128) >> 4, kChunkK = (BN * 128) >> 4;
           mma_ss(d, a_lo + (uint32_t)(kk >> 2) * kChunkQ + (uint32_t)(kk & 3) * 2,
-                 b_lo + (uint32_t)(kk >> 2) * kChunkK + (uint32_t)(kk & 3) * 2, idesc_qk, kk > 0 ? 1u : 0u);
+                 b_lo + (uint32_t)(kk >> 2) * kChunkK + (uint32_t)(kk & 3) * 2, idesc_qk, kk > 0 ? 1u : 0u, issue);
         }
-        if (t == 1 || !(j >= jb1 && j < je1)) tc_commit(bar_k_empty + 8 * s);
-        tc_commit(bar_s_full + 16 * t);
+        if (t == 1 || !(j >= jb1 && j < je1)) tc_commit(bar_k_empty + 8 * s, issue);
+        tc_commit(bar_s_full + 16 * t, issue);
         // the slot's last scores of this item: its Q buffer is free for the next item's Q from here on
-        if (j + 1 == (t ? je1 : je0)) tc_commit(bar_q_empty + 8 * t);
+        if (j + 1 == (t ? je1 : je0)) tc_commit(bar_q_empty + 8 * t, issue);
         return true;
       };
       // O_t (+)= P_t V_j, then either the next S_t or the end-of-item signals of slot t
@@ -708,22 +744,22 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (j >= jb && j < je) {
           const bool first = (j == jb);
           // the previous item's epilogue must have read O_t before it is overwritten
-          if (first && !mbar_wait(bar_o_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty)) return false;
-          if (!mbar_wait(bar_p_full + 16 * t, tcount & 1u, wctx, kWaitP)) return false;
+          if (first && !mbar_wait_warp(bar_o_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty)) return false;
+          if (!mbar_wait_warp(bar_p_full + 16 * t, tcount & 1u, wctx, kWaitP)) return false;
           const uint32_t vc = vc0 + (uint32_t)j, s = vc % NV;
-          if (!mbar_wait(bar_v_full + 8 * s, (vc / NV) & 1u, wctx, kWaitVFull)) return false;
+          if (!mbar_wait_warp(bar_v_full + 8 * s, (vc / NV) & 1u, wctx, kWaitVFull)) return false;
           tc_fence_after();
           const uint32_t a = tmem_base + Cfg::kTmemS + 128u * t;
           const uint32_t d = tmem_base + Cfg::kTmemO + (uint32_t)D * t;
           const uint32_t b_lo = v_lo0 + s * (Cfg::kKVBytes >> 4);
-          mma_ts(d, a, b_lo, idesc_pv, first ? 0u : 1u);
+          mma_ts(d, a, b_lo, idesc_pv, first ? 0u : 1u, issue);
 #pragma unroll
           for (int kk = 1; kk < BN / 16; ++kk)
-            mma_ts(d, a + kk * 8, b_lo + (uint32_t)kk * ((16 * 128) >> 4), idesc_pv, 1u);
+            mma_ts(d, a + kk * 8, b_lo + (uint32_t)kk * ((16 * 128) >> 4), idesc_pv, 1u, issue);
           ++tcount;
-          if (t == 1 || !(j >= jb1 && j < je1)) tc_commit(bar_v_empty + 8 * s);
+          if (t == 1 || !(j >= jb1 && j < je1)) tc_commit(bar_v_empty + 8 * s, issue);
           if (j + 1 < je) return issue_qk(t, j + 1);
-          tc_commit(bar_o_full + 8 * t);       // slot t is done with this item
+          tc_commit(bar_o_full + 8 * t, issue);       // slot t is done with this item
           return true;
         }
         if (j + 1 == jb && jb < je) return issue_qk(t, j + 1);   // slot t joins the key loop at the next tile
@@ -731,15 +767,15 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       };
       while (ok) {
         const uint32_t ring = it_n % kRing;
-        if (!mbar_wait(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull)) break;
+        if (!mbar_wait_warp(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull)) break;
         const volatile int* e = s_ring + ring * kRingInts;
-        const int w = e[0];
-        n = e[3]; jb1 = e[6]; je0 = e[7]; je1 = e[8];
-        mbar_arrive(bar_item_empty + 8 * ring);
+        const int w = uniform(e[0]);
+        n = uniform(e[3]); jb1 = uniform(e[6]); je0 = uniform(e[7]); je1 = uniform(e[8]);
+        if (issue) mbar_arrive(bar_item_empty + 8 * ring);
         if (w < 0) break;
         const uint32_t bar_q_ready = args.rope_table ? bar_q_rot : bar_q_full;
-        ok = mbar_wait(bar_q_ready + 0, it_n & 1u, wctx, kWaitQFull) &&
-             mbar_wait(bar_q_ready + 8, it_n & 1u, wctx, kWaitQFull);
+        ok = mbar_wait_warp(bar_q_ready + 0, it_n & 1u, wctx, kWaitQFull) &&
+             mbar_wait_warp(bar_q_ready + 8, it_n & 1u, wctx, kWaitQFull);
         if (!ok) break;
         if (je0 > 0) ok = issue_qk(0, 0);
         if (ok && jb1 == 0 && je1 > 0) ok = issue_qk(1, 0);
@@ -752,14 +788,12 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // before every softmax thread has seen the first, so wait until all of them are past the
         // previous item's o_full (they signal that on o_empty).
         if (je0 <= 0) {
-          if (!(ok = mbar_wait(bar_o_empty + 0, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
-          mbar_arrive(bar_q_empty + 0);
-          mbar_arrive(bar_o_full + 0);
+          if (!(ok = mbar_wait_warp(bar_o_empty + 0, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
+          if (issue) { mbar_arrive(bar_q_empty + 0); mbar_arrive(bar_o_full + 0); }
         }
         if (jb1 >= je1) {
-          if (!(ok = mbar_wait(bar_o_empty + 8, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
-          mbar_arrive(bar_q_empty + 8);
-          mbar_arrive(bar_o_full + 8);
+          if (!(ok = mbar_wait_warp(bar_o_empty + 8, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
+          if (issue) { mbar_arrive(bar_q_empty + 8); mbar_arrive(bar_o_full + 8); }
         }
         kc0 += (uint32_t)n;
         vc0 += (uint32_t)n;
