@@ -65,8 +65,8 @@ extern "C" const char* pp_last_cuda_error(void) { return pp::g_cuda_error; }
 
 extern "C" size_t pp_prefill_workspace_bytes(const pp_attn_params* params, int32_t k) {
   if (pp::check_params(params) != PP_OK || k < 1) return 0;
-  return sizeof(int32_t) * pp::prefill_table_ints(params->n_bins, params->capacity, k,
-                                                  params->n_q_heads / params->n_kv_heads);
+  return sizeof(int32_t) * pp::prefill_table_ints(params->n_bins, params->capacity, k, params->n_q_heads,
+                                                  params->n_kv_heads);
 }
 
 extern "C" int pp_prefill_attention(const pp_attn_params* params, const int32_t* bin_seg_ptr,
@@ -92,7 +92,7 @@ extern "C" int pp_prefill_attention(const pp_attn_params* params, const int32_t*
 
   pp::TableLayout L;
   st = pp::build_prefill_tables(params->n_bins, params->capacity, bin_seg_ptr, seg_start, seg_len, k,
-                                params->n_q_heads / params->n_kv_heads,
+                                params->n_q_heads, params->n_kv_heads,
                                 static_cast<int32_t*>(host_workspace), workspace_bytes / sizeof(int32_t), &L);
   if (st != PP_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -101,11 +101,11 @@ extern "C" int pp_prefill_attention(const pp_attn_params* params, const int32_t*
   if (e != cudaSuccess) return pp::note_cuda_error((int)e, "table upload");
   int32_t* d_table = static_cast<int32_t*>(workspace);
   if (do_rope) {
-    st = pp::launch_rope(*params, d_table, L, q, q, k_, stream);
+    st = pp::launch_rope(*params, d_table, L, q, k_, stream);
     if (st != PP_OK) return st;
   }
   if (do_attn) {
-    st = pp::launch_attention(*params, d_table, L, q, k_, v, o, nullptr, device_status, stream);
+    st = pp::launch_attention(*params, d_table, L, q, k_, v, o, nullptr, do_rope, device_status, stream);
     if (st != PP_OK) return st;
   }
   return PP_OK;
@@ -126,7 +126,7 @@ struct FusedLayout {
 FusedLayout fused_layout(const pp_attn_params& p, int32_t k) {
   auto up4 = [](size_t x) { return (x + 3) & ~size_t(3); };
   FusedLayout f;
-  f.table_ints = prefill_table_ints(p.n_bins, p.capacity, k, p.n_q_heads / p.n_kv_heads);
+  f.table_ints = prefill_table_ints(p.n_bins, p.capacity, k, p.n_q_heads, p.n_kv_heads);
   f.off_true_len = up4(f.table_ints);
   f.off_cap = f.off_true_len + up4((size_t)k);
   f.off_cache_off = f.off_cap + up4((size_t)k);          // multiple of 4 ints: 16-byte aligned int64 data
@@ -167,7 +167,7 @@ int launch_fused_kernels(const pp_attn_params& p, const TableLayout& L, const Fu
   }
   if (p.flags & PP_FLAG_ROPE_ONLY) return PP_OK;
   // the attention kernel rotates every Q tile in shared memory, so Q is read from HBM once
-  return launch_attention(p, d_table, L, q, k_, v, o, rope_table, device_status, stream);
+  return launch_attention(p, d_table, L, q, k_, v, o, rope_table, !(p.flags & PP_FLAG_SKIP_ROPE), device_status, stream);
 }
 
 // pp_prefill_fused, optionally cut in two: kUploadOnly validates, builds and uploads the tables,
@@ -211,7 +211,7 @@ int prefill_fused_impl(const pp_attn_params* params, const int32_t* bin_seg_ptr,
   if ((st = check_device()) != PP_OK) return st;
   TableLayout L;
   st = build_prefill_tables(params->n_bins, params->capacity, bin_seg_ptr, seg_start, seg_len, k,
-                            params->n_q_heads / params->n_kv_heads, h, f.table_ints, &L);
+                            params->n_q_heads, params->n_kv_heads, h, f.table_ints, &L);
   if (st != PP_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaMemcpyAsync(workspace, host_workspace, sizeof(int32_t) * f.upload_ints,

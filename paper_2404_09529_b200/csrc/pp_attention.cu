@@ -33,7 +33,8 @@
 //                (fused path) and run the previous item's epilogue
 //   warps 12-19  the same for slot 1
 // Softmax: tcgen05.ld the thread's scores, mask to the row's key range, lazy running maximum (O is
-// rescaled only when the maximum grows by more than 2^8), exp2, P written as bf16 over the S
+// rescaled only when the maximum grows by more than 2^8, or 2^90 in the shared-stream mode, where rows
+// whose scores are bounded drop the maximum altogether), exp2, P written as bf16 over the S
 // columns. Epilogue: O / l goes through a swizzled staging buffer and a TMA store.
 // TMEM: S0 | S1 | O0 | O1 = 512 columns. Every wait is an mbarrier wait with a time limit, also the
 // rendezvous between warps (no named barriers), so a failed wait ends the kernel with a status code.
@@ -60,6 +61,20 @@ constexpr int kRegsSoftmax = 104;          // setmaxnreg budgets: 640 threads st
 constexpr int kRegsSoftmaxIndep = 120;     // independent mode: 256 softmax threads at 120, 256 helper threads at 88
 constexpr int kRegsHelper = 88;
 constexpr int kRegsOther = 64;              // warps 0-3 give back 32 each, the 512 softmax threads take 8 each
+// Shared-stream mode, when a row needs no maximum any more. Its running maximum is lazy: it stays at the
+// maximum of the row's first visible tile until a score exceeds it by more than kLazyLog2 (log2 units).
+// Probabilities, sums and O have 8 exponent bits, so a common factor of up to 2^90 costs no precision, and
+// it leaves 2^37 for the number of keys times |v|. Where |q| |k| scale <= kBoundLog2 for every key
+// (Cauchy-Schwarz, norms taken before the rotation's rounding to bf16), two scores of a row differ by at
+// most 2 * 44 * (1 + 2^-7) < 90, so from its second tile on the row's maximum cannot move: neither the
+// 64 comparisons nor the exchange between the two threads of a row are needed, and the exponentials start
+// on the first 32 scores while the other 32 are still being loaded. The result does not depend on
+// whether the bound was known. Q and K of N(0, 1) values reach 17-30 (D = 64 / 128). Measured, whole step:
+// 16 prompts of up to 22 861 tokens, 32 heads, D = 128: 14.69 -> 12.2 ms (attention 14.1 -> 11.15 ms, 1156
+// TFLOP/s, from then on at the power cap: SM clock ~1620 MHz); 256 prompts of up to 3991, 32 / 8 heads:
+// 7.22 -> 6.48 ms. A wait for S took a softmax warp 2570 cycles per 128-key tile, now ~1250, of ~2900 in all.
+constexpr float kLazyLog2 = 90.f;
+constexpr float kBoundLog2 = 44.f;
 constexpr uint32_t kRing = 3;               // decoded work items in flight between the fetching thread and its readers
 constexpr int kRingInts = 20;              // ints per ring entry
 
@@ -244,6 +259,17 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr) : "memory");
 }
+// tcgen05.wait::ld with the loaded registers passed through it, so that nothing can be moved between
+// the load and the wait (used where other work stands between the two).
+__device__ __forceinline__ void tc_wait_ld32(uint32_t (&r)[32]) {
+  __syncwarp();
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+        "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+        "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+        "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+      :: "memory");
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   __syncwarp();
   asm volatile(
@@ -296,9 +322,55 @@ __device__ __forceinline__ uint64_t add_f2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+__device__ __forceinline__ uint64_t mul_f2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ float sum_f2x2(uint64_t a, uint64_t b) {
+  float x, y, z, w;
+  unpack_f2(a, x, y);
+  unpack_f2(b, z, w);
+  return (x + z) + (y + w);
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);     // .x (low 16 bits) = lo
   return *reinterpret_cast<uint32_t*>(&h);
+}
+
+// Probabilities of 32 scores: p = exp2(s * c - m), added up in sum_a / sum_b (two packed accumulators)
+// and packed to bf16.
+__device__ __forceinline__ void exp_chunk(const uint32_t* v, uint64_t c2, uint64_t negm2, uint64_t& sum_a, uint64_t& sum_b,
+                                          uint32_t (&pk)[16]) {
+#pragma unroll
+  for (int i = 0; i < 32; i += 4) {
+    float p0, p1, p2, p3;
+    unpack_f2(fma_f2(pack_f2(v[i], v[i + 1]), c2, negm2), p0, p1);
+    unpack_f2(fma_f2(pack_f2(v[i + 2], v[i + 3]), c2, negm2), p2, p3);
+    p0 = fast_exp2(p0); p1 = fast_exp2(p1); p2 = fast_exp2(p2); p3 = fast_exp2(p3);
+    sum_a = add_f2(sum_a, pack_f2(__float_as_uint(p0), __float_as_uint(p1)));
+    sum_b = add_f2(sum_b, pack_f2(__float_as_uint(p2), __float_as_uint(p3)));
+    pk[i >> 1] = pack_bf16(p0, p1);
+    pk[(i >> 1) + 1] = pack_bf16(p2, p3);
+  }
+}
+
+// Largest of 64 scores.
+__device__ __forceinline__ float max64(const uint32_t (&v)[64]) {
+  float m0 = fmax3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
+  float m1 = fmax3(__uint_as_float(v[3]), __uint_as_float(v[4]), __uint_as_float(v[5]));
+  float m2 = fmax3(__uint_as_float(v[6]), __uint_as_float(v[7]), __uint_as_float(v[8]));
+  float m3 = fmax3(__uint_as_float(v[9]), __uint_as_float(v[10]), __uint_as_float(v[11]));
+#pragma unroll
+  for (int i = 12; i + 7 < 64; i += 8) {
+    m0 = fmax3(m0, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
+    m1 = fmax3(m1, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
+    m2 = fmax3(m2, __uint_as_float(v[i + 4]), __uint_as_float(v[i + 5]));
+    m3 = fmax3(m3, __uint_as_float(v[i + 6]), __uint_as_float(v[i + 7]));
+  }
+  m0 = fmax3(m0, __uint_as_float(v[60]), __uint_as_float(v[61]));      // 12 + 8 * 6 = 60
+  m1 = fmax3(m1, __uint_as_float(v[62]), __uint_as_float(v[63]));
+  return fmaxf(fmax3(m0, m1, m2), m3);
 }
 
 // Bits [c_lo, c_hi] of a 64-bit word set (none if the interval is empty); c_hi <= 63, c_lo >= 0.
@@ -327,8 +399,11 @@ struct AttnArgs {
   int32_t capacity;              // rows per bin
   int32_t total_work;            // n_kv_heads * n_items * subs
   float scale_log2;              // softmax scale * log2(e)
+  float bound2;                  // (kBoundLog2 / scale_log2)^2: |q|^2 |k|^2 up to which scores are bounded
   __nv_bfloat16* o;
   const float2* rope_table;      // [D/4][capacity][2] (cos, sin) pairs, or null: Q arrives already rotated
+  const uint32_t* k_norm2;       // shared-stream mode: [Hkv] largest |k|^2 (float bits); null: no bound on the scores
+  const uint32_t* q_norm2;       // [Hq] largest |q|^2; used when Q arrives already rotated
   int32_t* status;
   unsigned long long wait_limit_ns;
 };
@@ -446,6 +521,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(misc + 400);
   volatile int* s_abort = reinterpret_cast<volatile int*>(misc + 404);
   volatile int* s_ring = reinterpret_cast<volatile int*>(misc + 416);   // [2 rings][kRing][kRingInts]
+  volatile uint8_t* s_bounded = misc + 1008;     // [2 slots][4 quadrants][2 halves] shared-stream mode: the warp's rows are bounded
   volatile float* s_xchg = reinterpret_cast<volatile float*>(misc + 1024);   // [2 slots][2 halves][128 rows]
   static_assert(416 + 2 * kRing * kRingInts * 4 <= 896, "ring does not fit");
   static_assert(NK <= 4 && NV <= 4, "barrier slots");
@@ -719,10 +795,13 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t it_n = 0, kc0 = 0, vc0 = 0, tc0 = 0, tc1 = 0;
       int n = 0, je0 = 0, jb1 = 0, je1 = 0;
       bool ok = true;
-      // S_t = Q_t K_j^T; the K stage is released after the last slot that reads it
-      auto issue_qk = [&](const int t, const int j) -> bool {
+      auto wait_k = [&](const int j) -> bool {
         const uint32_t kc = kc0 + (uint32_t)j, s = kc % NK;
-        if (!mbar_wait_warp(bar_k_full + 8 * s, (kc / NK) & 1u, wctx, kWaitKFull)) return false;
+        return mbar_wait_warp(bar_k_full + 8 * s, (kc / NK) & 1u, wctx, kWaitKFull);
+      };
+      // S_t = Q_t K_j^T (K_j has been waited for); the K stage is released after the last slot that reads it
+      auto issue_qk = [&](const int t, const int j) {
+        const uint32_t kc = kc0 + (uint32_t)j, s = kc % NK;
         tc_fence_after();
         const uint32_t d = tmem_base + Cfg::kTmemS + 128u * t;
         const uint32_t a_lo = q_lo0 + (uint32_t)t * (Cfg::kQBytes >> 4);
@@ -737,32 +816,37 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         tc_commit(bar_s_full + 16 * t, issue);
         // the slot's last scores of this item: its Q buffer is free for the next item's Q from here on
         if (j + 1 == (t ? je1 : je0)) tc_commit(bar_q_empty + 8 * t, issue);
-        return true;
       };
-      // O_t (+)= P_t V_j, then either the next S_t or the end-of-item signals of slot t
+      // O_t (+)= P_t V_j, then either the next S_t or the end-of-item signals of slot t. V_j and the next K
+      // tile are waited for first: they have been there for long, but even a wait that succeeds at once costs
+      // ~100 cycles, which then do not stand between P_t and its product.
       auto slot_step = [&](const int t, const int j, const int jb, const int je, uint32_t& tcount) -> bool {
         if (j >= jb && j < je) {
           const bool first = (j == jb);
           // the previous item's epilogue must have read O_t before it is overwritten
           if (first && !mbar_wait_warp(bar_o_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty)) return false;
-          if (!mbar_wait_warp(bar_p_full + 16 * t, tcount & 1u, wctx, kWaitP)) return false;
           const uint32_t vc = vc0 + (uint32_t)j, s = vc % NV;
           if (!mbar_wait_warp(bar_v_full + 8 * s, (vc / NV) & 1u, wctx, kWaitVFull)) return false;
+          if (j + 1 < je && !wait_k(j + 1)) return false;
+          if (!mbar_wait_warp(bar_p_full + 16 * t, tcount & 1u, wctx, kWaitP)) return false;
           tc_fence_after();
           const uint32_t a = tmem_base + Cfg::kTmemS + 128u * t;
           const uint32_t d = tmem_base + Cfg::kTmemO + (uint32_t)D * t;
           const uint32_t b_lo = v_lo0 + s * (Cfg::kKVBytes >> 4);
           mma_ts(d, a, b_lo, idesc_pv, first ? 0u : 1u, issue);
 #pragma unroll
-          for (int kk = 1; kk < BN / 16; ++kk)
-            mma_ts(d, a + kk * 8, b_lo + (uint32_t)kk * ((16 * 128) >> 4), idesc_pv, 1u, issue);
+          for (int kk = 1; kk < BN / 16; ++kk)        // P of the first 64 keys at column 0, of the others at column 64
+            mma_ts(d, a + (kk >> 2) * 64 + (kk & 3) * 8, b_lo + (uint32_t)kk * ((16 * 128) >> 4), idesc_pv, 1u, issue);
           ++tcount;
           if (t == 1 || !(j >= jb1 && j < je1)) tc_commit(bar_v_empty + 8 * s, issue);
-          if (j + 1 < je) return issue_qk(t, j + 1);
-          tc_commit(bar_o_full + 8 * t, issue);       // slot t is done with this item
+          if (j + 1 < je) issue_qk(t, j + 1);
+          else tc_commit(bar_o_full + 8 * t, issue);  // slot t is done with this item
           return true;
         }
-        if (j + 1 == jb && jb < je) return issue_qk(t, j + 1);   // slot t joins the key loop at the next tile
+        if (j + 1 == jb && jb < je) {        // slot t joins the key loop at the next tile
+          if (!wait_k(j + 1)) return false;
+          issue_qk(t, j + 1);
+        }
         return true;
       };
       while (ok) {
@@ -777,8 +861,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         ok = mbar_wait_warp(bar_q_ready + 0, it_n & 1u, wctx, kWaitQFull) &&
              mbar_wait_warp(bar_q_ready + 8, it_n & 1u, wctx, kWaitQFull);
         if (!ok) break;
-        if (je0 > 0) ok = issue_qk(0, 0);
-        if (ok && jb1 == 0 && je1 > 0) ok = issue_qk(1, 0);
+        if (!(ok = wait_k(0))) break;                     // every item has a first tile
+        if (je0 > 0) issue_qk(0, 0);
+        if (jb1 == 0 && je1 > 0) issue_qk(1, 0);
         for (int j = 0; ok && j < n; ++j) {
           ok = slot_step(0, j, 0, je0, tc0);
           if (ok) ok = slot_step(1, j, jb1, je1, tc1);
@@ -1109,12 +1194,16 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     const int32_t* tb = args.table;
     uint32_t it_n = 0, tcount = 0;
     bool ok = true;
-    // Rotates this thread's part of row `row` of Q_t in shared memory by the angles of position
-    // `pos` (<= 0: nothing to do), with the same fp32 arithmetic and rounding as the stand-alone
-    // kernel, then reports the slot's Q as ready. Waits for the TMA load of Q first.
-    auto rotate_q = [&](const int pos, const uint32_t parity) -> bool {
+    // Rotates this thread's part of row `row` of Q_t in shared memory by the angles of position `pos`
+    // (< 0: padding, nothing to do), with the same fp32 arithmetic and rounding as the stand-alone
+    // kernel, then reports the slot's Q as ready. Waits for the TMA load of Q first. The warp also says
+    // whether its half of every row is short enough for the bound on the scores: |half|^2 <= limit.
+    volatile uint8_t* const bounded_mine = s_bounded + (t * 4 + quad) * 2 + h;
+    volatile uint8_t* const bounded_other = s_bounded + (t * 4 + quad) * 2 + (h ^ 1);
+    auto rotate_q = [&](const int pos, const float limit, const uint32_t parity) -> bool {
       if (!__all_sync(0xffffffffu, mbar_wait(bar_q_full + 8 * t, parity, wctx, kWaitQFull))) return false;
-      if (pos > 0) {
+      uint64_t n2a = 0ull, n2b = 0ull;
+      if (pos >= 0) {
         constexpr int kUnits = D / 16;                 // 16-byte units per half of a row
         const uint32_t q_row = s_q + (uint32_t)t * Cfg::kQBytes + (uint32_t)row * 128;
         // table[g][pos] = (cos, sin) of j = 2g and 2g + 1: consecutive rows read consecutive 16 bytes
@@ -1141,6 +1230,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const __nv_bfloat162 l2 = *reinterpret_cast<__nv_bfloat162*>(&lo[i]);
             const __nv_bfloat162 h2 = *reinterpret_cast<__nv_bfloat162*>(&hi[i]);
             const float2 a = __bfloat1622float2(l2), b = __bfloat1622float2(h2);
+            const uint64_t a2 = pack_f2(__float_as_uint(a.x), __float_as_uint(a.y));
+            const uint64_t b2 = pack_f2(__float_as_uint(b.x), __float_as_uint(b.y));
+            n2a = fma_f2(a2, a2, n2a);
+            n2b = fma_f2(b2, b2, n2b);
             lo[i] = pack_bf16(__fmaf_rn(a.x, c.x, -__fmul_rn(b.x, c.y)), __fmaf_rn(a.y, c.z, -__fmul_rn(b.y, c.w)));
             hi[i] = pack_bf16(__fmaf_rn(b.x, c.x, __fmul_rn(a.x, c.y)), __fmaf_rn(b.y, c.z, __fmul_rn(a.y, c.w)));
           }
@@ -1149,6 +1242,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
       }
+      const bool short_rows = __all_sync(0xffffffffu, sum_f2x2(n2a, n2b) <= limit);
+      if (lane == 0) *bounded_mine = short_rows ? 1 : 0;
       mbar_arrive(bar_q_rot + 8 * t);
       return true;
     };
@@ -1162,7 +1257,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const int w = e[0];
       const int item_bin = e[1], item_kv_row0 = e[2];
       const int jb_t = f ? e[6] : 0, je_t = f ? e[8] : e[7];
-      const int q_row0_t = e[4 + f], head_t = e[9 + f];
+      const int q_row0_t = e[4 + f], head_t = e[9 + f], kv_head = e[11];
       const int bin_used = e[12], seg_end = e[13], key_lo_t = e[14 + f], seg_first_t = e[16 + f];
       const int single_seg = e[18] >> f;
       mbar_arrive(bar_item_empty + 8 * ring);
@@ -1176,17 +1271,55 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           lo = seg_start_at(tb + args.off_seg_start, seg_first_t + 1, seg_end, i_row, i_row - lane + 31, lo, lane);
         if (i_row < bin_used) { key_lo = lo; key_hi = i_row; }
       }
-      // Fused path: Q arrives raw and is rotated in shared memory.
+      // |q|^2 up to which every score of a row stays below the bound (0 if nothing is known about the keys)
+      float q2_limit = 0.f;
+      if (args.k_norm2) q2_limit = args.bound2 / fmaxf(__uint_as_float(__ldg(args.k_norm2 + kv_head)), 1e-30f);
+      bool bounded = false;
+      // Fused path: Q arrives raw and is rotated in shared memory. Each half of a row is held to half
+      // the limit, so that no sum over the two threads of a row is needed.
       if (args.rope_table) {
-        ok = rotate_q(used ? key_hi - key_lo : -1, it_n & 1u);
+        ok = rotate_q(used ? key_hi - key_lo : -1, 0.5f * q2_limit, it_n & 1u);
         if (!ok) break;
+      } else if (args.q_norm2) {
+        bounded = __uint_as_float(__ldg(args.q_norm2 + head_t)) <= q2_limit;
       }
       float m_run = -INFINITY;      // running maximum of the whole row, in scaled log2 units
-      float l_run = 0.f;            // this thread's share of the running sum of exp2(s * c - m_run)
+      uint64_t sum_a = 0ull, sum_b = 0ull;   // this thread's share of the running sum of exp2(s * c - m_run), in four parts
+      float neg_m = 0.f;
+      const uint64_t c2 = pack_f2(__float_as_uint(c_scale), __float_as_uint(c_scale));
+      bool fast = false;            // bounded, and every row of the warp has its maximum
+      // tiles [clean_jb, clean_je) of this half are visible to every row of the warp from end to end
+      constexpr int EPT = BN / 2;                            // scores per thread and tile
+      constexpr int NCH = EPT / 32;                          // 32-column TMEM round trips
+      const int half0 = item_kv_row0 + EPT * h;
+      const int clean_jb = (max(__reduce_max_sync(0xffffffffu, key_lo) - half0, 0) + BN - 1) / BN;
+      const int clean_je = (__reduce_min_sync(0xffffffffu, key_hi) - half0 + (BN - EPT + 1)) / BN;   // <= 0 with padding rows
+      // this half's P goes over the first half of its own scores' columns: no other thread reads them
+      const uint32_t tmem_sb = tmem_s + EPT * h;
 
       for (int j = jb_t; j < je_t; ++j) {
-        constexpr int EPT = BN / 2;                          // scores per thread and tile
-        constexpr int NCH = EPT / 32;                        // 32-column TMEM round trips
+        if (fast && j >= clean_jb && j < clean_je) {
+          // The common tile: nothing to mask, no maximum to find. The scores of the second chunk are
+          // loaded while the exponentials of the first are computed.
+          ok = mbar_wait_warp(bar_s_full + 16 * t, tcount & 1u, wctx, kWaitS);
+          if (!ok) break;                                    // warp-uniform
+          tc_fence_after();
+          const uint64_t negm2 = pack_f2(__float_as_uint(neg_m), __float_as_uint(neg_m));
+          uint32_t va[32], vb[32], pk[16];
+          tmem_ld32(tmem_sb, va);
+          tc_wait_ld32(va);
+          tmem_ld32(tmem_sb + 32, vb);
+          exp_chunk(va, c2, negm2, sum_a, sum_b, pk);
+          tmem_st16(tmem_sb, pk);
+          tc_wait_ld32(vb);
+          exp_chunk(vb, c2, negm2, sum_a, sum_b, pk);
+          tmem_st16(tmem_sb + 16, pk);
+          tc_wait_st();
+          tc_fence_before();
+          mbar_arrive(bar_p_full + 16 * t);
+          ++tcount;
+          continue;
+        }
         const int kv0 = item_kv_row0 + j * BN + EPT * h;     // first key of this thread's half
         const int c_lo = max(key_lo - kv0, 0);
         const int c_hi = min(key_hi - kv0, EPT - 1);         // visible columns [c_lo, c_hi] of the half
@@ -1200,19 +1333,14 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t warp_flags = __reduce_or_sync(0xffffffffu, lane_flags);
         const bool need[NCH] = {(warp_flags & 1u) != 0, (warp_flags & 2u) != 0};
         const bool cut = (warp_flags & 4u) != 0;
-        const uint32_t sbuf = 0u;
-        const uint32_t tparity = tcount & 1u;
-        const uint32_t tmem_sb = tmem_s;
-        ok = __all_sync(0xffffffffu, mbar_wait(bar_s_full + 8 * (2 * t + sbuf), tparity, wctx, kWaitS));
+        ok = mbar_wait_warp(bar_s_full + 16 * t, tcount & 1u, wctx, kWaitS);
         if (!ok) break;                                      // warp-uniform
         tc_fence_after();
-
-        // this thread's scores
         uint32_t v[EPT];
 #pragma unroll
         for (int ch = 0; ch < NCH; ++ch) {
           if (need[ch]) {
-            tmem_ld32(tmem_sb + EPT * h + 32 * ch, *reinterpret_cast<uint32_t(*)[32]>(&v[32 * ch]));
+            tmem_ld32(tmem_sb + 32 * ch, *reinterpret_cast<uint32_t(*)[32]>(&v[32 * ch]));
           } else {
 #pragma unroll
             for (int i = 0; i < 32; ++i) v[32 * ch + i] = 0xff800000u;        // -inf
@@ -1227,87 +1355,60 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
 #pragma unroll
           for (int i = 0; i < 32; ++i) v[32 + i] = (vis_hi & (1u << i)) ? v[32 + i] : 0xff800000u;
         }
-        float mx;
-        {
-          float m0 = fmax3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
-          float m1 = fmax3(__uint_as_float(v[3]), __uint_as_float(v[4]), __uint_as_float(v[5]));
-          float m2 = fmax3(__uint_as_float(v[6]), __uint_as_float(v[7]), __uint_as_float(v[8]));
-          float m3 = fmax3(__uint_as_float(v[9]), __uint_as_float(v[10]), __uint_as_float(v[11]));
-#pragma unroll
-          for (int i = 12; i + 7 < EPT; i += 8) {
-            m0 = fmax3(m0, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
-            m1 = fmax3(m1, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
-            m2 = fmax3(m2, __uint_as_float(v[i + 4]), __uint_as_float(v[i + 5]));
-            m3 = fmax3(m3, __uint_as_float(v[i + 6]), __uint_as_float(v[i + 7]));
-          }
-          // 12 + 8 * n = EPT - 4; the last four
-          m0 = fmax3(m0, __uint_as_float(v[EPT - 4]), __uint_as_float(v[EPT - 3]));
-          m1 = fmax3(m1, __uint_as_float(v[EPT - 2]), __uint_as_float(v[EPT - 1]));
-          mx = fmaxf(fmax3(m0, m1, m2), m3);
-        }
-        // Row maximum over both halves. The barrier also orders the two halves' S reads before
-        // either writes P over the S columns.
-        *x_mine = mx;
-        if (!(ok = rendezvous(bar_pair, pair_ph, kWaitPair))) break;
-        mx = fmaxf(mx, *x_other);
-        // lazy running-maximum update: keep the stale maximum while the new one is < 2^8 above it
-        const float m_tile = mx * c_scale;
-        float m_new = m_run;
-        if (m_tile > m_run + 8.f) m_new = m_tile;
-        const bool rescale = (m_new != m_run) && (m_run != -INFINITY);
-        const float alpha = rescale ? fast_exp2(m_run - m_new) : 1.f;
-        if (j > jb_t && __any_sync(0xffffffffu, rescale)) {
-          // (S_t ready implies that the previous P_t V product has finished.) Each half rescales its
-          // own D/2 columns of the row.
+        if (!fast) {
+          // Row maximum over both halves. (The exchange slot is not written again before both halves
+          // have announced their P of this tile.)
+          float mx = max64(v);
+          *x_mine = mx;
+          if (!(ok = rendezvous(bar_pair, pair_ph, kWaitPair))) break;
+          mx = fmaxf(mx, *x_other);
+          if (j == jb_t && args.rope_table) bounded = (*bounded_mine & *bounded_other) != 0;
+          const float m_tile = mx * c_scale;
+          float m_new = m_run;
+          if (m_tile > m_run + kLazyLog2) m_new = m_tile;
+          const bool rescale = (m_new != m_run) && (m_run != -INFINITY);
+          if (j > jb_t && __any_sync(0xffffffffu, rescale)) {
+            const float alpha = rescale ? fast_exp2(m_run - m_new) : 1.f;
+            // (S_t ready implies that the previous P_t V product has finished.) Each half rescales its
+            // own D/2 columns of the row.
 #pragma unroll 1
-          for (int ch = 0; ch < D / 32; ++ch) {          // rare path: keep it small
-            uint32_t ov[16];
-            tmem_ld16(tmem_o + (D / 2) * h + ch * 16, ov);
-            tc_wait_ld();
+            for (int ch = 0; ch < D / 32; ++ch) {          // rare path: keep it small
+              uint32_t ov[16];
+              tmem_ld16(tmem_o + (D / 2) * h + ch * 16, ov);
+              tc_wait_ld();
 #pragma unroll
-            for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
-            tmem_st16(tmem_o + (D / 2) * h + ch * 16, ov);
+              for (int i = 0; i < 16; ++i) ov[i] = __float_as_uint(__uint_as_float(ov[i]) * alpha);
+              tmem_st16(tmem_o + (D / 2) * h + ch * 16, ov);
+            }
+            const uint64_t alpha2 = pack_f2(__float_as_uint(alpha), __float_as_uint(alpha));
+            sum_a = mul_f2(sum_a, alpha2);
+            sum_b = mul_f2(sum_b, alpha2);
           }
+          m_run = m_new;
+          neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
+          // rows that see nothing at all (padding) do not hold the others back
+          fast = bounded && __all_sync(0xffffffffu, m_run != -INFINITY || key_hi < key_lo);
         }
-        l_run *= alpha;
-        m_run = m_new;
-        const float neg_m = (m_run == -INFINITY) ? 0.f : -m_run;
-
         // p = exp2(s * c - m), row sum, P (bf16) written over the S columns
-        const uint64_t c2 = pack_f2(__float_as_uint(c_scale), __float_as_uint(c_scale));
-        const uint64_t negm2 = pack_f2(__float_as_uint(neg_m), __float_as_uint(neg_m));
-        uint64_t sum_a = 0ull, sum_b = 0ull;                 // two packed accumulators
+        const uint64_t negm2_tile = pack_f2(__float_as_uint(neg_m), __float_as_uint(neg_m));
 #pragma unroll
         for (int ch = 0; ch < NCH; ++ch) {
           uint32_t pk[16];
           if (need[ch]) {
-#pragma unroll
-            for (int i = 0; i < 32; i += 4) {
-              float p0, p1, p2, p3;
-              unpack_f2(fma_f2(pack_f2(v[ch * 32 + i], v[ch * 32 + i + 1]), c2, negm2), p0, p1);
-              unpack_f2(fma_f2(pack_f2(v[ch * 32 + i + 2], v[ch * 32 + i + 3]), c2, negm2), p2, p3);
-              p0 = fast_exp2(p0); p1 = fast_exp2(p1); p2 = fast_exp2(p2); p3 = fast_exp2(p3);
-              sum_a = add_f2(sum_a, pack_f2(__float_as_uint(p0), __float_as_uint(p1)));
-              sum_b = add_f2(sum_b, pack_f2(__float_as_uint(p2), __float_as_uint(p3)));
-              pk[i >> 1] = pack_bf16(p0, p1);
-              pk[(i >> 1) + 1] = pack_bf16(p2, p3);
-            }
+            exp_chunk(&v[32 * ch], c2, negm2_tile, sum_a, sum_b, pk);
           } else {
 #pragma unroll
             for (int i = 0; i < 16; ++i) pk[i] = 0u;
           }
-          tmem_st16(tmem_sb + (EPT / 2) * h + ch * 16, pk);
+          tmem_st16(tmem_sb + ch * 16, pk);
         }
-        float sum0, sum1, sum2, sum3;
-        unpack_f2(sum_a, sum0, sum1);
-        unpack_f2(sum_b, sum2, sum3);
-        l_run += (sum0 + sum2) + (sum1 + sum3);
         tc_wait_st();
         tc_fence_before();
-        mbar_arrive(bar_p_full + 8 * (2 * t + sbuf));
+        mbar_arrive(bar_p_full + 16 * t);
         ++tcount;
       }
       if (!ok) break;
+      const float l_run = sum_f2x2(sum_a, sum_b);
 
       // epilogue: O_t / l -> bf16 -> shared memory (128-byte swizzle) -> TMA store
       ok = __all_sync(0xffffffffu, mbar_wait(bar_o_full + 8 * t, it_n & 1u, wctx, kWaitOFull));
@@ -1457,8 +1558,8 @@ int sm_count() {
 
 template <int D, bool kIndep>
 int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const void* q,
-                       const void* k, const void* v, void* o, const void* rope_table, int32_t* device_status,
-                       cudaStream_t stream) {
+                       const void* k, const void* v, void* o, const void* rope_table, bool have_norms,
+                       int32_t* device_status, cudaStream_t stream) {
   constexpr int BN = kIndep ? kTileNShort : kTileN;
   using Cfg = AttnCfg<D, BN>;
   CUtensorMap mq, mk, mv, mo;
@@ -1502,6 +1603,10 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.total_work = (int32_t)total;
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf((float)D);
   a.scale_log2 = scale * 1.4426950408889634f;
+  a.bound2 = (kBoundLog2 / a.scale_log2) * (kBoundLog2 / a.scale_log2);
+  const bool norms = have_norms && !kIndep && p.n_q_heads + p.n_kv_heads <= kMaxNormHeads;
+  a.k_norm2 = norms ? reinterpret_cast<const uint32_t*>(d_table + L.norms) : nullptr;
+  a.q_norm2 = norms && !rope_table ? a.k_norm2 + p.n_kv_heads : nullptr;
   a.o = static_cast<__nv_bfloat16*>(o);
   a.rope_table = static_cast<const float2*>(rope_table);
   a.status = device_status;
@@ -1522,15 +1627,15 @@ int launch_bounded_wait_selftest(int32_t* device_status, uint64_t limit_ns, void
 }
 
 int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const void* q,
-                     const void* k, const void* v, void* o, const void* rope_table, int32_t* device_status,
-                     void* stream) {
+                     const void* k, const void* v, void* o, const void* rope_table, bool have_norms,
+                     int32_t* device_status, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (L.independent_slots) {
-    if (p.head_dim == 128) return launch_attention_t<128, true>(p, d_table, L, q, k, v, o, rope_table, device_status, s);
-    return launch_attention_t<64, true>(p, d_table, L, q, k, v, o, rope_table, device_status, s);
+    if (p.head_dim == 128) return launch_attention_t<128, true>(p, d_table, L, q, k, v, o, rope_table, have_norms, device_status, s);
+    return launch_attention_t<64, true>(p, d_table, L, q, k, v, o, rope_table, have_norms, device_status, s);
   }
-  if (p.head_dim == 128) return launch_attention_t<128, false>(p, d_table, L, q, k, v, o, rope_table, device_status, s);
-  return launch_attention_t<64, false>(p, d_table, L, q, k, v, o, rope_table, device_status, s);
+  if (p.head_dim == 128) return launch_attention_t<128, false>(p, d_table, L, q, k, v, o, rope_table, have_norms, device_status, s);
+  return launch_attention_t<64, false>(p, d_table, L, q, k, v, o, rope_table, have_norms, device_status, s);
 }
 
 }  // namespace pp

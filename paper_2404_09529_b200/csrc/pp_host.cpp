@@ -189,13 +189,13 @@ int32_t max_fold(int32_t group) {
   return 1;
 }
 
-size_t prefill_table_ints(int32_t n_bins, int32_t capacity, int32_t k, int32_t group) {
+size_t prefill_table_ints(int32_t n_bins, int32_t capacity, int32_t k, int32_t n_q_heads, int32_t n_kv_heads) {
   // sized for the shortest query tiles any mode can choose (head folding shortens them)
-  const int32_t rq = kTileM / max_fold(group);
+  const int32_t rq = kTileM / max_fold(n_q_heads / n_kv_heads);
   const int64_t q_tiles = (int64_t)n_bins * ((capacity + rq - 1) / rq);
-  // header + bin_seg_ptr + bin_used + seg_start + items (kItemInts ints each), each block 4-int aligned
+  // header + norms + bin_seg_ptr + bin_used + seg_start + items (kItemInts ints each), each block 4-int aligned
   auto up4 = [](int64_t x) { return (x + 3) & ~int64_t(3); };
-  return (size_t)(kHeaderInts + up4(n_bins + 1) + up4(n_bins) + up4(k) + kItemInts * q_tiles);
+  return (size_t)(kHeaderInts + up4((int64_t)n_q_heads + n_kv_heads) + up4(n_bins + 1) + up4(n_bins) + up4(k) + kItemInts * q_tiles);
 }
 
 namespace {
@@ -219,8 +219,9 @@ double mean_key_tiles(int32_t n_bins, const int32_t* bin_seg_ptr, const int32_t*
 }  // namespace
 
 int build_prefill_tables(int32_t n_bins, int32_t capacity, const int32_t* bin_seg_ptr,
-                         const int32_t* seg_start, const int32_t* seg_len, int32_t k, int32_t group,
-                         int32_t* out, size_t out_ints, TableLayout* layout) {
+                         const int32_t* seg_start, const int32_t* seg_len, int32_t k, int32_t n_q_heads,
+                         int32_t n_kv_heads, int32_t* out, size_t out_ints, TableLayout* layout) {
+  const int32_t group = n_q_heads / n_kv_heads;
   // How the two query-tile slots of a CTA are fed:
   //  - even number of query heads per KV head: two heads over the same rows share a K/V stream;
   //  - otherwise, long items: two consecutive row tiles of one head share a K/V stream (halves the
@@ -238,11 +239,12 @@ int build_prefill_tables(int32_t n_bins, int32_t capacity, const int32_t* bin_se
   const int32_t rq = kTileM / fold;                            // bin rows per query tile
   auto up4 = [](int64_t x) { return (x + 3) & ~int64_t(3); };
   TableLayout L;
-  L.bin_seg_ptr = kHeaderInts;
+  L.norms = kHeaderInts;
+  L.bin_seg_ptr = L.norms + (int32_t)up4((int64_t)n_q_heads + n_kv_heads);
   L.bin_used = L.bin_seg_ptr + (int32_t)up4(n_bins + 1);
   L.seg_start = L.bin_used + (int32_t)up4(n_bins);
   L.items = L.seg_start + (int32_t)up4(k);
-  if (out_ints < prefill_table_ints(n_bins, capacity, k, group)) return PP_ERR_BUFFER_TOO_SMALL;
+  if (out_ints < prefill_table_ints(n_bins, capacity, k, n_q_heads, n_kv_heads)) return PP_ERR_BUFFER_TOO_SMALL;
   std::memset(out, 0, sizeof(int32_t) * (size_t)L.items);
   std::memcpy(out + L.bin_seg_ptr, bin_seg_ptr, sizeof(int32_t) * (size_t)(n_bins + 1));
   std::memcpy(out + L.seg_start, seg_start, sizeof(int32_t) * (size_t)k);
@@ -352,11 +354,11 @@ extern "C" int pp_prefill_schedule_info(const pp_attn_params* params, const int3
   int st = pp::validate_packing(params->n_bins, params->capacity, bin_seg_ptr, seg_start, seg_len, k);
   if (st != PP_OK) return st;
   try {
-    const int32_t group = params->n_q_heads / params->n_kv_heads;
-    std::vector<int32_t> table(pp::prefill_table_ints(params->n_bins, params->capacity, k, group));
+    std::vector<int32_t> table(pp::prefill_table_ints(params->n_bins, params->capacity, k, params->n_q_heads,
+                                                      params->n_kv_heads));
     pp::TableLayout L;
     st = pp::build_prefill_tables(params->n_bins, params->capacity, bin_seg_ptr, seg_start, seg_len, k,
-                                  group, table.data(), table.size(), &L);
+                                  params->n_q_heads, params->n_kv_heads, table.data(), table.size(), &L);
     if (st != PP_OK) return st;
     const pp::WorkItem* items = reinterpret_cast<const pp::WorkItem*>(table.data() + L.items);
     int64_t steps = 0;

@@ -16,6 +16,7 @@ constexpr int kHeaderInts = 16;  // table header, see build_prefill_tables
 constexpr int kHeaderCounter = 10;   // header word the persistent CTAs draw work indices from
 constexpr int kItemInts = 16;
 constexpr int kMaxFold = 8;      // most query heads of one KV head folded into the rows of a query tile
+constexpr int kMaxNormHeads = 512;   // Hq + Hkv up to which the rotation kernels track the norms (shared memory)
 
 // One entry of the attention work list: two query-tile slots sharing one key/value tile stream.
 struct WorkItem {
@@ -37,6 +38,8 @@ struct WorkItem {
 // Offsets (in int32 units) of the blocks inside the prefill table that is built on the host and
 // copied to the device workspace.
 struct TableLayout {
+  int32_t norms = 0;        // [Hkv + Hq] largest |k|^2 per KV head and |q|^2 per query head (float bits), filled by the
+                            // rotation kernels (shared-stream mode); zero in the uploaded table
   int32_t bin_seg_ptr = 0;  // [R+1]
   int32_t bin_used = 0;     // [R]   occupied rows per bin
   int32_t seg_start = 0;    // [k]   bin-local first row of each segment
@@ -50,28 +53,29 @@ struct TableLayout {
 
 int validate_packing(int32_t n_bins, int32_t capacity, const int32_t* bin_seg_ptr,
                      const int32_t* seg_start, const int32_t* seg_len, int32_t k);
-size_t prefill_table_ints(int32_t n_bins, int32_t capacity, int32_t k, int32_t group);
+size_t prefill_table_ints(int32_t n_bins, int32_t capacity, int32_t k, int32_t n_q_heads, int32_t n_kv_heads);
 int32_t max_fold(int32_t group);   // largest power of two <= kMaxFold that divides the GQA group
 int build_prefill_tables(int32_t n_bins, int32_t capacity, const int32_t* bin_seg_ptr,
-                         const int32_t* seg_start, const int32_t* seg_len, int32_t k, int32_t group,
-                         int32_t* out, size_t out_ints, TableLayout* layout);
+                         const int32_t* seg_start, const int32_t* seg_len, int32_t k, int32_t n_q_heads,
+                         int32_t n_kv_heads, int32_t* out, size_t out_ints, TableLayout* layout);
 
 // Records a failed CUDA call for pp_last_cuda_error(); returns PP_ERR_CUDA.
 int note_cuda_error(int cuda_error, const char* what);
 
 // Kernel launchers (device pointers, stream = cudaStream_t as void*). Return a PP_* status.
-// Rotates the n_q_heads heads of q into q_out (may be the same buffer) and the n_kv_heads heads of k
-// in place; pass n_q_heads or n_kv_heads = 0 in `p` to rotate only the other tensor.
-int launch_rope(const pp_attn_params& p, const int32_t* d_table, const TableLayout& L,
-                const void* q, void* q_out, void* k, void* stream);
+// Rotates q and k in place; in the shared-stream mode it also leaves the largest |k|^2 and |q|^2 of every
+// head in the table (L.norms).
+int launch_rope(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, void* q, void* k, void* stream);
 // rope_table: device [D/4][capacity][2] (cos, sin) pairs, or null. When given, q holds the raw
-// queries and the kernel rotates each Q tile in shared memory before use.
+// queries and the kernel rotates each Q tile in shared memory before use. have_norms: a rotation kernel
+// of the same call has filled the norms of the table (of the keys, and without rope_table of the queries).
 int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayout& L,
                      const void* q, const void* k, const void* v, void* o, const void* rope_table,
-                     int32_t* device_status, void* stream);
+                     bool have_norms, int32_t* device_status, void* stream);
 // Fused K rotation + UNPACK; the three offsets locate per-segment arrays inside the table
-// (true length, cache capacity: int32; cache element offset: int64).
-int launch_rope_unpack(const pp_attn_params& p, const int32_t* d_table, const TableLayout& L,
+// (true length, cache capacity: int32; cache element offset: int64). In the shared-stream mode it also leaves
+// the largest |k|^2 of every KV head in the table (L.norms).
+int launch_rope_unpack(const pp_attn_params& p, int32_t* d_table, const TableLayout& L,
                        int32_t off_true_len, int32_t off_cap, int32_t off_cache_off, const void* rope_table,
                        void* k, const void* v, void* k_cache, void* v_cache, void* stream);
 // Fills rope_table for positions 0 .. capacity-1.

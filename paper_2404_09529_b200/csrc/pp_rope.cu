@@ -41,10 +41,32 @@ __device__ __forceinline__ void rotate8(uint4& lo, uint4& hi, const float* cs, c
   }
 }
 
+// Largest |row|^2 per head, for the bound on the scores that the attention kernel uses (shared-stream
+// mode): a (row, head) is held by kLanes neighbouring lanes, each with the sum of squares of its part in
+// `part` (>= 0; all lanes of the warp call). Non-negative floats order like their bit patterns.
+template <int kLanes>
+__device__ __forceinline__ void note_norm(float part, bool real, uint32_t* s_max_of_head) {
+#pragma unroll
+  for (int o = kLanes / 2; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+  if (real && (threadIdx.x & (kLanes - 1)) == 0) atomicMax(s_max_of_head, __float_as_uint(part));
+}
+__device__ __forceinline__ float sum_squares(const uint4& lo, const uint4& hi) {
+  const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+  float a = 0.f, b = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float2 f = bf2_to_f2(w[i]);
+    a = fmaf(f.x, f.x, a);
+    b = fmaf(f.y, f.y, b);
+  }
+  return a + b;
+}
+
+// norms: null, or [Hkv] then [Hq] words that receive the largest |k|^2 / |q|^2 of each head.
 template <int D>
 __global__ void __launch_bounds__(kRopeThreads)
-rope_kernel(const __nv_bfloat16* q, __nv_bfloat16* q_out, __nv_bfloat16* __restrict__ k,
-            const int32_t* __restrict__ table, int32_t off_bin_seg_ptr, int32_t off_bin_used,
+rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32_t* norms,
+            const int32_t* table, int32_t off_bin_seg_ptr, int32_t off_bin_used,
             int32_t off_seg_start, int32_t n_bins, int32_t capacity, int32_t n_q_heads,
             int32_t n_kv_heads, const __grid_constant__ RopeFreq freq) {
   constexpr int kHalf = D / 2;
@@ -52,12 +74,16 @@ rope_kernel(const __nv_bfloat16* q, __nv_bfloat16* q_out, __nv_bfloat16* __restr
   __shared__ int32_t s_pos[kRopeRows];              // restart position, -1 for padding rows
   __shared__ float s_cos[kRopeRows][kHalf];
   __shared__ float s_sin[kRopeRows][kHalf];
+  __shared__ uint32_t s_norm[kMaxNormHeads];        // [Hkv] of k, then [Hq] of q
 
   pdl_launch_dependents();      // the attention kernel may set up while this one runs
   const int64_t row0 = (int64_t)blockIdx.x * kRopeRows;
   const int64_t n_rows = (int64_t)n_bins * capacity;
   const int tid = threadIdx.x;
 
+  const int n_heads = n_q_heads + n_kv_heads;
+  if (norms)
+    for (int h = tid; h < n_heads; h += kRopeThreads) s_norm[h] = 0u;
   if (tid < kRopeRows) {
     const int64_t row = row0 + tid;
     int32_t pos = -1;
@@ -96,25 +122,35 @@ rope_kernel(const __nv_bfloat16* q, __nv_bfloat16* q_out, __nv_bfloat16* __restr
   }
   __syncthreads();
 
-  const int units_per_row = (n_q_heads + n_kv_heads) * kUnitsPerHead;
-  for (int u = tid; u < kRopeRows * units_per_row; u += kRopeThreads) {
+  const int units_per_row = n_heads * kUnitsPerHead;
+  const int units = kRopeRows * units_per_row;
+  for (int u0 = 0; u0 < units; u0 += kRopeThreads) {          // whole warps: the norms are summed across lanes
+    const int u = u0 + tid;
     const int r = u / units_per_row;
     const int w = u - r * units_per_row;
-    const bool in_place = (q_out == q);
-    // padding rows are skipped; position 0 is the identity (copied only when Q goes elsewhere)
-    if (s_pos[r] < 0 || (s_pos[r] == 0 && (in_place || w >= n_q_heads * kUnitsPerHead))) continue;
+    const int32_t pos = u < units ? s_pos[r] : -1;
     const int head = w / kUnitsPerHead;
     const int c = w - head * kUnitsPerHead;
     const int64_t row = row0 + r;
     const bool is_q = head < n_q_heads;
-    const int64_t off = is_q ? (row * n_q_heads + head) * D : (row * n_kv_heads + (head - n_q_heads)) * D;
-    const __nv_bfloat16* src = is_q ? q + off : k + off;
-    __nv_bfloat16* dst = is_q ? q_out + off : k + off;
-    uint4 lo = *reinterpret_cast<const uint4*>(src + c * 8);
-    uint4 hi = *reinterpret_cast<const uint4*>(src + kHalf + c * 8);
-    if (s_pos[r] > 0) rotate8(lo, hi, &s_cos[r][c * 8], &s_sin[r][c * 8]);
-    *reinterpret_cast<uint4*>(dst + c * 8) = lo;
-    *reinterpret_cast<uint4*>(dst + kHalf + c * 8) = hi;
+    float n2 = 0.f;
+    if (pos > 0 || (norms && pos == 0)) {                     // padding rows are skipped, position 0 is the identity
+      __nv_bfloat16* p = is_q ? q + (row * n_q_heads + head) * D : k + (row * n_kv_heads + (head - n_q_heads)) * D;
+      uint4 lo = *reinterpret_cast<const uint4*>(p + c * 8);
+      uint4 hi = *reinterpret_cast<const uint4*>(p + kHalf + c * 8);
+      if (norms) n2 = sum_squares(lo, hi);
+      if (pos > 0) {
+        rotate8(lo, hi, &s_cos[r][c * 8], &s_sin[r][c * 8]);
+        *reinterpret_cast<uint4*>(p + c * 8) = lo;
+        *reinterpret_cast<uint4*>(p + kHalf + c * 8) = hi;
+      }
+    }
+    if (norms) note_norm<kUnitsPerHead>(n2, pos >= 0, s_norm + (is_q ? n_kv_heads + head : head - n_q_heads));
+  }
+  if (norms) {
+    __syncthreads();
+    for (int h = tid; h < n_heads; h += kRopeThreads)
+      if (s_norm[h] > __ldcg(norms + h)) atomicMax(norms + h, s_norm[h]);
   }
 }
 
@@ -154,9 +190,9 @@ constexpr int kRuV = 8;      // 16-byte V copies in flight per thread
 constexpr int kRuK = 2;      // (lower, upper) K pairs in flight per thread
 template <int D, int kRuRows>
 __global__ void __launch_bounds__(kRopeThreads)
-rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v,
+rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, uint32_t* norms,
                    __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
-                   const int32_t* __restrict__ table, int32_t off_bin_seg_ptr, int32_t off_bin_used,
+                   const int32_t* table, int32_t off_bin_seg_ptr, int32_t off_bin_used,
                    int32_t off_seg_start, SegExt ext, const float2* __restrict__ rope_table,
                    int32_t n_bins, int32_t capacity, int32_t n_kv_heads) {
   constexpr int kHalf = D / 2;
@@ -166,11 +202,14 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
   __shared__ int64_t s_dst[kRuRows];              // cache element offset of (head 0, this position); -1: not cached
   __shared__ int64_t s_head_stride[kRuRows];      // cache_cap * D
   __shared__ float4 s_tab[kRuRows][D / 4];          // (cos, sin) of j = 2g, 2g + 1 at each row's position
+  __shared__ uint32_t s_norm[kMaxNormHeads];        // largest |k|^2 of the block's rows, per KV head
 
   pdl_launch_dependents();      // the attention kernel may set up while this one runs
   const int64_t row0 = (int64_t)blockIdx.x * kRuRows;
   const int64_t n_rows = (int64_t)n_bins * capacity;
   const int tid = threadIdx.x;
+  if (norms)
+    for (int h = tid; h < n_kv_heads; h += kRopeThreads) s_norm[h] = 0u;
   if (tid < kRuRows) {
     const int64_t row = row0 + tid;
     int32_t pos = -1;
@@ -230,13 +269,15 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
   __syncthreads();
   // K rows: rotate, write back to the packed tensor and into the cache; two pairs in flight
   const int units_k = n_kv_heads * kPairUnits;
-  for (int u0 = tid; u0 < kRuRows * units_k; u0 += kRuK * kRopeThreads) {
+  for (int base_u = 0; base_u < kRuRows * units_k; base_u += kRuK * kRopeThreads) {   // whole warps (norms)
+    const int u0 = base_u + tid;
     uint4 lo[kRuK], hi[kRuK];
     int rr[kRuK], hh[kRuK], cc[kRuK];
 #pragma unroll
     for (int i = 0; i < kRuK; ++i) {
       const int u = u0 + i * kRopeThreads;
       rr[i] = -1;
+      hh[i] = 0;
       if (u < kRuRows * units_k) {
         const int r = u / units_k, w = u - r * units_k;
         if (s_pos[r] >= 0) {
@@ -249,6 +290,7 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
     }
 #pragma unroll
     for (int i = 0; i < kRuK; ++i) {
+      if (norms) note_norm<kPairUnits>(rr[i] < 0 ? 0.f : sum_squares(lo[i], hi[i]), rr[i] >= 0, s_norm + hh[i]);
       if (rr[i] < 0) continue;
       const int r = rr[i], head = hh[i], c = cc[i];
       const int32_t pos = s_pos[r];
@@ -271,6 +313,18 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
       }
     }
   }
+  if (norms) {
+    __syncthreads();
+    for (int h = tid; h < n_kv_heads; h += kRopeThreads)
+      if (s_norm[h] > __ldcg(norms + h)) atomicMax(norms + h, s_norm[h]);
+  }
+}
+
+// Where the rotation kernels leave the norms: the table's norm words in the shared-stream mode, which uses
+// them; null in the independent mode and where there are more heads than the kernels' shared memory holds.
+uint32_t* norm_words(const pp_attn_params& p, int32_t* d_table, const TableLayout& L) {
+  if (L.independent_slots || p.n_q_heads + p.n_kv_heads > kMaxNormHeads) return nullptr;
+  return reinterpret_cast<uint32_t*>(d_table + L.norms);
 }
 
 RopeFreq make_freq(const pp_attn_params& p) {
@@ -293,7 +347,7 @@ int launch_rope_table(const pp_attn_params& p, void* table, void* stream) {
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope table kernel launch");
 }
 
-int launch_rope_unpack(const pp_attn_params& p, const int32_t* d_table, const TableLayout& L,
+int launch_rope_unpack(const pp_attn_params& p, int32_t* d_table, const TableLayout& L,
                        int32_t off_true_len, int32_t off_cap, int32_t off_cache_off, const void* rope_table,
                        void* k, const void* v, void* k_cache, void* v_cache, void* stream) {
   const int64_t n_rows = (int64_t)p.n_bins * p.capacity;
@@ -305,7 +359,8 @@ int launch_rope_unpack(const pp_attn_params& p, const int32_t* d_table, const Ta
   cudaError_t launch_err = cudaSuccess;
 #define PP_RU_LAUNCH(DD, RR)                                                                                      \
   launch_err = launch_dependent(rope_unpack_kernel<DD, RR>, dim3(grid), dim3(kRopeThreads), 0, s,                 \
-      (__nv_bfloat16*)k, (const __nv_bfloat16*)v, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, d_table,      \
+      (__nv_bfloat16*)k, (const __nv_bfloat16*)v, norm_words(p, d_table, L), (__nv_bfloat16*)k_cache,             \
+      (__nv_bfloat16*)v_cache, (const int32_t*)d_table,                                                           \
       L.bin_seg_ptr, L.bin_used, L.seg_start, ext, (const float2*)rope_table, p.n_bins, p.capacity, p.n_kv_heads)
   if (p.head_dim == 128) {
     if (narrow) PP_RU_LAUNCH(128, kRuRowsNarrow); else PP_RU_LAUNCH(128, kRuRowsWide);
@@ -317,19 +372,18 @@ int launch_rope_unpack(const pp_attn_params& p, const int32_t* d_table, const Ta
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope+unpack kernel launch");
 }
 
-int launch_rope(const pp_attn_params& p, const int32_t* d_table, const TableLayout& L, const void* q,
-                void* q_out, void* k, void* stream) {
+int launch_rope(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, void* q, void* k, void* stream) {
   const RopeFreq freq = make_freq(p);
   const int64_t n_rows = (int64_t)p.n_bins * p.capacity;
   const unsigned grid = (unsigned)((n_rows + kRopeRows - 1) / kRopeRows);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (p.head_dim == 128) {
     rope_kernel<128><<<grid, kRopeThreads, 0, s>>>(
-        (const __nv_bfloat16*)q, (__nv_bfloat16*)q_out, (__nv_bfloat16*)k, d_table, L.bin_seg_ptr, L.bin_used, L.seg_start,
+        (__nv_bfloat16*)q, (__nv_bfloat16*)k, norm_words(p, d_table, L), d_table, L.bin_seg_ptr, L.bin_used, L.seg_start,
         p.n_bins, p.capacity, p.n_q_heads, p.n_kv_heads, freq);
   } else {
     rope_kernel<64><<<grid, kRopeThreads, 0, s>>>(
-        (const __nv_bfloat16*)q, (__nv_bfloat16*)q_out, (__nv_bfloat16*)k, d_table, L.bin_seg_ptr, L.bin_used, L.seg_start,
+        (__nv_bfloat16*)q, (__nv_bfloat16*)k, norm_words(p, d_table, L), d_table, L.bin_seg_ptr, L.bin_used, L.seg_start,
         p.n_bins, p.capacity, p.n_q_heads, p.n_kv_heads, freq);
   }
   const cudaError_t e = cudaGetLastError();
