@@ -1,15 +1,28 @@
 // One generation step over the per-prompt caches that UNPACK produced (Section 7 of the prepacking
 // paper, "prepacking for generation"): the caches are never padded, so the step reads exactly the
-// keys and values every prompt has. Three kernels:
-//   decode_append_kernel     rotates the new token's q and k by its position (= tokens cached so far),
-//                            appends k' and v to the prompt's caches, leaves q' in the workspace
-//   decode_partial_kernel    one CTA per (chunk of 256 or 64 cached keys, KV head): scores, online softmax
-//                            and P V for the query heads of that KV head, partial (m, l, o) out
-//   decode_combine_kernel    merges a prompt's chunks into o
-// HBM-bound: K and V of every cached token are read once.
+// keys and values every prompt has. Two kernels:
+//   decode_kernel            one CTA per (chunk of a prompt's cached keys, KV head): rotates the query heads of
+//                            that KV head by the new token's position (= tokens cached so far), scores, online
+//                            softmax and P V over the chunk; the CTA of a prompt's last chunk also rotates the
+//                            new key, appends k' and v to the caches and attends to them. A prompt of one
+//                            chunk gets its O at once, the others leave (m, l, o) of every chunk.
+//   decode_combine_kernel    merges the chunks of those prompts into O (launched only if there are any)
+//
+// Bound: HBM, K and V of every cached token are read once. The arithmetic therefore runs on the tensor cores
+// through mma.m16n8k16 with the query heads of a KV head as the N = 8 columns (absent ones are zero): with
+// four heads per KV head the dot products of a warp per key row, each summed over 32 lanes by five shuffles,
+// took 541 us for 240 k cached tokens, 3.6 times what their 983 MB take to copy. Fragments are read straight
+// from global memory (no shared memory in between): the order of the contraction index is free as long as
+// both operands use the same, so a thread's 16-byte piece of a K row serves two products, and its 16-byte
+// pieces of four V rows (paired with byte permutes) serve eight. P is split into three bf16 numbers (24 bits
+// of it), so P V is as exact as with P in fp32.
+// Measured, whole step (D = 128): 256 prompts, 240 k cached tokens, 32 / 8 heads 568 -> 177 us (decode_kernel 159 us,
+// 6.2 TB/s, 96 % of the copy peak); 64 prompts, 17.5 k tokens, 32 / 32 heads 77 -> 59 us (54 us); ten prompts, 1009
+// tokens 41 -> 36 us (host-bound; the three kernels and the copy took 17.6 us, these two overlap to ~12).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "pp_internal.h"
@@ -18,259 +31,434 @@ namespace pp {
 namespace {
 
 constexpr int kDecodeThreads = 128;     // 4 warps per CTA
-constexpr int kMaxGroup = 8;            // query heads per KV head supported by the partial kernel
+constexpr int kDecodeWarps = kDecodeThreads / 32;
+constexpr int kMaxGroup = 8;            // query heads per KV head: the N of the tensor-core product
+constexpr int kTileKeys = 16;           // keys per warp and step: the M of the score product
 
-struct DecodeFreq {
+// What the kernels know about a prompt. For up to kInlineMany prompts the entries travel in the kernel's
+// parameters (a launch takes up to 32 KB of them), so that a step needs no table upload, a copy and a gap in
+// the stream in front of it; beyond that they are read from the workspace.
+struct DecodePrompt {
+  int64_t cache_off;                    // elements
+  int32_t length, cap;                  // tokens cached so far, rows of the block
+};
+struct DecodeArgs {
+  const __nv_bfloat16 *q_new, *k_new, *v_new;
+  __nv_bfloat16 *o, *k_cache, *v_cache;
+  float2* part_ml;                      // [chunk][Hq] (m, l), m in scaled log2 units
+  float* part_o;                        // [chunk][Hq][D]
+  const DecodePrompt* prompts;          // [k], chunk_ptr: read where the parameters do not hold them
+  const int32_t* chunk_ptr;             // [k + 1] first chunk of every prompt
+  int32_t n_prompts, n_q_heads, n_kv_heads, group, chunk_keys;
+  float scale_log2;
   double inv_freq[64];                  // theta_j = base^(-2j/D), computed in double on the host
 };
-
-// Offsets (int32 units) inside the uploaded table: chunks[n_chunks][3] = (prompt, first key, keys),
-// chunk_ptr[k + 1], lengths[k], cache_cap[k], cache_off int64[k].
-struct DecodeTable {
-  int32_t chunks, chunk_ptr, lengths, cache_cap, cache_off;
+template <int N>
+struct DecodeInline {
+  DecodePrompt prompts[N];
+  int32_t chunk_ptr[N + 1];
 };
+template <>
+struct DecodeInline<0> {};
+constexpr int kInlineFew = 32, kInlineMany = 512;
+
+template <int N>
+__device__ __forceinline__ int32_t chunk_ptr_at(const DecodeArgs& a, const DecodeInline<N>& in, int i) {
+  if constexpr (N > 0) return in.chunk_ptr[i]; else return __ldg(a.chunk_ptr + i);
+}
+template <int N>
+__device__ __forceinline__ DecodePrompt prompt_at(const DecodeArgs& a, const DecodeInline<N>& in, int i) {
+  if constexpr (N > 0) return in.prompts[i]; else return a.prompts[i];
+}
+
+__device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+// 8 x 8 transpose of 16-bit elements across the warp
+__device__ __forceinline__ uint32_t transpose8x8(uint32_t x) {
+  uint32_t y;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+  return y;
+}
+__device__ __forceinline__ uint4 load16(const __nv_bfloat16* p) {      // read once: do not keep in L1
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ uint32_t word_of(const uint4& v, int i) { return i == 0 ? v.x : i == 1 ? v.y : i == 2 ? v.z : v.w; }
+
+// Fragments of one 16-key step of a warp. Lane = 4 g + t. K: rows g and g + 8, 16-byte pieces t, t + 4, ...
+// of a row. V: rows 2t, 2t + 1, 2t + 8, 2t + 9, the 16-byte piece g of a row (and, at D = 128, piece g + 8).
+template <int D>
+struct StepK { uint4 r[2][D / 32]; };
+template <int D>
+struct StepV { uint4 r[4][D / 64]; };
 
 template <int D>
-__global__ void __launch_bounds__(kDecodeThreads)
-decode_append_kernel(const __nv_bfloat16* __restrict__ q_new, const __nv_bfloat16* __restrict__ k_new,
-                     const __nv_bfloat16* __restrict__ v_new, __nv_bfloat16* __restrict__ q_rot,
-                     __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
-                     const int32_t* __restrict__ table, DecodeTable T, int32_t n_q_heads, int32_t n_kv_heads,
-                     const __grid_constant__ DecodeFreq freq) {
-  constexpr int kHalf = D / 2;
-  __shared__ float s_cos[kHalf], s_sin[kHalf];
-  pdl_launch_dependents();      // the partial kernel may set up while this one runs
-  const int i = blockIdx.x;
-  const int32_t pos = table[T.lengths + i];                      // position of the new token
-  const int64_t cap = table[T.cache_cap + i];
-  const int64_t base = reinterpret_cast<const int64_t*>(table + T.cache_off)[i];
-  if (threadIdx.x < kHalf) {
-    float sn = 0.f, cs = 1.f;
-    if (pos > 0) {      // same reduction as the prefill kernels
-      const double ang = (double)pos * freq.inv_freq[threadIdx.x];
-      const double n = rint(ang * 0.15915494309189535);
-      double red = fma(-n, 6.283185307179586, ang);
-      red = fma(-n, 2.4492935982947064e-16, red);
-      sincosf((float)red, &sn, &cs);
-    }
-    s_cos[threadIdx.x] = cs;
-    s_sin[threadIdx.x] = sn;
+__device__ __forceinline__ void load_k(StepK<D>& f, const __nv_bfloat16* base, int key, int last, int g, int t) {
+#pragma unroll
+  for (int x = 0; x < 2; ++x) {
+    const __nv_bfloat16* p = base + (int64_t)min(key + g + 8 * x, last) * D + 8 * t;   // rows past the chunk: a row of it
+#pragma unroll
+    for (int i = 0; i < D / 32; ++i) f.r[x][i] = load16(p + 32 * i);
   }
-  __syncthreads();
-  // Units of eight (j, j + D/2) pairs: (head, group of eight j) of q, then of k. 16-byte accesses, and
-  // the loads of up to four units are issued before the first store (the compiler cannot prove
-  // that the destinations do not alias the sources, so it would serialise them otherwise).
-  constexpr int kGroups = kHalf / 8;
-  const int n_units = (n_q_heads + n_kv_heads) * kGroups;
-  for (int u0 = threadIdx.x; u0 < n_units; u0 += 4 * kDecodeThreads) {
-    uint4 lo[4], hi[4];
-    __nv_bfloat16* dst[4];
+}
+template <int D>
+__device__ __forceinline__ void load_v(StepV<D>& f, const __nv_bfloat16* base, int key, int last, int g, int t) {
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      const int u = u0 + x * kDecodeThreads;
-      dst[x] = nullptr;
-      if (u < n_units) {
-        const int head = u / kGroups, g = u - head * kGroups;
-        const bool is_k = head >= n_q_heads;
-        const __nv_bfloat16* src = is_k ? k_new + ((int64_t)i * n_kv_heads + (head - n_q_heads)) * D
-                                        : q_new + ((int64_t)i * n_q_heads + head) * D;
-        dst[x] = (is_k ? k_cache + base + ((int64_t)(head - n_q_heads) * cap + pos) * D
-                       : q_rot + ((int64_t)i * n_q_heads + head) * D) + 8 * g;
-        lo[x] = __ldg(reinterpret_cast<const uint4*>(src + 8 * g));
-        hi[x] = __ldg(reinterpret_cast<const uint4*>(src + 8 * g + kHalf));
-      }
-    }
+  for (int x = 0; x < 4; ++x) {
+    const __nv_bfloat16* p = base + (int64_t)min(key + 2 * t + (x & 1) + 8 * (x >> 1), last) * D + 8 * g;
 #pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      if (!dst[x]) continue;
-      const int j0 = (int)((u0 + x * kDecodeThreads) % kGroups) * 8;
-      uint32_t* l32 = reinterpret_cast<uint32_t*>(&lo[x]);
-      uint32_t* h32 = reinterpret_cast<uint32_t*>(&hi[x]);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&l32[e]));
-        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h32[e]));
-        const float c0 = s_cos[j0 + 2 * e], s0 = s_sin[j0 + 2 * e], c1 = s_cos[j0 + 2 * e + 1], s1 = s_sin[j0 + 2 * e + 1];
-        const __nv_bfloat162 lo2 = __floats2bfloat162_rn(__fmaf_rn(a.x, c0, -__fmul_rn(b.x, s0)),
-                                                         __fmaf_rn(a.y, c1, -__fmul_rn(b.y, s1)));
-        const __nv_bfloat162 hi2 = __floats2bfloat162_rn(__fmaf_rn(b.x, c0, __fmul_rn(a.x, s0)),
-                                                         __fmaf_rn(b.y, c1, __fmul_rn(a.y, s1)));
-        l32[e] = *reinterpret_cast<const uint32_t*>(&lo2);
-        h32[e] = *reinterpret_cast<const uint32_t*>(&hi2);
-      }
-      *reinterpret_cast<uint4*>(dst[x]) = lo[x];
-      *reinterpret_cast<uint4*>(dst[x] + kHalf) = hi[x];
-    }
-  }
-  // v is copied as it is
-  for (int u = threadIdx.x; u < n_kv_heads * (D / 8); u += kDecodeThreads) {
-    const int head = u / (D / 8), g = u - head * (D / 8);
-    *reinterpret_cast<uint4*>(v_cache + base + ((int64_t)head * cap + pos) * D + 8 * g) =
-        __ldg(reinterpret_cast<const uint4*>(v_new + ((int64_t)i * n_kv_heads + head) * D + 8 * g));
+    for (int i = 0; i < D / 64; ++i) f.r[x][i] = load16(p + 64 * i);
   }
 }
 
-// partial results: [chunk][query head][D + 2] floats = (m, l, o[D]), m in scaled log2 units.
-// G: compile-time bound on the query heads per KV head (1, 2, 4 or 8), so that a small group does
-// not pay registers for a large one.
-template <int D, int G>
-__global__ void __launch_bounds__(kDecodeThreads)
-decode_partial_kernel(const __nv_bfloat16* __restrict__ q_rot, const __nv_bfloat16* __restrict__ k_cache,
-                      const __nv_bfloat16* __restrict__ v_cache, float* __restrict__ partial,
-                      const int32_t* __restrict__ table, DecodeTable T, int32_t n_q_heads, int32_t n_kv_heads,
-                      int32_t group, float scale_log2) {
-  constexpr int E = D / 32;                       // elements of a row per lane
-  __shared__ float s_m[4][G], s_l[4][G], s_o[4][G][D];
-  const int chunk = blockIdx.x, kvh = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int i = table[T.chunks + 3 * chunk], key0 = table[T.chunks + 3 * chunk + 1], n_keys = table[T.chunks + 3 * chunk + 2];
-  const int64_t cap = table[T.cache_cap + i];
-  const int64_t base = reinterpret_cast<const int64_t*>(table + T.cache_off)[i] + (int64_t)kvh * cap * D;
-  pdl_launch_dependents();      // the combine kernel may set up while this one runs
-  pdl_wait();                   // rotated queries and the appended K / V rows come from the append kernel
-  float q[G][E], acc[G][E], m[G], l[G];
+template <int D>
+struct Softmax {
+  float m[2] = {-INFINITY, -INFINITY};    // running maximum of query heads 2t and 2t + 1 (all lanes of equal t agree)
+  float l[2] = {0.f, 0.f};                // this thread's keys' share of the running sum
+  float acc[D / 16][4];                   // O^T: product j, rows d (see pv), columns = heads 2t, 2t + 1
+};
+
+// Scores of 16 keys against 8 query heads (c: keys g, g + 8 by heads 2t, 2t + 1).
+template <int D>
+__device__ __forceinline__ void scores(float (&c)[4], const StepK<D>& f, const uint4 (&q)[D / 32]) {
+  c[0] = c[1] = c[2] = c[3] = 0.f;
 #pragma unroll
-  for (int h = 0; h < G; ++h) {
-    m[h] = -INFINITY;
-    l[h] = 0.f;
+  for (int i = 0; i < D / 32; ++i) {
+    mma16816(c, f.r[0][i].x, f.r[1][i].x, f.r[0][i].y, f.r[1][i].y, q[i].x, q[i].y);
+    mma16816(c, f.r[0][i].z, f.r[1][i].z, f.r[0][i].w, f.r[1][i].w, q[i].z, q[i].w);
+  }
+}
+
+// Online softmax over the 16 keys (those at or past n_real are hidden); leaves P in c.
+template <int D>
+__device__ __forceinline__ void softmax_step(Softmax<D>& s, float (&c)[4], float scale, int n_real, int g) {
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-      acc[h][e] = 0.f;
-      q[h][e] = (h < group) ? __bfloat162float(q_rot[((int64_t)i * n_q_heads + kvh * group + h) * D + lane * E + e]) : 0.f;
+  for (int x = 0; x < 4; ++x) c[x] = g + 8 * (x >> 1) < n_real ? c[x] * scale : -INFINITY;
+  float mx[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    mx[h] = fmaxf(c[h], c[2 + h]);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) mx[h] = fmaxf(mx[h], __shfl_xor_sync(0xffffffffu, mx[h], o));
+  }
+  if (__any_sync(0xffffffffu, mx[0] > s.m[0] || mx[1] > s.m[1])) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float m_new = fmaxf(s.m[h], mx[h]);          // every step has a real key: finite
+      const float alpha = ex2(s.m[h] - m_new);           // 0 on the first step
+      s.m[h] = m_new;
+      s.l[h] *= alpha;
+#pragma unroll
+      for (int j = 0; j < D / 16; ++j) { s.acc[j][h] *= alpha; s.acc[j][2 + h] *= alpha; }
     }
   }
-  // one 4- or 8-byte load per lane and row; four keys per iteration keep eight loads in flight
-  auto load_row = [&](const __nv_bfloat16* p, float (&out)[E]) {
-    if constexpr (E == 4) {
-      const uint2 u = __ldg(reinterpret_cast<const uint2*>(p));
-      const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
-      const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
-      out[0] = a.x; out[1] = a.y; out[2] = b.x; out[3] = b.y;
-    } else {
-      const uint32_t u = __ldg(reinterpret_cast<const uint32_t*>(p));
-      const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u));
-      out[0] = a.x; out[1] = a.y;
-    }
-  };
-  auto one_key = [&](const float (&kk)[E], const float (&vv)[E]) {
 #pragma unroll
-    for (int h = 0; h < G; ++h) {
-      if (h >= group) break;
-      float s = 0.f;
-#pragma unroll
-      for (int e = 0; e < E; ++e) s = fmaf(q[h][e], kk[e], s);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      s *= scale_log2;
-      const float m_new = fmaxf(m[h], s);
-      const float alpha = exp2f(m[h] - m_new), p = exp2f(s - m_new);      // exp2f(-inf) = 0 on the first key
-      l[h] = l[h] * alpha + p;
-#pragma unroll
-      for (int e = 0; e < E; ++e) acc[h][e] = acc[h][e] * alpha + p * vv[e];
-      m[h] = m_new;
-    }
-  };
-  const __nv_bfloat16* kbase = k_cache + base + (int64_t)key0 * D + lane * E;
-  const __nv_bfloat16* vbase = v_cache + base + (int64_t)key0 * D + lane * E;
-  int t = warp;
-  for (; t + 12 < n_keys; t += 16) {
-    float kx[4][E], vx[4][E];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      load_row(kbase + (int64_t)(t + 4 * u) * D, kx[u]);
-      load_row(vbase + (int64_t)(t + 4 * u) * D, vx[u]);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) one_key(kx[u], vx[u]);
+  for (int h = 0; h < 2; ++h) {
+    c[h] = ex2(c[h] - s.m[h]);
+    c[2 + h] = ex2(c[2 + h] - s.m[h]);
+    s.l[h] += c[h] + c[2 + h];
   }
-  for (; t < n_keys; t += 4) {
-    float k0[E], v0[E];
-    load_row(kbase + (int64_t)t * D, k0);
-    load_row(vbase + (int64_t)t * D, v0);
-    one_key(k0, v0);
+}
+
+// O^T += V^T P. Product j: row g is d = 8g + j, row g + 8 is d = 64 + 8g + j (D = 128) or 8g + 4 + j (D = 64).
+template <int D>
+__device__ __forceinline__ void pv(Softmax<D>& s, const StepV<D>& f, const float (&p)[4]) {
+  uint32_t b[3][2];
+  float r[4] = {p[0], p[1], p[2], p[3]};
+#pragma unroll
+  for (int part = 0; part < 3; ++part)
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+      const __nv_bfloat162 v = __floats2bfloat162_rn(r[2 * x], r[2 * x + 1]);
+      b[part][x] = transpose8x8(*reinterpret_cast<const uint32_t*>(&v));
+      const float2 back = __bfloat1622float2(v);
+      r[2 * x] -= back.x;
+      r[2 * x + 1] -= back.y;
+    }
+#pragma unroll
+  for (int j = 0; j < D / 16; ++j) {
+    uint32_t a[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {      // a0: row g, keys 2t, 2t + 1; a1: row g + 8; a2, a3: the same for keys 2t + 8, 2t + 9
+      const int e = (D == 128) ? j : j + 4 * (x & 1), piece = (D == 128) ? (x & 1) : 0;
+      const uint32_t k0 = word_of(f.r[2 * (x >> 1)][piece], e >> 1), k1 = word_of(f.r[2 * (x >> 1) + 1][piece], e >> 1);
+      a[x] = __byte_perm(k0, k1, (e & 1) ? 0x7632 : 0x5410);
+    }
+#pragma unroll
+    for (int part = 2; part >= 0; --part) mma16816(s.acc[j], a[0], a[1], a[2], a[3], b[part][0], b[part][1]);
   }
-  // merge the four warps
-#pragma unroll
-  for (int h = 0; h < G; ++h) {
-    if (h >= group) break;
-    if (lane == 0) { s_m[warp][h] = m[h]; s_l[warp][h] = l[h]; }
-#pragma unroll
-    for (int e = 0; e < E; ++e) s_o[warp][h][lane * E + e] = acc[h][e];
+}
+
+template <int D, int N>
+__global__ void __launch_bounds__(kDecodeThreads, D == 128 ? 3 : 4)
+decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeInline<N> in) {
+  constexpr int kHalf = D / 2;
+  __shared__ float s_cos[kHalf], s_sin[kHalf];
+  __shared__ __align__(16) __nv_bfloat16 s_q[kMaxGroup + 1][D];       // rotated query heads, then the rotated new key
+  __shared__ float s_m[kDecodeWarps][kMaxGroup], s_l[kDecodeWarps][kMaxGroup];
+  __shared__ float s_o[kDecodeWarps][kMaxGroup][D];
+  const int chunk = blockIdx.x, kvh = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = lane >> 2, t = lane & 3;
+  pdl_launch_dependents();              // the combine kernel may set up while this one runs
+  int lo = 0, hi = a.n_prompts - 1;     // last prompt whose first chunk is <= chunk
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (chunk_ptr_at(a, in, mid) <= chunk) lo = mid; else hi = mid - 1;
+  }
+  const int i = lo;
+  const int c0 = chunk_ptr_at(a, in, i), n_chunks = chunk_ptr_at(a, in, i + 1) - c0;
+  const DecodePrompt pr = prompt_at(a, in, i);
+  const int key0 = (chunk - c0) * a.chunk_keys, key_end = min(key0 + a.chunk_keys, pr.length);
+  const bool last_chunk = chunk - c0 == n_chunks - 1;
+  const int64_t base = pr.cache_off + (int64_t)kvh * pr.cap * D;
+  const __nv_bfloat16 *kb = a.k_cache + base, *vb = a.v_cache + base;
+
+  // the first step's K and V are on their way while the queries are rotated
+  StepK<D> fk;
+  StepV<D> fv;
+  int key = key0 + kTileKeys * warp;
+  if (key < key_end) {
+    load_k<D>(fk, kb, key, key_end - 1, g, t);
+    load_v<D>(fv, vb, key, key_end - 1, g, t);
+  }
+  if (tid < kHalf) {      // the position is >= 1; same reduction as the prefill kernels
+    const double ang = (double)pr.length * a.inv_freq[tid];
+    const double n = rint(ang * 0.15915494309189535);
+    double red = fma(-n, 6.283185307179586, ang);
+    red = fma(-n, 2.4492935982947064e-16, red);
+    float sn, cs;
+    sincosf((float)red, &sn, &cs);
+    s_cos[tid] = cs;
+    s_sin[tid] = sn;
   }
   __syncthreads();
-  for (int u = threadIdx.x; u < group * D; u += kDecodeThreads) {
+  // heads of the group, zeros for the absent ones, and the new key; four (j, j + D/2) pairs at a time
+  for (int u = tid; u < (kMaxGroup + 1) * (kHalf / 4); u += kDecodeThreads) {
+    const int h = u / (kHalf / 4), j = 4 * (u - h * (kHalf / 4));
+    uint2 lo2 = make_uint2(0u, 0u), hi2 = make_uint2(0u, 0u);
+    if (h < a.group || (h == kMaxGroup && last_chunk)) {
+      const __nv_bfloat16* src = h == kMaxGroup ? a.k_new + ((int64_t)i * a.n_kv_heads + kvh) * D
+                                                : a.q_new + ((int64_t)i * a.n_q_heads + kvh * a.group + h) * D;
+      lo2 = __ldg(reinterpret_cast<const uint2*>(src + j));
+      hi2 = __ldg(reinterpret_cast<const uint2*>(src + j + kHalf));
+      uint32_t* l32 = reinterpret_cast<uint32_t*>(&lo2);
+      uint32_t* h32 = reinterpret_cast<uint32_t*>(&hi2);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&l32[e]));
+        const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h32[e]));
+        const float ca = s_cos[j + 2 * e], sa = s_sin[j + 2 * e], cb = s_cos[j + 2 * e + 1], sb = s_sin[j + 2 * e + 1];
+        const __nv_bfloat162 rl = __floats2bfloat162_rn(__fmaf_rn(x.x, ca, -__fmul_rn(y.x, sa)), __fmaf_rn(x.y, cb, -__fmul_rn(y.y, sb)));
+        const __nv_bfloat162 rh = __floats2bfloat162_rn(__fmaf_rn(y.x, ca, __fmul_rn(x.x, sa)), __fmaf_rn(y.y, cb, __fmul_rn(x.y, sb)));
+        l32[e] = *reinterpret_cast<const uint32_t*>(&rl);
+        h32[e] = *reinterpret_cast<const uint32_t*>(&rh);
+      }
+    }
+    *reinterpret_cast<uint2*>(&s_q[h][j]) = lo2;
+    *reinterpret_cast<uint2*>(&s_q[h][j + kHalf]) = hi2;
+  }
+  __syncthreads();
+  uint4 q[D / 32];        // head g, the pieces of a row that this thread's K pieces meet
+#pragma unroll
+  for (int x = 0; x < D / 32; ++x) q[x] = *reinterpret_cast<const uint4*>(&s_q[g][8 * t + 32 * x]);
+
+  Softmax<D> s;
+#pragma unroll
+  for (int j = 0; j < D / 16; ++j)
+#pragma unroll
+    for (int x = 0; x < 4; ++x) s.acc[j][x] = 0.f;
+  float c[4];
+  // K of the next 16 keys is loaded as soon as the scores of these are there, V after its product, so a warp
+  // has 4 to 8 KB in flight (D = 128), three CTAs of four warps per SM 48 to 96 KB.
+  while (key < key_end) {
+    scores<D>(c, fk, q);
+    const int next = key + kTileKeys * kDecodeWarps;
+    if (next < key_end) load_k<D>(fk, kb, next, key_end - 1, g, t);
+    softmax_step<D>(s, c, a.scale_log2, key_end - key, g);
+    pv<D>(s, fv, c);
+    if (next < key_end) load_v<D>(fv, vb, next, key_end - 1, g, t);
+    key = next;
+  }
+  if (last_chunk && warp == 0) {        // the new token, as a step with one real key
+    const __nv_bfloat16* vn = a.v_new + ((int64_t)i * a.n_kv_heads + kvh) * D;
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+      for (int y = 0; y < D / 32; ++y)
+        fk.r[x][y] = x == 0 && g == 0 ? *reinterpret_cast<const uint4*>(&s_q[kMaxGroup][8 * t + 32 * y]) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+      for (int y = 0; y < D / 64; ++y)
+        fv.r[x][y] = x == 0 && t == 0 ? __ldg(reinterpret_cast<const uint4*>(vn + 8 * g + 64 * y)) : make_uint4(0u, 0u, 0u, 0u);
+    scores<D>(c, fk, q);
+    softmax_step<D>(s, c, a.scale_log2, 1, g);
+    pv<D>(s, fv, c);
+    // and its rows of the caches
+    const int64_t row = base + (int64_t)pr.length * D;
+    if (lane < D / 8) {
+      *reinterpret_cast<uint4*>(a.k_cache + row + 8 * lane) = *reinterpret_cast<const uint4*>(&s_q[kMaxGroup][8 * lane]);
+      *reinterpret_cast<uint4*>(a.v_cache + row + 8 * lane) = __ldg(reinterpret_cast<const uint4*>(vn + 8 * lane));
+    }
+  }
+  // merge the four warps (one without keys has m = -inf, l = 0)
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float l = s.l[h];
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    const int head = 2 * t + h;
+    if (head < a.group) {
+      if (g == 0) { s_m[warp][head] = s.m[h]; s_l[warp][head] = l; }
+#pragma unroll
+      for (int j = 0; j < D / 16; ++j) {
+        s_o[warp][head][8 * g + j] = s.acc[j][h];
+        s_o[warp][head][(D == 128 ? 64 + 8 * g : 8 * g + 4) + j] = s.acc[j][2 + h];
+      }
+    }
+  }
+  __syncthreads();
+  for (int u = tid; u < a.group * D; u += kDecodeThreads) {
     const int h = u / D, d = u - h * D;
-    float mm = -INFINITY;
-    for (int w = 0; w < 4; ++w) mm = fmaxf(mm, s_m[w][h]);
+    float mm = s_m[0][h];
+#pragma unroll
+    for (int w = 1; w < kDecodeWarps; ++w) mm = fmaxf(mm, s_m[w][h]);
     float ll = 0.f, oo = 0.f;
-    for (int w = 0; w < 4; ++w) {
-      const float f = (s_m[w][h] == -INFINITY) ? 0.f : exp2f(s_m[w][h] - mm);
+#pragma unroll
+    for (int w = 0; w < kDecodeWarps; ++w) {
+      const float f = ex2(s_m[w][h] - mm);
       ll += s_l[w][h] * f;
       oo += s_o[w][h][d] * f;
     }
-    float* out = partial + ((int64_t)chunk * n_q_heads + kvh * group + h) * (D + 2);
-    if (d == 0) { out[0] = mm; out[1] = ll; }
-    out[2 + d] = oo;
+    const int head = kvh * a.group + h;
+    if (n_chunks == 1) {
+      a.o[((int64_t)i * a.n_q_heads + head) * D + d] = __float2bfloat16_rn(oo / ll);
+    } else {
+      const int64_t at = (int64_t)chunk * a.n_q_heads + head;
+      if (d == 0) a.part_ml[at] = make_float2(mm, ll);
+      a.part_o[at * D + d] = oo;
+    }
   }
 }
 
-template <int D>
-__global__ void __launch_bounds__(D)
-decode_combine_kernel(const float* __restrict__ partial, __nv_bfloat16* __restrict__ o,
-                      const int32_t* __restrict__ table, DecodeTable T, int32_t n_q_heads) {
-  const int i = blockIdx.x, head = blockIdx.y, d = threadIdx.x;
-  const int c0 = table[T.chunk_ptr + i], c1 = table[T.chunk_ptr + i + 1];
-  pdl_wait();                   // the partial results come from the kernel before this one
+// One warp per (prompt, query head); prompts of one chunk are done already.
+template <int D, int N>
+__global__ void __launch_bounds__(kDecodeThreads)
+decode_combine_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeInline<N> in) {
+  constexpr int E = D / 32;             // consecutive elements per lane
+  const int i = blockIdx.x, head = blockIdx.y * kDecodeWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  const int c0 = chunk_ptr_at(a, in, i), c1 = chunk_ptr_at(a, in, i + 1);
+  if (c1 - c0 < 2 || head >= a.n_q_heads) return;
+  pdl_wait();                           // the partial results come from the kernel before this one
   float mm = -INFINITY;
-  for (int c = c0; c < c1; ++c) mm = fmaxf(mm, partial[((int64_t)c * n_q_heads + head) * (D + 2)]);
-  float ll = 0.f, oo = 0.f;
+  for (int c = c0 + lane; c < c1; c += 32) mm = fmaxf(mm, a.part_ml[(int64_t)c * a.n_q_heads + head].x);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+  float ll = 0.f, oo[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) oo[e] = 0.f;
+#pragma unroll 4
   for (int c = c0; c < c1; ++c) {
-    const float* p = partial + ((int64_t)c * n_q_heads + head) * (D + 2);
-    const float f = exp2f(p[0] - mm);
-    ll += p[1] * f;
-    oo += p[2 + d] * f;
+    const int64_t at = (int64_t)c * a.n_q_heads + head;
+    const float2 ml = a.part_ml[at];
+    const float f = ex2(ml.x - mm);
+    ll += ml.y * f;
+    float p[E];
+    if constexpr (E == 4) {
+      const float4 x = *reinterpret_cast<const float4*>(a.part_o + at * D + E * lane);
+      p[0] = x.x; p[1] = x.y; p[2] = x.z; p[3] = x.w;
+    } else {
+      const float2 x = *reinterpret_cast<const float2*>(a.part_o + at * D + E * lane);
+      p[0] = x.x; p[1] = x.y;
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e) oo[e] += p[e] * f;
   }
-  o[((int64_t)i * n_q_heads + head) * D + d] = __float2bfloat16_rn(oo / ll);
+  uint32_t r[E / 2];
+#pragma unroll
+  for (int e = 0; e < E / 2; ++e) {
+    const __nv_bfloat162 x = __floats2bfloat162_rn(oo[2 * e] / ll, oo[2 * e + 1] / ll);
+    r[e] = *reinterpret_cast<const uint32_t*>(&x);
+  }
+  __nv_bfloat16* dst = a.o + ((int64_t)i * a.n_q_heads + head) * D + E * lane;
+  if constexpr (E == 4) *reinterpret_cast<uint2*>(dst) = make_uint2(r[0], r[1]);
+  else *reinterpret_cast<uint32_t*>(dst) = r[0];
 }
 
-// Keys per chunk: 256 when that already gives every SM several CTAs, else 64, so that a small batch
-// (a few prompts, one of them long) is spread over more CTAs and each warp's chain of dependent row
-// loads is a quarter as long.
-constexpr int kChunkKeysLarge = 256, kChunkKeysSmall = 64;
-constexpr int64_t kChunkCtasWanted = 148 * 8;
-
-int64_t count_chunks(const int32_t* lengths, int32_t k, int chunk_keys) {
-  int64_t n = 0;
-  for (int32_t i = 0; i < k; ++i) n += ((int64_t)lengths[i] + 1 + chunk_keys - 1) / chunk_keys;
-  return n;
-}
-size_t up4(size_t x) { return (x + 3) & ~size_t(3); }
+// Keys per chunk. Enough (chunk, KV head) CTAs for about four rounds of the 3 x 148 that run at once, so that
+// the last round is a small part of the whole; at least one 16-key step for each of the four warps, at most
+// 512 keys (a CTA's set-up is then a few per cent of its loads), and more only where a very long prompt would
+// otherwise be cut into more pieces than one warp merges quickly.
+constexpr int64_t kChunkCtasWanted = 148 * 3 * 4;
+constexpr int kMostChunksPerPrompt = 64;
 
 struct DecodeLayout {
-  DecodeTable T;
-  size_t table_ints, q_rot_bytes_off, partial_bytes_off, total_bytes;
+  size_t chunk_ptr_off, table_bytes;    // table: prompts, chunk_ptr (uploaded where they do not fit the parameters)
+  size_t ml_off, o_off, total_bytes;
   int64_t n_chunks;
-  int chunk_keys;
+  int32_t chunk_keys;
 };
 DecodeLayout decode_layout(const pp_attn_params& p, const int32_t* lengths, int32_t k) {
   DecodeLayout L;
-  L.chunk_keys = kChunkKeysLarge;
-  L.n_chunks = count_chunks(lengths, k, L.chunk_keys);
-  if (L.n_chunks * p.n_kv_heads < kChunkCtasWanted) {
-    L.chunk_keys = kChunkKeysSmall;
-    L.n_chunks = count_chunks(lengths, k, L.chunk_keys);
+  int64_t total = 0;
+  int32_t longest = 0;
+  for (int32_t i = 0; i < k; ++i) {
+    total += lengths[i];
+    longest = std::max(longest, lengths[i]);
   }
-  size_t off = 0;
-  L.T.chunks = (int32_t)off; off += up4(3 * (size_t)L.n_chunks);
-  L.T.chunk_ptr = (int32_t)off; off += up4((size_t)k + 1);
-  L.T.lengths = (int32_t)off; off += up4((size_t)k);
-  L.T.cache_cap = (int32_t)off; off += up4((size_t)k);
-  L.T.cache_off = (int32_t)off; off += 2 * (size_t)k;
-  L.table_ints = off;
-  L.q_rot_bytes_off = (off * 4 + 255) & ~size_t(255);
-  L.partial_bytes_off = (L.q_rot_bytes_off + (size_t)k * p.n_q_heads * p.head_dim * 2 + 255) & ~size_t(255);
-  L.total_bytes = L.partial_bytes_off + (size_t)L.n_chunks * p.n_q_heads * (p.head_dim + 2) * sizeof(float);
+  const int64_t unit = kTileKeys * kDecodeWarps;
+  int64_t keys = std::min<int64_t>(std::max<int64_t>(total * p.n_kv_heads / kChunkCtasWanted, 1), 512);
+  keys = std::max<int64_t>(keys, ((int64_t)longest + kMostChunksPerPrompt - 1) / kMostChunksPerPrompt);
+  L.chunk_keys = (int32_t)((keys + unit - 1) / unit * unit);
+  L.n_chunks = 0;
+  for (int32_t i = 0; i < k; ++i) L.n_chunks += ((int64_t)lengths[i] + L.chunk_keys - 1) / L.chunk_keys;
+  auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
+  L.chunk_ptr_off = (size_t)k * sizeof(DecodePrompt);
+  L.table_bytes = L.chunk_ptr_off + ((size_t)k + 1) * sizeof(int32_t);
+  L.ml_off = up(L.table_bytes);
+  L.o_off = up(L.ml_off + (size_t)L.n_chunks * p.n_q_heads * sizeof(float2));
+  L.total_bytes = L.o_off + (size_t)L.n_chunks * p.n_q_heads * p.head_dim * sizeof(float);
   return L;
+}
+
+void fill_table(const DecodeLayout& L, const int32_t* lengths, int32_t k, const int64_t* cache_off,
+                const int32_t* cache_cap, DecodePrompt* prompts, int32_t* chunk_ptr) {
+  int32_t c = 0;
+  for (int32_t i = 0; i < k; ++i) {
+    prompts[i] = DecodePrompt{cache_off[i], lengths[i], cache_cap[i]};
+    chunk_ptr[i] = c;
+    c += (int32_t)(((int64_t)lengths[i] + L.chunk_keys - 1) / L.chunk_keys);
+  }
+  chunk_ptr[k] = c;
+}
+
+template <int D, int N>
+cudaError_t launch_decode(const DecodeArgs& a, const DecodeInline<N>& in, const DecodeLayout& L, cudaStream_t s) {
+  decode_kernel<D, N><<<dim3((unsigned)L.n_chunks, (unsigned)a.n_kv_heads), kDecodeThreads, 0, s>>>(a, in);
+  if (L.n_chunks == a.n_prompts) return cudaGetLastError();       // one chunk each: O is complete
+  const dim3 grid((unsigned)a.n_prompts, (unsigned)((a.n_q_heads + kDecodeWarps - 1) / kDecodeWarps));
+  const cudaError_t e = launch_dependent(decode_combine_kernel<D, N>, grid, dim3(kDecodeThreads), 0, s, a, in);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+template <int N>
+cudaError_t launch_decode_d(int head_dim, const DecodeArgs& a, const DecodeInline<N>& in, const DecodeLayout& L, cudaStream_t s) {
+  return head_dim == 128 ? launch_decode<128, N>(a, in, L, s) : launch_decode<64, N>(a, in, L, s);
+}
+template <int N>
+cudaError_t launch_decode_inline(int head_dim, const DecodeArgs& a, const DecodeLayout& L, const int32_t* lengths, int32_t k,
+                                 const int64_t* cache_off, const int32_t* cache_cap, cudaStream_t s) {
+  DecodeInline<N> in;
+  fill_table(L, lengths, k, cache_off, cache_cap, in.prompts, in.chunk_ptr);
+  return launch_decode_d(head_dim, a, in, L, s);
 }
 
 int check_decode_params(const pp_attn_params* p) {
@@ -314,53 +502,41 @@ extern "C" int pp_decode_step(const pp_attn_params* params, const int32_t* lengt
   const pp::DecodeLayout L = pp::decode_layout(*params, lengths, k);
   if (L.n_chunks > INT32_MAX / 4) return PP_ERR_UNSUPPORTED;
   if (workspace_bytes < L.total_bytes) return PP_ERR_BUFFER_TOO_SMALL;
-  int32_t* h = static_cast<int32_t*>(host_workspace);
-  int64_t* h_off = reinterpret_cast<int64_t*>(h + L.T.cache_off);
-  int32_t c = 0;
-  for (int32_t i = 0; i < k; ++i) {
-    h[L.T.chunk_ptr + i] = c;
-    const int32_t n = lengths[i] + 1;                     // the new token is attended too
-    for (int32_t key0 = 0; key0 < n; key0 += L.chunk_keys, ++c) {
-      h[L.T.chunks + 3 * c] = i;
-      h[L.T.chunks + 3 * c + 1] = key0;
-      h[L.T.chunks + 3 * c + 2] = n - key0 < L.chunk_keys ? n - key0 : L.chunk_keys;
-    }
-    h[L.T.lengths + i] = lengths[i];
-    h[L.T.cache_cap + i] = cache_cap[i];
-    h_off[i] = cache_off[i];
-  }
-  h[L.T.chunk_ptr + k] = c;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaMemcpyAsync(workspace, host_workspace, L.table_ints * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return pp::note_cuda_error((int)e, "decode table upload");
-  const int32_t* d_table = static_cast<const int32_t*>(workspace);
-  __nv_bfloat16* q_rot = reinterpret_cast<__nv_bfloat16*>(static_cast<char*>(workspace) + L.q_rot_bytes_off);
-  float* partial = reinterpret_cast<float*>(static_cast<char*>(workspace) + L.partial_bytes_off);
-  pp::DecodeFreq freq;
+  char* ws = static_cast<char*>(workspace);
+  pp::DecodeArgs a;
+  a.q_new = static_cast<const __nv_bfloat16*>(q_new);
+  a.k_new = static_cast<const __nv_bfloat16*>(k_new);
+  a.v_new = static_cast<const __nv_bfloat16*>(v_new);
+  a.o = static_cast<__nv_bfloat16*>(o);
+  a.k_cache = static_cast<__nv_bfloat16*>(k_cache);
+  a.v_cache = static_cast<__nv_bfloat16*>(v_cache);
+  a.part_ml = reinterpret_cast<float2*>(ws + L.ml_off);
+  a.part_o = reinterpret_cast<float*>(ws + L.o_off);
+  a.prompts = reinterpret_cast<const pp::DecodePrompt*>(ws);
+  a.chunk_ptr = reinterpret_cast<const int32_t*>(ws + L.chunk_ptr_off);
+  a.n_prompts = k;
+  a.n_q_heads = params->n_q_heads;
+  a.n_kv_heads = params->n_kv_heads;
+  a.group = params->n_q_heads / params->n_kv_heads;
+  a.chunk_keys = L.chunk_keys;
+  const float scale = params->softmax_scale > 0.f ? params->softmax_scale : 1.0f / sqrtf((float)params->head_dim);
+  a.scale_log2 = scale * 1.4426950408889634f;
   const int half = params->head_dim / 2;
   for (int j = 0; j < 64; ++j)
-    freq.inv_freq[j] = j < half ? pow((double)params->rope_base, -2.0 * j / (double)params->head_dim) : 0.0;
-  const float scale = params->softmax_scale > 0.f ? params->softmax_scale : 1.0f / sqrtf((float)params->head_dim);
-  const float scale_log2 = scale * 1.4426950408889634f;
-  const int group = params->n_q_heads / params->n_kv_heads;
-  const dim3 grid_p((unsigned)L.n_chunks, (unsigned)params->n_kv_heads), grid_c((unsigned)k, (unsigned)params->n_q_heads);
-  cudaError_t le = cudaSuccess;
-#define PP_DECODE_PARTIAL(DD, GG)                                                                                \
-  le = pp::launch_dependent(pp::decode_partial_kernel<DD, GG>, grid_p, dim3(pp::kDecodeThreads), 0, s,           \
-      (const __nv_bfloat16*)q_rot, (const __nv_bfloat16*)k_cache, (const __nv_bfloat16*)v_cache, partial, d_table, L.T, \
-      params->n_q_heads, params->n_kv_heads, group, scale_log2)
-#define PP_DECODE_LAUNCH(DD)                                                                                     \
-  pp::decode_append_kernel<DD><<<k, pp::kDecodeThreads, 0, s>>>(                                                 \
-      (const __nv_bfloat16*)q_new, (const __nv_bfloat16*)k_new, (const __nv_bfloat16*)v_new, q_rot,              \
-      (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, d_table, L.T, params->n_q_heads, params->n_kv_heads, freq); \
-  if (group == 1) PP_DECODE_PARTIAL(DD, 1); else if (group == 2) PP_DECODE_PARTIAL(DD, 2);                       \
-  else if (group <= 4) PP_DECODE_PARTIAL(DD, 4); else PP_DECODE_PARTIAL(DD, 8);                                  \
-  if (le == cudaSuccess)                                                                                         \
-    le = pp::launch_dependent(pp::decode_combine_kernel<DD>, grid_c, dim3(DD), 0, s, (const float*)partial,      \
-                              (__nv_bfloat16*)o, d_table, L.T, params->n_q_heads)
-  if (params->head_dim == 128) { PP_DECODE_LAUNCH(128); } else { PP_DECODE_LAUNCH(64); }
-#undef PP_DECODE_LAUNCH
-#undef PP_DECODE_PARTIAL
-  e = le != cudaSuccess ? le : cudaGetLastError();
+    a.inv_freq[j] = j < half ? pow((double)params->rope_base, -2.0 * j / (double)params->head_dim) : 0.0;
+  cudaError_t e;
+  if (k <= pp::kInlineFew) {
+    e = pp::launch_decode_inline<pp::kInlineFew>(params->head_dim, a, L, lengths, k, cache_off, cache_cap, s);
+  } else if (k <= pp::kInlineMany) {
+    e = pp::launch_decode_inline<pp::kInlineMany>(params->head_dim, a, L, lengths, k, cache_off, cache_cap, s);
+  } else {
+    char* h = static_cast<char*>(host_workspace);
+    pp::fill_table(L, lengths, k, cache_off, cache_cap, reinterpret_cast<pp::DecodePrompt*>(h),
+                   reinterpret_cast<int32_t*>(h + L.chunk_ptr_off));
+    e = cudaMemcpyAsync(workspace, host_workspace, L.table_bytes, cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return pp::note_cuda_error((int)e, "decode table upload");
+    e = pp::launch_decode_d(params->head_dim, a, pp::DecodeInline<0>{}, L, s);
+  }
   return e == cudaSuccess ? PP_OK : pp::note_cuda_error((int)e, "decode kernel launch");
 }

@@ -77,3 +77,38 @@ def test_decode_argument_checks():
     with pytest.raises(pp.PrepackError):       # workspace too small
         pp.pp_decode_step(params, lengths, x, x, x, x.clone(), cache, cache.clone(), off, np.array([8, 8], np.int32),
                           ws, host, 16)
+
+
+@pytest.mark.parametrize("lengths,hq,hkv,d", [
+    # every remainder of a 16-key step and of a 64-key chunk, in one chunk and in several; group 8
+    (np.array([1, 2, 15, 16, 17, 31, 32, 33, 47, 48, 49, 63, 64, 65, 127, 128, 129, 191, 192, 193], np.int32), 16, 2, 128),
+    (np.array([1, 15, 16, 17, 63, 64, 65, 129, 255, 257], np.int32), 6, 2, 64),          # group 3: absent head columns
+    (np.array([5000, 3], np.int32), 2, 1, 128),                                          # most chunks per prompt
+    (np.arange(600, dtype=np.int32) % 37 + 1, 2, 2, 64),                                 # table uploaded, not in the parameters
+    (np.array([70] * 40 + [200], np.int32), 4, 1, 128),                                  # the larger parameter block
+    (np.array([3000] * 3 + [512, 513], np.int32), 128, 32, 64),                          # chunks of 512 keys
+])
+def test_decode_chunks_and_tables(lengths, hq, hkv, d):
+    """The generation step on caches of random contents at the edges of its steps, chunks and table forms,
+    spare rows untouched."""
+    from paper_2404_09529_b200.runner import DecodeBatch
+    dec = DecodeBatch(lengths, hq, hkv, d, 10000.0, room=2)
+    g = torch.Generator().manual_seed(int(lengths.sum()))
+    for pool in (dec.k_cache, dec.v_cache):
+        pool.copy_(torch.randn(pool.shape, generator=g).to(torch.bfloat16))
+    before = [tuple(c.clone() for c in dec.caches(i)) for i in range(dec.k)]
+    qn, kn, vn = (torch.randn(dec.k, h, d, generator=g).to(torch.bfloat16) for h in (hq, hkv, hkv))
+    got = to64(dec.step(qn.cuda(), kn.cuda(), vn.cuda()))
+    errs = []
+    for i in range(dec.k):
+        l = int(lengths[i])
+        kc, vc = (to64(c[:, :l]) for c in before[i])
+        o_ref, k_ref, v_ref = orc.decode_step(to64(qn[i]), to64(kn[i]), to64(vn[i]), kc, vc, 10000.0)
+        errs.append(np.abs(got[i] - o_ref).ravel())
+        ck, cv = dec.caches(i)
+        assert np.max(np.abs(to64(ck[:, l]) - k_ref[:, l])) <= MAX_ABS_TOL
+        assert torch.equal(cv[:, l].cpu(), vn[i])
+        for now, was in zip((ck, cv), before[i]):
+            assert torch.equal(now[:, :l], was[:, :l]) and torch.equal(now[:, l + 1:], was[:, l + 1:])
+    e = np.concatenate(errs)
+    assert e.max() <= MAX_ABS_TOL and e.mean() <= MEAN_ABS_TOL, (e.max(), e.mean())
