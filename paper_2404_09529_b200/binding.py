@@ -1,5 +1,6 @@
-"""ctypes binding of libprepack_b200.so. Argument marshalling only: no arithmetic of the
-method lives here. Function names and argument order follow ``include/pp.h``."""
+"""Binding of libprepack_b200.so. Argument marshalling only: no arithmetic of the method lives here.
+Function names and argument order follow ``include/pp.h``. The calls that a program makes once per step
+go through the compiled module ``_native``, the others through ctypes."""
 from __future__ import annotations
 
 import ctypes
@@ -83,6 +84,22 @@ def load_library():
     return lib
 
 
+_native = None
+
+
+def _load_native():
+    """The compiled marshalling of the per-step calls (built together with the library)."""
+    global _native
+    load_library()
+    try:
+        from . import _native as module
+    except ImportError as e:
+        raise ImportError(f"paper_2404_09529_b200._native cannot be loaded ({e}): build it with "
+                          "`python -m paper_2404_09529_b200.build`") from e
+    _native = module
+    return module
+
+
 def _i32(a) -> np.ndarray:
     return np.ascontiguousarray(np.asarray(a, dtype=np.int32))
 
@@ -151,16 +168,10 @@ class Packing:
 
 
 def pp_pack(lengths, capacity: int = 0) -> Packing:
-    lib = load_library()
-    l = _i32(lengths)
-    k = int(l.shape[0])
-    n_bins, cap = ctypes.c_int32(0), ctypes.c_int32(0)
-    ptr = np.zeros(k + 1, np.int32)
-    outs = [np.zeros(max(k, 1), np.int32) for _ in range(5)]
-    st = lib.pp_pack(_p32(l), k, capacity, ctypes.byref(n_bins), ctypes.byref(cap), _p32(ptr),
-                     *[_p32(o) for o in outs])
-    _check(st, "pp_pack")
-    return Packing(n_bins.value, cap.value, ptr[:n_bins.value + 1].copy(), *[o[:k] for o in outs])
+    st, n_bins, cap, *arrays = (_native or _load_native()).pack(lengths, capacity)
+    if st != 0:
+        raise PrepackError(st, "pp_pack")
+    return Packing(n_bins, cap, *arrays)
 
 
 def pp_fill_position_ids(pack: Packing):
@@ -202,30 +213,20 @@ def pp_prefill_fused_host_bytes(params: AttnParams, k: int) -> int:
 def pp_prefill_fused(params: AttnParams, pack: Packing, lengths, q, k, v, o, k_cache, v_cache, cache_off,
                      cache_cap, workspace, host_workspace, workspace_bytes: int, device_status=None,
                      stream: int = 0) -> None:
-    l, cc = _i32(lengths), _i32(cache_cap)
-    co = np.ascontiguousarray(np.asarray(cache_off, dtype=np.int64))
-    st = load_library().pp_prefill_fused(
-        ctypes.byref(params), _p32(pack.bin_seg_ptr), _p32(pack.seg_start), _p32(pack.seg_len),
-        _p32(pack.seg_prompt), pack.k, _p32(l), _addr(q), _addr(k), _addr(v), _addr(o), _addr(k_cache),
-        _addr(v_cache), co.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), _p32(cc), _addr(workspace),
-        _addr(host_workspace), workspace_bytes, _addr(device_status), stream)
-    _check(st, "pp_prefill_fused")
+    _check((_native or _load_native()).prefill_fused(
+        params, pack.bin_seg_ptr, pack.seg_start, pack.seg_len, pack.seg_prompt, lengths, q, k, v, o, k_cache, v_cache,
+        cache_off, cache_cap, workspace, host_workspace, workspace_bytes, device_status, stream), "pp_prefill_fused")
 
 
 def pp_decode_workspace_bytes(params: AttnParams, lengths) -> int:
-    l = _i32(lengths)
-    return int(load_library().pp_decode_workspace_bytes(ctypes.byref(params), _p32(l), int(l.shape[0])))
+    return (_native or _load_native()).decode_workspace_bytes(params, lengths)
 
 
 def pp_decode_step(params: AttnParams, lengths, q_new, k_new, v_new, o, k_cache, v_cache, cache_off, cache_cap,
                    workspace, host_workspace, workspace_bytes: int, stream: int = 0) -> None:
-    l, cc = _i32(lengths), _i32(cache_cap)
-    co = np.ascontiguousarray(np.asarray(cache_off, dtype=np.int64))
-    st = load_library().pp_decode_step(
-        ctypes.byref(params), _p32(l), int(l.shape[0]), _addr(q_new), _addr(k_new), _addr(v_new), _addr(o),
-        _addr(k_cache), _addr(v_cache), co.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), _p32(cc),
-        _addr(workspace), _addr(host_workspace), workspace_bytes, stream)
-    _check(st, "pp_decode_step")
+    _check((_native or _load_native()).decode_step(
+        params, lengths, q_new, k_new, v_new, o, k_cache, v_cache, cache_off, cache_cap, workspace, host_workspace,
+        workspace_bytes, stream), "pp_decode_step")
 
 
 def pp_selftest_bounded_wait(device_status, limit_ms: int, stream: int = 0) -> None:
@@ -239,22 +240,16 @@ def pp_unpack_workspace_bytes(k: int) -> int:
 
 def pp_prefill_attention(params: AttnParams, pack: Packing, q, k, v, o, workspace, host_workspace,
                          workspace_bytes: int, device_status=None, stream: int = 0) -> None:
-    st = load_library().pp_prefill_attention(
-        ctypes.byref(params), _p32(pack.bin_seg_ptr), _p32(pack.seg_start), _p32(pack.seg_len), pack.k,
-        _addr(q), _addr(k), _addr(v), _addr(o), _addr(workspace), _addr(host_workspace), workspace_bytes,
-        _addr(device_status), stream)
-    _check(st, "pp_prefill_attention")
+    _check((_native or _load_native()).prefill_attention(
+        params, pack.bin_seg_ptr, pack.seg_start, pack.seg_len, q, k, v, o, workspace, host_workspace, workspace_bytes,
+        device_status, stream), "pp_prefill_attention")
 
 
 def pp_unpack_kv(params: AttnParams, bin_of, off_of, lengths, k_rot, v, k_cache, v_cache, cache_off, cache_cap,
                  workspace, host_workspace, workspace_bytes: int, stream: int = 0) -> None:
-    b, o, l, cc = _i32(bin_of), _i32(off_of), _i32(lengths), _i32(cache_cap)
-    co = np.ascontiguousarray(np.asarray(cache_off, dtype=np.int64))
-    st = load_library().pp_unpack_kv(
-        ctypes.byref(params), _p32(b), _p32(o), _p32(l), int(l.shape[0]), _addr(k_rot), _addr(v),
-        _addr(k_cache), _addr(v_cache), co.ctypes.data_as(ctypes.POINTER(ctypes.c_int64)), _p32(cc),
-        _addr(workspace), _addr(host_workspace), workspace_bytes, stream)
-    _check(st, "pp_unpack_kv")
+    _check((_native or _load_native()).unpack_kv(
+        params, bin_of, off_of, lengths, k_rot, v, k_cache, v_cache, cache_off, cache_cap, workspace, host_workspace,
+        workspace_bytes, stream), "pp_unpack_kv")
 
 
 def pp_unpack_static_max_prompts() -> int:
@@ -293,6 +288,17 @@ def pp_prefill_host(params: AttnParams, lengths, q_host, k_host, v_host, o_host,
     _check(st, "pp_prefill_host")
 
 
+def current_stream() -> int:
+    """The cudaStream_t of torch's current stream on the current device, as an integer."""
+    import torch
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+def fence():
+    """An event to wait for on the host: record(stream), synchronize()."""
+    return (_native or _load_native()).Fence()
+
+
 class Workspaces:
     """Device workspaces plus a small ring of pinned host staging buffers for the two calls that
     upload tables. Memory plumbing only (torch allocations and events); a staging buffer is
@@ -313,18 +319,15 @@ class Workspaces:
         self._fused_host = [torch.empty(pp_prefill_fused_host_bytes(params, k), dtype=torch.uint8).pin_memory()
                             for _ in range(ring)]
         self._ring = [(torch.empty(self.attn_bytes, dtype=torch.uint8).pin_memory(),
-                       torch.empty(self.unpack_bytes, dtype=torch.uint8).pin_memory(),
-                       torch.cuda.Event()) for _ in range(ring)]
+                       torch.empty(self.unpack_bytes, dtype=torch.uint8).pin_memory(), fence()) for _ in range(ring)]
         self._next = 0
-        self._used = [False] * ring
 
     def acquire(self):
         """Next (attn_host, unpack_host, slot); blocks until the slot's previous copies are done."""
         i = self._next
         self._next = (i + 1) % len(self._ring)
-        a, u, ev = self._ring[i]
-        if self._used[i]:
-            ev.synchronize()
+        a, u, fence = self._ring[i]
+        fence.synchronize()
         return a, u, i
 
     def fused_host(self, slot: int):
@@ -332,5 +335,8 @@ class Workspaces:
 
     def release(self, slot: int, stream=None) -> None:
         """Record, on the stream the copies were enqueued on, that slot's buffers may be reused after it."""
-        self._ring[slot][2].record(stream if stream is not None else self._torch.cuda.current_stream())
-        self._used[slot] = True
+        if stream is None:
+            self._ring[slot][2].record(current_stream())
+        else:
+            with self._torch.cuda.device(stream.device):
+                self._ring[slot][2].record(stream.cuda_stream)

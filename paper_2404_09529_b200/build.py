@@ -1,16 +1,20 @@
-"""Builds the C-ABI shared library (libprepack_b200.so) in-tree with nvcc for sm_100a."""
+"""Builds the C-ABI shared library (libprepack_b200.so) in-tree with nvcc for sm_100a, and the Python
+module over it (_native)."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libprepack_b200.so")
+MODULE_PATH = os.path.join(PKG_DIR, "_native" + sysconfig.get_config_var("EXT_SUFFIX"))
 SOURCES = ["pp_host.cpp", "pp_api.cu", "pp_rope.cu", "pp_attention.cu", "pp_unpack.cu", "pp_unpack_static.cu",
            "pp_tensorize.cu", "pp_decode.cu"]
+MODULE_SOURCE = "pp_python.cpp"
 HEADERS = ["pp_internal.h", "pp_device_once.h", os.path.join("..", "..", "include", "pp.h")]
 
 
@@ -22,11 +26,21 @@ def _nvcc() -> str:
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB_PATH):
-        return True
-    t = os.path.getmtime(LIB_PATH)
-    deps = [os.path.join(CSRC, s) for s in SOURCES + HEADERS]
-    return any(os.path.getmtime(d) > t for d in deps)
+    for path, sources in ((LIB_PATH, SOURCES), (MODULE_PATH, [MODULE_SOURCE])):
+        if not os.path.exists(path):
+            return True
+        t = os.path.getmtime(path)
+        if any(os.path.getmtime(os.path.join(CSRC, s)) > t for s in sources + HEADERS):
+            return True
+    return False
+
+
+def _run(cmd: list, verbose: bool) -> None:
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
+    if verbose:
+        sys.stderr.write(res.stderr)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -39,11 +53,11 @@ def build(force: bool = False, verbose: bool = False) -> str:
         cmd += ["-Xptxas", "-v"]
     cmd += [os.path.join(CSRC, s) for s in SOURCES]
     cmd += ["-o", LIB_PATH]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
-    if verbose:
-        sys.stderr.write(res.stderr)
+    _run(cmd, verbose)
+    import numpy
+    _run([_nvcc(), "-O2", "-std=c++17", "-shared", "-Xcompiler", "-fPIC", "-I", sysconfig.get_paths()["include"],
+          "-I", numpy.get_include(), os.path.join(CSRC, MODULE_SOURCE), "-o", MODULE_PATH, "-L", PKG_DIR,
+          "-l:" + os.path.basename(LIB_PATH), "-Xlinker", "-rpath=$ORIGIN"], verbose)
     return LIB_PATH
 
 

@@ -119,7 +119,7 @@ class PrefillBatch:
         """One pass of the hot path on the current stream (asynchronous)."""
         if repack:
             self._pack()
-        stream = torch.cuda.current_stream().cuda_stream
+        stream = B.current_stream()
         host_attn, host_unpack, slot = self.ws.acquire()
         self.params.flags = flags
         B.pp_prefill_attention(self.params, self.pack, self.q, self.kk, self.v, self.o, self.ws.attn_dev,
@@ -136,7 +136,7 @@ class PrefillBatch:
         same capacity on, the cos/sin table in it is declared valid (PP_FLAG_KEEP_ROPE_TABLE)."""
         if repack:
             self._pack()
-        stream = torch.cuda.current_stream().cuda_stream
+        stream = B.current_stream()
         _, _, slot = self.ws.acquire()
         if keep_rope_table and getattr(self, "_rope_table_capacity", None) == self.pack.capacity:
             flags |= B.PP_FLAG_KEEP_ROPE_TABLE
@@ -148,7 +148,7 @@ class PrefillBatch:
         self.ws.release(slot)
 
     def run_unpack_only(self) -> None:
-        stream = torch.cuda.current_stream().cuda_stream
+        stream = B.current_stream()
         _, host_unpack, slot = self.ws.acquire()
         B.pp_unpack_kv(self.params, self.bin_of, self.off_of, self.lengths, self.kk, self.v, self.k_cache,
                        self.v_cache, self.cache_off, self.cache_cap, self.ws.unpack_dev, host_unpack,
@@ -238,16 +238,15 @@ class DecodeBatch:
             self._ws_bytes = need + (need >> 2)        # lengths grow by one per step
             self._ws = torch.empty(self._ws_bytes, dtype=torch.uint8, device=self.device)
             self._host = [torch.empty(self._ws_bytes, dtype=torch.uint8).pin_memory() for _ in range(2)]
-            self._copied = [None, None]                # event after the upload that last read each staging buffer
+            self._copied = [B.fence() for _ in range(2)]   # after the upload that last read each staging buffer
             self._turn = 0
         slot = self._turn & 1
         self._turn += 1
-        if self._copied[slot] is not None:
-            self._copied[slot].synchronize()
+        self._copied[slot].synchronize()
+        stream = B.current_stream()
         B.pp_decode_step(self.params, self.lengths, q_new, k_new, v_new, self.o, self.k_cache, self.v_cache,
                          self.cache_off, self.cache_cap, self._ws, self._host[slot], self._ws_bytes,
-                         torch.cuda.current_stream().cuda_stream)
-        self._copied[slot] = torch.cuda.Event()
-        self._copied[slot].record()
+                         stream)
+        self._copied[slot].record(stream)
         self.lengths += 1
         return self.o
