@@ -110,8 +110,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count));
 }
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes, uint32_t issue) {
+  asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n@q mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}"
+               ::"r"(bar), "r"(bytes), "r"(issue) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -179,19 +180,34 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, co
   return true;
 }
 
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar,
-                                            int c0, int c1, int c2, int c3) {
+// The warps that issue TMA loads and MMAs run in uniform control flow: all 32 lanes execute the loop, the waits
+// and the address arithmetic, and a predicate (`issue`, set on one lane by elect.sync) picks the lane that
+// issues. With a branch on the lane index instead, every tcgen05.mma takes ~50 cycles to issue whatever its size
+// (a group of 8: 400 cycles against 101-136 in this form, one CTA per SM, with or without 16 busy warps
+// beside it), which held the tensor pipe below its rate of one 128 x 128 x 16 product per 64 cycles. A TMA
+// load with its expect_tx and the wait for an earlier one takes a warp 307 ns with the branch and 259 ns in this
+// form, for any box from 2 to 32 KB, so a tile is one load: whole steps 3.5 % faster for 256 prompts of up to
+// 3991 tokens on 32 / 8 heads, 2.7 % for 2048 short ones, 1 to 2 % for the others.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t r;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(r));
+  return r;
+}
+// Coordinates: column (0), head, row, chunk (0), bin; see make_map. Issued, like the MMAs below, by one lane of a
+// warp in uniform control flow.
+__device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, uint32_t bar, int head, int row, int bin,
+                                         uint32_t issue) {
   asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4, %5, %6}], [%2];"
-      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %6, 0;\n"
+      "@q cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%7, %3, %4, %7, %5}], [%2];\n}"
+      ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(head), "r"(row), "r"(bin), "r"(issue), "r"(0)
       : "memory");
 }
-__device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t src, int c0, int c1,
-                                             int c2, int c3) {
+__device__ __forceinline__ void tma_store(const CUtensorMap* map, uint32_t src, int head, int row, int chunk, int bin) {
   asm volatile(
-      "cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];"
-      ::"l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+      "cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%6, %2, %3, %4, %5}], [%1];"
+      ::"l"(reinterpret_cast<uint64_t>(map)), "r"(src), "r"(head), "r"(row), "r"(chunk), "r"(bin), "r"(0)
       : "memory");
 }
 __device__ __forceinline__ void tma_store_wait_read() {
@@ -200,16 +216,6 @@ __device__ __forceinline__ void tma_store_wait_read() {
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-// The MMA-issuing warps run in uniform control flow: all 32 lanes execute the loop, the waits and the
-// address arithmetic, and a predicate (`issue`, set on one lane by elect.sync) picks the lane that issues.
-// With a branch on the lane index instead, every tcgen05.mma takes ~50 cycles to issue whatever its size
-// (a group of 8: 400 cycles against 101-136 in this form, one CTA per SM, with or without 16 busy warps
-// beside it), which held the tensor pipe below its rate of one 128 x 128 x 16 product per 64 cycles.
-__device__ __forceinline__ uint32_t elect_one() {
-  uint32_t r;
-  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(r));
-  return r;
-}
 __device__ __forceinline__ void tc_commit(uint32_t bar, uint32_t issue) {
   asm volatile(
       "{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
@@ -433,6 +439,14 @@ __device__ __forceinline__ void decode_work(const AttnArgs& a, int w, Work& wk) 
   }
 }
 
+// The next work index of a CTA or slot, -1 when there is none left (a whole warp calls).
+__device__ __forceinline__ int draw_work(const AttnArgs& a, int lane) {
+  int w = 0;
+  if (lane == 0) w = atomicAdd(a.counter, 1);
+  w = __shfl_sync(0xffffffffu, w, 0);
+  return w < a.total_work ? w : -1;
+}
+
 // Second half of a work-list entry: what the softmax threads need to place their rows.
 __device__ __forceinline__ void decode_rows(const AttnArgs& a, int w, Work& wk) {
   const int gi = (w / a.subs) % a.n_items;
@@ -572,50 +586,46 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
     if constexpr (kIndep) {
-      if (warp >= 2 && lane == 0) {
+      if (warp >= 2) {
         // -------------------------------------------------------------- producer of slot t:
         // draws the slot's own items, loads Q and the item's K / V tiles (one stage each)
         const int t = warp - 2;
+        const uint32_t issue = elect_one();
         const uint32_t ring_bar = 8 * (uint32_t)t * kRing;
         volatile int* ring_base = s_ring + t * (int)kRing * kRingInts;
         uint32_t it_n = 0, kc = 0;
         Work wk;
         while (true) {
-          int w = atomicAdd(args.counter, 1);
-          if (w >= args.total_work) w = -1;
+          const int w = draw_work(args, lane);
           if (w >= 0) {
             decode_work(args, w, wk);
             decode_rows(args, w, wk);
           }
           const uint32_t ring = it_n % kRing;
-          if (!mbar_wait(bar_item_empty + ring_bar + 8 * ring, ((it_n / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) break;
-          if (w >= 0) ring_write(ring_base + ring * kRingInts, w, wk);
-          else ring_base[ring * kRingInts] = -1;
-          mbar_arrive(bar_item_full + ring_bar + 8 * ring);
+          if (!mbar_wait_warp(bar_item_empty + ring_bar + 8 * ring, ((it_n / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) break;
+          if (issue) {
+            if (w >= 0) ring_write(ring_base + ring * kRingInts, w, wk);
+            else ring_base[ring * kRingInts] = -1;
+            mbar_arrive(bar_item_full + ring_bar + 8 * ring);
+          }
           if (w < 0) break;
           // the slot's last Q.K^T of the previous item must have finished reading the Q buffer
-          if (!mbar_wait(bar_q_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitQEmpty)) break;
-          mbar_expect_tx(bar_q_full + 8 * t, Cfg::kQBytes);
-          for (int c = 0; c < kChunks; ++c)
-            tma_load_4d(s_q + t * Cfg::kQBytes + c * (BM * 128), &map_q, bar_q_full + 8 * t,
-                        c * 64, wk.head[0], wk.q_row0[0], wk.bin);
+          if (!mbar_wait_warp(bar_q_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitQEmpty)) break;
+          mbar_expect_tx(bar_q_full + 8 * t, Cfg::kQBytes, issue);
+          tma_load(s_q + t * Cfg::kQBytes, &map_q, bar_q_full + 8 * t, wk.head[0], wk.q_row0[0], wk.bin, issue);
           bool ok = true;
           for (int j = 0; ok && j < wk.n; ++j, ++kc) {
             const int kv0 = wk.kv_row0 + j * BN;
             const uint32_t st = 2u * (uint32_t)t + (kc & 1u);          // the slot's stage for this tile
             const uint32_t free_parity = ((kc >> 1) & 1u) ^ 1u;
-            ok = mbar_wait(bar_k_empty + 8 * st, free_parity, wctx, kWaitKEmpty);
+            ok = mbar_wait_warp(bar_k_empty + 8 * st, free_parity, wctx, kWaitKEmpty);
             if (!ok) break;
-            mbar_expect_tx(bar_k_full + 8 * st, Cfg::kKVBytes);
-            for (int c = 0; c < kChunks; ++c)
-              tma_load_4d(s_k + st * Cfg::kKVBytes + c * (BN * 128), &map_k, bar_k_full + 8 * st,
-                          c * 64, wk.kv_head, kv0, wk.bin);
-            ok = mbar_wait(bar_v_empty + 8 * st, free_parity, wctx, kWaitVEmpty);
+            mbar_expect_tx(bar_k_full + 8 * st, Cfg::kKVBytes, issue);
+            tma_load(s_k + st * Cfg::kKVBytes, &map_k, bar_k_full + 8 * st, wk.kv_head, kv0, wk.bin, issue);
+            ok = mbar_wait_warp(bar_v_empty + 8 * st, free_parity, wctx, kWaitVEmpty);
             if (!ok) break;
-            mbar_expect_tx(bar_v_full + 8 * st, Cfg::kKVBytes);
-            for (int c = 0; c < kChunks; ++c)
-              tma_load_4d(s_v + st * Cfg::kKVBytes + c * (BN * 128), &map_v, bar_v_full + 8 * st,
-                          c * 64, wk.kv_head, kv0, wk.bin);
+            mbar_expect_tx(bar_v_full + 8 * st, Cfg::kKVBytes, issue);
+            tma_load(s_v + st * Cfg::kKVBytes, &map_v, bar_v_full + 8 * st, wk.kv_head, kv0, wk.bin, issue);
           }
           if (!ok) break;
           ++it_n;
@@ -720,65 +730,62 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
       }
     } else {
-    if (warp == 0 && lane == 0) {
+    if (warp == 0) {
       // ---------------------------------------------------------------- work fetch + K/V producer
+      const uint32_t issue = elect_one();
       uint32_t it_n = 0, kc = 0;
       Work wk;
       while (true) {
-        int w = atomicAdd(args.counter, 1);
-        if (w >= args.total_work) w = -1;
+        const int w = draw_work(args, lane);
         if (w >= 0) {
           decode_work(args, w, wk);
           decode_rows(args, w, wk);
         }
         const uint32_t ring = it_n % kRing;
-        if (!mbar_wait(bar_item_empty + 8 * ring, ((it_n / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) break;
-        if (w >= 0) ring_write(s_ring + ring * kRingInts, w, wk);
-        else s_ring[ring * kRingInts] = -1;
-        mbar_arrive(bar_item_full + 8 * ring);
+        if (!mbar_wait_warp(bar_item_empty + 8 * ring, ((it_n / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) break;
+        if (issue) {
+          if (w >= 0) ring_write(s_ring + ring * kRingInts, w, wk);
+          else s_ring[ring * kRingInts] = -1;
+          mbar_arrive(bar_item_full + 8 * ring);
+        }
         if (w < 0) break;
         bool ok = true;
         for (int j = 0; ok && j < wk.n; ++j, ++kc) {
           const int kv0 = wk.kv_row0 + j * BN;
           uint32_t s = kc % NK;
-          ok = mbar_wait(bar_k_empty + 8 * s, ((kc / NK) & 1u) ^ 1u, wctx, kWaitKEmpty);
+          ok = mbar_wait_warp(bar_k_empty + 8 * s, ((kc / NK) & 1u) ^ 1u, wctx, kWaitKEmpty);
           if (!ok) break;
-          mbar_expect_tx(bar_k_full + 8 * s, Cfg::kKVBytes);
-          for (int c = 0; c < kChunks; ++c)
-            tma_load_4d(s_k + s * Cfg::kKVBytes + c * (BN * 128), &map_k, bar_k_full + 8 * s,
-                        c * 64, wk.kv_head, kv0, wk.bin);
+          mbar_expect_tx(bar_k_full + 8 * s, Cfg::kKVBytes, issue);
+          tma_load(s_k + s * Cfg::kKVBytes, &map_k, bar_k_full + 8 * s, wk.kv_head, kv0, wk.bin, issue);
           s = kc % NV;
-          ok = mbar_wait(bar_v_empty + 8 * s, ((kc / NV) & 1u) ^ 1u, wctx, kWaitVEmpty);
+          ok = mbar_wait_warp(bar_v_empty + 8 * s, ((kc / NV) & 1u) ^ 1u, wctx, kWaitVEmpty);
           if (!ok) break;
-          mbar_expect_tx(bar_v_full + 8 * s, Cfg::kKVBytes);
-          for (int c = 0; c < kChunks; ++c)
-            tma_load_4d(s_v + s * Cfg::kKVBytes + c * (BN * 128), &map_v, bar_v_full + 8 * s,
-                        c * 64, wk.kv_head, kv0, wk.bin);
+          mbar_expect_tx(bar_v_full + 8 * s, Cfg::kKVBytes, issue);
+          tma_load(s_v + s * Cfg::kKVBytes, &map_v, bar_v_full + 8 * s, wk.kv_head, kv0, wk.bin, issue);
         }
         if (!ok) break;
         ++it_n;
       }
-    } else if (warp >= 2 && lane == 0) {
+    } else if (warp >= 2) {
       // ---------------------------------------------------------------- Q loader of slot t
       const int t = warp - 2;
+      const uint32_t issue = elect_one();
       uint32_t it_n = 0;
       while (true) {
         const uint32_t ring = it_n % kRing;
-        if (!mbar_wait(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull)) break;
+        if (!mbar_wait_warp(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull)) break;
         const volatile int* e = s_ring + ring * kRingInts;
-        const int w = e[0], bin = e[1];
-        const int q_row0 = e[4 + t], head = e[9 + t];
-        const bool used = t ? (e[6] < e[8]) : (e[7] > 0);
-        mbar_arrive(bar_item_empty + 8 * ring);
+        const int w = uniform(e[0]), bin = uniform(e[1]);
+        const int q_row0 = uniform(e[4 + t]), head = uniform(e[9 + t]);
+        const bool used = uniform(t ? (e[6] < e[8]) : (e[7] > 0)) != 0;
+        if (issue) mbar_arrive(bar_item_empty + 8 * ring);
         if (w < 0) break;
         // the slot's last Q.K^T of the previous item must have finished reading the buffer
-        if (!mbar_wait(bar_q_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitQEmpty)) break;
+        if (!mbar_wait_warp(bar_q_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitQEmpty)) break;
         if (used) {
-          mbar_expect_tx(bar_q_full + 8 * t, Cfg::kQBytes);
-          for (int c = 0; c < kChunks; ++c)
-            tma_load_4d(s_q + t * Cfg::kQBytes + c * (BM * 128), &map_q, bar_q_full + 8 * t,
-                        c * 64, head, q_row0, bin);
-        } else {
+          mbar_expect_tx(bar_q_full + 8 * t, Cfg::kQBytes, issue);
+          tma_load(s_q + t * Cfg::kQBytes, &map_q, bar_q_full + 8 * t, head, q_row0, bin, issue);
+        } else if (issue) {
           mbar_arrive(bar_q_full + 8 * t);
         }
         ++it_n;
@@ -1161,7 +1168,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
               __syncwarp();
               if (lane == 0 && p_row0 < args.capacity) {
-                tma_store_4d(&map_o, stage, hh * 64, p_head, p_row0, p_bin);
+                tma_store(&map_o, stage, p_head, p_row0, hh, p_bin);
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
               }
             }
@@ -1453,7 +1460,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0 && row0_w < args.capacity) {
-              tma_store_4d(&map_o, stage, hh * 64, head_t, row0_w, item_bin);
+              tma_store(&map_o, stage, head_t, row0_w, hh, item_bin);
               asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             }
           }
@@ -1517,16 +1524,17 @@ EncodeFn get_encode_fn() {
   return fn;
 }
 
-// 4-D map over a dense [R, M, H, D] bf16 tensor; box = 64 elements x `heads` heads x `rows` rows x 1 bin
-// (in shared memory: row-major over (row, head), 128 bytes each).
-int make_map(CUtensorMap* map, const void* ptr, int64_t R, int64_t M, int64_t H, int64_t D, int rows, int heads = 1) {
+// 5-D map (column, head, row, chunk of 64 columns, bin) over a dense [R, M, H, D] bf16 tensor; box = 64 columns x
+// `heads` heads x `rows` rows x `chunks` chunks x 1 bin: in shared memory the chunks lie one behind the other, each
+// row-major over (row, head) with 128 bytes per row, swizzled. So a whole tile is one load.
+int make_map(CUtensorMap* map, const void* ptr, int64_t R, int64_t M, int64_t H, int64_t D, int rows, int heads, int chunks) {
   EncodeFn enc = get_encode_fn();
   if (!enc) return note_cuda_error(-1, "cuTensorMapEncodeTiled entry point not found");
-  cuuint64_t dims[4] = {(cuuint64_t)D, (cuuint64_t)H, (cuuint64_t)M, (cuuint64_t)R};
-  cuuint64_t strides[3] = {(cuuint64_t)(D * 2), (cuuint64_t)(H * D * 2), (cuuint64_t)(M * H * D * 2)};
-  cuuint32_t box[4] = {64u, (cuuint32_t)heads, (cuuint32_t)rows, 1u};
-  cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
-  const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(ptr), dims, strides,
+  cuuint64_t dims[5] = {64u, (cuuint64_t)H, (cuuint64_t)M, (cuuint64_t)(D / 64), (cuuint64_t)R};
+  cuuint64_t strides[4] = {(cuuint64_t)(D * 2), (cuuint64_t)(H * D * 2), 128u, (cuuint64_t)(M * H * D * 2)};
+  cuuint32_t box[5] = {64u, (cuuint32_t)heads, (cuuint32_t)rows, (cuuint32_t)chunks, 1u};
+  cuuint32_t estr[5] = {1u, 1u, 1u, 1u, 1u};
+  const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(ptr), dims, strides,
                          box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? PP_OK : note_cuda_error((int)r, "cuTensorMapEncodeTiled");
@@ -1567,10 +1575,10 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   const int fold = kIndep ? L.fold : 1;
   int fold_shift = 0;
   while ((1 << fold_shift) < fold) ++fold_shift;
-  if ((st = make_map(&mq, q, p.n_bins, p.capacity, p.n_q_heads, D, BM / fold, fold)) != PP_OK) return st;
-  if ((st = make_map(&mk, k, p.n_bins, p.capacity, p.n_kv_heads, D, BN)) != PP_OK) return st;
-  if ((st = make_map(&mv, v, p.n_bins, p.capacity, p.n_kv_heads, D, BN)) != PP_OK) return st;
-  if ((st = make_map(&mo, o, p.n_bins, p.capacity, p.n_q_heads, D, 32 / fold, fold)) != PP_OK) return st;   // one warp's rows per store
+  if ((st = make_map(&mq, q, p.n_bins, p.capacity, p.n_q_heads, D, BM / fold, fold, D / 64)) != PP_OK) return st;
+  if ((st = make_map(&mk, k, p.n_bins, p.capacity, p.n_kv_heads, D, BN, 1, D / 64)) != PP_OK) return st;
+  if ((st = make_map(&mv, v, p.n_bins, p.capacity, p.n_kv_heads, D, BN, 1, D / 64)) != PP_OK) return st;
+  if ((st = make_map(&mo, o, p.n_bins, p.capacity, p.n_q_heads, D, 32 / fold, fold, 1)) != PP_OK) return st;   // one warp's rows per store
   // the shared-memory opt-in of a kernel is a per-device attribute
   static DeviceOnce configured;     // per template instance
   int dev = 0;
