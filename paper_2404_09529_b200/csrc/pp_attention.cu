@@ -27,10 +27,10 @@
 // the f heads, a short prompt fills a tile with heads instead of empty rows, and an item's key
 // tiles start at the first row of the first prompt it touches rather than at a tile boundary.
 //   warps 0-1    issue the tcgen05.mma of slot 0 / slot 1
-//   warps 2-3    draw items and TMA-load Q, K, V of slot 0 / slot 1 (two K and two V stages each)
+//   warps 2-3    draw items and TMA-load Q (two tiles: the next item's is there early), K, V of slot 0 / slot 1
 //   warps 4-7    softmax threads of slot 0, one per query row; they never leave the tile loop
-//   warps 8-11   helper threads of slot 0, one per row: rotate the next item's Q in shared memory
-//                (fused path) and run the previous item's epilogue
+//   warps 8-11   helper threads of slot 0, one per row: find the first key of each row of the next item,
+//                rotate its Q in shared memory (fused path) and run the previous item's epilogue
 //   warps 12-19  the same for slot 1
 // Softmax: tcgen05.ld the thread's scores, mask to the row's key range, lazy running maximum (O is
 // rescaled only when the maximum grows by more than 2^8, or 2^90 in the shared-stream mode, where rows
@@ -78,19 +78,24 @@ constexpr float kBoundLog2 = 44.f;
 constexpr uint32_t kRing = 3;               // decoded work items in flight between the fetching thread and its readers
 constexpr int kRingInts = 20;              // ints per ring entry
 
-// BN: key rows per tile. 128 in shared-stream mode; 64 in independent mode, where every slot owns
-// two K and two V stages and two S buffers (see the kernel).
+// BN: key rows per tile. 128 in shared-stream mode: one Q tile per slot, rings of K and V tiles that both
+// slots read, an O staging buffer per slot. 64 in independent mode: per slot two Q tiles (that of the
+// next item is loaded and rotated while the current item is computed) and one ring in which K and V tiles
+// alternate; at D = 128, where there is no room for a staging buffer, O is staged in the Q tile of its own
+// item. At D = 128 both modes come to exactly 227 KB.
 template <int D, int BN> struct AttnCfg {
-  static constexpr int kKStages = (D == 128 && BN == 128) ? 2 : 4;
-  static constexpr int kVStages = (D == 128 && BN == 128) ? 2 : 4;
-  static constexpr int kChunks = D / 64;                     // 128-byte swizzle spans per row
-  static constexpr int kQBytes = BM * D * 2;                 // per slot
+  static constexpr bool kIndep = BN == kTileNShort;
+  static constexpr int kKStages = D == 128 ? 2 : 4, kVStages = kKStages;   // shared-stream mode
+  static constexpr int kKVStages = D == 128 ? 3 : 4;         // independent mode, per slot
+  static constexpr bool kStageInQ = D == 128;                // independent mode
+  static constexpr int kQBytes = BM * D * 2;                 // one Q tile
   static constexpr int kKVBytes = BN * D * 2;
   // barriers + work ring (1024) and the row-maximum exchange buffer [slot][half][row] (2048), placed
-  // in front of the 1024-byte-aligned tiles; at D = 128 the total is exactly the 227 KB limit
+  // in front of the 1024-byte-aligned tiles
   static constexpr int kMiscBytes = 3072;
   static constexpr int kStageOBytes = BM * 128;              // per slot: one 64-column box of O
-  static constexpr int kTileBytes = 2 * kQBytes + (kKStages + kVStages) * kKVBytes + 2 * kStageOBytes;
+  static constexpr int kTileBytes = kIndep ? 2 * (2 * kQBytes + kKVStages * kKVBytes + (kStageInQ ? 0 : kStageOBytes))
+                                           : 2 * kQBytes + (kKStages + kVStages) * kKVBytes + 2 * kStageOBytes;
   static constexpr int kSmemBytes = kMiscBytes + kTileBytes;
   static constexpr uint32_t kTmemS = 0;                      // S_t at 128 * t
   static constexpr uint32_t kTmemO = 256;                    // O_t at 256 + D * t
@@ -492,6 +497,12 @@ __device__ __forceinline__ int seg_start_at(const int32_t* starts, int seg_begin
 //   sequences, GQA head pairs). kIndep = true: every slot draws its own single-tile items and loads
 //   its own K/V tiles (64 rows each), so neither slot ever waits for the other (short prompts, where
 //   pairing two row tiles of different length would leave one slot idle for a tile per item).
+// Independent mode: place in the slot's K / V ring sequence K0 K1 V0 K2 V1 K3 V2 ... of the k-th key tile of the slot.
+// With three stages K(k+3) then follows V(k) and V(k+2) follows K(k+2) in a stage: either load has more than a
+// tile's time (in the sequence K0 V0 K1 V1 ..., K(k+3) followed V(k+1), and its load was waited for every time).
+__device__ __forceinline__ uint32_t kv_index_k(uint32_t k) { return k ? 2u * k - 1u : 0u; }
+__device__ __forceinline__ uint32_t kv_index_v(uint32_t k) { return 2u * k + 2u; }
+
 template <int D, bool kIndep>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -499,19 +510,20 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                  const AttnArgs args) {
   constexpr int BN = kIndep ? kTileNShort : kTileN;
   using Cfg = AttnCfg<D, BN>;
-  constexpr int NK = Cfg::kKStages, NV = Cfg::kVStages, kChunks = Cfg::kChunks;
+  constexpr int NK = Cfg::kKStages, NV = Cfg::kVStages;
 
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t s_misc = smem_u32(smem_raw);
   uint8_t* misc = smem_raw;
-  const uint32_t s_q = (s_misc + 3072u + 1023u) & ~1023u;       // [2] slots; tiles need 1024-byte alignment
-  const uint32_t s_k = s_q + 2 * Cfg::kQBytes;                  // [NK]
+  const uint32_t s_q = (s_misc + 3072u + 1023u) & ~1023u;       // tiles need 1024-byte alignment
+  const uint32_t s_kv = s_q + 4 * Cfg::kQBytes;                 // independent mode: [2 slots][kKVStages] behind [2][2] Q tiles
+  const uint32_t s_k = s_q + 2 * Cfg::kQBytes;                  // shared-stream mode: [NK] behind [2] Q tiles
   const uint32_t s_v = s_k + NK * Cfg::kKVBytes;                // [NV]
-  const uint32_t s_stage_o = s_v + NV * Cfg::kKVBytes;          // [2] slots, epilogue staging
+  const uint32_t s_stage_o = kIndep ? s_kv + 2 * Cfg::kKVStages * Cfg::kKVBytes : s_v + NV * Cfg::kKVBytes;   // [2] slots, epilogue staging
   {
     uint32_t dyn_bytes;
     asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
-    if (s_stage_o + 2 * Cfg::kStageOBytes > s_misc + dyn_bytes) {   // base less aligned than expected
+    if (s_q + Cfg::kTileBytes > s_misc + dyn_bytes) {           // base less aligned than expected
       if (threadIdx.x == 0 && args.status) atomicCAS(args.status, 0, 100);
       return;
     }
@@ -519,18 +531,22 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // mbarriers, 8 bytes each
   const uint32_t bar_item_full = s_misc + 0;     // [2 rings][kRing]
   const uint32_t bar_item_empty = s_misc + 64;   // [2 rings][kRing]
-  const uint32_t bar_q_full = s_misc + 128;      // [2]
-  const uint32_t bar_q_empty = s_misc + 144;     // [2]
+  const uint32_t bar_q_full = s_misc + (kIndep ? 896 : 128);    // [2]; independent mode: [2 slots][2 Q tiles]
+  const uint32_t bar_q_empty = s_misc + (kIndep ? 128 : 144);   // [2]; independent mode: [2 slots][2 Q tiles]
   const uint32_t bar_s_full = s_misc + 160;      // [2 slots][2 S buffers]; shared mode uses [t][0]
   const uint32_t bar_p_full = s_misc + 192;      // [2 slots][2 S buffers]
   const uint32_t bar_o_full = s_misc + 224;      // [2]
   const uint32_t bar_o_empty = s_misc + 240;     // [2]
-  const uint32_t bar_k_full = s_misc + 256;      // [4]; independent mode: [2 slots][2 stages]
+  const uint32_t bar_k_full = s_misc + 256;      // [4]
   const uint32_t bar_k_empty = s_misc + 288;     // [4]
   const uint32_t bar_v_full = s_misc + 320;      // [4]
   const uint32_t bar_v_empty = s_misc + 352;     // [4]
-  const uint32_t bar_q_rot = s_misc + 384;       // [2] Q_t has been rotated in place (fused path)
-  const uint32_t bar_pair0 = s_misc + 896;       // [2 slots][4 quadrants] rendezvous of the two warps that share rows
+  const uint32_t bar_kv_full = s_misc + 256;     // independent mode, in their place: [2 slots][4 stages]
+  const uint32_t bar_kv_empty = s_misc + 320;    // [2 slots][4 stages]
+  const uint32_t bar_q_rot = s_misc + (kIndep ? 928 : 384);     // [2] Q_t has been rotated in place (fused path);
+                                                 // independent mode: [2 slots][2 Q tiles], its rows' first keys are there too
+  const uint32_t bar_pv_done = s_misc + 384;     // [2] independent mode: P(k) V(k) has been computed
+  const uint32_t bar_pair0 = s_misc + 896;       // [2 slots][4 quadrants] shared-stream mode: rendezvous of the two warps that share rows
   const uint32_t bar_l_ready = s_misc + 976;     // [2][2] independent mode: the slot's row sums of item i are in shared memory ([slot][i & 1])
   uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(misc + 400);
   volatile int* s_abort = reinterpret_cast<volatile int*>(misc + 404);
@@ -538,7 +554,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   volatile uint8_t* s_bounded = misc + 1008;     // [2 slots][4 quadrants][2 halves] shared-stream mode: the warp's rows are bounded
   volatile float* s_xchg = reinterpret_cast<volatile float*>(misc + 1024);   // [2 slots][2 halves][128 rows]
   static_assert(416 + 2 * kRing * kRingInts * 4 <= 896, "ring does not fit");
-  static_assert(NK <= 4 && NV <= 4, "barrier slots");
+  static_assert(NK <= 4 && NV <= 4 && Cfg::kKVStages <= 4, "barrier slots");
 
   const int warp = uniform((int)(threadIdx.x >> 5));
   const int lane = threadIdx.x & 31;
@@ -552,21 +568,32 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       mbar_init(bar_item_empty + 8 * i, kIndep ? 1 + kSoftmaxThreads : 1 + 2 + 2 * kSoftmaxThreads);
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(bar_q_full + 8 * i, 1);
-      mbar_init(bar_q_empty + 8 * i, 1);
-      mbar_init(bar_q_rot + 8 * i, kIndep ? kSoftmaxThreads / 2 : kSoftmaxThreads);
       for (int b = 0; b < 2; ++b) {
         mbar_init(bar_s_full + 8 * (2 * i + b), 1);
         mbar_init(bar_p_full + 8 * (2 * i + b), kIndep ? kSoftmaxThreads / 2 : kSoftmaxThreads);
+        mbar_init(bar_l_ready + 8 * (2 * i + b), kSoftmaxThreads / 2);
       }
       mbar_init(bar_o_full + 8 * i, 1);
       mbar_init(bar_o_empty + 8 * i, kIndep ? kSoftmaxThreads / 2 : kSoftmaxThreads);
-      mbar_init(bar_l_ready + 16 * i, kSoftmaxThreads / 2);
-      mbar_init(bar_l_ready + 16 * i + 8, kSoftmaxThreads / 2);
-      for (int qd = 0; qd < 4; ++qd) mbar_init(bar_pair0 + 8 * (4 * i + qd), 64);
     }
-    for (int s = 0; s < NK; ++s) { mbar_init(bar_k_full + 8 * s, 1); mbar_init(bar_k_empty + 8 * s, 1); }
-    for (int s = 0; s < NV; ++s) { mbar_init(bar_v_full + 8 * s, 1); mbar_init(bar_v_empty + 8 * s, 1); }
+    if constexpr (kIndep) {
+      for (int i = 0; i < 4; ++i) {
+        mbar_init(bar_q_full + 8 * i, 1);
+        mbar_init(bar_q_empty + 8 * i, Cfg::kStageInQ ? 4 : 1);   // one lane of each helper warp, or a commit
+        mbar_init(bar_q_rot + 8 * i, kSoftmaxThreads / 2);
+      }
+      for (int i = 0; i < 8; ++i) { mbar_init(bar_kv_full + 8 * i, 1); mbar_init(bar_kv_empty + 8 * i, 1); }
+      for (int i = 0; i < 2; ++i) mbar_init(bar_pv_done + 8 * i, 1);
+    } else {
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(bar_q_full + 8 * i, 1);
+        mbar_init(bar_q_empty + 8 * i, 1);
+        mbar_init(bar_q_rot + 8 * i, kSoftmaxThreads);
+        for (int qd = 0; qd < 4; ++qd) mbar_init(bar_pair0 + 8 * (4 * i + qd), 64);
+      }
+      for (int s = 0; s < NK; ++s) { mbar_init(bar_k_full + 8 * s, 1); mbar_init(bar_k_empty + 8 * s, 1); }
+      for (int s = 0; s < NV; ++s) { mbar_init(bar_v_full + 8 * s, 1); mbar_init(bar_v_empty + 8 * s, 1); }
+    }
     *s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -588,47 +615,63 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     if constexpr (kIndep) {
       if (warp >= 2) {
         // -------------------------------------------------------------- producer of slot t:
-        // draws the slot's own items, loads Q and the item's K / V tiles (one stage each)
+        // draws the slot's own items, loads Q and the item's K / V tiles. The next item is drawn and announced
+        // at the start of the current one and its Q loaded behind the first two key tiles, so that the helper
+        // threads rotate it under the current item (loaded behind the last scores of an item and rotated
+        // then, Q kept the slot waiting 5500 cycles per item of 5.3 key tiles, 2000 without the rotation; whole
+        // steps: 34 bins of a stream 1197 -> 1116 us, 64 prompts 315 -> 307, both 32 heads, D = 128). K runs
+        // one tile ahead of V, over the end of the item too: the order in which the MMAs want them.
         const int t = warp - 2;
+        constexpr int NS = Cfg::kKVStages;
         const uint32_t issue = elect_one();
         const uint32_t ring_bar = 8 * (uint32_t)t * kRing;
         volatile int* ring_base = s_ring + t * (int)kRing * kRingInts;
-        uint32_t it_n = 0, kc = 0;
-        Work wk;
-        while (true) {
-          const int w = draw_work(args, lane);
+        auto announce = [&](const uint32_t it, const int w, Work& wk) -> bool {      // w < 0: there is no item `it`
           if (w >= 0) {
             decode_work(args, w, wk);
             decode_rows(args, w, wk);
           }
-          const uint32_t ring = it_n % kRing;
-          if (!mbar_wait_warp(bar_item_empty + ring_bar + 8 * ring, ((it_n / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) break;
+          const uint32_t ring = it % kRing;
+          if (!mbar_wait_warp(bar_item_empty + ring_bar + 8 * ring, ((it / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) return false;
           if (issue) {
             if (w >= 0) ring_write(ring_base + ring * kRingInts, w, wk);
             else ring_base[ring * kRingInts] = -1;
             mbar_arrive(bar_item_full + ring_bar + 8 * ring);
           }
-          if (w < 0) break;
-          // the slot's last Q.K^T of the previous item must have finished reading the Q buffer
-          if (!mbar_wait_warp(bar_q_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitQEmpty)) break;
-          mbar_expect_tx(bar_q_full + 8 * t, Cfg::kQBytes, issue);
-          tma_load(s_q + t * Cfg::kQBytes, &map_q, bar_q_full + 8 * t, wk.head[0], wk.q_row0[0], wk.bin, issue);
-          bool ok = true;
+          return true;
+        };
+        auto load_q = [&](const uint32_t it, const Work& wk) -> bool {
+          // O of the item before the previous one must have left this Q tile (or, where O is staged
+          // elsewhere, its last scores must have been computed)
+          const uint32_t qb = 2u * (uint32_t)t + (it & 1u);
+          if (!mbar_wait_warp(bar_q_empty + 8 * qb, ((it >> 1) & 1u) ^ 1u, wctx, kWaitQEmpty)) return false;
+          mbar_expect_tx(bar_q_full + 8 * qb, Cfg::kQBytes, issue);
+          tma_load(s_q + qb * Cfg::kQBytes, &map_q, bar_q_full + 8 * qb, wk.head[0], wk.q_row0[0], wk.bin, issue);
+          return true;
+        };
+        auto load_kv = [&](const CUtensorMap* map, const uint32_t idx, const Work& wk, const int j) -> bool {
+          const uint32_t st = idx % NS, bar = 8 * (4u * (uint32_t)t + st);
+          if (!mbar_wait_warp(bar_kv_empty + bar, ((idx / NS) & 1u) ^ 1u, wctx, kWaitKEmpty)) return false;
+          mbar_expect_tx(bar_kv_full + bar, Cfg::kKVBytes, issue);
+          tma_load(s_kv + ((uint32_t)t * NS + st) * Cfg::kKVBytes, map, bar_kv_full + bar, wk.kv_head, wk.kv_row0 + j * BN, wk.bin, issue);
+          return true;
+        };
+        int w = draw_work(args, lane);
+        Work wk, wk_next;
+        bool ok = announce(0, w, wk);
+        if (ok && w >= 0) ok = load_q(0, wk) && load_kv(&map_k, kv_index_k(0), wk, 0);
+        uint32_t kc = 0;                      // key tiles of the slot's stream whose V has been loaded
+        for (uint32_t it_n = 0; ok && w >= 0; ++it_n) {
+          const int w_next = draw_work(args, lane);
+          if (!(ok = announce(it_n + 1u, w_next, wk_next))) break;
           for (int j = 0; ok && j < wk.n; ++j, ++kc) {
-            const int kv0 = wk.kv_row0 + j * BN;
-            const uint32_t st = 2u * (uint32_t)t + (kc & 1u);          // the slot's stage for this tile
-            const uint32_t free_parity = ((kc >> 1) & 1u) ^ 1u;
-            ok = mbar_wait_warp(bar_k_empty + 8 * st, free_parity, wctx, kWaitKEmpty);
-            if (!ok) break;
-            mbar_expect_tx(bar_k_full + 8 * st, Cfg::kKVBytes, issue);
-            tma_load(s_k + st * Cfg::kKVBytes, &map_k, bar_k_full + 8 * st, wk.kv_head, kv0, wk.bin, issue);
-            ok = mbar_wait_warp(bar_v_empty + 8 * st, free_parity, wctx, kWaitVEmpty);
-            if (!ok) break;
-            mbar_expect_tx(bar_v_full + 8 * st, Cfg::kKVBytes, issue);
-            tma_load(s_v + st * Cfg::kKVBytes, &map_v, bar_v_full + 8 * st, wk.kv_head, kv0, wk.bin, issue);
+            if (j + 1 < wk.n) ok = load_kv(&map_k, kv_index_k(kc + 1), wk, j + 1);
+            else if (w_next >= 0) ok = load_kv(&map_k, kv_index_k(kc + 1), wk_next, 0);
+            if (ok) ok = load_kv(&map_v, kv_index_v(kc), wk, j);
+            if (ok && j == min(1, wk.n - 1) && w_next >= 0) ok = load_q(it_n + 1u, wk_next);
           }
-          if (!ok) break;
-          ++it_n;
+          w = w_next;
+          wk = wk_next;
         }
       } else if (warp < 2) {
         // -------------------------------------------------------------- MMA issuer of slot t
@@ -642,42 +685,42 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t issue = elect_one();
         constexpr uint32_t idesc_qk = instr_desc(BN, false);
         constexpr uint32_t idesc_pv = instr_desc(D, true);
-        const uint32_t a_lo = desc_lo(s_q, 0) + (uint32_t)t * (Cfg::kQBytes >> 4);
-        const uint32_t k_lo = desc_lo(s_k, 0) + 2u * (uint32_t)t * (Cfg::kKVBytes >> 4);
-        const uint32_t v_lo = desc_lo(s_v, BN * 128) + 2u * (uint32_t)t * (Cfg::kKVBytes >> 4);
+        constexpr int NS = Cfg::kKVStages;
+        const uint32_t q_lo = desc_lo(s_q, 0) + 2u * (uint32_t)t * (Cfg::kQBytes >> 4);
+        const uint32_t k_lo = desc_lo(s_kv, 0) + (uint32_t)(t * NS) * (Cfg::kKVBytes >> 4);
+        const uint32_t v_lo = desc_lo(s_kv, BN * 128) + (uint32_t)(t * NS) * (Cfg::kKVBytes >> 4);
         const uint32_t tm_s = tmem_base + Cfg::kTmemS + 128u * (uint32_t)t;
         const uint32_t tm_o = tmem_base + Cfg::kTmemO + (uint32_t)D * (uint32_t)t;
-        const uint32_t bar_q_ready = (args.rope_table ? bar_q_rot : bar_q_full) + 8 * t;
+        const uint32_t b_q_ready = bar_q_rot + 16 * t;         // [Q tile]
         const uint32_t b_item_full = bar_item_full + 8 * (uint32_t)t * kRing;
         const uint32_t b_item_empty = bar_item_empty + 8 * (uint32_t)t * kRing;
-        const uint32_t b_k_full = bar_k_full + 16 * t, b_k_empty = bar_k_empty + 16 * t;   // [stage]
-        const uint32_t b_v_full = bar_v_full + 16 * t, b_v_empty = bar_v_empty + 16 * t;
+        const uint32_t b_kv_full = bar_kv_full + 32 * t, b_kv_empty = bar_kv_empty + 32 * t;   // [stage]
         const uint32_t b_s_full = bar_s_full + 16 * t, b_p_full = bar_p_full + 16 * t;     // [buffer]
         const uint32_t b_o_full = bar_o_full + 8 * t, b_o_empty = bar_o_empty + 8 * t;
-        const uint32_t b_q_empty = bar_q_empty + 8 * t;
         uint32_t it_n = 0, kc = 0;       // items and key tiles consumed
         bool ok = true;
-        // S(kq) = Q_t K(kq)^T into buffer kq & 1
-        auto issue_qk = [&](const uint32_t kq, const bool last_of_item) -> bool {
-          const uint32_t b = kq & 1u;
-          if (!mbar_wait_warp(b_k_full + 8 * b, (kq >> 1) & 1u, wctx, kWaitKFull)) return false;
+        // S(kq) = Q_t K(kq)^T into buffer kq & 1, for the slot's item `item`
+        auto issue_qk = [&](const uint32_t kq, const uint32_t item, const bool last_of_item) -> bool {
+          const uint32_t idx = kv_index_k(kq), st = idx % NS;
+          if (!mbar_wait_warp(b_kv_full + 8 * st, (idx / NS) & 1u, wctx, kWaitKFull)) return false;
           tc_fence_after();
-          const uint32_t d = tm_s + 64u * b;
-          const uint32_t kb = k_lo + b * (Cfg::kKVBytes >> 4);
+          const uint32_t d = tm_s + 64u * (kq & 1u);
+          const uint32_t a_lo = q_lo + (item & 1u) * (Cfg::kQBytes >> 4);
+          const uint32_t kb = k_lo + st * (Cfg::kKVBytes >> 4);
 #pragma unroll
           for (int kk = 0; kk < D / 16; ++kk) {
             constexpr uint32_t kChunkQ = (BM * 128) >> 4, kChunkK = (BN * 128) >> 4;
             mma_ss(d, a_lo + (uint32_t)(kk >> 2) * kChunkQ + (uint32_t)(kk & 3) * 2,
                    kb + (uint32_t)(kk >> 2) * kChunkK + (uint32_t)(kk & 3) * 2, idesc_qk, kk > 0 ? 1u : 0u, issue);
           }
-          tc_commit(b_k_empty + 8 * b, issue);
-          tc_commit(b_s_full + 8 * b, issue);
-          if (last_of_item) tc_commit(b_q_empty, issue);     // last read of Q_t in this item
+          tc_commit(b_kv_empty + 8 * st, issue);
+          tc_commit(b_s_full + 8 * (kq & 1u), issue);
+          if (!Cfg::kStageInQ && last_of_item) tc_commit(bar_q_empty + 16 * t + 8 * (item & 1u), issue);   // last read of Q
           return true;
         };
         // The slot's tiles form one stream across items: while the softmax threads work on tile k,
         // the scores of the stream's next tile are computed, also when that tile opens the slot's
-        // next item (its Q was loaded as soon as this item's last scores had been issued).
+        // next item (its Q has been loaded and rotated under this item).
         int w = -1, n = 0, j = 0;
         {
           if (!mbar_wait_warp(b_item_full, 0u, wctx, kWaitItemFull)) ok = false;
@@ -687,38 +730,37 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             if (issue) mbar_arrive(b_item_empty);
           }
         }
-        if (ok && w >= 0) ok = mbar_wait_warp(bar_q_ready, 0u, wctx, kWaitQFull) && issue_qk(kc, n == 1);
+        if (ok && w >= 0) ok = mbar_wait_warp(b_q_ready, 0u, wctx, kWaitQFull) && issue_qk(kc, 0u, n == 1);
         while (ok && w >= 0) {
           const bool last_tile = (j + 1 == n);
           int w_next = w, n_next = n;
-          bool have = true, last_flag = (j + 2 == n);
           // With one tile per item the next item's scores would be issued before the previous item's
           // epilogue has read O_t; the softmax threads must not get that far ahead of it.
           if (j == 0 && last_tile && !(ok = mbar_wait_warp(b_o_empty, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
+          const uint32_t item = it_n + (last_tile ? 1u : 0u);         // whose tile comes next
           if (last_tile) {
-            const uint32_t item = it_n + 1u, ring = item % kRing;
+            const uint32_t ring = item % kRing;
             if (!(ok = mbar_wait_warp(b_item_full + 8 * ring, (item / kRing) & 1u, wctx, kWaitItemFull))) break;
             const volatile int* e = s_ring + (t * (int)kRing + (int)ring) * kRingInts;
             w_next = uniform(e[0]); n_next = uniform(e[3]);
             if (issue) mbar_arrive(b_item_empty + 8 * ring);
-            have = w_next >= 0;
-            last_flag = n_next == 1;
-            if (have && !(ok = mbar_wait_warp(bar_q_ready, item & 1u, wctx, kWaitQFull))) break;
+            if (w_next >= 0 && !(ok = mbar_wait_warp(b_q_ready + 8 * (item & 1u), (item >> 1) & 1u, wctx, kWaitQFull))) break;
           }
-          if (have && !(ok = issue_qk(kc + 1, last_flag))) break;
+          if (w_next >= 0 && !(ok = issue_qk(kc + 1, item, last_tile ? n_next == 1 : j + 2 == n))) break;
           // the previous item's epilogue must have read O_t before it is overwritten
           if (j == 0 && !last_tile && !(ok = mbar_wait_warp(b_o_empty, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
-          const uint32_t b = kc & 1u, parity = (kc >> 1) & 1u;
-          if (!(ok = mbar_wait_warp(b_p_full + 8 * b, parity, wctx, kWaitP))) break;
-          if (!(ok = mbar_wait_warp(b_v_full + 8 * b, parity, wctx, kWaitVFull))) break;
+          const uint32_t idx = kv_index_v(kc), st = idx % NS;
+          if (!(ok = mbar_wait_warp(b_kv_full + 8 * st, (idx / NS) & 1u, wctx, kWaitVFull))) break;
+          if (!(ok = mbar_wait_warp(b_p_full + 8 * (kc & 1u), (kc >> 1) & 1u, wctx, kWaitP))) break;
           tc_fence_after();            // O_t (+)= P(k) V(k)
-          const uint32_t a = tm_s + 64u * b;
-          const uint32_t vb = v_lo + b * (Cfg::kKVBytes >> 4);
+          const uint32_t a = tm_s + 64u * (kc & 1u);
+          const uint32_t vb = v_lo + st * (Cfg::kKVBytes >> 4);
           mma_ts(tm_o, a, vb, idesc_pv, j == 0 ? 0u : 1u, issue);
 #pragma unroll
           for (int kk = 1; kk < BN / 16; ++kk)
             mma_ts(tm_o, a + kk * 8, vb + (uint32_t)kk * ((16 * 128) >> 4), idesc_pv, 1u, issue);
-          tc_commit(b_v_empty + 8 * b, issue);
+          tc_commit(b_kv_empty + 8 * st, issue);
+          tc_commit(bar_pv_done + 8 * t, issue);
           ++kc;
           if (last_tile) {
             tc_commit(b_o_full, issue);
@@ -917,7 +959,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       volatile float* x_l = s_xchg + t * 128 + row;            // + 256 * (item & 1)
       bool ok = true;
       // key range [key_lo, key_hi] of this thread's row from a ring entry (empty for padding rows)
-      // (all lanes of the warp call it together: the prompts' start rows are loaded once per warp)
+      // (all lanes of the warp call it together: the prompts' start rows are loaded once per warp). The helper
+      // threads do this ahead of time; the softmax threads get the first key from them.
       auto row_range = [&](const volatile int* e, int& key_lo, int& key_hi) {
         const int i_row = e[4] + (row >> fs);
         int lo = e[14];
@@ -936,10 +979,13 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (!ok) break;
           const volatile int* e = s_ring + ring * kRingInts;
           const int w = e[0], item_kv_row0 = e[2], n_tiles = e[3];
-          int key_lo, key_hi;
-          if (w >= 0) row_range(e, key_lo, key_hi);
+          const int i_row = e[4] + (row >> fs), bin_used = e[12];
           mbar_arrive(bar_item_empty + 8 * ring);
           if (w < 0) break;
+          ok = mbar_wait_warp(bar_q_rot + 8 * (2 * t + (it_n & 1u)), (it_n >> 1) & 1u, wctx, kWaitQFull);
+          if (!ok) break;
+          const int key_lo = __float_as_int(x_l[256 * (it_n & 1u)]);
+          const int key_hi = i_row < bin_used ? i_row : 0;       // padding rows: key_lo = 1, an empty range
           float m_run = -INFINITY;      // running maximum of the row, in scaled log2 units
           float l_run = 0.f;            // running sum of exp2(s * c - m_run)
           for (int j = 0; j < n_tiles; ++j) {
@@ -960,7 +1006,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const bool cut = (warp_flags & 4u) != 0;
             const uint32_t sbuf = tcount & 1u;                   // tile k of the stream lives in S buffer k & 1
             const uint32_t tmem_sb = tmem_s + 64u * sbuf;
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_s_full + 8 * (2 * t + sbuf), (tcount >> 1) & 1u, wctx, kWaitS));
+            ok = mbar_wait_warp(bar_s_full + 8 * (2 * t + sbuf), (tcount >> 1) & 1u, wctx, kWaitS);
             if (!ok) break;
             tc_fence_after();
             uint32_t v[EPT];
@@ -1006,10 +1052,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const bool rescale = (m_new != m_run) && (m_run != -INFINITY);
             const float alpha = rescale ? fast_exp2(m_run - m_new) : 1.f;
             if (j > 0 && __any_sync(0xffffffffu, rescale)) {
-              // S(k) is computed ahead of P(k-1) V(k-1), so O_t is stable only once that product has
-              // been committed: the release of the V stage it read is the same event
-              const uint32_t kp = tcount - 1u;
-              ok = __all_sync(0xffffffffu, mbar_wait(bar_v_empty + 8 * (2 * t + (kp & 1u)), (kp >> 1) & 1u, wctx, kWaitVEmpty));
+              // S(k) is computed ahead of P(k-1) V(k-1): O_t is stable only once that product is there
+              ok = mbar_wait_warp(bar_pv_done + 8 * t, (tcount - 1u) & 1u, wctx, kWaitVEmpty);
               if (!ok) break;
               tc_fence_after();
 #pragma unroll 1
@@ -1080,17 +1124,25 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const volatile int* e = s_ring + ring * kRingInts;
           const int w = e[0], c_bin = e[1], c_q_row0 = e[4], c_head = e[9];
           int key_lo = 1, key_hi = 0;
-          if (w >= 0 && args.rope_table) row_range(e, key_lo, key_hi);
+          if (w >= 0) row_range(e, key_lo, key_hi);
           mbar_arrive(bar_item_empty + 8 * ring);
-          if (w >= 0 && args.rope_table) {
+          const uint32_t qb = 2u * (uint32_t)t + (it_n & 1u);      // Q tile of this item
+          // the O tile that was stored last has left its Q tile by now, or will soon: hand the tile back
+          if (Cfg::kStageInQ && it_n > 1 && lane == 0) {
+            tma_store_wait_read();
+            mbar_arrive(bar_q_empty + 8 * qb);
+          }
+          if (w >= 0) {
             // rotate row `row` of this item's Q in shared memory by the angles of its position, with
-            // the same fp32 arithmetic and rounding as the stand-alone kernel, then report Q_t ready
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_q_full + 8 * t, it_n & 1u, wctx, kWaitQFull));
+            // the same fp32 arithmetic and rounding as the stand-alone kernel, leave the row's first key
+            // where its row sum will be (this thread has read that of the item before the previous one
+            // from there), then report Q_t ready
+            ok = mbar_wait_warp(bar_q_full + 8 * qb, (it_n >> 1) & 1u, wctx, kWaitQFull);
             if (!ok) break;
             const int pos = key_hi - key_lo;             // < 0 for padding rows
-            if (pos > 0) {
+            if (args.rope_table && pos > 0) {
               constexpr int kUnits = D / 16;             // 16-byte (lower, upper) unit pairs per row
-              const uint32_t q_row = s_q + (uint32_t)t * Cfg::kQBytes + (uint32_t)row * 128;
+              const uint32_t q_row = s_q + qb * Cfg::kQBytes + (uint32_t)row * 128;
               // table[g][pos] = (cos, sin) of j = 2g and 2g + 1: consecutive rows read consecutive 16 bytes
               const float4* tab = reinterpret_cast<const float4*>(args.rope_table) + pos;
 #pragma unroll 1
@@ -1126,28 +1178,31 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
               asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
             }
-            mbar_arrive(bar_q_rot + 8 * t);
+            x_l[256 * (it_n & 1u)] = __int_as_float(key_lo);
+            mbar_arrive(bar_q_rot + 8 * qb);
           }
           if (it_n > 0) {
             // epilogue of the previous item: O_t / l -> bf16 -> shared memory (128-byte swizzle) -> TMA store
             const uint32_t pi = it_n - 1u;
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_o_full + 8 * t, pi & 1u, wctx, kWaitOFull));
+            ok = mbar_wait_warp(bar_o_full + 8 * t, pi & 1u, wctx, kWaitOFull);
             if (!ok) break;
-            ok = __all_sync(0xffffffffu, mbar_wait(bar_l_ready + 16 * t + 8 * (pi & 1u), (pi >> 1) & 1u, wctx, kWaitRowSum));
+            ok = mbar_wait_warp(bar_l_ready + 16 * t + 8 * (pi & 1u), (pi >> 1) & 1u, wctx, kWaitRowSum);
             if (!ok) break;
             tc_fence_after();
             const float l_row = x_l[256 * (pi & 1u)];
             const float inv_l = l_row > 0.f ? 1.f / l_row : 0.f;
             // Each warp stages and stores its own 32 rows (a 32-row TMA box), so the epilogue needs
-            // no rendezvous between warps: lane 0 issues the warp's stores and is the one to wait
-            // until the previous store has read the staging rows.
-            const uint32_t stage = s_stage_o + (uint32_t)t * Cfg::kStageOBytes + (uint32_t)quad * (32 * 128);
-            const uint32_t stage_row = stage + (uint32_t)lane * 128;
+            // no rendezvous between warps.
+            const uint32_t stage = (Cfg::kStageInQ ? s_q + (qb ^ 1u) * Cfg::kQBytes : s_stage_o + (uint32_t)t * Cfg::kStageOBytes) +
+                                   (uint32_t)quad * (32 * 128);
             const int p_row0 = p_q_row0 + ((32 * quad) >> fs);   // the warp's 32 tile rows: 32 >> fs bin rows x fold heads
 #pragma unroll 1
             for (int hh = 0; hh < D / 64; ++hh) {          // 64 columns (one TMA box) at a time
-              if (lane == 0) tma_store_wait_read();
-              __syncwarp();
+              const uint32_t box = stage + (uint32_t)hh * (BM * 128);
+              if (!Cfg::kStageInQ) {                       // the previous item's store must have read the staging rows
+                if (lane == 0) tma_store_wait_read();
+                __syncwarp();
+              }
               uint32_t ov[64];
               tmem_ld32(tmem_o + hh * 64, *reinterpret_cast<uint32_t(*)[32]>(&ov[0]));
               tmem_ld32(tmem_o + hh * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&ov[32]));
@@ -1158,7 +1213,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               }
 #pragma unroll
               for (int c16 = 0; c16 < 8; ++c16) {
-                const uint32_t addr = stage_row + (((uint32_t)c16 ^ ((uint32_t)lane & 7u)) << 4);
+                const uint32_t addr = box + (uint32_t)lane * 128 + (((uint32_t)c16 ^ ((uint32_t)lane & 7u)) << 4);
                 const uint32_t w0 = pack_bf16(__uint_as_float(ov[c16 * 8 + 0]) * inv_l, __uint_as_float(ov[c16 * 8 + 1]) * inv_l);
                 const uint32_t w1 = pack_bf16(__uint_as_float(ov[c16 * 8 + 2]) * inv_l, __uint_as_float(ov[c16 * 8 + 3]) * inv_l);
                 const uint32_t w2 = pack_bf16(__uint_as_float(ov[c16 * 8 + 4]) * inv_l, __uint_as_float(ov[c16 * 8 + 5]) * inv_l);
@@ -1168,11 +1223,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
               __syncwarp();
               if (lane == 0 && p_row0 < args.capacity) {
-                tma_store(&map_o, stage, p_head, p_row0, hh, p_bin);
+                tma_store(&map_o, box, p_head, p_row0, hh, p_bin);
                 asm volatile("cp.async.bulk.commit_group;" ::: "memory");
               }
             }
-            if (!ok) break;
           }
           if (w < 0) break;
           p_q_row0 = c_q_row0; p_head = c_head; p_bin = c_bin;
