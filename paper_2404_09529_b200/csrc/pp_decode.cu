@@ -16,9 +16,11 @@
 // both operands use the same, so a thread's 16-byte piece of a K row serves two products, and its 16-byte
 // pieces of four V rows (paired with byte permutes) serve eight. P is split into three bf16 numbers (24 bits
 // of it), so P V is as exact as with P in fp32.
-// Measured, whole step (D = 128): 256 prompts, 240 k cached tokens, 32 / 8 heads 568 -> 177 us (decode_kernel 159 us,
-// 6.2 TB/s, 96 % of the copy peak); 64 prompts, 17.5 k tokens, 32 / 32 heads 77 -> 59 us (54 us); ten prompts, 1009
-// tokens 41 -> 36 us (host-bound; the three kernels and the copy took 17.6 us, these two overlap to ~12).
+// Measured, whole step (D = 128): 256 prompts, 240 k cached tokens, 32 / 8 heads 568 -> 167 us (decode_kernel 159 us,
+// 6.2 TB/s, 96 % of the copy peak); 64 prompts, 17.5 k tokens, 32 / 32 heads 76 -> 57.5 us (54 us); ten prompts, 1009
+// tokens 38.5 -> 12.6 us, where the latencies in front of the first product count: the search for the prompt and
+// the angles run while the kernel before is finishing (programmatic dependent launch), and the loads of q, k
+// and the first keys and values are all issued before any is waited for (16.0 us without the two).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -222,14 +224,8 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Deco
   const int64_t base = pr.cache_off + (int64_t)kvh * pr.cap * D;
   const __nv_bfloat16 *kb = a.k_cache + base, *vb = a.v_cache + base;
 
-  // the first step's K and V are on their way while the queries are rotated
-  StepK<D> fk;
-  StepV<D> fv;
-  int key = key0 + kTileKeys * warp;
-  if (key < key_end) {
-    load_k<D>(fk, kb, key, key_end - 1, g, t);
-    load_v<D>(fv, vb, key, key_end - 1, g, t);
-  }
+  // Everything up to here, and the angles, come from the parameters alone (up to kInlineMany prompts): with a
+  // programmatic dependent launch this runs while the kernel before this one is finishing.
   if (tid < kHalf) {      // the position is >= 1; same reduction as the prefill kernels
     const double ang = (double)pr.length * a.inv_freq[tid];
     const double n = rint(ang * 0.15915494309189535);
@@ -240,31 +236,48 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Deco
     s_cos[tid] = cs;
     s_sin[tid] = sn;
   }
-  __syncthreads();
-  // heads of the group, zeros for the absent ones, and the new key; four (j, j + D/2) pairs at a time
-  for (int u = tid; u < (kMaxGroup + 1) * (kHalf / 4); u += kDecodeThreads) {
-    const int h = u / (kHalf / 4), j = 4 * (u - h * (kHalf / 4));
-    uint2 lo2 = make_uint2(0u, 0u), hi2 = make_uint2(0u, 0u);
-    if (h < a.group || (h == kMaxGroup && last_chunk)) {
+  pdl_wait();
+  // heads of the group, zeros for the absent ones, and the new key; four (j, j + D/2) pairs at a time. These and
+  // the first step's K and V are all on their way before any of them is used.
+  constexpr int kRotUnits = (kMaxGroup + 1) * (kHalf / 4), kRotTrips = (kRotUnits + kDecodeThreads - 1) / kDecodeThreads;
+  uint2 lo2[kRotTrips], hi2[kRotTrips];
+#pragma unroll
+  for (int x = 0; x < kRotTrips; ++x) {
+    const int u = tid + x * kDecodeThreads, h = u / (kHalf / 4), j = 4 * (u - h * (kHalf / 4));
+    lo2[x] = hi2[x] = make_uint2(0u, 0u);
+    if (u < kRotUnits && (h < a.group || (h == kMaxGroup && last_chunk))) {
       const __nv_bfloat16* src = h == kMaxGroup ? a.k_new + ((int64_t)i * a.n_kv_heads + kvh) * D
                                                 : a.q_new + ((int64_t)i * a.n_q_heads + kvh * a.group + h) * D;
-      lo2 = __ldg(reinterpret_cast<const uint2*>(src + j));
-      hi2 = __ldg(reinterpret_cast<const uint2*>(src + j + kHalf));
-      uint32_t* l32 = reinterpret_cast<uint32_t*>(&lo2);
-      uint32_t* h32 = reinterpret_cast<uint32_t*>(&hi2);
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const float2 x = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&l32[e]));
-        const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h32[e]));
-        const float ca = s_cos[j + 2 * e], sa = s_sin[j + 2 * e], cb = s_cos[j + 2 * e + 1], sb = s_sin[j + 2 * e + 1];
-        const __nv_bfloat162 rl = __floats2bfloat162_rn(__fmaf_rn(x.x, ca, -__fmul_rn(y.x, sa)), __fmaf_rn(x.y, cb, -__fmul_rn(y.y, sb)));
-        const __nv_bfloat162 rh = __floats2bfloat162_rn(__fmaf_rn(y.x, ca, __fmul_rn(x.x, sa)), __fmaf_rn(y.y, cb, __fmul_rn(x.y, sb)));
-        l32[e] = *reinterpret_cast<const uint32_t*>(&rl);
-        h32[e] = *reinterpret_cast<const uint32_t*>(&rh);
-      }
+      lo2[x] = __ldg(reinterpret_cast<const uint2*>(src + j));
+      hi2[x] = __ldg(reinterpret_cast<const uint2*>(src + j + kHalf));
     }
-    *reinterpret_cast<uint2*>(&s_q[h][j]) = lo2;
-    *reinterpret_cast<uint2*>(&s_q[h][j + kHalf]) = hi2;
+  }
+  StepK<D> fk;
+  StepV<D> fv;
+  int key = key0 + kTileKeys * warp;
+  if (key < key_end) {
+    load_k<D>(fk, kb, key, key_end - 1, g, t);
+    load_v<D>(fv, vb, key, key_end - 1, g, t);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int x = 0; x < kRotTrips; ++x) {
+    const int u = tid + x * kDecodeThreads, h = u / (kHalf / 4), j = 4 * (u - h * (kHalf / 4));
+    if (u >= kRotUnits) break;
+    uint32_t* l32 = reinterpret_cast<uint32_t*>(&lo2[x]);
+    uint32_t* h32 = reinterpret_cast<uint32_t*>(&hi2[x]);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float2 p = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&l32[e]));
+      const float2 y = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h32[e]));
+      const float ca = s_cos[j + 2 * e], sa = s_sin[j + 2 * e], cb = s_cos[j + 2 * e + 1], sb = s_sin[j + 2 * e + 1];
+      const __nv_bfloat162 rl = __floats2bfloat162_rn(__fmaf_rn(p.x, ca, -__fmul_rn(y.x, sa)), __fmaf_rn(p.y, cb, -__fmul_rn(y.y, sb)));
+      const __nv_bfloat162 rh = __floats2bfloat162_rn(__fmaf_rn(y.x, ca, __fmul_rn(p.x, sa)), __fmaf_rn(y.y, cb, __fmul_rn(p.y, sb)));
+      l32[e] = *reinterpret_cast<const uint32_t*>(&rl);
+      h32[e] = *reinterpret_cast<const uint32_t*>(&rh);
+    }
+    *reinterpret_cast<uint2*>(&s_q[h][j]) = lo2[x];
+    *reinterpret_cast<uint2*>(&s_q[h][j + kHalf]) = hi2[x];
   }
   __syncthreads();
   uint4 q[D / 32];        // head g, the pieces of a row that this thread's K pieces meet
@@ -359,29 +372,40 @@ decode_combine_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
   const int c0 = chunk_ptr_at(a, in, i), c1 = chunk_ptr_at(a, in, i + 1);
   if (c1 - c0 < 2 || head >= a.n_q_heads) return;
   pdl_wait();                           // the partial results come from the kernel before this one
-  float mm = -INFINITY;
-  for (int c = c0 + lane; c < c1; c += 32) mm = fmaxf(mm, a.part_ml[(int64_t)c * a.n_q_heads + head].x);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
-  float ll = 0.f, oo[E];
+  float mm = -INFINITY, ll = 0.f, oo[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) oo[e] = 0.f;
-#pragma unroll 4
-  for (int c = c0; c < c1; ++c) {
-    const int64_t at = (int64_t)c * a.n_q_heads + head;
-    const float2 ml = a.part_ml[at];
-    const float f = ex2(ml.x - mm);
-    ll += ml.y * f;
-    float p[E];
-    if constexpr (E == 4) {
-      const float4 x = *reinterpret_cast<const float4*>(a.part_o + at * D + E * lane);
-      p[0] = x.x; p[1] = x.y; p[2] = x.z; p[3] = x.w;
-    } else {
-      const float2 x = *reinterpret_cast<const float2*>(a.part_o + at * D + E * lane);
-      p[0] = x.x; p[1] = x.y;
-    }
+  for (int base = c0; base < c1; base += 32) {           // 32 chunks at a time: one (m, l) per lane
+    const int n = min(32, c1 - base);
+    const float2 ml = lane < n ? a.part_ml[(int64_t)(base + lane) * a.n_q_heads + head] : make_float2(-INFINITY, 0.f);
+    float m_new = ml.x;
 #pragma unroll
-    for (int e = 0; e < E; ++e) oo[e] += p[e] * f;
+    for (int o = 16; o > 0; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));
+    m_new = fmaxf(mm, m_new);
+    const float alpha = ex2(mm - m_new), f = ex2(ml.x - m_new);
+    mm = m_new;
+    float l = ml.y * f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    ll = ll * alpha + l;
+#pragma unroll
+    for (int e = 0; e < E; ++e) oo[e] *= alpha;
+    const float* src = a.part_o + ((int64_t)base * a.n_q_heads + head) * D + E * lane;
+    const int64_t stride = (int64_t)a.n_q_heads * D;
+#pragma unroll 8
+    for (int c = 0; c < n; ++c) {
+      const float fc = __shfl_sync(0xffffffffu, f, c);
+      float p[E];
+      if constexpr (E == 4) {
+        const float4 x = *reinterpret_cast<const float4*>(src + c * stride);
+        p[0] = x.x; p[1] = x.y; p[2] = x.z; p[3] = x.w;
+      } else {
+        const float2 x = *reinterpret_cast<const float2*>(src + c * stride);
+        p[0] = x.x; p[1] = x.y;
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) oo[e] += p[e] * fc;
+    }
   }
   uint32_t r[E / 2];
 #pragma unroll
@@ -443,11 +467,12 @@ void fill_table(const DecodeLayout& L, const int32_t* lengths, int32_t k, const 
 
 template <int D, int N>
 cudaError_t launch_decode(const DecodeArgs& a, const DecodeInline<N>& in, const DecodeLayout& L, cudaStream_t s) {
-  decode_kernel<D, N><<<dim3((unsigned)L.n_chunks, (unsigned)a.n_kv_heads), kDecodeThreads, 0, s>>>(a, in);
-  if (L.n_chunks == a.n_prompts) return cudaGetLastError();       // one chunk each: O is complete
+  const dim3 chunks((unsigned)L.n_chunks, (unsigned)a.n_kv_heads);
+  const cudaError_t first = launch_dependent(decode_kernel<D, N>, chunks, dim3(kDecodeThreads), 0, s, a, in);
+  if (first != cudaSuccess || L.n_chunks == a.n_prompts) return first;       // one chunk each: O is complete
   const dim3 grid((unsigned)a.n_prompts, (unsigned)((a.n_q_heads + kDecodeWarps - 1) / kDecodeWarps));
   const cudaError_t e = launch_dependent(decode_combine_kernel<D, N>, grid, dim3(kDecodeThreads), 0, s, a, in);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return e;
 }
 template <int N>
 cudaError_t launch_decode_d(int head_dim, const DecodeArgs& a, const DecodeInline<N>& in, const DecodeLayout& L, cudaStream_t s) {
