@@ -96,16 +96,19 @@ extern "C" int pp_prefill_attention(const pp_attn_params* params, const int32_t*
                                 static_cast<int32_t*>(host_workspace), workspace_bytes / sizeof(int32_t), &L);
   if (st != PP_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaMemcpyAsync(workspace, host_workspace, sizeof(int32_t) * (size_t)L.total_ints,
-                                  cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return pp::note_cuda_error((int)e, "table upload");
+  // a small table travels in the kernels' parameters (the rotation kernel resets the work counter then)
+  const int32_t* small = do_rope && L.independent_slots && L.total_ints <= pp::kInlineInts ? static_cast<int32_t*>(host_workspace) : nullptr;
+  if (!small) {
+    cudaError_t e = cudaMemcpyAsync(workspace, host_workspace, sizeof(int32_t) * (size_t)L.total_ints, cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return pp::note_cuda_error((int)e, "table upload");
+  }
   int32_t* d_table = static_cast<int32_t*>(workspace);
   if (do_rope) {
-    st = pp::launch_rope(*params, d_table, L, q, k_, stream);
+    st = pp::launch_rope(*params, d_table, L, small, q, k_, stream);
     if (st != PP_OK) return st;
   }
   if (do_attn) {
-    st = pp::launch_attention(*params, d_table, L, q, k_, v, o, nullptr, do_rope, device_status, stream);
+    st = pp::launch_attention(*params, d_table, L, small, q, k_, v, o, nullptr, do_rope, device_status, stream);
     if (st != PP_OK) return st;
   }
   return PP_OK;
@@ -150,8 +153,9 @@ extern "C" size_t pp_prefill_fused_host_bytes(const pp_attn_params* params, int3
 
 namespace pp {
 namespace {
-// The kernels of the fused path on tables that are (or will be, in stream order) in `workspace`.
-int launch_fused_kernels(const pp_attn_params& p, const TableLayout& L, const FusedLayout& f, const void* q,
+// The kernels of the fused path on tables that are (or will be, in stream order) in `workspace`, or on the small
+// table in host memory that is handed to them as a parameter.
+int launch_fused_kernels(const pp_attn_params& p, const TableLayout& L, const FusedLayout& f, const int32_t* small, const void* q,
                          void* k_, const void* v, void* o, void* k_cache, void* v_cache, void* workspace,
                          int32_t* device_status, void* stream) {
   int st;
@@ -161,13 +165,13 @@ int launch_fused_kernels(const pp_attn_params& p, const TableLayout& L, const Fu
     if ((st = launch_rope_table(p, rope_table, stream)) != PP_OK) return st;
   }
   if (!(p.flags & PP_FLAG_SKIP_ROPE)) {       // flag: k_ is rotated and the caches are filled already
-    st = launch_rope_unpack(p, d_table, L, (int32_t)f.off_true_len, (int32_t)f.off_cap,
+    st = launch_rope_unpack(p, d_table, L, small, (int32_t)f.off_true_len, (int32_t)f.off_cap,
                             (int32_t)f.off_cache_off, rope_table, k_, v, k_cache, v_cache, stream);
     if (st != PP_OK) return st;
   }
   if (p.flags & PP_FLAG_ROPE_ONLY) return PP_OK;
   // the attention kernel rotates every Q tile in shared memory, so Q is read from HBM once
-  return launch_attention(p, d_table, L, q, k_, v, o, rope_table, !(p.flags & PP_FLAG_SKIP_ROPE), device_status, stream);
+  return launch_attention(p, d_table, L, small, q, k_, v, o, rope_table, !(p.flags & PP_FLAG_SKIP_ROPE), device_status, stream);
 }
 
 // pp_prefill_fused, optionally cut in two: kUploadOnly validates, builds and uploads the tables,
@@ -184,7 +188,7 @@ int prefill_fused_impl(const pp_attn_params* params, const int32_t* bin_seg_ptr,
   if (st != PP_OK) return st;
   if (step == TableStep::kLaunchOnly) {
     const FusedLayout f = fused_layout(*params, k);
-    return launch_fused_kernels(*params, *layout, f, q, k_, v, o, k_cache, v_cache, workspace, device_status, stream);
+    return launch_fused_kernels(*params, *layout, f, nullptr, q, k_, v, o, k_cache, v_cache, workspace, device_status, stream);
   }
   if (!q || !k_ || !v || !o || !k_cache || !v_cache || !cache_off || !cache_cap || !seg_prompt || !lengths ||
       !workspace || !host_workspace)
@@ -214,12 +218,15 @@ int prefill_fused_impl(const pp_attn_params* params, const int32_t* bin_seg_ptr,
                             params->n_q_heads, params->n_kv_heads, h, f.table_ints, &L);
   if (st != PP_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaError_t e = cudaMemcpyAsync(workspace, host_workspace, sizeof(int32_t) * f.upload_ints,
-                                  cudaMemcpyHostToDevice, s);
-  if (e != cudaSuccess) return note_cuda_error((int)e, "table upload");
+  const int32_t* small = step == TableStep::kUploadAndLaunch && !(params->flags & PP_FLAG_SKIP_ROPE) && L.independent_slots &&
+                                 f.upload_ints <= (size_t)kInlineInts ? h : nullptr;
+  if (!small) {
+    cudaError_t e = cudaMemcpyAsync(workspace, host_workspace, sizeof(int32_t) * f.upload_ints, cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return note_cuda_error((int)e, "table upload");
+  }
   if (layout) *layout = L;
   if (step == TableStep::kUploadOnly) return PP_OK;
-  return launch_fused_kernels(*params, L, f, q, k_, v, o, k_cache, v_cache, workspace, device_status, stream);
+  return launch_fused_kernels(*params, L, f, small, q, k_, v, o, k_cache, v_cache, workspace, device_status, stream);
 }
 }  // namespace
 }  // namespace pp

@@ -45,6 +45,7 @@
 
 #include <cmath>
 #include <cstdlib>
+#include <cstring>
 #include <type_traits>
 
 #include "pp_device_once.h"
@@ -397,7 +398,6 @@ __host__ __device__ constexpr uint32_t instr_desc(uint32_t n, bool b_mn_major) {
 }
 
 struct AttnArgs {
-  const int32_t* table;
   int32_t* counter;              // global work counter (a header word of the table)
   int32_t off_bin_seg_ptr, off_bin_used, off_seg_start, off_items;
   int32_t n_items;               // geometry entries in the work list
@@ -425,13 +425,14 @@ struct Work {
   int bin_used, seg_end, key_lo[2], seg_first[2], single_seg;
 };
 
-__device__ __forceinline__ void decode_work(const AttnArgs& a, int w, Work& wk) {
+template <class Table>
+__device__ __forceinline__ void decode_work(const AttnArgs& a, const Table& tab, int w, Work& wk) {
   const int sub = w % a.subs;
   const int rest = w / a.subs;
   const int gi = rest % a.n_items;
   wk.kv_head = rest / a.n_items;
-  const int4* p = reinterpret_cast<const int4*>(a.table + a.off_items + kItemInts * gi);
-  const int4 x = __ldg(p), y = __ldg(p + 1);
+  const int at = a.off_items + kItemInts * gi;
+  const int4 x = tab.i128(at), y = tab.i128(at + 4);
   wk.bin = x.x; wk.kv_row0 = x.y; wk.n = x.z; wk.q_row0[0] = x.w; wk.q_row0[1] = y.x;
   wk.jb[0] = 0; wk.je[0] = y.z;
   wk.jb[1] = y.y; wk.je[1] = (y.x >= 0) ? x.z : y.y;       // unused slot: empty range
@@ -444,19 +445,21 @@ __device__ __forceinline__ void decode_work(const AttnArgs& a, int w, Work& wk) 
   }
 }
 
-// The next work index of a CTA or slot, -1 when there is none left (a whole warp calls).
-__device__ __forceinline__ int draw_work(const AttnArgs& a, int lane) {
+// The next work index of a CTA or slot, -1 when there is none left (a whole warp calls). The first one is the
+// drawer's own number, of `drawers` (no round trip to the counter in front of the first loads).
+__device__ __forceinline__ int draw_work(const AttnArgs& a, int lane, int drawers) {
   int w = 0;
-  if (lane == 0) w = atomicAdd(a.counter, 1);
+  if (lane == 0) w = drawers + atomicAdd(a.counter, 1);
   w = __shfl_sync(0xffffffffu, w, 0);
   return w < a.total_work ? w : -1;
 }
 
 // Second half of a work-list entry: what the softmax threads need to place their rows.
-__device__ __forceinline__ void decode_rows(const AttnArgs& a, int w, Work& wk) {
+template <class Table>
+__device__ __forceinline__ void decode_rows(const AttnArgs& a, const Table& tab, int w, Work& wk) {
   const int gi = (w / a.subs) % a.n_items;
-  const int4* p = reinterpret_cast<const int4*>(a.table + a.off_items + kItemInts * gi);
-  const int4 x = __ldg(p + 2), y = __ldg(p + 3);
+  const int at = a.off_items + kItemInts * gi;
+  const int4 x = tab.i128(at + 8), y = tab.i128(at + 12);
   wk.bin_used = x.x; wk.seg_end = x.y; wk.key_lo[0] = x.z; wk.key_lo[1] = x.w;
   wk.seg_first[0] = y.x; wk.seg_first[1] = y.y; wk.single_seg = y.z;
 }
@@ -475,15 +478,16 @@ enum WaitCode { kWaitItemFull = 1, kWaitItemEmpty, kWaitQFull, kWaitQEmpty, kWai
                 kWaitVFull, kWaitVEmpty, kWaitS, kWaitP, kWaitOFull, kWaitOEmpty, kWaitPair, kWaitRowSum };
 
 // Start row of the prompt that holds bin-local row `i_row`, among the prompts seg_begin .. seg_end-1
-// of a bin whose start rows (ascending) are in `starts`; `lo` if none of them starts at or before the
+// of a bin whose start rows (ascending) are in the table from `starts` on; `lo` if none of them starts at or before the
 // row. All 32 lanes call it with the same range and with row_max = the largest row of the warp: the
 // starts are loaded 32 at a time, one per lane, and handed round with shuffles, so the walk costs one
 // memory round trip per 32 prompts.
-__device__ __forceinline__ int seg_start_at(const int32_t* starts, int seg_begin, int seg_end, int i_row, int row_max,
+template <class Table>
+__device__ __forceinline__ int seg_start_at(const Table& tab, int starts, int seg_begin, int seg_end, int i_row, int row_max,
                                             int lo, int lane) {
   for (int base = seg_begin; base < seg_end; base += 32) {
     const int cnt = min(32, seg_end - base);
-    const int mine = (lane < cnt) ? __ldg(starts + base + lane) : 0x7fffffff;
+    const int mine = (lane < cnt) ? tab.i32(starts + base + lane) : 0x7fffffff;
     for (int sg = 0; sg < cnt; ++sg) {
       const int st = __shfl_sync(0xffffffffu, mine, sg);
       if (st > row_max) return lo;                     // warp-uniform: no later prompt starts in these rows
@@ -503,11 +507,11 @@ __device__ __forceinline__ int seg_start_at(const int32_t* starts, int seg_begin
 __device__ __forceinline__ uint32_t kv_index_k(uint32_t k) { return k ? 2u * k - 1u : 0u; }
 __device__ __forceinline__ uint32_t kv_index_v(uint32_t k) { return 2u * k + 2u; }
 
-template <int D, bool kIndep>
+template <int D, bool kIndep, class Table>
 __global__ void __launch_bounds__(kAttnThreads, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
-                 const AttnArgs args) {
+                 const __grid_constant__ AttnArgs args, const __grid_constant__ Table tab) {
   constexpr int BN = kIndep ? kTileNShort : kTileN;
   using Cfg = AttnCfg<D, BN>;
   constexpr int NK = Cfg::kKStages, NV = Cfg::kVStages;
@@ -628,8 +632,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         volatile int* ring_base = s_ring + t * (int)kRing * kRingInts;
         auto announce = [&](const uint32_t it, const int w, Work& wk) -> bool {      // w < 0: there is no item `it`
           if (w >= 0) {
-            decode_work(args, w, wk);
-            decode_rows(args, w, wk);
+            decode_work(args, tab, w, wk);
+            decode_rows(args, tab, w, wk);
           }
           const uint32_t ring = it % kRing;
           if (!mbar_wait_warp(bar_item_empty + ring_bar + 8 * ring, ((it / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) return false;
@@ -656,13 +660,15 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           tma_load(s_kv + ((uint32_t)t * NS + st) * Cfg::kKVBytes, map, bar_kv_full + bar, wk.kv_head, wk.kv_row0 + j * BN, wk.bin, issue);
           return true;
         };
-        int w = draw_work(args, lane);
+        const int drawers = 2 * (int)gridDim.x;
+        int w = (int)blockIdx.x + t * (int)gridDim.x;
+        if (w >= args.total_work) w = -1;
         Work wk, wk_next;
         bool ok = announce(0, w, wk);
         if (ok && w >= 0) ok = load_q(0, wk) && load_kv(&map_k, kv_index_k(0), wk, 0);
         uint32_t kc = 0;                      // key tiles of the slot's stream whose V has been loaded
         for (uint32_t it_n = 0; ok && w >= 0; ++it_n) {
-          const int w_next = draw_work(args, lane);
+          const int w_next = draw_work(args, lane, drawers);
           if (!(ok = announce(it_n + 1u, w_next, wk_next))) break;
           for (int j = 0; ok && j < wk.n; ++j, ++kc) {
             if (j + 1 < wk.n) ok = load_kv(&map_k, kv_index_k(kc + 1), wk, j + 1);
@@ -778,10 +784,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t it_n = 0, kc = 0;
       Work wk;
       while (true) {
-        const int w = draw_work(args, lane);
+        const int w = it_n == 0 ? (int)blockIdx.x : draw_work(args, lane, (int)gridDim.x);   // (at most one CTA per index)
         if (w >= 0) {
-          decode_work(args, w, wk);
-          decode_rows(args, w, wk);
+          decode_work(args, tab, w, wk);
+          decode_rows(args, tab, w, wk);
         }
         const uint32_t ring = it_n % kRing;
         if (!mbar_wait_warp(bar_item_empty + 8 * ring, ((it_n / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) break;
@@ -952,7 +958,6 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       // rotate the next item's Q in shared memory (fused path) and run the epilogue of the previous
       // item, both off the softmax threads' critical path.
       const float c_scale = args.scale_log2;
-      const int32_t* tb = args.table;
       const int fs = args.fold_shift;                  // tile row m holds bin row q_row0 + (m >> fs)
       const uint32_t ring0 = (uint32_t)t * kRing;
       // row sums travel from the softmax thread to the helper of the same row, double-buffered by item
@@ -965,7 +970,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const int i_row = e[4] + (row >> fs);
         int lo = e[14];
         if (!(e[18] & 1))
-          lo = seg_start_at(tb + args.off_seg_start, e[16] + 1, e[13], i_row, e[4] + ((quad * 32 + 31) >> fs), lo, lane);
+          lo = seg_start_at(tab, args.off_seg_start, e[16] + 1, e[13], i_row, e[4] + ((quad * 32 + 31) >> fs), lo, lane);
         const bool real = i_row < e[12];
         key_lo = real ? lo : 1;
         key_hi = real ? i_row : 0;
@@ -1252,7 +1257,6 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       return r;
     };
     const float c_scale = args.scale_log2;
-    const int32_t* tb = args.table;
     uint32_t it_n = 0, tcount = 0;
     bool ok = true;
     // Rotates this thread's part of row `row` of Q_t in shared memory by the angles of position `pos`
@@ -1329,7 +1333,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       if (used) {                                      // warp-uniform
         int lo = key_lo_t;
         if (!(single_seg & 1))                         // several prompts in this tile: find this row's
-          lo = seg_start_at(tb + args.off_seg_start, seg_first_t + 1, seg_end, i_row, i_row - lane + 31, lo, lane);
+          lo = seg_start_at(tab, args.off_seg_start, seg_first_t + 1, seg_end, i_row, i_row - lane + 31, lo, lane);
         if (i_row < bin_used) { key_lo = lo; key_hi = i_row; }
       }
       // |q|^2 up to which every score of a row stays below the bound (0 if nothing is known about the keys)
@@ -1618,8 +1622,8 @@ int sm_count() {
   return cached;
 }
 
-template <int D, bool kIndep>
-int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const void* q,
+template <int D, bool kIndep, class Table>
+int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const Table& tab, const void* q,
                        const void* k, const void* v, void* o, const void* rope_table, bool have_norms,
                        int32_t* device_status, cudaStream_t stream) {
   constexpr int BN = kIndep ? kTileNShort : kTileN;
@@ -1638,7 +1642,7 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return note_cuda_error(-1, "cudaGetDevice");
   if (!configured.done(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(attention_kernel<D, kIndep>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(attention_kernel<D, kIndep, Table>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          Cfg::kSmemBytes);
     if (e != cudaSuccess) return note_cuda_error((int)e, "cudaFuncSetAttribute(smem)");
     configured.mark(dev);
@@ -1646,7 +1650,6 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   const int sms = sm_count();
   if (sms <= 0) return note_cuda_error(-1, "multiprocessor count");
   AttnArgs a;
-  a.table = d_table;
   a.counter = d_table + kHeaderCounter;
   a.off_bin_seg_ptr = L.bin_seg_ptr;
   a.off_bin_used = L.bin_used;
@@ -1674,8 +1677,8 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.status = device_status;
   a.wait_limit_ns = wait_limit_ns();
   const unsigned grid = (unsigned)(total < sms ? total : sms);
-  const cudaError_t launch_err = launch_dependent(attention_kernel<D, kIndep>, dim3(grid), dim3(kAttnThreads),
-                                                  (size_t)Cfg::kSmemBytes, stream, mq, mk, mv, mo, a);
+  const cudaError_t launch_err = launch_dependent(attention_kernel<D, kIndep, Table>, dim3(grid), dim3(kAttnThreads),
+                                                  (size_t)Cfg::kSmemBytes, stream, mq, mk, mv, mo, a, tab);
   const cudaError_t e = launch_err != cudaSuccess ? launch_err : cudaGetLastError();
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "attention kernel launch");
 }
@@ -1688,16 +1691,23 @@ int launch_bounded_wait_selftest(int32_t* device_status, uint64_t limit_ns, void
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "self-test kernel launch");
 }
 
-int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const void* q,
+int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table, const void* q,
                      const void* k, const void* v, void* o, const void* rope_table, bool have_norms,
                      int32_t* device_status, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (L.independent_slots) {
-    if (p.head_dim == 128) return launch_attention_t<128, true>(p, d_table, L, q, k, v, o, rope_table, have_norms, device_status, s);
-    return launch_attention_t<64, true>(p, d_table, L, q, k, v, o, rope_table, have_norms, device_status, s);
+  if (inline_table) {                 // independent mode only
+    TableInline tab;
+    std::memcpy(tab.w, inline_table, sizeof(int32_t) * (size_t)(L.total_ints < kInlineInts ? L.total_ints : kInlineInts));
+    if (p.head_dim == 128) return launch_attention_t<128, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
+    return launch_attention_t<64, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
   }
-  if (p.head_dim == 128) return launch_attention_t<128, false>(p, d_table, L, q, k, v, o, rope_table, have_norms, device_status, s);
-  return launch_attention_t<64, false>(p, d_table, L, q, k, v, o, rope_table, have_norms, device_status, s);
+  const TableInMemory tab{d_table};
+  if (L.independent_slots) {
+    if (p.head_dim == 128) return launch_attention_t<128, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
+    return launch_attention_t<64, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
+  }
+  if (p.head_dim == 128) return launch_attention_t<128, false>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
+  return launch_attention_t<64, false>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
 }
 
 }  // namespace pp

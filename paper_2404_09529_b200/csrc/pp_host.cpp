@@ -326,7 +326,7 @@ int build_prefill_tables(int32_t n_bins, int32_t capacity, const int32_t* bin_se
   out[1] = L.n_items;
   out[2] = n_bins;
   out[3] = capacity;
-  out[4] = k;
+  out[kHeaderSegments] = k;
   out[5] = L.bin_seg_ptr;
   out[6] = L.bin_used;
   out[7] = L.seg_start;

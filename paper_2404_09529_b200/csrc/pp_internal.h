@@ -13,6 +13,7 @@ constexpr int kTileM = 128;      // query rows per work item (tcgen05 MMA M)
 constexpr int kTileN = 128;      // key rows per inner step (tcgen05 MMA N of Q.K^T), shared-stream mode
 constexpr int kTileNShort = 64;  // the same in independent-slot mode (short work items)
 constexpr int kHeaderInts = 16;  // table header, see build_prefill_tables
+constexpr int kHeaderSegments = 4;   // header word with the number of segments
 constexpr int kHeaderCounter = 10;   // header word the persistent CTAs draw work indices from
 constexpr int kItemInts = 16;
 constexpr int kMaxFold = 8;      // most query heads of one KV head folded into the rows of a query tile
@@ -65,17 +66,20 @@ int note_cuda_error(int cuda_error, const char* what);
 // Kernel launchers (device pointers, stream = cudaStream_t as void*). Return a PP_* status.
 // Rotates q and k in place; in the shared-stream mode it also leaves the largest |k|^2 and |q|^2 of every
 // head in the table (L.norms).
-int launch_rope(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, void* q, void* k, void* stream);
+// inline_table (here and below): null, or the host copy of a table that was not uploaded and travels in the
+// kernel's parameters; the rotation kernel then resets the work counter in d_table.
+int launch_rope(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table, void* q, void* k,
+                void* stream);
 // rope_table: device [D/4][capacity][2] (cos, sin) pairs, or null. When given, q holds the raw
 // queries and the kernel rotates each Q tile in shared memory before use. have_norms: a rotation kernel
 // of the same call has filled the norms of the table (of the keys, and without rope_table of the queries).
-int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayout& L,
+int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
                      const void* q, const void* k, const void* v, void* o, const void* rope_table,
                      bool have_norms, int32_t* device_status, void* stream);
 // Fused K rotation + UNPACK; the three offsets locate per-segment arrays inside the table
 // (true length, cache capacity: int32; cache element offset: int64). In the shared-stream mode it also leaves
 // the largest |k|^2 of every KV head in the table (L.norms).
-int launch_rope_unpack(const pp_attn_params& p, int32_t* d_table, const TableLayout& L,
+int launch_rope_unpack(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
                        int32_t off_true_len, int32_t off_cap, int32_t off_cache_off, const void* rope_table,
                        void* k, const void* v, void* k_cache, void* v_cache, void* stream);
 // Fills rope_table for positions 0 .. capacity-1.
@@ -98,7 +102,28 @@ int launch_bounded_wait_selftest(int32_t* device_status, uint64_t limit_ns, void
 // cache_cap[k], cache_off as int64[k] (8-byte aligned).
 size_t unpack_table_bytes(int32_t k);
 
+// A table of at most this many ints is not uploaded but handed to the kernels as a parameter (independent mode:
+// the shared-stream mode wants words of it zeroed in memory). Without the copy, the gap behind it and the wait
+// for it a step of 8 prompts on 4 heads takes 13.5 us instead of 16.9, one of 16 prompts on 32 heads 54 instead
+// of 65 (the rotation kernel's look-ups then run under the end of the kernel before). Larger tables would
+// slow every launch down.
+constexpr int kInlineInts = 896;
+
 #ifdef __CUDACC__
+// The prefill table as the kernels see it.
+struct TableInMemory {
+  const int32_t* p;
+  __device__ __forceinline__ int32_t i32(int i) const { return __ldg(p + i); }
+  __device__ __forceinline__ int4 i128(int i) const { return __ldg(reinterpret_cast<const int4*>(p + i)); }
+  __device__ __forceinline__ int64_t i64(int base, int i) const { return __ldg(reinterpret_cast<const long long*>(p + base) + i); }
+};
+struct alignas(16) TableInline {
+  int32_t w[kInlineInts];
+  __device__ __forceinline__ int32_t i32(int i) const { return w[i]; }
+  __device__ __forceinline__ int4 i128(int i) const { return *reinterpret_cast<const int4*>(w + i); }
+  __device__ __forceinline__ int64_t i64(int base, int i) const { return *reinterpret_cast<const int64_t*>(w + base + 2 * i); }
+};
+
 // Programmatic dependent launch. A kernel of the path that is launched with launch_dependent() may
 // start while the kernel before it in the stream is still finishing: its blocks are scheduled once
 // every block of that kernel has called pdl_launch_dependents() (or exited), run their set-up, and

@@ -4,6 +4,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <cstring>
+
 #include "pp_internal.h"
 
 namespace pp {
@@ -63,10 +65,11 @@ __device__ __forceinline__ float sum_squares(const uint4& lo, const uint4& hi) {
 }
 
 // norms: null, or [Hkv] then [Hq] words that receive the largest |k|^2 / |q|^2 of each head.
-template <int D>
+// counter: null, or the work counter to reset for the attention kernel.
+template <int D, class Table>
 __global__ void __launch_bounds__(kRopeThreads)
-rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32_t* norms,
-            const int32_t* table, int32_t off_bin_seg_ptr, int32_t off_bin_used,
+rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32_t* norms, int32_t* counter,
+            const __grid_constant__ Table tab, int32_t off_bin_seg_ptr, int32_t off_bin_used,
             int32_t off_seg_start, int32_t n_bins, int32_t capacity, int32_t n_q_heads,
             int32_t n_kv_heads, const __grid_constant__ RopeFreq freq) {
   constexpr int kHalf = D / 2;
@@ -90,14 +93,14 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32
     if (row < n_rows) {
       const int32_t b = (int32_t)(row / capacity);
       const int32_t t = (int32_t)(row - (int64_t)b * capacity);
-      if (t < table[off_bin_used + b]) {
+      if (t < tab.i32(off_bin_used + b)) {
         // last segment of bin b whose start row is <= t
-        int32_t lo = table[off_bin_seg_ptr + b], hi = table[off_bin_seg_ptr + b + 1] - 1;
+        int32_t lo = tab.i32(off_bin_seg_ptr + b), hi = tab.i32(off_bin_seg_ptr + b + 1) - 1;
         while (lo < hi) {
           const int32_t mid = (lo + hi + 1) >> 1;
-          if (table[off_seg_start + mid] <= t) lo = mid; else hi = mid - 1;
+          if (tab.i32(off_seg_start + mid) <= t) lo = mid; else hi = mid - 1;
         }
-        pos = t - table[off_seg_start + lo];
+        pos = t - tab.i32(off_seg_start + lo);
       }
     }
     s_pos[tid] = pos;
@@ -120,6 +123,8 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32
     s_cos[r][j] = cs;
     s_sin[r][j] = sn;
   }
+  pdl_wait();                   // (the set-up above reads parameters or an uploaded table only)
+  if (counter && blockIdx.x == 0 && tid == 0) *counter = 0;
   __syncthreads();
 
   const int units_per_row = n_heads * kUnitsPerHead;
@@ -186,13 +191,16 @@ struct SegExt {                    // per-segment arrays appended to the prefill
 // where it is at most 2 KB, so that a block always has tens of KB to move for its set-up cost.
 constexpr int kRuRowsWide = 8, kRuRowsNarrow = 32;
 constexpr int kRuNarrowRowElems = 1024;   // n_kv_heads * D up to which a row counts as narrow
+// ... and only where that still gives every SM a few blocks: a few hundred rows in blocks of 32 leave most of the chip
+// idle (448 rows of 4 heads, D = 64: 14 blocks; with 56 blocks of 8 rows and the table as a parameter 5.8 -> 3.3 us).
+constexpr int64_t kRuNarrowRows = 32 * 148 * 4;
 constexpr int kRuV = 8;      // 16-byte V copies in flight per thread
 constexpr int kRuK = 2;      // (lower, upper) K pairs in flight per thread
-template <int D, int kRuRows>
+template <int D, int kRuRows, class Table>
 __global__ void __launch_bounds__(kRopeThreads)
 rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, uint32_t* norms,
-                   __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
-                   const int32_t* table, int32_t off_bin_seg_ptr, int32_t off_bin_used,
+                   int32_t* counter, __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
+                   const __grid_constant__ Table tab, int32_t off_bin_seg_ptr, int32_t off_bin_used,
                    int32_t off_seg_start, SegExt ext, const float2* __restrict__ rope_table,
                    int32_t n_bins, int32_t capacity, int32_t n_kv_heads) {
   constexpr int kHalf = D / 2;
@@ -217,17 +225,16 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
     if (row < n_rows) {
       const int32_t b = (int32_t)(row / capacity);
       const int32_t t = (int32_t)(row - (int64_t)b * capacity);
-      if (t < table[off_bin_used + b]) {
-        int32_t lo = table[off_bin_seg_ptr + b], hi = table[off_bin_seg_ptr + b + 1] - 1;
+      if (t < tab.i32(off_bin_used + b)) {
+        int32_t lo = tab.i32(off_bin_seg_ptr + b), hi = tab.i32(off_bin_seg_ptr + b + 1) - 1;
         while (lo < hi) {
           const int32_t mid = (lo + hi + 1) >> 1;
-          if (table[off_seg_start + mid] <= t) lo = mid; else hi = mid - 1;
+          if (tab.i32(off_seg_start + mid) <= t) lo = mid; else hi = mid - 1;
         }
-        pos = t - table[off_seg_start + lo];
-        if (pos < table[ext.off_true_len + lo]) {   // rows past the prompt's true length are not cached
-          const int64_t* coff = reinterpret_cast<const int64_t*>(table + ext.off_cache_off);
-          stride = (int64_t)table[ext.off_cap + lo] * D;
-          dst = coff[lo] + (int64_t)pos * D;
+        pos = t - tab.i32(off_seg_start + lo);
+        if (pos < tab.i32(ext.off_true_len + lo)) {   // rows past the prompt's true length are not cached
+          stride = (int64_t)tab.i32(ext.off_cap + lo) * D;
+          dst = tab.i64(ext.off_cache_off, lo) + (int64_t)pos * D;
         }
       }
     }
@@ -237,6 +244,7 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
   }
   __syncthreads();
   pdl_wait();                   // the rotation table is written by the kernel before this one
+  if (counter && blockIdx.x == 0 && tid == 0) *counter = 0;
   // each row's D/2 (cos, sin) pairs once, for all heads: D/4 16-byte loads per row, one per thread
   for (int u = tid; u < kRuRows * (D / 4); u += kRopeThreads) {
     const int r = u / (D / 4), g = u - r * (D / 4);
@@ -335,6 +343,49 @@ RopeFreq make_freq(const pp_attn_params& p) {
   return freq;
 }
 
+template <class Table>
+int launch_rope_unpack_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const Table& tab, int32_t* counter,
+                         const SegExt& ext, const void* rope_table, void* k, const void* v, void* k_cache, void* v_cache,
+                         cudaStream_t s) {
+  const int64_t n_rows = (int64_t)p.n_bins * p.capacity;
+  const bool narrow = p.n_kv_heads * p.head_dim <= kRuNarrowRowElems && n_rows >= kRuNarrowRows;
+  const int rows = narrow ? kRuRowsNarrow : kRuRowsWide;
+  const unsigned grid = (unsigned)((n_rows + rows - 1) / rows);
+  auto launch = [&](auto kernel) {
+    return launch_dependent(kernel, dim3(grid), dim3(kRopeThreads), 0, s, (__nv_bfloat16*)k, (const __nv_bfloat16*)v,
+                            norm_words(p, d_table, L), counter, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, tab,
+                            L.bin_seg_ptr, L.bin_used, L.seg_start, ext, (const float2*)rope_table, p.n_bins, p.capacity,
+                            p.n_kv_heads);
+  };
+  cudaError_t e;
+  if (p.head_dim == 128)
+    e = narrow ? launch(rope_unpack_kernel<128, kRuRowsNarrow, Table>) : launch(rope_unpack_kernel<128, kRuRowsWide, Table>);
+  else
+    e = narrow ? launch(rope_unpack_kernel<64, kRuRowsNarrow, Table>) : launch(rope_unpack_kernel<64, kRuRowsWide, Table>);
+  return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope+unpack kernel launch");
+}
+
+template <class Table>
+int launch_rope_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const Table& tab, int32_t* counter, void* q,
+                  void* k, cudaStream_t s) {
+  const RopeFreq freq = make_freq(p);
+  const int64_t n_rows = (int64_t)p.n_bins * p.capacity;
+  const unsigned grid = (unsigned)((n_rows + kRopeRows - 1) / kRopeRows);
+  auto launch = [&](auto kernel) {
+    return launch_dependent(kernel, dim3(grid), dim3(kRopeThreads), 0, s, (__nv_bfloat16*)q, (__nv_bfloat16*)k,
+                            norm_words(p, d_table, L), counter, tab, L.bin_seg_ptr, L.bin_used, L.seg_start, p.n_bins,
+                            p.capacity, p.n_q_heads, p.n_kv_heads, freq);
+  };
+  const cudaError_t e = p.head_dim == 128 ? launch(rope_kernel<128, Table>) : launch(rope_kernel<64, Table>);
+  return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope kernel launch");
+}
+
+TableInline inline_copy(const int32_t* table, size_t ints) {
+  TableInline t;
+  std::memcpy(t.w, table, sizeof(int32_t) * (ints < (size_t)kInlineInts ? ints : (size_t)kInlineInts));
+  return t;
+}
+
 }  // namespace
 
 int launch_rope_table(const pp_attn_params& p, void* table, void* stream) {
@@ -347,47 +398,23 @@ int launch_rope_table(const pp_attn_params& p, void* table, void* stream) {
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope table kernel launch");
 }
 
-int launch_rope_unpack(const pp_attn_params& p, int32_t* d_table, const TableLayout& L,
+int launch_rope_unpack(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
                        int32_t off_true_len, int32_t off_cap, int32_t off_cache_off, const void* rope_table,
                        void* k, const void* v, void* k_cache, void* v_cache, void* stream) {
-  const int64_t n_rows = (int64_t)p.n_bins * p.capacity;
-  const bool narrow = p.n_kv_heads * p.head_dim <= kRuNarrowRowElems;
-  const int rows = narrow ? kRuRowsNarrow : kRuRowsWide;
-  const unsigned grid = (unsigned)((n_rows + rows - 1) / rows);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const SegExt ext{off_true_len, off_cap, off_cache_off};
-  cudaError_t launch_err = cudaSuccess;
-#define PP_RU_LAUNCH(DD, RR)                                                                                      \
-  launch_err = launch_dependent(rope_unpack_kernel<DD, RR>, dim3(grid), dim3(kRopeThreads), 0, s,                 \
-      (__nv_bfloat16*)k, (const __nv_bfloat16*)v, norm_words(p, d_table, L), (__nv_bfloat16*)k_cache,             \
-      (__nv_bfloat16*)v_cache, (const int32_t*)d_table,                                                           \
-      L.bin_seg_ptr, L.bin_used, L.seg_start, ext, (const float2*)rope_table, p.n_bins, p.capacity, p.n_kv_heads)
-  if (p.head_dim == 128) {
-    if (narrow) PP_RU_LAUNCH(128, kRuRowsNarrow); else PP_RU_LAUNCH(128, kRuRowsWide);
-  } else {
-    if (narrow) PP_RU_LAUNCH(64, kRuRowsNarrow); else PP_RU_LAUNCH(64, kRuRowsWide);
-  }
-#undef PP_RU_LAUNCH
-  const cudaError_t e = launch_err != cudaSuccess ? launch_err : cudaGetLastError();
-  return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope+unpack kernel launch");
+  if (inline_table)      // the per-segment arrays lie behind the work list, the cache offsets last
+    return launch_rope_unpack_t(p, d_table, L, inline_copy(inline_table, (size_t)off_cache_off + 2 * (size_t)inline_table[kHeaderSegments]),
+                                d_table + kHeaderCounter, ext, rope_table, k, v, k_cache, v_cache, s);
+  return launch_rope_unpack_t(p, d_table, L, TableInMemory{d_table}, nullptr, ext, rope_table, k, v, k_cache, v_cache, s);
 }
 
-int launch_rope(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, void* q, void* k, void* stream) {
-  const RopeFreq freq = make_freq(p);
-  const int64_t n_rows = (int64_t)p.n_bins * p.capacity;
-  const unsigned grid = (unsigned)((n_rows + kRopeRows - 1) / kRopeRows);
+int launch_rope(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table, void* q, void* k,
+                void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (p.head_dim == 128) {
-    rope_kernel<128><<<grid, kRopeThreads, 0, s>>>(
-        (__nv_bfloat16*)q, (__nv_bfloat16*)k, norm_words(p, d_table, L), d_table, L.bin_seg_ptr, L.bin_used, L.seg_start,
-        p.n_bins, p.capacity, p.n_q_heads, p.n_kv_heads, freq);
-  } else {
-    rope_kernel<64><<<grid, kRopeThreads, 0, s>>>(
-        (__nv_bfloat16*)q, (__nv_bfloat16*)k, norm_words(p, d_table, L), d_table, L.bin_seg_ptr, L.bin_used, L.seg_start,
-        p.n_bins, p.capacity, p.n_q_heads, p.n_kv_heads, freq);
-  }
-  const cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope kernel launch");
+  if (inline_table)
+    return launch_rope_t(p, d_table, L, inline_copy(inline_table, (size_t)L.total_ints), d_table + kHeaderCounter, q, k, s);
+  return launch_rope_t(p, d_table, L, TableInMemory{d_table}, nullptr, q, k, s);
 }
 
 }  // namespace pp

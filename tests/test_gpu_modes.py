@@ -192,3 +192,31 @@ def test_keep_rope_table_flag_gives_identical_results():
     assert b.device_status() == 0
     for a, c in zip(ref, (b.o_tokens(), b.k_cache, b.v_cache)):
         assert torch.equal(a, c)
+
+
+@pytest.mark.parametrize("k", [1, 30, 45])        # small tables travel as kernel parameters (1, 30), larger ones are uploaded
+@pytest.mark.parametrize("hq,hkv,d", [(4, 4, 64), (4, 2, 128)])
+def test_table_as_parameter_or_uploaded(k, hq, hkv, d):
+    """Both forms of the prefill table give the oracle's results, on the first and on a repeated call on the
+    same workspace (the work counter starts anew), and whole or split by flags."""
+    lengths = np.asarray([100 - 3 * (i % 7) for i in range(k)], np.int32)
+    base = 10000.0
+    q, kk, v = _case(lengths, hq, hkv, d, seed=k + d)
+    refs = oracle_refs(lengths, q, kk, v, base)
+    fused = PrefillBatch(lengths, hq, hkv, d, base, guard=True)
+    three = PrefillBatch(lengths, hq, hkv, d, base, guard=True)
+    for _ in range(2):
+        for b, call in ((fused, fused.run_fused), (three, three.run)):
+            b.load(q, kk, v)
+            call()
+            torch.cuda.synchronize()
+            assert b.device_status() == 0
+            b.assert_untouched()
+            compare_with_refs(b, lengths, refs)
+    o = fused.o.clone()
+    fused.load(q, kk, v)
+    fused.o.zero_()
+    fused.run_fused(flags=pp.PP_FLAG_ROPE_ONLY)
+    fused.run_fused(flags=pp.PP_FLAG_SKIP_ROPE)
+    torch.cuda.synchronize()
+    assert fused.device_status() == 0 and torch.equal(fused.o_tokens(), o.view(-1, hq, d)[fused.token_rows])
