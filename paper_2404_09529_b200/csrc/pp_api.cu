@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <new>
@@ -177,18 +178,19 @@ int launch_fused_kernels(const pp_attn_params& p, const TableLayout& L, const Fu
 // pp_prefill_fused, optionally cut in two: kUploadOnly validates, builds and uploads the tables,
 // launches nothing and hands the table layout back through `layout`; kLaunchOnly takes that layout,
 // touches neither the host staging buffer (its upload may still be in flight) nor the arguments
-// already checked, and launches the kernels on the tables in `workspace`.
+// already checked, and launches the kernels on the tables in `workspace`. small_table: where not null, a small
+// table need not be uploaded; the first step then leaves its address in the staging buffer there, for the second.
 int prefill_fused_impl(const pp_attn_params* params, const int32_t* bin_seg_ptr, const int32_t* seg_start,
                        const int32_t* seg_len, const int32_t* seg_prompt, int32_t k, const int32_t* lengths,
                        const void* q, void* k_, const void* v, void* o, void* k_cache, void* v_cache,
                        const int64_t* cache_off, const int32_t* cache_cap, void* workspace,
                        void* host_workspace, size_t workspace_bytes, int32_t* device_status, void* stream,
-                       TableStep step, TableLayout* layout) {
+                       TableStep step, TableLayout* layout, const int32_t** small_table = nullptr) {
   int st = check_params(params);
   if (st != PP_OK) return st;
   if (step == TableStep::kLaunchOnly) {
     const FusedLayout f = fused_layout(*params, k);
-    return launch_fused_kernels(*params, *layout, f, nullptr, q, k_, v, o, k_cache, v_cache, workspace, device_status, stream);
+    return launch_fused_kernels(*params, *layout, f, small_table ? *small_table : nullptr, q, k_, v, o, k_cache, v_cache, workspace, device_status, stream);
   }
   if (!q || !k_ || !v || !o || !k_cache || !v_cache || !cache_off || !cache_cap || !seg_prompt || !lengths ||
       !workspace || !host_workspace)
@@ -218,13 +220,14 @@ int prefill_fused_impl(const pp_attn_params* params, const int32_t* bin_seg_ptr,
                             params->n_q_heads, params->n_kv_heads, h, f.table_ints, &L);
   if (st != PP_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const int32_t* small = step == TableStep::kUploadAndLaunch && !(params->flags & PP_FLAG_SKIP_ROPE) && L.independent_slots &&
+  const int32_t* small = (step == TableStep::kUploadAndLaunch || small_table) && !(params->flags & PP_FLAG_SKIP_ROPE) && L.independent_slots &&
                                  f.upload_ints <= (size_t)kInlineInts ? h : nullptr;
   if (!small) {
     cudaError_t e = cudaMemcpyAsync(workspace, host_workspace, sizeof(int32_t) * f.upload_ints, cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return note_cuda_error((int)e, "table upload");
   }
   if (layout) *layout = L;
+  if (small_table) *small_table = small;
   if (step == TableStep::kUploadOnly) return PP_OK;
   return launch_fused_kernels(*params, L, f, small, q, k_, v, o, k_cache, v_cache, workspace, device_status, stream);
 }
@@ -452,6 +455,73 @@ int host_pipe(HostPipe** out) {
   return PP_OK;
 }
 
+// Device address of `bytes` of pinned host memory at p that kernels can work on in 16-byte pieces; null if it is
+// anything else (pageable memory, an odd address).
+void* mapped(const void* p, size_t bytes) {
+  if (!aligned16(p)) return nullptr;
+  void* dev[2];
+  for (int end = 0; end < 2; ++end) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, static_cast<const char*>(p) + (end ? bytes - 1 : 0)) != cudaSuccess) {
+      (void)cudaGetLastError();
+      return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
+    dev[end] = a.devicePointer;
+  }
+  return static_cast<char*>(dev[1]) - static_cast<char*>(dev[0]) == (std::ptrdiff_t)(bytes - 1) ? dev[0] : nullptr;
+}
+
+// pp_prefill_host for one group whose six tensors are mapped: the kernels read and write them where they are, on the
+// caller's stream: six launches at most instead of nineteen copies, kernels and events, which took a small batch
+// longer than its bytes on the bus (1.1 MB both ways 132 -> 70 us, 3.9 MB 177 -> 125, 11 MB 312 -> 269, 39 MB 941
+// -> 881). Sets *done if it took the call.
+int prefill_host_mapped(const pp_attn_params& p, const HostPlan& h, const int32_t* lengths, int32_t k, const void* q_host,
+                        const void* k_host, const void* v_host, void* o_host, void* k_cache_host, void* v_cache_host, char* base,
+                        HostPipe* pipe, cudaStream_t s, bool* done) {
+  *done = false;
+  const size_t q_bytes = (size_t)h.total_tokens * p.n_q_heads * p.head_dim * 2;
+  const size_t kv_bytes = (size_t)h.total_tokens * p.n_kv_heads * p.head_dim * 2;
+  HostRows r;
+  r.q = base + h.q; r.k = base + h.k; r.v = base + h.v; r.o = base + h.o;
+  r.q_host = mapped(q_host, q_bytes); r.k_host = mapped(k_host, kv_bytes); r.v_host = mapped(v_host, kv_bytes);
+  r.o_host = mapped(o_host, q_bytes);
+  void *kc = mapped(k_cache_host, kv_bytes), *vc = mapped(v_cache_host, kv_bytes);
+  if (!r.q_host || !r.k_host || !r.v_host || !r.o_host || !kc || !vc) return PP_OK;
+  const HostGroup& G = h.groups[0];
+  const FusedLayout f = fused_layout(p, k);
+  void* stage = nullptr;
+  int st = host_staging(pipe, 0, 256 + f.total_bytes, &stage);
+  if (st != PP_OK) return st;
+  r.status = reinterpret_cast<int32_t*>(base + h.status);
+  r.host_status = static_cast<int32_t*>(stage);
+  *r.host_status = 0;
+  void* tables = static_cast<char*>(stage) + 256;
+  std::vector<int64_t> cache_off(k);
+  int64_t t = 0;
+  for (int32_t i = 0; i < k; ++i) {
+    cache_off[i] = t * p.n_kv_heads * p.head_dim;
+    t += lengths[i];
+  }
+  *done = true;
+  TableLayout L;
+  const int32_t* small = nullptr;
+  auto fused = [&](TableStep step) {
+    return prefill_fused_impl(&p, G.bin_seg_ptr.data(), G.seg_start.data(), G.seg_len.data(), G.seg_prompt.data(), k, lengths,
+                              r.q, r.k, r.v, r.o, kc, vc, cache_off.data(), lengths, base + h.ws, tables, f.total_bytes, r.status,
+                              s, step, &L, &small);
+  };
+  if ((st = fused(TableStep::kUploadOnly)) != PP_OK) return st;
+  int32_t* d_table = reinterpret_cast<int32_t*>(base + h.ws);
+  st = launch_host_rows(true, p, d_table, L, small, (int32_t)f.off_cache_off, r, s);
+  if (st == PP_OK) st = fused(TableStep::kLaunchOnly);
+  if (st == PP_OK) st = launch_host_rows(false, p, d_table, L, small, (int32_t)f.off_cache_off, r, s);
+  const cudaError_t e = cudaStreamSynchronize(s);      // also after an error: queued work uses the caller's buffers
+  if (st != PP_OK) return st;
+  if (e != cudaSuccess) return note_cuda_error((int)e, "stream synchronize");
+  return *static_cast<volatile int32_t*>(r.host_status) == 0 ? PP_OK : PP_ERR_DEVICE_TIMEOUT;
+}
+
 }  // namespace
 }  // namespace pp
 
@@ -514,6 +584,11 @@ extern "C" int pp_prefill_host(pp_attn_params* params, const int32_t* lengths, i
     };
 #define PP_TRY(call, what) do { e = (call); if (e != cudaSuccess) return bail(pp::note_cuda_error((int)e, what)); } while (0)
     const int n_groups = (int)h.groups.size();
+    if (n_groups == 1) {
+      bool done = false;
+      st = pp::prefill_host_mapped(*params, h, lengths, k, q_host, k_host, v_host, o_host, k_cache_host, v_cache_host, base, pipe, s, &done);
+      if (done || st != PP_OK) return st;
+    }
     PP_TRY(cudaMemsetAsync(base + h.status, 0, 4, s), "memset status");
     PP_TRY(cudaEventRecord(pipe->start, s), "event record");
     std::vector<int64_t> g_cache_off;

@@ -45,7 +45,6 @@
 
 #include <cmath>
 #include <cstdlib>
-#include <cstring>
 #include <type_traits>
 
 #include "pp_device_once.h"
@@ -1696,8 +1695,7 @@ int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayou
                      int32_t* device_status, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (inline_table) {                 // independent mode only
-    TableInline tab;
-    std::memcpy(tab.w, inline_table, sizeof(int32_t) * (size_t)(L.total_ints < kInlineInts ? L.total_ints : kInlineInts));
+    const TableInline tab = inline_copy(inline_table, (size_t)L.total_ints);
     if (p.head_dim == 128) return launch_attention_t<128, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
     return launch_attention_t<64, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
   }

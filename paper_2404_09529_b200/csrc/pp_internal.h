@@ -92,6 +92,18 @@ int launch_unpack(const pp_attn_params& p, const int32_t* d_table, int32_t k, in
 int launch_tensorize(bool to_packed, void* packed, void* tokens, const int64_t* d_map, int32_t n_prompts,
                      int64_t total_tokens, int32_t row_bytes, void* stream);
 
+// Token-major tensors in mapped host memory <-> packed tensors, by packed row (the row's token is found in the prefill
+// table: the cache offsets of its prompt are those of token-major caches). to_packed: q, k, v into the packed tensors,
+// padding rows zeroed, *status zeroed. Back: O into the host tensor, *status copied to *host_status.
+struct HostRows {
+  void *q, *k, *v, *o;                         // packed
+  const void *q_host, *k_host, *v_host;
+  void* o_host;
+  int32_t *status, *host_status;
+};
+int launch_host_rows(bool to_packed, const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
+                     int32_t off_cache_off, const HostRows& rows, void* stream);
+
 // Zeroes rows [bin_used[b], capacity) of every bin of the packed q / k / v (null pointers are skipped).
 int launch_zero_pad_rows(void* q, void* k, void* v, int32_t q_row_bytes, int32_t kv_row_bytes,
                          const int64_t* d_bin_used, int32_t n_bins, int32_t capacity, void* stream);
@@ -123,6 +135,12 @@ struct alignas(16) TableInline {
   __device__ __forceinline__ int4 i128(int i) const { return *reinterpret_cast<const int4*>(w + i); }
   __device__ __forceinline__ int64_t i64(int base, int i) const { return *reinterpret_cast<const int64_t*>(w + base + 2 * i); }
 };
+
+inline TableInline inline_copy(const int32_t* table, size_t ints) {
+  TableInline t;
+  for (size_t i = 0; i < (ints < (size_t)kInlineInts ? ints : (size_t)kInlineInts); ++i) t.w[i] = table[i];
+  return t;
+}
 
 // Programmatic dependent launch. A kernel of the path that is launched with launch_dependent() may
 // start while the kernel before it in the stream is still finishing: its blocks are scheduled once

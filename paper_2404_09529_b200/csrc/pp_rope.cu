@@ -4,8 +4,6 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
-#include <cstring>
-
 #include "pp_internal.h"
 
 namespace pp {
@@ -378,12 +376,6 @@ int launch_rope_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& 
   };
   const cudaError_t e = p.head_dim == 128 ? launch(rope_kernel<128, Table>) : launch(rope_kernel<64, Table>);
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope kernel launch");
-}
-
-TableInline inline_copy(const int32_t* table, size_t ints) {
-  TableInline t;
-  std::memcpy(t.w, table, sizeof(int32_t) * (ints < (size_t)kInlineInts ? ints : (size_t)kInlineInts));
-  return t;
 }
 
 }  // namespace

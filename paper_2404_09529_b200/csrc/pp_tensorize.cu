@@ -6,6 +6,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "pp_internal.h"
 
 namespace pp {
@@ -80,7 +82,94 @@ zero_pad_rows_kernel(PadTensors t, const int64_t* __restrict__ bin_used, int32_t
   }
 }
 
+// A batch in mapped (pinned) host memory: the rows are read and written over the bus by the kernel itself, so one
+// launch takes the place of three copies, the zeroing and three scatters (or of a gather and a copy). For a small
+// batch those are a queue of 2 us operations (see launch_host_rows); the bus runs at 51 GB/s up and 52 GB/s down this
+// way against 55 and 53 of the copy engines.
+struct RowTable {
+  int32_t off_bin_seg_ptr, off_bin_used, off_seg_start, off_cache_off;
+  int32_t capacity, kv_elems;                  // kv_elems: n_kv_heads * head_dim, one token of a token-major cache
+  int32_t rows_per_block;                      // at most kTzTokens
+  int64_t n_rows;
+};
+template <bool kToPacked, class Table>
+__global__ void __launch_bounds__(kTzThreads)
+host_rows_kernel(HostRows h, RowTable m, int32_t q_vec, int32_t kv_vec, const __grid_constant__ Table tab) {
+  __shared__ int64_t s_tok[kTzTokens];           // token of each packed row, -1 for padding
+  const int64_t row0 = (int64_t)blockIdx.x * m.rows_per_block;
+  if (threadIdx.x < m.rows_per_block) {
+    const int64_t row = row0 + threadIdx.x;
+    int64_t tok = -1;
+    if (row < m.n_rows) {
+      const int32_t b = (int32_t)(row / m.capacity);
+      const int32_t t = (int32_t)(row - (int64_t)b * m.capacity);
+      if (t < tab.i32(m.off_bin_used + b)) {
+        int32_t lo = tab.i32(m.off_bin_seg_ptr + b), hi = tab.i32(m.off_bin_seg_ptr + b + 1) - 1;
+        while (lo < hi) {                        // last prompt that starts at or before the row
+          const int32_t mid = (lo + hi + 1) >> 1;
+          if (tab.i32(m.off_seg_start + mid) <= t) lo = mid; else hi = mid - 1;
+        }
+        tok = tab.i64(m.off_cache_off, lo) / m.kv_elems + (t - tab.i32(m.off_seg_start + lo));
+      }
+    }
+    s_tok[threadIdx.x] = tok;
+  }
+  if (!kToPacked) pdl_wait();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (kToPacked) *h.status = 0; else *h.host_status = *h.status;
+  }
+  __syncthreads();
+  const int per_row = kToPacked ? q_vec + 2 * kv_vec : q_vec;
+  const int rows = (int)(m.n_rows - row0 < m.rows_per_block ? m.n_rows - row0 : m.rows_per_block);
+  for (int u0 = threadIdx.x; u0 < rows * per_row; u0 += 4 * kTzThreads) {
+    uint4 val[4];
+    uint4* dst[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int u = u0 + i * kTzThreads;
+      dst[i] = nullptr;
+      if (u < rows * per_row) {
+        const int r = u / per_row, w = u - r * per_row;
+        const int64_t tok = s_tok[r], row = row0 + r;
+        if (kToPacked) {
+          const int which = w < q_vec ? 0 : w < q_vec + kv_vec ? 1 : 2;
+          const int vec = which == 0 ? q_vec : kv_vec, c = w - (which == 0 ? 0 : which == 1 ? q_vec : q_vec + kv_vec);
+          const uint4* src = static_cast<const uint4*>(which == 0 ? h.q_host : which == 1 ? h.k_host : h.v_host);
+          dst[i] = static_cast<uint4*>(which == 0 ? h.q : which == 1 ? h.k : h.v) + row * vec + c;
+          val[i] = tok >= 0 ? src[tok * vec + c] : make_uint4(0u, 0u, 0u, 0u);
+        } else if (tok >= 0) {
+          dst[i] = static_cast<uint4*>(h.o_host) + tok * q_vec + w;
+          val[i] = static_cast<const uint4*>(h.o)[row * q_vec + w];
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (dst[i]) *dst[i] = val[i];
+  }
+}
+
 }  // namespace
+
+int launch_host_rows(bool to_packed, const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
+                     int32_t off_cache_off, const HostRows& rows, void* stream) {
+  RowTable m{L.bin_seg_ptr, L.bin_used, L.seg_start, off_cache_off, p.capacity, p.n_kv_heads * p.head_dim, 1,
+             (int64_t)p.n_bins * p.capacity};
+  // a bus read takes 1 to 2 us, so few rows are spread over as many blocks as there are
+  while (m.rows_per_block < kTzTokens && m.n_rows > (int64_t)m.rows_per_block * 148 * 2) m.rows_per_block *= 2;
+  const dim3 grid((unsigned)((m.n_rows + m.rows_per_block - 1) / m.rows_per_block)), block(kTzThreads);
+  const int32_t q_vec = p.n_q_heads * p.head_dim / 8, kv_vec = m.kv_elems / 8;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  auto launch = [&](const auto& tab) {
+    using Table = std::decay_t<decltype(tab)>;
+    if (!to_packed) return launch_dependent(host_rows_kernel<false, Table>, grid, block, 0, s, rows, m, q_vec, kv_vec, tab);
+    host_rows_kernel<true, Table><<<grid, block, 0, s>>>(rows, m, q_vec, kv_vec, tab);
+    return cudaGetLastError();
+  };
+  const cudaError_t e = inline_table ? launch(inline_copy(inline_table, (size_t)off_cache_off + 2 * (size_t)inline_table[kHeaderSegments]))
+                                     : launch(TableInMemory{d_table});
+  return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "host rows kernel launch");
+}
 
 int launch_zero_pad_rows(void* q, void* k, void* v, int32_t q_row_bytes, int32_t kv_row_bytes,
                          const int64_t* d_bin_used, int32_t n_bins, int32_t capacity, void* stream) {

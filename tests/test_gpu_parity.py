@@ -305,3 +305,30 @@ def test_kernel_gives_up_cleanly_when_its_waits_expire(name, monkeypatch):
     torch.cuda.synchronize()
     assert b.device_status() == 0
     compare_sampled(b, lengths, q, k, v, cfg.rope_base, prompts=[0, 3], kv_heads=[0], n_rows=16, seed=2)
+
+
+@pytest.mark.parametrize("lengths,hq,hkv,d", [
+    ([1], 4, 4, 64),                                    # a single row
+    ([70, 3, 64, 1, 33], 6, 2, 128),                    # several prompts per bin, padding rows
+    ([61] * 700, 2, 1, 64),                             # several rows per block, table uploaded
+])
+@pytest.mark.parametrize("pinned", [True, False])
+def test_host_entry_point_one_group_mapped_or_copied(lengths, hq, hkv, d, pinned):
+    """One group: kernels work on pinned host tensors in place, pageable ones are copied; both bit-identical to
+    the device route, call after call on the same arena."""
+    import paper_2404_09529_b200 as pp
+    lengths = np.array(lengths, np.int32)
+    q, k, v = _random_case(lengths, hq, hkv, d, seed=int(lengths.sum()))
+    ref = run_cuda(lengths, q, k, v, hq, hkv, d, 10000.0)
+    params = pp.AttnParams(hq, hkv, d, 10000.0, 0.0, 0, 0, 0)
+    nbytes = pp.pp_prefill_host_arena_bytes(params, lengths)
+    arena = torch.full((nbytes,), 255, dtype=torch.uint8, device="cuda")
+    new = lambda n: torch.full((n + 16,), -7.0, dtype=torch.bfloat16)
+    bufs = [q.contiguous(), k.contiguous(), v.contiguous(), new(q.numel()), new(k.numel()), new(v.numel())]
+    if pinned:
+        bufs = [b.pin_memory() for b in bufs]
+    for _ in range(2):
+        pp.pp_prefill_host(params, lengths, *bufs, arena, nbytes, torch.cuda.current_stream().cuda_stream)
+        for got, want in zip(bufs[3:], (ref.o_tokens(), ref.k_cache, ref.v_cache)):
+            assert torch.equal(got[:-16], want.cpu().flatten()) and bool((got[-16:] == -7.0).all())
+            got[:-16].zero_()
