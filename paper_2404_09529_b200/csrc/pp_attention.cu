@@ -32,6 +32,7 @@
 //   warps 8-11   helper threads of slot 0, one per row: find the first key of each row of the next item,
 //                rotate its Q in shared memory (fused path) and run the previous item's epilogue
 //   warps 12-19  the same for slot 1
+//   warps 20-21  (kFill) write the V rows of the slots' own query tiles from shared memory to the caches
 // Softmax: tcgen05.ld the thread's scores, mask to the row's key range, lazy running maximum (O is
 // rescaled only when the maximum grows by more than 2^8, or 2^90 in the shared-stream mode, where rows
 // whose scores are bounded drop the maximum altogether), exp2, P written as bf16 over the S
@@ -55,12 +56,16 @@ namespace {
 
 constexpr int BM = kTileM;
 constexpr int kAttnThreads = 640;
+constexpr int kAttnThreadsFill = 768;      // one warpgroup more, two of its warps fill the V caches
 constexpr int kSoftmaxThreads = 256;       // per slot: two threads per query row
 constexpr uint32_t kTmemCols = 512;
 constexpr int kRegsSoftmax = 104;          // setmaxnreg budgets: 640 threads start with 96 registers each;
 constexpr int kRegsSoftmaxIndep = 120;     // independent mode: 256 softmax threads at 120, 256 helper threads at 88
 constexpr int kRegsHelper = 88;
 constexpr int kRegsOther = 64;              // warps 0-3 give back 32 each, the 512 softmax threads take 8 each
+constexpr int kRegsSoftmaxFill = 112;      // with cache writers: 768 threads start with 80 registers each; the 256 softmax
+constexpr int kRegsOtherFill = 56;         //   threads take 32 each from warps 0-3 (24 each) and the cache writers'
+constexpr int kRegsWriter = 40;            //   warpgroup (40 each); the 256 helper threads keep their 80
 // Shared-stream mode, when a row needs no maximum any more. Its running maximum is lazy: it stays at the
 // maximum of the row's first visible tile until a score exceeds it by more than kLazyLog2 (log2 units).
 // Probabilities, sums and O have 8 exponent bits, so a common factor of up to 2^90 costs no precision, and
@@ -416,6 +421,8 @@ struct AttnArgs {
   const uint32_t* q_norm2;       // [Hq] largest |q|^2; used when Q arrives already rotated
   int32_t* status;
   unsigned long long wait_limit_ns;
+  __nv_bfloat16* v_cache;                         // kFill: the V caches
+  int32_t off_true_len, off_cap, off_cache_off;   // per-segment arrays in the table, for them
 };
 
 // What one work index means for a CTA.
@@ -506,8 +513,8 @@ __device__ __forceinline__ int seg_start_at(const Table& tab, int starts, int se
 __device__ __forceinline__ uint32_t kv_index_k(uint32_t k) { return k ? 2u * k - 1u : 0u; }
 __device__ __forceinline__ uint32_t kv_index_v(uint32_t k) { return 2u * k + 2u; }
 
-template <int D, bool kIndep, class Table>
-__global__ void __launch_bounds__(kAttnThreads, 1)
+template <int D, bool kIndep, bool kFill, class Table>
+__global__ void __launch_bounds__(kFill ? kAttnThreadsFill : kAttnThreads, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
                  const __grid_constant__ AttnArgs args, const __grid_constant__ Table tab) {
@@ -550,6 +557,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                                                  // independent mode: [2 slots][2 Q tiles], its rows' first keys are there too
   const uint32_t bar_pv_done = s_misc + 384;     // [2] independent mode: P(k) V(k) has been computed
   const uint32_t bar_pair0 = s_misc + 896;       // [2 slots][4 quadrants] shared-stream mode: rendezvous of the two warps that share rows
+  const uint32_t bar_v_seen0 = s_misc + 960, bar_v_seen1 = s_misc + 1008;   // [2] each, independent mode: the slot's MMA warp has seen V(k)
   const uint32_t bar_l_ready = s_misc + 976;     // [2][2] independent mode: the slot's row sums of item i are in shared memory ([slot][i & 1])
   uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(misc + 400);
   volatile int* s_abort = reinterpret_cast<volatile int*>(misc + 404);
@@ -568,7 +576,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       mbar_init(bar_item_full + 8 * i, 1);
       // readers of a ring entry: the MMA thread and the softmax threads of the slot(s) it feeds;
       // in shared mode also the two Q loaders
-      mbar_init(bar_item_empty + 8 * i, kIndep ? 1 + kSoftmaxThreads : 1 + 2 + 2 * kSoftmaxThreads);
+      // (and in independent mode the slot's cache writer, where caches are filled)
+      mbar_init(bar_item_empty + 8 * i, kIndep ? 1 + kSoftmaxThreads + (kFill ? 1 : 0) : 1 + 2 + 2 * kSoftmaxThreads);
     }
     for (int i = 0; i < 2; ++i) {
       for (int b = 0; b < 2; ++b) {
@@ -585,8 +594,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         mbar_init(bar_q_empty + 8 * i, Cfg::kStageInQ ? 4 : 1);   // one lane of each helper warp, or a commit
         mbar_init(bar_q_rot + 8 * i, kSoftmaxThreads / 2);
       }
-      for (int i = 0; i < 8; ++i) { mbar_init(bar_kv_full + 8 * i, 1); mbar_init(bar_kv_empty + 8 * i, 1); }
-      for (int i = 0; i < 2; ++i) mbar_init(bar_pv_done + 8 * i, 1);
+      // a stage is free when its product has been computed and, where caches are filled, its rows have been read
+      for (int i = 0; i < 8; ++i) { mbar_init(bar_kv_full + 8 * i, 1); mbar_init(bar_kv_empty + 8 * i, kFill ? 2 : 1); }
+      for (int i = 0; i < 2; ++i) { mbar_init(bar_pv_done + 8 * i, 1); if (kFill) { mbar_init(bar_v_seen0 + 8 * i, 1); mbar_init(bar_v_seen1 + 8 * i, 1); } }
     } else {
       for (int i = 0; i < 2; ++i) {
         mbar_init(bar_q_full + 8 * i, 1);
@@ -614,7 +624,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   pdl_wait();
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFill ? kRegsOtherFill : kRegsOther));
     if constexpr (kIndep) {
       if (warp >= 2) {
         // -------------------------------------------------------------- producer of slot t:
@@ -719,6 +729,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                    kb + (uint32_t)(kk >> 2) * kChunkK + (uint32_t)(kk & 3) * 2, idesc_qk, kk > 0 ? 1u : 0u, issue);
           }
           tc_commit(b_kv_empty + 8 * st, issue);
+          if (kFill && issue) mbar_arrive(b_kv_empty + 8 * st);      // (no row of a K tile is written to a cache)
           tc_commit(b_s_full + 8 * (kq & 1u), issue);
           if (!Cfg::kStageInQ && last_of_item) tc_commit(bar_q_empty + 16 * t + 8 * (item & 1u), issue);   // last read of Q
           return true;
@@ -756,6 +767,14 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (j == 0 && !last_tile && !(ok = mbar_wait_warp(b_o_empty, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
           const uint32_t idx = kv_index_v(kc), st = idx % NS;
           if (!(ok = mbar_wait_warp(b_kv_full + 8 * st, (idx / NS) & 1u, wctx, kWaitVFull))) break;
+          if constexpr (kFill) {
+            // The cache writer must have seen V(kc - 2), whose barrier this is again, before V(kc) is announced. K(kc + 1)
+            // could not have been loaded otherwise (three stages; with four, V(kc)); the slot's last tile has none.
+            const uint32_t before = kv_index_v(kc - 2u);
+            if (last_tile && w_next < 0 && kc >= 2u &&
+                !(ok = mbar_wait_warp(b_kv_empty + 8 * (before % NS), (before / NS) & 1u, wctx, kWaitVEmpty))) break;
+            if (issue) mbar_arrive((t ? bar_v_seen1 : bar_v_seen0) + 8 * (kc & 1u));
+          }
           if (!(ok = mbar_wait_warp(b_p_full + 8 * (kc & 1u), (kc >> 1) & 1u, wctx, kWaitP))) break;
           tc_fence_after();            // O_t (+)= P(k) V(k)
           const uint32_t a = tm_s + 64u * (kc & 1u);
@@ -940,6 +959,81 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
     }
     }   // shared-stream roles
+  } else if (kFill && warp >= 20) {
+    // ------------------------------------------------------------------ cache writer of slot t (warps 20, 21)
+    // UNPACK of V: every row of V passes through shared memory here anyway, so the warp writes it to its prompt's
+    // cache from there while the slot's other warps compute, and the kernel in front of this one reads and writes K
+    // only. An item writes the rows of its own query tile, which are its last key rows; with as many KV heads as
+    // query heads (the only use) every row has one such item. The bound is memory, as without: 17 554 tokens of 32
+    // heads of 128, rotation kernel 121 -> 77 us, this one 194 -> 210 (they overlap), both 299 -> 292.
+    // (K' written the same way made this kernel 58 us longer, as much as the rotation kernel got shorter: a K stage
+    // is wanted back as soon as the scores are there, a V stage is held for the softmax's time in any case.)
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsWriter));
+    if (warp < 22) {
+      const int t = warp - 20;
+      const uint32_t bar_v_seen = t ? bar_v_seen1 : bar_v_seen0;
+      constexpr int NS = Cfg::kKVStages;
+      constexpr int kPieces = D / 8;                 // 16-byte pieces of a row, one per lane
+      constexpr int kRowsAtOnce = 32 / kPieces;
+      const int piece = lane & (kPieces - 1);
+      uint32_t kc = 0;
+      bool ok = true;
+      for (uint32_t it_n = 0; ok; ++it_n) {
+        const uint32_t ring = (uint32_t)t * kRing + it_n % kRing;
+        if (!mbar_wait_warp(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull)) break;
+        const volatile int* e = s_ring + ring * kRingInts;
+        const int w = uniform(e[0]), kv_row0 = e[2], n = uniform(e[3]), q_row0 = e[4], kv_head = e[11];
+        const int bin_used = e[12], seg_end = e[13], seg_first = e[16];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_item_empty + 8 * ring);
+        if (w < 0) break;
+        const int own_end = min(q_row0 + BM, bin_used);      // rows [q_row0, own_end)
+        // The prompt under the cursor, all lanes alike: its rows [.., cached) go to offset base + row * D, the next
+        // prompt starts at row `next`.
+        int seg = seg_first, cached = 0, next = 0;
+        int64_t seg_base = 0;
+        auto load_seg = [&]() {
+          const int start = tab.i32(args.off_seg_start + seg);
+          next = seg + 1 < seg_end ? tab.i32(args.off_seg_start + seg + 1) : own_end;
+          cached = start + tab.i32(args.off_true_len + seg);
+          seg_base = tab.i64(args.off_cache_off, seg) + ((int64_t)kv_head * tab.i32(args.off_cap + seg) - start) * D;
+        };
+        load_seg();
+        for (int j = 0; ok && j < n; ++j, ++kc) {
+          const int r0 = kv_row0 + j * BN;
+          const int lo = max(r0, q_row0), hi = min(r0 + BN, own_end);
+          const uint32_t st = kv_index_v(kc) % NS;
+          ok = mbar_wait_warp(bar_v_seen + 8 * (kc & 1u), (kc >> 1) & 1u, wctx, kWaitVFull);
+          if (!ok) break;
+          const uint32_t tile = s_kv + ((uint32_t)t * NS + st) * Cfg::kKVBytes + (uint32_t)(piece >> 3) * (BN * 128);
+          __nv_bfloat16* cache = args.v_cache + 8 * piece;
+          for (int row = lo; row < hi;) {                      // prompt by prompt
+            if (row >= next) {
+              ++seg;
+              load_seg();
+              continue;
+            }
+            const int stop = min(hi, next), copy_end = min(stop, cached);
+            for (int at = row + lane / kPieces; at < copy_end + lane / kPieces; at += 4 * kRowsAtOnce) {
+              uint4 val[4];
+#pragma unroll
+              for (int x = 0; x < 4; ++x) {
+                const uint32_t r = (uint32_t)(min(at + x * kRowsAtOnce, copy_end - 1) - r0);
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(val[x].x), "=r"(val[x].y), "=r"(val[x].z), "=r"(val[x].w)
+                             : "r"(tile + r * 128 + ((((uint32_t)piece & 7u) ^ (r & 7u)) << 4)));
+              }
+#pragma unroll
+              for (int x = 0; x < 4; ++x)
+                if (at + x * kRowsAtOnce < copy_end)
+                  *reinterpret_cast<uint4*>(cache + seg_base + (int64_t)(at + x * kRowsAtOnce) * D) = val[x];
+            }
+            row = stop;
+          }
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_kv_empty + 8 * (4 * t + st));
+        }
+      }
+    }
   } else {
     // ------------------------------------------------------------------ softmax + epilogue
     const int t = (warp - 4) >> 3;                   // slot
@@ -975,7 +1069,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         key_hi = real ? i_row : 0;
       };
       if (h == 0) {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmaxIndep));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kFill ? kRegsSoftmaxFill : kRegsSoftmaxIndep));
         uint32_t it_n = 0, tcount = 0;
         while (true) {
           const uint32_t ring = ring0 + it_n % kRing;
@@ -1118,7 +1212,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ++it_n;
         }
       } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsHelper));
+        if (!kFill) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsHelper));
         uint32_t it_n = 0;
         int p_q_row0 = 0, p_head = 0, p_bin = 0;         // coordinates of the previous item (its epilogue is due)
         while (true) {
@@ -1621,10 +1715,10 @@ int sm_count() {
   return cached;
 }
 
-template <int D, bool kIndep, class Table>
+template <int D, bool kIndep, bool kFill, class Table>
 int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const Table& tab, const void* q,
                        const void* k, const void* v, void* o, const void* rope_table, bool have_norms,
-                       int32_t* device_status, cudaStream_t stream) {
+                       const CacheFill* caches, int32_t* device_status, cudaStream_t stream) {
   constexpr int BN = kIndep ? kTileNShort : kTileN;
   using Cfg = AttnCfg<D, BN>;
   CUtensorMap mq, mk, mv, mo;
@@ -1641,7 +1735,7 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return note_cuda_error(-1, "cudaGetDevice");
   if (!configured.done(dev)) {
-    cudaError_t e = cudaFuncSetAttribute(attention_kernel<D, kIndep, Table>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(attention_kernel<D, kIndep, kFill, Table>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          Cfg::kSmemBytes);
     if (e != cudaSuccess) return note_cuda_error((int)e, "cudaFuncSetAttribute(smem)");
     configured.mark(dev);
@@ -1650,6 +1744,10 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   if (sms <= 0) return note_cuda_error(-1, "multiprocessor count");
   AttnArgs a;
   a.counter = d_table + kHeaderCounter;
+  a.v_cache = kFill ? static_cast<__nv_bfloat16*>(caches->v_cache) : nullptr;
+  a.off_true_len = caches ? caches->off_true_len : 0;
+  a.off_cap = caches ? caches->off_cap : 0;
+  a.off_cache_off = caches ? caches->off_cache_off : 0;
   a.off_bin_seg_ptr = L.bin_seg_ptr;
   a.off_bin_used = L.bin_used;
   a.off_seg_start = L.seg_start;
@@ -1676,7 +1774,7 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.status = device_status;
   a.wait_limit_ns = wait_limit_ns();
   const unsigned grid = (unsigned)(total < sms ? total : sms);
-  const cudaError_t launch_err = launch_dependent(attention_kernel<D, kIndep, Table>, dim3(grid), dim3(kAttnThreads),
+  const cudaError_t launch_err = launch_dependent(attention_kernel<D, kIndep, kFill, Table>, dim3(grid), dim3(kFill ? kAttnThreadsFill : kAttnThreads),
                                                   (size_t)Cfg::kSmemBytes, stream, mq, mk, mv, mo, a, tab);
   const cudaError_t e = launch_err != cudaSuccess ? launch_err : cudaGetLastError();
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "attention kernel launch");
@@ -1692,20 +1790,25 @@ int launch_bounded_wait_selftest(int32_t* device_status, uint64_t limit_ns, void
 
 int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table, const void* q,
                      const void* k, const void* v, void* o, const void* rope_table, bool have_norms,
-                     int32_t* device_status, void* stream) {
+                     const CacheFill* caches, int32_t* device_status, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const auto launch = [&](auto d, auto indep, auto fill, const auto& tab) {
+    return launch_attention_t<d(), indep(), fill()>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, caches, device_status, s);
+  };
+  using D64 = std::integral_constant<int, 64>;
+  using D128 = std::integral_constant<int, 128>;
+  using Yes = std::true_type;
+  using No = std::false_type;
   if (inline_table) {                 // independent mode only
-    const TableInline tab = inline_copy(inline_table, (size_t)L.total_ints);
-    if (p.head_dim == 128) return launch_attention_t<128, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
-    return launch_attention_t<64, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
+    const TableInline tab = inline_copy(inline_table, caches ? (size_t)caches->off_cache_off + 2 * (size_t)L.n_segments
+                                                             : (size_t)L.total_ints);
+    if (caches) return launch(D128{}, Yes{}, Yes{}, tab);
+    return p.head_dim == 128 ? launch(D128{}, Yes{}, No{}, tab) : launch(D64{}, Yes{}, No{}, tab);
   }
   const TableInMemory tab{d_table};
-  if (L.independent_slots) {
-    if (p.head_dim == 128) return launch_attention_t<128, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
-    return launch_attention_t<64, true>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
-  }
-  if (p.head_dim == 128) return launch_attention_t<128, false>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
-  return launch_attention_t<64, false>(p, d_table, L, tab, q, k, v, o, rope_table, have_norms, device_status, s);
+  if (caches) return launch(D128{}, Yes{}, Yes{}, tab);
+  if (L.independent_slots) return p.head_dim == 128 ? launch(D128{}, Yes{}, No{}, tab) : launch(D64{}, Yes{}, No{}, tab);
+  return p.head_dim == 128 ? launch(D128{}, No{}, No{}, tab) : launch(D64{}, No{}, No{}, tab);
 }
 
 }  // namespace pp

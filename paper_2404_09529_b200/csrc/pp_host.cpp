@@ -255,6 +255,7 @@ int build_prefill_tables(int32_t n_bins, int32_t capacity, const int32_t* bin_se
       const int32_t s_lo = bin_seg_ptr[b], s_hi = bin_seg_ptr[b + 1];
       const int32_t used = seg_start[s_hi - 1] + seg_len[s_hi - 1];
       out[L.bin_used + b] = used;
+      L.rows_used += used;
       int32_t s = s_lo, s_slot0 = s_lo;     // cursors over the bin's segments: query rows only move forward
       // first key row that query tile q0 can see: the start of the prompt that holds row q0, rounded
       // down to a key tile where two slots share the stream (their tiles must coincide)
@@ -339,6 +340,7 @@ int build_prefill_tables(int32_t n_bins, int32_t capacity, const int32_t* bin_se
   L.independent_slots = independent;
   L.pair_rows = pair_rows;
   L.fold = fold;
+  L.n_segments = k;
   if (layout) *layout = L;
   return PP_OK;
 }

@@ -49,6 +49,8 @@ struct TableLayout {
   int32_t total_ints = 0;
   bool independent_slots = false;   // items are single tiles, drawn by each slot on its own
   bool pair_rows = false;           // shared-stream mode: the two slots are consecutive row tiles of one head
+  int64_t rows_used = 0;            // occupied rows of all bins
+  int32_t n_segments = 0;           // prompts
   int32_t fold = 1;                 // independent mode: query heads folded into a query tile (128 / fold bin rows each)
 };
 
@@ -73,11 +75,18 @@ int launch_rope(const pp_attn_params& p, int32_t* d_table, const TableLayout& L,
 // rope_table: device [D/4][capacity][2] (cos, sin) pairs, or null. When given, q holds the raw
 // queries and the kernel rotates each Q tile in shared memory before use. have_norms: a rotation kernel
 // of the same call has filled the norms of the table (of the keys, and without rope_table of the queries).
+// caches: null, or the per-prompt V caches, which the kernel fills from the V tiles it loads (independent mode, head_dim
+// 128, as many KV heads as query heads).
+struct CacheFill {
+  void* v_cache;
+  int32_t off_true_len, off_cap, off_cache_off;   // per-segment arrays inside the table, as for launch_rope_unpack
+};
 int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
                      const void* q, const void* k, const void* v, void* o, const void* rope_table,
-                     bool have_norms, int32_t* device_status, void* stream);
+                     bool have_norms, const CacheFill* caches, int32_t* device_status, void* stream);
 // Fused K rotation + UNPACK; the three offsets locate per-segment arrays inside the table
-// (true length, cache capacity: int32; cache element offset: int64). In the shared-stream mode it also leaves
+// (true length, cache capacity: int32; cache element offset: int64). v null: the V caches are filled elsewhere.
+// In the shared-stream mode it also leaves
 // the largest |k|^2 of every KV head in the table (L.norms).
 int launch_rope_unpack(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
                        int32_t off_true_len, int32_t off_cap, int32_t off_cache_off, const void* rope_table,

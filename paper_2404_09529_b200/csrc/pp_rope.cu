@@ -251,7 +251,7 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
   }
 
   // V rows first: plain 16-byte copies, four in flight per thread
-  const int units_v = n_kv_heads * kVecs;
+  const int units_v = v ? n_kv_heads * kVecs : 0;
   for (int u0 = tid; u0 < kRuRows * units_v; u0 += kRuV * kRopeThreads) {
     uint4 val[kRuV];
     int64_t dsts[kRuV];

@@ -220,3 +220,25 @@ def test_table_as_parameter_or_uploaded(k, hq, hkv, d):
     fused.run_fused(flags=pp.PP_FLAG_SKIP_ROPE)
     torch.cuda.synchronize()
     assert fused.device_status() == 0 and torch.equal(fused.o_tokens(), o.view(-1, hq, d)[fused.token_rows])
+
+
+# Multi-head, D = 128, independent mode: the attention kernel fills the V caches from 32 rows per prompt on, the rotation
+# kernel below that. Prompts at the edges of the 64-key and the 128-row tiles, many in a tile, and streams of many items.
+@pytest.mark.parametrize("lengths,room", [
+    ([1], 0), ([32], 0), ([63, 1, 64, 65, 127], 3), ([128, 129, 1, 1, 1, 191, 193], 0), ([700, 3, 640, 257], 5),
+    ([31] * 9, 0), ([32] * 9, 2), ([97 + i % 64 for i in range(70)], 0)])
+@pytest.mark.parametrize("h", [1, 3])
+def test_v_caches_filled_by_either_kernel(lengths, room, h):
+    lengths = np.asarray(lengths, np.int32)
+    base = 10000.0
+    q, k, v = _case(lengths, h, h, 128, seed=int(lengths.sum()) + h)
+    b = PrefillBatch(lengths, h, h, 128, base, room=room, guard=True)
+    _assert_schedule(b, h, h, 1, 2)
+    refs = oracle_refs(lengths, q, k, v, base)
+    for _ in range(2):
+        b.load(q, k, v)
+        b.run_fused()
+        torch.cuda.synchronize()
+        assert b.device_status() == 0
+        b.assert_untouched()
+        compare_with_refs(b, lengths, refs)
