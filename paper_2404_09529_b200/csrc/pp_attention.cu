@@ -1431,7 +1431,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       // |q|^2 up to which every score of a row stays below the bound (0 if nothing is known about the keys)
       float q2_limit = 0.f;
-      if (args.k_norm2) q2_limit = args.bound2 / fmaxf(__uint_as_float(__ldg(args.k_norm2 + kv_head)), 1e-30f);
+      if (args.k_norm2) {
+        const float k2 = __uint_as_float(__ldg(args.k_norm2 + kv_head));
+        if (k2 < INFINITY) q2_limit = args.bound2 / fmaxf(k2, 1e-30f);      // (a NaN among the keys bounds nothing)
+      }
       bool bounded = false;
       // Fused path: Q arrives raw and is rotated in shared memory. Each half of a row is held to half
       // the limit, so that no sum over the two threads of a row is needed.

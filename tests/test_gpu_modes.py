@@ -242,3 +242,55 @@ def test_v_caches_filled_by_either_kernel(lengths, room, h):
         assert b.device_status() == 0
         b.assert_untouched()
         compare_with_refs(b, lengths, refs)
+
+
+def _scaled_inputs(kind, lengths, hq, hkv, d):
+    q, k, v = _case(lengths, hq, hkv, d, seed=d + hq)
+    t = q.shape[0]
+    pos = torch.cat([torch.arange(int(l)) / int(l) for l in lengths]).view(-1, 1, 1)
+    if kind == "unbounded":
+        q, k = q * 4, k * 4
+    elif kind == "rising":                       # later key tiles exceed the first one by far more than 2^90
+        q, k = q * 6, k * (0.1 + 16 * pos)
+    elif kind == "mixed":                        # rows within and beyond the bound side by side
+        q = q * (0.5 + 8 * (torch.arange(t) % 3 == 0)).view(-1, 1, 1)
+    elif kind == "nan":                          # one key is not a number: rows that do not see it stay right
+        q, k = q * 4, k * 4
+        k[int(lengths[0]) - 1] = float("nan")
+    return q.to(torch.bfloat16), k.to(torch.bfloat16), v
+
+
+@pytest.mark.parametrize("kind", ["bounded", "unbounded", "rising", "mixed", "nan"])
+@pytest.mark.parametrize("lengths,hq,hkv,d", [([2432, 640], 2, 2, 128), ([3000, 1500, 700], 4, 1, 64)])
+def test_rows_with_and_without_a_running_maximum(lengths, hq, hkv, d, kind):
+    """Shared-stream mode: rows whose scores the norms bound drop the running maximum, others rescale. Reference: float64
+    attention on the rotated q and k that the library returns (their own parity is tested above), so that the
+    scores agree to fp32 and the rest is rounding: P to bf16 (2^-9 of each term, of which the sum of weights is 1),
+    the sum of weights with or without it (as much again) and O to bf16, together below 2^-7 of the largest |v|."""
+    lengths = np.asarray(lengths, np.int32)
+    q, k, v = _scaled_inputs(kind, lengths, hq, hkv, d)
+    fused = PrefillBatch(lengths, hq, hkv, d, 10000.0, guard=True)
+    three = PrefillBatch(lengths, hq, hkv, d, 10000.0, guard=True)
+    for b, call in ((fused, fused.run_fused), (three, three.run)):
+        _assert_schedule(b, hq, hkv, 0, 0 if (hq // hkv) % 2 == 0 else 1)
+        b.load(q, k, v)
+        call()
+        torch.cuda.synchronize()
+        assert b.device_status() == 0
+        b.assert_untouched()
+    rows = three.token_rows.long()
+    qr = three.q.reshape(-1, hq, d)[rows].double()
+    kr = three.kk.reshape(-1, hkv, d)[rows].double().repeat_interleave(hq // hkv, 1)
+    vr = v.cuda().double().repeat_interleave(hq // hkv, 1)
+    tol = 2.0 ** -7 * float(v.abs().max())
+    start = 0
+    for i, l in enumerate(int(x) for x in lengths):
+        part = slice(start, start + l)
+        seen = l - 1 if kind == "nan" and i == 0 else l
+        s = torch.einsum("qhd,khd->hqk", qr[part], kr[part]) / d ** 0.5
+        s = s.masked_fill(torch.ones(l, l, dtype=torch.bool, device=s.device).triu(1), float("-inf"))
+        ref = torch.einsum("hqk,khd->qhd", torch.softmax(s, -1), vr[part])
+        for b in (fused, three):
+            err = (b.o_tokens()[part].double() - ref).abs()[:seen].max().item()
+            assert err <= tol, (i, err, tol)
+        start += l
