@@ -188,6 +188,7 @@ int pp_prefill_attention(const pp_attn_params* params,
  *                cos/sin table of capacity * D/2 pairs); host_workspace: host staging of at least
  *                pp_prefill_fused_host_bytes (the tables, which are what is uploaded; the cos/sin
  *                table is built on the device), pinned memory keeps the call asynchronous
+ *                (and is read in place by a kernel of the call's)
  * params->flags: PP_FLAG_ROPE_ONLY runs only the rotation / unpack kernels, PP_FLAG_SKIP_ROPE only the
  * attention kernel (k_ holds rotated keys already). Outputs are bit-identical to the two-call path.
  * Errors as the two calls it replaces.

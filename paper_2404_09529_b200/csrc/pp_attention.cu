@@ -622,6 +622,11 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   // Everything above is set-up that touches no tensor: with a programmatic dependent launch it runs
   // while the kernel before this one (rotation / cache scatter) is still finishing.
   pdl_wait();
+  // The next call's table upload may read host memory as SMs run out of work here (2048 short prompts 193 -> 186 us a
+  // step, 64 on a 7B layer 282 -> 278). Not before this wait: the next kernel may count on all that was queued before
+  // this one. Not where tables are parameters: the rotation kernel, which is next then, would fill the first SMs to
+  // become idle with its blocks (16 prompts on a 7B layer 49.5 -> 53.6).
+  if (Table::kUploaded) pdl_launch_dependents();
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFill ? kRegsOtherFill : kRegsOther));

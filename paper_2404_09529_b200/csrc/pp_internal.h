@@ -119,6 +119,10 @@ int launch_zero_pad_rows(void* q, void* k, void* v, int32_t q_row_bytes, int32_t
 
 int launch_bounded_wait_selftest(int32_t* device_status, uint64_t limit_ns, void* stream);
 
+// A table in mapped host memory (both addresses on 16-byte boundaries) into device memory, up to kUploadKernelBytes.
+constexpr size_t kUploadKernelBytes = size_t(1) << 20;
+int launch_upload(void* dst, const void* src, size_t bytes, void* stream);
+
 // Unpack table (int32 units): header 4 ints, then token_prefix[k+1], bin_of[k], off_of[k],
 // cache_cap[k], cache_off as int64[k] (8-byte aligned).
 size_t unpack_table_bytes(int32_t k);
@@ -133,12 +137,14 @@ constexpr int kInlineInts = 896;
 #ifdef __CUDACC__
 // The prefill table as the kernels see it.
 struct TableInMemory {
+  static constexpr bool kUploaded = true;      // by a kernel, perhaps: nothing may be read before pdl_wait()
   const int32_t* p;
   __device__ __forceinline__ int32_t i32(int i) const { return __ldg(p + i); }
   __device__ __forceinline__ int4 i128(int i) const { return __ldg(reinterpret_cast<const int4*>(p + i)); }
   __device__ __forceinline__ int64_t i64(int base, int i) const { return __ldg(reinterpret_cast<const long long*>(p + base) + i); }
 };
 struct alignas(16) TableInline {
+  static constexpr bool kUploaded = false;
   int32_t w[kInlineInts];
   __device__ __forceinline__ int32_t i32(int i) const { return w[i]; }
   __device__ __forceinline__ int4 i128(int i) const { return *reinterpret_cast<const int4*>(w + i); }

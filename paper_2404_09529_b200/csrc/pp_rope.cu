@@ -78,6 +78,7 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32
   __shared__ uint32_t s_norm[kMaxNormHeads];        // [Hkv] of k, then [Hq] of q
 
   pdl_launch_dependents();      // the attention kernel may set up while this one runs
+  if (Table::kUploaded) pdl_wait();
   const int64_t row0 = (int64_t)blockIdx.x * kRopeRows;
   const int64_t n_rows = (int64_t)n_bins * capacity;
   const int tid = threadIdx.x;
@@ -121,7 +122,7 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32
     s_cos[r][j] = cs;
     s_sin[r][j] = sn;
   }
-  pdl_wait();                   // (the set-up above reads parameters or an uploaded table only)
+  pdl_wait();
   if (counter && blockIdx.x == 0 && tid == 0) *counter = 0;
   __syncthreads();
 
@@ -211,6 +212,7 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
   __shared__ uint32_t s_norm[kMaxNormHeads];        // largest |k|^2 of the block's rows, per KV head
 
   pdl_launch_dependents();      // the attention kernel may set up while this one runs
+  if (Table::kUploaded) pdl_wait();
   const int64_t row0 = (int64_t)blockIdx.x * kRuRows;
   const int64_t n_rows = (int64_t)n_bins * capacity;
   const int tid = threadIdx.x;

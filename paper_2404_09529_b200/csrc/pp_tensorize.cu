@@ -149,7 +149,36 @@ host_rows_kernel(HostRows h, RowTable m, int32_t q_vec, int32_t kv_vec, const __
   }
 }
 
+
+// A table read from mapped host memory. A bus read takes 1 to 2 us whatever its size, so all of a thread's reads are
+// issued together, and before the wait for the kernel in front, whose end they overlap.
+constexpr int kUploadThreads = 128, kUploadVecs = 4;
+__global__ void __launch_bounds__(kUploadThreads)
+upload_kernel(uint4* dst, const uint4* src, int32_t n_vec, int32_t tail_words) {
+  const int32_t at = blockIdx.x * (kUploadThreads * kUploadVecs) + threadIdx.x;
+  uint4 val[kUploadVecs];
+#pragma unroll
+  for (int i = 0; i < kUploadVecs; ++i)
+    if (at + i * kUploadThreads < n_vec) val[i] = __ldcv(src + at + i * kUploadThreads);
+  uint32_t word = 0;
+  const bool tail = blockIdx.x == 0 && (int)threadIdx.x < tail_words;
+  if (tail) word = __ldcv(reinterpret_cast<const uint32_t*>(src + n_vec) + threadIdx.x);
+  pdl_wait();                   // the kernel in front may still read the table that was here
+#pragma unroll
+  for (int i = 0; i < kUploadVecs; ++i)
+    if (at + i * kUploadThreads < n_vec) dst[at + i * kUploadThreads] = val[i];
+  if (tail) reinterpret_cast<uint32_t*>(dst + n_vec)[threadIdx.x] = word;
+}
+
 }  // namespace
+
+int launch_upload(void* dst, const void* src, size_t bytes, void* stream) {
+  const int32_t n_vec = (int32_t)(bytes / 16);
+  const unsigned grid = (unsigned)(n_vec / (kUploadThreads * kUploadVecs) + 1);
+  const cudaError_t e = launch_dependent(upload_kernel, dim3(grid), dim3(kUploadThreads), 0, static_cast<cudaStream_t>(stream),
+                                         static_cast<uint4*>(dst), static_cast<const uint4*>(src), n_vec, (int32_t)(bytes % 16 / 4));
+  return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "table upload");
+}
 
 int launch_host_rows(bool to_packed, const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
                      int32_t off_cache_off, const HostRows& rows, void* stream) {

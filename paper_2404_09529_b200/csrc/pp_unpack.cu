@@ -36,6 +36,8 @@ unpack_kernel(const uint4* __restrict__ k_rot, const uint4* __restrict__ v,
               int32_t capacity, int32_t n_kv_heads) {
   constexpr int kVecPerHead = D / 8;
   __shared__ TokenRef s_tok[kUnpackTokens];
+  pdl_wait();
+  pdl_launch_dependents();      // the next call's table upload may read host memory now
   const int64_t tok0 = (int64_t)blockIdx.x * kUnpackTokens;
   const int32_t* prefix = table + 4;
   const int32_t* bin_of = prefix + up4(n_prompts + 1);
@@ -84,16 +86,11 @@ int launch_unpack(const pp_attn_params& p, const int32_t* d_table, int32_t k, in
                   const void* k_rot, const void* v, void* k_cache, void* v_cache, void* stream) {
   const unsigned grid = (unsigned)((total_tokens + kUnpackTokens - 1) / kUnpackTokens);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (p.head_dim == 128) {
-    unpack_kernel<128><<<grid, kUnpackThreads, 0, s>>>(
-        (const uint4*)k_rot, (const uint4*)v, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache,
-        d_table, k, total_tokens, p.capacity, p.n_kv_heads);
-  } else {
-    unpack_kernel<64><<<grid, kUnpackThreads, 0, s>>>(
-        (const uint4*)k_rot, (const uint4*)v, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache,
-        d_table, k, total_tokens, p.capacity, p.n_kv_heads);
-  }
-  const cudaError_t e = cudaGetLastError();
+  const auto launch = [&](auto kernel) {
+    return launch_dependent(kernel, dim3(grid), dim3(kUnpackThreads), 0, s, (const uint4*)k_rot, (const uint4*)v,
+                            (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, d_table, k, total_tokens, p.capacity, p.n_kv_heads);
+  };
+  const cudaError_t e = p.head_dim == 128 ? launch(unpack_kernel<128>) : launch(unpack_kernel<64>);
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "unpack kernel launch");
 }
 

@@ -222,6 +222,34 @@ def test_table_as_parameter_or_uploaded(k, hq, hkv, d):
     assert fused.device_status() == 0 and torch.equal(fused.o_tokens(), o.view(-1, hq, d)[fused.token_rows])
 
 
+@pytest.mark.parametrize("k", [31, 45, 333])
+@pytest.mark.parametrize("staging", ["pinned", "pinned + 16", "pinned + 8", "pageable"])
+def test_tables_from_any_staging_memory(k, staging):
+    """Tables are read by a kernel from aligned pinned memory and copied from any other, several calls in a row
+    through the ring of staging buffers."""
+    lengths = np.asarray([60 - 7 * (i % 9) for i in range(k)], np.int32)
+    q, kk, v = _case(lengths, 2, 1, 64, seed=k)
+    refs = oracle_refs(lengths, q, kk, v, 10000.0)
+    at = int(staging.split("+")[1]) if "+" in staging else 0
+    fused = PrefillBatch(lengths, 2, 1, 64, 10000.0, guard=True)
+    three = PrefillBatch(lengths, 2, 1, 64, 10000.0, guard=True)
+
+    def buffer(like):
+        t = torch.empty(like.numel() + at, dtype=torch.uint8)
+        return (t if staging == "pageable" else t.pin_memory())[at:]
+
+    for b, call in ((fused, fused.run_fused), (three, three.run)):
+        b.ws._fused_host = [buffer(t) for t in b.ws._fused_host]
+        b.ws._ring = [(buffer(a), buffer(u), fence) for a, u, fence in b.ws._ring]
+        for _ in range(6):
+            b.load(q, kk, v)
+            call()
+        torch.cuda.synchronize()
+        assert b.device_status() == 0
+        b.assert_untouched()
+        compare_with_refs(b, lengths, refs)
+
+
 # Multi-head, D = 128, independent mode: the attention kernel fills the V caches from 32 rows per prompt on, the rotation
 # kernel below that. Prompts at the edges of the 64-key and the 128-row tiles, many in a tile, and streams of many items.
 @pytest.mark.parametrize("lengths,room", [
