@@ -4,7 +4,7 @@
 // row carries the key range [start row of its prompt, its own row], and the host work list
 // restricts each query tile to the key tiles that can intersect such a range.
 //
-// Persistent kernel, one CTA per SM, 640 threads, two 128-row query-tile slots per CTA. CTAs draw
+// Persistent kernel, one CTA per SM, 640 threads (768 with kFill), two 128-row query-tile slots per CTA. CTAs draw
 // work from a global counter (items are listed KV-head-major, longest first). Two modes, chosen on
 // the host from the mean number of key tiles per query tile:
 //
