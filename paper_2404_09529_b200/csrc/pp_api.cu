@@ -132,10 +132,11 @@ extern "C" int pp_prefill_attention(const pp_attn_params* params, const int32_t*
   if (!small && (st = pp::upload_table(workspace, host_workspace, sizeof(int32_t) * (size_t)L.total_ints, s)) != PP_OK) return st;
   int32_t* d_table = static_cast<int32_t*>(workspace);
   if (do_rope) {
-    st = pp::launch_rope(*params, d_table, L, small, q, k_, stream);
+    st = pp::launch_rope(*params, d_table, L, small, q, k_, do_attn ? v : nullptr, stream);
     if (st != PP_OK) return st;
   }
   if (do_attn) {
+    if (!do_rope && pp::tracks_ranges(*params, L) && (st = pp::launch_value_range(*params, d_table, L, v, stream)) != PP_OK) return st;
     st = pp::launch_attention(*params, d_table, L, small, q, k_, v, o, nullptr, do_rope, nullptr, device_status, stream);
     if (st != PP_OK) return st;
   }
@@ -209,6 +210,7 @@ int launch_fused_kernels(const pp_attn_params& p, const TableLayout& L, const Fu
     if (st != PP_OK) return st;
   }
   if (!attend) return PP_OK;
+  if (!rotate && tracks_ranges(p, L) && (st = launch_value_range(p, d_table, L, v, stream)) != PP_OK) return st;
   // the attention kernel rotates every Q tile in shared memory, so Q is read from HBM once
   const CacheFill caches{v_cache, (int32_t)f.off_true_len, (int32_t)f.off_cap, (int32_t)f.off_cache_off};
   return launch_attention(p, d_table, L, small, q, k_, v, o, rope_table, rotate, fill ? &caches : nullptr, device_status, stream);

@@ -69,17 +69,21 @@ constexpr int kRegsWriter = 40;            //   warpgroup (40 each); the 256 hel
 // Shared-stream mode, when a row needs no maximum any more. Its running maximum is lazy: it stays at the
 // maximum of the row's first visible tile until a score exceeds it by more than kLazyLog2 (log2 units).
 // Probabilities, sums and O have 8 exponent bits, so a common factor of up to 2^90 costs no precision, and
-// it leaves 2^37 for the number of keys times |v|. Where |q| |k| scale <= kBoundLog2 for every key
+// it leaves 2^37 for the number of keys times |v|: that much room there must be (kValueRoomLog2, with a bit to
+// spare; the largest |v| of the batch is found on the way), or the factor is kept to 2^kLazyLog2Wide and every row
+// has its maximum found. Where |q| |k| scale <= kBoundLog2 for every key
 // (Cauchy-Schwarz, norms taken before the rotation's rounding to bf16), two scores of a row differ by at
 // most 2 * 44 * (1 + 2^-7) < 90, so from its second tile on the row's maximum cannot move: neither the
 // 64 comparisons nor the exchange between the two threads of a row are needed, and the exponentials start
 // on the first 32 scores while the other 32 are still being loaded. The result does not depend on
-// whether the bound was known. Q and K of N(0, 1) values reach 17-30 (D = 64 / 128). Measured, whole step:
+// whether the bound was known, so all routes give the same bits. Q and K of N(0, 1) values reach 17-30 (D = 64 / 128). Measured, whole step:
 // 16 prompts of up to 22 861 tokens, 32 heads, D = 128: 14.69 -> 12.2 ms (attention 14.1 -> 11.15 ms, 1156
 // TFLOP/s, from then on at the power cap: SM clock ~1620 MHz); 256 prompts of up to 3991, 32 / 8 heads:
 // 7.22 -> 6.48 ms. A wait for S took a softmax warp 2570 cycles per 128-key tile, now ~1250, of ~2900 in all.
 constexpr float kLazyLog2 = 90.f;
 constexpr float kBoundLog2 = 44.f;
+constexpr float kLazyLog2Wide = 8.f;
+constexpr int kValueRoomLog2 = 36;
 constexpr uint32_t kRing = 3;               // decoded work items in flight between the fetching thread and its readers
 constexpr int kRingInts = 20;              // ints per ring entry
 
@@ -419,6 +423,8 @@ struct AttnArgs {
   const float2* rope_table;      // [D/4][capacity][2] (cos, sin) pairs, or null: Q arrives already rotated
   const uint32_t* k_norm2;       // shared-stream mode: [Hkv] largest |k|^2 (float bits); null: no bound on the scores
   const uint32_t* q_norm2;       // [Hq] largest |q|^2; used when Q arrives already rotated
+  const uint32_t* v_max;         // shared-stream mode: largest |v| (bf16 bits); null: not known
+  float v_room;                  // 2^kValueRoomLog2 / capacity: |v| up to which kLazyLog2 holds
   int32_t* status;
   unsigned long long wait_limit_ns;
   __nv_bfloat16* v_cache;                         // kFill: the V caches
@@ -1355,6 +1361,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       return r;
     };
     const float c_scale = args.scale_log2;
+    // (a NaN among the values, too, leaves no room)
+    const float lazy_log2 = args.v_max && __uint_as_float(__ldcg(args.v_max) << 16) <= args.v_room ? kLazyLog2 : kLazyLog2Wide;
     uint32_t it_n = 0, tcount = 0;
     bool ok = true;
     // Rotates this thread's part of row `row` of Q_t in shared memory by the angles of position `pos`
@@ -1436,7 +1444,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       // |q|^2 up to which every score of a row stays below the bound (0 if nothing is known about the keys)
       float q2_limit = 0.f;
-      if (args.k_norm2) {
+      if (args.k_norm2 && lazy_log2 == kLazyLog2) {
         const float k2 = __uint_as_float(__ldg(args.k_norm2 + kv_head));
         if (k2 < INFINITY) q2_limit = args.bound2 / fmaxf(k2, 1e-30f);      // (a NaN among the keys bounds nothing)
       }
@@ -1531,7 +1539,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (j == jb_t && args.rope_table) bounded = (*bounded_mine & *bounded_other) != 0;
           const float m_tile = mx * c_scale;
           float m_new = m_run;
-          if (m_tile > m_run + kLazyLog2) m_new = m_tile;
+          if (m_tile > m_run + lazy_log2) m_new = m_tile;
           const bool rescale = (m_new != m_run) && (m_run != -INFINITY);
           if (j > jb_t && __any_sync(0xffffffffu, rescale)) {
             const float alpha = rescale ? fast_exp2(m_run - m_new) : 1.f;
@@ -1712,17 +1720,6 @@ unsigned long long wait_limit_ns() {
   return 2000000000ull;   // 2 s
 }
 
-int sm_count() {
-  static thread_local int cached_dev = -1, cached = 0;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (dev != cached_dev) {
-    if (cudaDeviceGetAttribute(&cached, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    cached_dev = dev;
-  }
-  return cached;
-}
-
 template <int D, bool kIndep, bool kFill, class Table>
 int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const Table& tab, const void* q,
                        const void* k, const void* v, void* o, const void* rope_table, bool have_norms,
@@ -1774,9 +1771,11 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf((float)D);
   a.scale_log2 = scale * 1.4426950408889634f;
   a.bound2 = (kBoundLog2 / a.scale_log2) * (kBoundLog2 / a.scale_log2);
-  const bool norms = have_norms && !kIndep && p.n_q_heads + p.n_kv_heads <= kMaxNormHeads;
+  const bool norms = have_norms && tracks_ranges(p, L);
   a.k_norm2 = norms ? reinterpret_cast<const uint32_t*>(d_table + L.norms) : nullptr;
   a.q_norm2 = norms && !rope_table ? a.k_norm2 + p.n_kv_heads : nullptr;
+  a.v_max = tracks_ranges(p, L) ? reinterpret_cast<const uint32_t*>(d_table + kHeaderValueMax) : nullptr;
+  a.v_room = ldexpf(1.f, kValueRoomLog2) / (float)p.capacity;
   a.o = static_cast<__nv_bfloat16*>(o);
   a.rope_table = static_cast<const float2*>(rope_table);
   a.status = device_status;
@@ -1789,6 +1788,17 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
 }
 
 }  // namespace
+
+int sm_count() {
+  static thread_local int cached_dev = -1, cached = 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (dev != cached_dev) {
+    if (cudaDeviceGetAttribute(&cached, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    cached_dev = dev;
+  }
+  return cached;
+}
 
 int launch_bounded_wait_selftest(int32_t* device_status, uint64_t limit_ns, void* stream) {
   bounded_wait_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(device_status, limit_ns);

@@ -336,6 +336,7 @@ int build_prefill_tables(int32_t n_bins, int32_t capacity, const int32_t* bin_se
   for (const WorkItem& it : items) tiles += it.cost;
   out[9] = (int32_t)std::min<int64_t>(tiles, INT32_MAX);
   out[kHeaderCounter] = 0;   // work counter the CTAs draw from; reset by every upload
+  out[kHeaderValueMax] = 0;  // largest |v|, as far as a kernel has looked
   L.total_ints = (int32_t)(L.items + kItemInts * (int64_t)items.size());
   L.independent_slots = independent;
   L.pair_rows = pair_rows;

@@ -15,6 +15,7 @@ constexpr int kTileNShort = 64;  // the same in independent-slot mode (short wor
 constexpr int kHeaderInts = 16;  // table header, see build_prefill_tables
 constexpr int kHeaderSegments = 4;   // header word with the number of segments
 constexpr int kHeaderCounter = 10;   // header word the persistent CTAs draw work indices from
+constexpr int kHeaderValueMax = 11;  // header word with the largest |v| (bf16 bits), shared-stream mode; zero in the uploaded table
 constexpr int kItemInts = 16;
 constexpr int kMaxFold = 8;      // most query heads of one KV head folded into the rows of a query tile
 constexpr int kMaxNormHeads = 512;   // Hq + Hkv up to which the rotation kernels track the norms (shared memory)
@@ -62,16 +63,18 @@ int build_prefill_tables(int32_t n_bins, int32_t capacity, const int32_t* bin_se
                          const int32_t* seg_start, const int32_t* seg_len, int32_t k, int32_t n_q_heads,
                          int32_t n_kv_heads, int32_t* out, size_t out_ints, TableLayout* layout);
 
+int sm_count();     // multiprocessors of the current device; 0 if it cannot be asked
+
 // Records a failed CUDA call for pp_last_cuda_error(); returns PP_ERR_CUDA.
 int note_cuda_error(int cuda_error, const char* what);
 
 // Kernel launchers (device pointers, stream = cudaStream_t as void*). Return a PP_* status.
 // Rotates q and k in place; in the shared-stream mode it also leaves the largest |k|^2 and |q|^2 of every
-// head in the table (L.norms).
+// head (L.norms) and, unless v is null, the largest |v| (kHeaderValueMax) in the table.
 // inline_table (here and below): null, or the host copy of a table that was not uploaded and travels in the
 // kernel's parameters; the rotation kernel then resets the work counter in d_table.
 int launch_rope(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table, void* q, void* k,
-                void* stream);
+                const void* v, void* stream);
 // rope_table: device [D/4][capacity][2] (cos, sin) pairs, or null. When given, q holds the raw
 // queries and the kernel rotates each Q tile in shared memory before use. have_norms: a rotation kernel
 // of the same call has filled the norms of the table (of the keys, and without rope_table of the queries).
@@ -84,10 +87,15 @@ struct CacheFill {
 int launch_attention(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
                      const void* q, const void* k, const void* v, void* o, const void* rope_table,
                      bool have_norms, const CacheFill* caches, int32_t* device_status, void* stream);
+// Whether the kernels leave norms and the largest |v| in the table and use them: shared-stream mode, and as many heads
+// as the rotation kernels' shared memory has room for.
+bool tracks_ranges(const pp_attn_params& p, const TableLayout& L);
+// Largest |v| of the packed batch into the table (kHeaderValueMax), where no rotation kernel of the call has read v.
+int launch_value_range(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const void* v, void* stream);
 // Fused K rotation + UNPACK; the three offsets locate per-segment arrays inside the table
 // (true length, cache capacity: int32; cache element offset: int64). v null: the V caches are filled elsewhere.
-// In the shared-stream mode it also leaves
-// the largest |k|^2 of every KV head in the table (L.norms).
+// In the shared-stream mode (v is not null there) it also leaves the largest |k|^2 of every KV head (L.norms) and the
+// largest |v| (kHeaderValueMax) in the table.
 int launch_rope_unpack(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table,
                        int32_t off_true_len, int32_t off_cap, int32_t off_cache_off, const void* rope_table,
                        void* k, const void* v, void* k_cache, void* v_cache, void* stream);

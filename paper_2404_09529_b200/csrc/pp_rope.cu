@@ -4,6 +4,9 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "pp_internal.h"
 
 namespace pp {
@@ -62,11 +65,36 @@ __device__ __forceinline__ float sum_squares(const uint4& lo, const uint4& hi) {
   return a + b;
 }
 
-// norms: null, or [Hkv] then [Hq] words that receive the largest |k|^2 / |q|^2 of each head.
+// Largest |x| of bf16 pairs, a NaN if there is one.
+__device__ __forceinline__ __nv_bfloat162 max_abs(__nv_bfloat162 m, const uint4& x) {
+  const uint32_t w[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) m = __hmax2_nan(m, __habs2(*reinterpret_cast<const __nv_bfloat162*>(&w[i])));
+  return m;
+}
+// ... of a warp into *s_max as bits, which order like the values and a NaN above all
+__device__ __forceinline__ void note_max_abs(__nv_bfloat162 m2, uint32_t* s_max) {
+  const uint32_t bits = *reinterpret_cast<const uint32_t*>(&m2);
+  const uint32_t m = __reduce_max_sync(0xffffffffu, max(bits >> 16, bits & 0xffffu));
+  if ((threadIdx.x & 31) == 0) atomicMax(s_max, m);
+}
+// A block's maxima to global memory: s_max[0 .. n) to out[0 .. n), s_max[n] to *out_v.
+__device__ __forceinline__ void publish_ranges(const uint32_t* s_max, int n, uint32_t* out, uint32_t* out_v) {
+  __syncthreads();
+  for (int h = threadIdx.x; h <= n; h += kRopeThreads) {
+    uint32_t* dst = h < n ? out + h : out_v;
+    if (s_max[h] > __ldcg(dst)) atomicMax(dst, s_max[h]);
+  }
+}
+
+// kRange (shared-stream mode): norms, [Hkv] then [Hq] words, receive the largest |k|^2 / |q|^2 of each head, v_max the
+// largest |v| of the real rows of v (null: not wanted). Reading V here costs its bytes (four prompts of 3000 to 4096
+// tokens on 32 / 32 heads of 128, three calls: 638 -> 655 us; as a kernel of its own 633 -> 664).
 // counter: null, or the work counter to reset for the attention kernel.
-template <int D, class Table>
+template <int D, bool kRange, class Table>
 __global__ void __launch_bounds__(kRopeThreads)
-rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32_t* norms, int32_t* counter,
+rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, uint32_t* norms,
+            uint32_t* v_max, int32_t* counter,
             const __grid_constant__ Table tab, int32_t off_bin_seg_ptr, int32_t off_bin_used,
             int32_t off_seg_start, int32_t n_bins, int32_t capacity, int32_t n_q_heads,
             int32_t n_kv_heads, const __grid_constant__ RopeFreq freq) {
@@ -75,7 +103,7 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32
   __shared__ int32_t s_pos[kRopeRows];              // restart position, -1 for padding rows
   __shared__ float s_cos[kRopeRows][kHalf];
   __shared__ float s_sin[kRopeRows][kHalf];
-  __shared__ uint32_t s_norm[kMaxNormHeads];        // [Hkv] of k, then [Hq] of q
+  __shared__ uint32_t s_norm[kMaxNormHeads + 1];    // [Hkv] of k, then [Hq] of q, then v
 
   pdl_launch_dependents();      // the attention kernel may set up while this one runs
   if (Table::kUploaded) pdl_wait();
@@ -84,8 +112,8 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32
   const int tid = threadIdx.x;
 
   const int n_heads = n_q_heads + n_kv_heads;
-  if (norms)
-    for (int h = tid; h < n_heads; h += kRopeThreads) s_norm[h] = 0u;
+  if (kRange)
+    for (int h = tid; h <= n_heads; h += kRopeThreads) s_norm[h] = 0u;
   if (tid < kRopeRows) {
     const int64_t row = row0 + tid;
     int32_t pos = -1;
@@ -138,23 +166,37 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, uint32
     const int64_t row = row0 + r;
     const bool is_q = head < n_q_heads;
     float n2 = 0.f;
-    if (pos > 0 || (norms && pos == 0)) {                     // padding rows are skipped, position 0 is the identity
+    if (pos > 0 || (kRange && pos == 0)) {                     // padding rows are skipped, position 0 is the identity
       __nv_bfloat16* p = is_q ? q + (row * n_q_heads + head) * D : k + (row * n_kv_heads + (head - n_q_heads)) * D;
       uint4 lo = *reinterpret_cast<const uint4*>(p + c * 8);
       uint4 hi = *reinterpret_cast<const uint4*>(p + kHalf + c * 8);
-      if (norms) n2 = sum_squares(lo, hi);
+      if (kRange) n2 = sum_squares(lo, hi);
       if (pos > 0) {
         rotate8(lo, hi, &s_cos[r][c * 8], &s_sin[r][c * 8]);
         *reinterpret_cast<uint4*>(p + c * 8) = lo;
         *reinterpret_cast<uint4*>(p + kHalf + c * 8) = hi;
       }
     }
-    if (norms) note_norm<kUnitsPerHead>(n2, pos >= 0, s_norm + (is_q ? n_kv_heads + head : head - n_q_heads));
+    if (kRange) note_norm<kUnitsPerHead>(n2, pos >= 0, s_norm + (is_q ? n_kv_heads + head : head - n_q_heads));
   }
-  if (norms) {
-    __syncthreads();
-    for (int h = tid; h < n_heads; h += kRopeThreads)
-      if (s_norm[h] > __ldcg(norms + h)) atomicMax(norms + h, s_norm[h]);
+  if (kRange) {
+    if (v) {
+      constexpr int kAtOnce = 4;
+      const int vecs = n_kv_heads * (D / 8);
+      __nv_bfloat162 m = __float2bfloat162_rn(0.f);
+      for (int u0 = tid; u0 < kRopeRows * vecs; u0 += kAtOnce * kRopeThreads) {
+        uint4 val[kAtOnce];
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) {
+          const int u = u0 + i * kRopeThreads, r = u / vecs;
+          val[i] = u < kRopeRows * vecs && s_pos[r] >= 0 ? __ldg(reinterpret_cast<const uint4*>(v) + row0 * vecs + u) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int i = 0; i < kAtOnce; ++i) m = max_abs(m, val[i]);
+      }
+      note_max_abs(m, s_norm + n_heads);
+    }
+    publish_ranges(s_norm, n_heads, norms, v_max);
   }
 }
 
@@ -195,10 +237,11 @@ constexpr int kRuNarrowRowElems = 1024;   // n_kv_heads * D up to which a row co
 constexpr int64_t kRuNarrowRows = 32 * 148 * 4;
 constexpr int kRuV = 8;      // 16-byte V copies in flight per thread
 constexpr int kRuK = 2;      // (lower, upper) K pairs in flight per thread
-template <int D, int kRuRows, class Table>
+// kRange: the norms and the largest |v| are wanted (shared-stream mode).
+template <int D, int kRuRows, bool kRange, class Table>
 __global__ void __launch_bounds__(kRopeThreads)
 rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, uint32_t* norms,
-                   int32_t* counter, __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
+                   uint32_t* v_max, int32_t* counter, __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
                    const __grid_constant__ Table tab, int32_t off_bin_seg_ptr, int32_t off_bin_used,
                    int32_t off_seg_start, SegExt ext, const float2* __restrict__ rope_table,
                    int32_t n_bins, int32_t capacity, int32_t n_kv_heads) {
@@ -209,15 +252,15 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
   __shared__ int64_t s_dst[kRuRows];              // cache element offset of (head 0, this position); -1: not cached
   __shared__ int64_t s_head_stride[kRuRows];      // cache_cap * D
   __shared__ float4 s_tab[kRuRows][D / 4];          // (cos, sin) of j = 2g, 2g + 1 at each row's position
-  __shared__ uint32_t s_norm[kMaxNormHeads];        // largest |k|^2 of the block's rows, per KV head
+  __shared__ uint32_t s_norm[kMaxNormHeads + 1];    // largest |k|^2 of the block's rows, per KV head, then their largest |v|
 
   pdl_launch_dependents();      // the attention kernel may set up while this one runs
   if (Table::kUploaded) pdl_wait();
   const int64_t row0 = (int64_t)blockIdx.x * kRuRows;
   const int64_t n_rows = (int64_t)n_bins * capacity;
   const int tid = threadIdx.x;
-  if (norms)
-    for (int h = tid; h < n_kv_heads; h += kRopeThreads) s_norm[h] = 0u;
+  if (kRange)
+    for (int h = tid; h <= n_kv_heads; h += kRopeThreads) s_norm[h] = 0u;
   if (tid < kRuRows) {
     const int64_t row = row0 + tid;
     int32_t pos = -1;
@@ -252,8 +295,10 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
     if (pos > 0) s_tab[r][g] = __ldg(reinterpret_cast<const float4*>(rope_table) + (size_t)g * (size_t)capacity + pos);
   }
 
-  // V rows first: plain 16-byte copies, four in flight per thread
+  // V rows first: plain 16-byte copies, kRuV in flight per thread (rows that are attended to but not cached are
+  // read for their largest value only)
   const int units_v = v ? n_kv_heads * kVecs : 0;
+  __nv_bfloat162 my_v_max = __float2bfloat162_rn(0.f);
   for (int u0 = tid; u0 < kRuRows * units_v; u0 += kRuV * kRopeThreads) {
     uint4 val[kRuV];
     int64_t dsts[kRuV];
@@ -263,16 +308,18 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
       dsts[i] = -1;
       if (u < kRuRows * units_v) {
         const int r = u / units_v, w = u - r * units_v;
-        if (s_dst[r] >= 0) {
+        if (s_dst[r] >= 0 || (kRange && s_pos[r] >= 0)) {
           const int head = w / kVecs, c = w - head * kVecs;
           val[i] = __ldg(reinterpret_cast<const uint4*>(v + ((row0 + r) * n_kv_heads + head) * D + c * 8));
-          dsts[i] = s_dst[r] + head * s_head_stride[r] + c * 8;
+          dsts[i] = !kRange || s_dst[r] >= 0 ? s_dst[r] + head * s_head_stride[r] + c * 8 : -2;
         }
       }
     }
 #pragma unroll
-    for (int i = 0; i < kRuV; ++i)
+    for (int i = 0; i < kRuV; ++i) {
       if (dsts[i] >= 0) *reinterpret_cast<uint4*>(v_cache + dsts[i]) = val[i];
+      if (kRange && dsts[i] != -1) my_v_max = max_abs(my_v_max, val[i]);
+    }
   }
   __syncthreads();
   // K rows: rotate, write back to the packed tensor and into the cache; two pairs in flight
@@ -298,7 +345,7 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
     }
 #pragma unroll
     for (int i = 0; i < kRuK; ++i) {
-      if (norms) note_norm<kPairUnits>(rr[i] < 0 ? 0.f : sum_squares(lo[i], hi[i]), rr[i] >= 0, s_norm + hh[i]);
+      if (kRange) note_norm<kPairUnits>(rr[i] < 0 ? 0.f : sum_squares(lo[i], hi[i]), rr[i] >= 0, s_norm + hh[i]);
       if (rr[i] < 0) continue;
       const int r = rr[i], head = hh[i], c = cc[i];
       const int32_t pos = s_pos[r];
@@ -321,18 +368,44 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
       }
     }
   }
-  if (norms) {
-    __syncthreads();
-    for (int h = tid; h < n_kv_heads; h += kRopeThreads)
-      if (s_norm[h] > __ldcg(norms + h)) atomicMax(norms + h, s_norm[h]);
+  if (kRange) {
+    note_max_abs(my_v_max, s_norm + n_kv_heads);
+    publish_ranges(s_norm, n_kv_heads, norms, v_max);
   }
 }
 
-// Where the rotation kernels leave the norms: the table's norm words in the shared-stream mode, which uses
-// them; null in the independent mode and where there are more heads than the kernels' shared memory holds.
+// The largest |v| of the occupied rows where no rotation kernel of the call has read V (attention alone). HBM-bound.
+// grid = (bins, slices of a bin).
+constexpr int kRangeVecs = 8;      // 16-byte loads in flight per thread
+__global__ void __launch_bounds__(kRopeThreads)
+value_range_kernel(const uint4* __restrict__ v, const TableInMemory tab, int32_t off_bin_used, int32_t capacity, int32_t vec_per_row,
+                   uint32_t* v_max) {
+  __shared__ uint32_t s_max;
+  if (threadIdx.x == 0) s_max = 0u;
+  pdl_launch_dependents();
+  pdl_wait();
+  __syncthreads();
+  const int64_t n = (int64_t)tab.i32(off_bin_used + blockIdx.x) * vec_per_row;
+  const uint4* src = v + (int64_t)blockIdx.x * capacity * vec_per_row;
+  const int64_t stride = (int64_t)gridDim.y * kRopeThreads;
+  __nv_bfloat162 m = __float2bfloat162_rn(0.f);
+  for (int64_t at = (int64_t)blockIdx.y * kRopeThreads + threadIdx.x; at < n; at += kRangeVecs * stride) {
+    uint4 val[kRangeVecs];
+#pragma unroll
+    for (int i = 0; i < kRangeVecs; ++i) val[i] = at + i * stride < n ? __ldg(src + at + i * stride) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int i = 0; i < kRangeVecs; ++i) m = max_abs(m, val[i]);
+  }
+  note_max_abs(m, &s_max);
+  publish_ranges(&s_max, 0, nullptr, v_max);
+}
+
+// Where the kernels leave the norms and the largest |v|: words of the table, or null where nothing uses them.
 uint32_t* norm_words(const pp_attn_params& p, int32_t* d_table, const TableLayout& L) {
-  if (L.independent_slots || p.n_q_heads + p.n_kv_heads > kMaxNormHeads) return nullptr;
-  return reinterpret_cast<uint32_t*>(d_table + L.norms);
+  return tracks_ranges(p, L) ? reinterpret_cast<uint32_t*>(d_table + L.norms) : nullptr;
+}
+uint32_t* value_word(const pp_attn_params& p, int32_t* d_table, const TableLayout& L) {
+  return tracks_ranges(p, L) ? reinterpret_cast<uint32_t*>(d_table + kHeaderValueMax) : nullptr;
 }
 
 RopeFreq make_freq(const pp_attn_params& p) {
@@ -353,34 +426,64 @@ int launch_rope_unpack_t(const pp_attn_params& p, int32_t* d_table, const TableL
   const unsigned grid = (unsigned)((n_rows + rows - 1) / rows);
   auto launch = [&](auto kernel) {
     return launch_dependent(kernel, dim3(grid), dim3(kRopeThreads), 0, s, (__nv_bfloat16*)k, (const __nv_bfloat16*)v,
-                            norm_words(p, d_table, L), counter, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, tab,
+                            norm_words(p, d_table, L), value_word(p, d_table, L), counter, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, tab,
                             L.bin_seg_ptr, L.bin_used, L.seg_start, ext, (const float2*)rope_table, p.n_bins, p.capacity,
                             p.n_kv_heads);
   };
   cudaError_t e;
-  if (p.head_dim == 128)
-    e = narrow ? launch(rope_unpack_kernel<128, kRuRowsNarrow, Table>) : launch(rope_unpack_kernel<128, kRuRowsWide, Table>);
+  const auto launch_d = [&](auto range) {
+    constexpr bool kRange = decltype(range)::value;
+    if (p.head_dim == 128)
+      return narrow ? launch(rope_unpack_kernel<128, kRuRowsNarrow, kRange, Table>) : launch(rope_unpack_kernel<128, kRuRowsWide, kRange, Table>);
+    return narrow ? launch(rope_unpack_kernel<64, kRuRowsNarrow, kRange, Table>) : launch(rope_unpack_kernel<64, kRuRowsWide, kRange, Table>);
+  };
+  if constexpr (Table::kUploaded)           // (tables as parameters: independent mode only)
+    e = tracks_ranges(p, L) ? launch_d(std::true_type{}) : launch_d(std::false_type{});
   else
-    e = narrow ? launch(rope_unpack_kernel<64, kRuRowsNarrow, Table>) : launch(rope_unpack_kernel<64, kRuRowsWide, Table>);
+    e = launch_d(std::false_type{});
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope+unpack kernel launch");
 }
 
 template <class Table>
 int launch_rope_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const Table& tab, int32_t* counter, void* q,
-                  void* k, cudaStream_t s) {
+                  void* k, const void* v, cudaStream_t s) {
   const RopeFreq freq = make_freq(p);
   const int64_t n_rows = (int64_t)p.n_bins * p.capacity;
   const unsigned grid = (unsigned)((n_rows + kRopeRows - 1) / kRopeRows);
   auto launch = [&](auto kernel) {
-    return launch_dependent(kernel, dim3(grid), dim3(kRopeThreads), 0, s, (__nv_bfloat16*)q, (__nv_bfloat16*)k,
-                            norm_words(p, d_table, L), counter, tab, L.bin_seg_ptr, L.bin_used, L.seg_start, p.n_bins,
+    return launch_dependent(kernel, dim3(grid), dim3(kRopeThreads), 0, s, (__nv_bfloat16*)q, (__nv_bfloat16*)k, (const __nv_bfloat16*)v,
+                            norm_words(p, d_table, L), value_word(p, d_table, L), counter, tab, L.bin_seg_ptr, L.bin_used, L.seg_start, p.n_bins,
                             p.capacity, p.n_q_heads, p.n_kv_heads, freq);
   };
-  const cudaError_t e = p.head_dim == 128 ? launch(rope_kernel<128, Table>) : launch(rope_kernel<64, Table>);
+  const auto launch_d = [&](auto range) {
+    constexpr bool kRange = decltype(range)::value;
+    return p.head_dim == 128 ? launch(rope_kernel<128, kRange, Table>) : launch(rope_kernel<64, kRange, Table>);
+  };
+  cudaError_t e;
+  if constexpr (Table::kUploaded)           // (tables as parameters: independent mode only)
+    e = tracks_ranges(p, L) ? launch_d(std::true_type{}) : launch_d(std::false_type{});
+  else
+    e = launch_d(std::false_type{});
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "rope kernel launch");
 }
 
 }  // namespace
+
+bool tracks_ranges(const pp_attn_params& p, const TableLayout& L) {
+  return !L.independent_slots && p.n_q_heads + p.n_kv_heads <= kMaxNormHeads;
+}
+
+int launch_value_range(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const void* v, void* stream) {
+  const int32_t vec_per_row = p.n_kv_heads * p.head_dim / 8;
+  // about four blocks per SM, but no slice of a bin shorter than one pass of a block
+  const int64_t per_bin = ((int64_t)p.capacity * vec_per_row + kRopeThreads * kRangeVecs - 1) / (kRopeThreads * kRangeVecs);
+  const int64_t wanted = (4 * (int64_t)std::max(sm_count(), 1) + p.n_bins - 1) / p.n_bins;
+  const unsigned slices = (unsigned)std::min<int64_t>(std::min(per_bin, wanted), 65535);
+  const cudaError_t e = launch_dependent(value_range_kernel, dim3((unsigned)p.n_bins, slices), dim3(kRopeThreads), 0,
+                                         static_cast<cudaStream_t>(stream), static_cast<const uint4*>(v), TableInMemory{d_table},
+                                         L.bin_used, p.capacity, vec_per_row, value_word(p, d_table, L));
+  return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "value range kernel launch");
+}
 
 int launch_rope_table(const pp_attn_params& p, void* table, void* stream) {
   const RopeFreq freq = make_freq(p);
@@ -404,11 +507,11 @@ int launch_rope_unpack(const pp_attn_params& p, int32_t* d_table, const TableLay
 }
 
 int launch_rope(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const int32_t* inline_table, void* q, void* k,
-                void* stream) {
+                const void* v, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (inline_table)
-    return launch_rope_t(p, d_table, L, inline_copy(inline_table, (size_t)L.total_ints), d_table + kHeaderCounter, q, k, s);
-  return launch_rope_t(p, d_table, L, TableInMemory{d_table}, nullptr, q, k, s);
+    return launch_rope_t(p, d_table, L, inline_copy(inline_table, (size_t)L.total_ints), d_table + kHeaderCounter, q, k, v, s);
+  return launch_rope_t(p, d_table, L, TableInMemory{d_table}, nullptr, q, k, v, s);
 }
 
 }  // namespace pp

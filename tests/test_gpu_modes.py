@@ -322,3 +322,59 @@ def test_rows_with_and_without_a_running_maximum(lengths, hq, hkv, d, kind):
             err = (b.o_tokens()[part].double() - ref).abs()[:seen].max().item()
             assert err <= tol, (i, err, tol)
         start += l
+
+
+def _climbing_scores(climb, lengths, hq, hkv, d):
+    """q and k along one slowly turning direction, so that a row's scores climb from -climb to climb (log2 units) with
+    the key's place in its prompt; a little noise on top."""
+    q, k, v = _case(lengths, hq, hkv, d, seed=d + hq)
+    pos = torch.cat([torch.arange(int(l)) / int(l) for l in lengths]).view(-1, 1)
+    amp = (climb * d ** 0.5 / 1.4426950408889634) ** 0.5
+    q, k = q * 0.02, k * 0.02
+    q[:, :, d // 2 - 1] += amp
+    k[:, :, d // 2 - 1] += amp * (2 * pos - 1)
+    return q.to(torch.bfloat16), k.to(torch.bfloat16), v
+
+
+def _float64_attention(rotated, values, lengths, scale):
+    """O of every prompt in float64 from the rotated q and k that the library handed back."""
+    qr, kr = (x.double() for x in rotated)
+    group = qr.shape[1] // kr.shape[1]
+    kr, vr = kr.repeat_interleave(group, 1), values.cuda().double().repeat_interleave(group, 1)
+    out, start = [], 0
+    for l in (int(x) for x in lengths):
+        part = slice(start, start + l)
+        s = torch.einsum("qhd,khd->hqk", qr[part], kr[part]) * scale
+        s = s.masked_fill(torch.ones(l, l, dtype=torch.bool, device=s.device).triu(1), float("-inf"))
+        out.append(torch.einsum("hqk,khd->qhd", torch.softmax(s, -1), vr[part]))
+        start += l
+    return torch.cat(out)
+
+
+@pytest.mark.parametrize("v_scale", [1.0, 2.0 ** 60, 2.0 ** 100])
+@pytest.mark.parametrize("climb", [38, 300])           # within the bound on the scores, beyond it
+@pytest.mark.parametrize("lengths,hq,hkv,d", [([2432, 640], 2, 2, 128), ([3000, 1500, 700], 4, 1, 64)])
+def test_large_values_where_scores_climb(lengths, hq, hkv, d, climb, v_scale):
+    """Shared-stream mode: however far a row's scores climb above those of its first key tile, O stays finite for values up
+    to 2^100, and all routes give the same bits. Tolerance as in test_rows_with_and_without_a_running_maximum."""
+    lengths = np.asarray(lengths, np.int32)
+    q, k, v = _climbing_scores(climb, lengths, hq, hkv, d)
+    v = (v * v_scale).to(torch.bfloat16)
+    routes = {"three calls": lambda b: b.run(), "fused": lambda b: b.run_fused(),
+              "three calls, split": lambda b: (b.run(flags=pp.PP_FLAG_ROPE_ONLY, unpack=False), b.run(flags=pp.PP_FLAG_SKIP_ROPE)),
+              "fused, split": lambda b: (b.run_fused(flags=pp.PP_FLAG_ROPE_ONLY), b.run_fused(flags=pp.PP_FLAG_SKIP_ROPE))}
+    first = None
+    for name, call in routes.items():
+        b = PrefillBatch(lengths, hq, hkv, d, 10000.0)
+        _assert_schedule(b, hq, hkv, 0, 0 if (hq // hkv) % 2 == 0 else 1)
+        b.load(q, k, v)
+        call(b)
+        torch.cuda.synchronize()
+        assert b.device_status() == 0
+        got = (b.o_tokens(), b.k_cache, b.v_cache)
+        if first is None:
+            first = got
+            err = (got[0].double() - _float64_attention(b.rotated_tokens(), v, lengths, d ** -0.5)).abs().max().item()
+            assert err <= 2.0 ** -7 * float(v.abs().max()), err
+        for x, y in zip(first, got):
+            assert torch.equal(x, y), name
