@@ -1368,7 +1368,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // Rotates this thread's part of row `row` of Q_t in shared memory by the angles of position `pos`
     // (< 0: padding, nothing to do), with the same fp32 arithmetic and rounding as the stand-alone
     // kernel, then reports the slot's Q as ready. Waits for the TMA load of Q first. The warp also says
-    // whether its half of every row is short enough for the bound on the scores: |half|^2 <= limit.
+    // whether its half of every row is short enough for the bound on the scores: |half|^2 <= limit (0: there is no bound,
+    // not even for a row whose squares come to 0).
     volatile uint8_t* const bounded_mine = s_bounded + (t * 4 + quad) * 2 + h;
     volatile uint8_t* const bounded_other = s_bounded + (t * 4 + quad) * 2 + (h ^ 1);
     auto rotate_q = [&](const int pos, const float limit, const uint32_t parity) -> bool {
@@ -1413,7 +1414,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
       }
-      const bool short_rows = __all_sync(0xffffffffu, sum_f2x2(n2a, n2b) <= limit);
+      const bool short_rows = __all_sync(0xffffffffu, limit > 0.f && sum_f2x2(n2a, n2b) <= limit);
       if (lane == 0) *bounded_mine = short_rows ? 1 : 0;
       mbar_arrive(bar_q_rot + 8 * t);
       return true;
@@ -1455,7 +1456,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         ok = rotate_q(used ? key_hi - key_lo : -1, 0.5f * q2_limit, it_n & 1u);
         if (!ok) break;
       } else if (args.q_norm2) {
-        bounded = __uint_as_float(__ldg(args.q_norm2 + head_t)) <= q2_limit;
+        bounded = q2_limit > 0.f && __uint_as_float(__ldg(args.q_norm2 + head_t)) <= q2_limit;
       }
       float m_run = -INFINITY;      // running maximum of the whole row, in scaled log2 units
       uint64_t sum_a = 0ull, sum_b = 0ull;   // this thread's share of the running sum of exp2(s * c - m_run), in four parts

@@ -378,3 +378,30 @@ def test_large_values_where_scores_climb(lengths, hq, hkv, d, climb, v_scale):
             assert err <= 2.0 ** -7 * float(v.abs().max()), err
         for x, y in zip(first, got):
             assert torch.equal(x, y), name
+
+
+@pytest.mark.parametrize("end", ["no bound"])
+@pytest.mark.parametrize("lengths,hq,hkv,d", [([2432, 640], 2, 2, 128), ([3000, 1500, 700], 4, 1, 64)])
+def test_bound_on_the_scores_at_its_ends(lengths, hq, hkv, d, end):
+    """Shared-stream mode, scores that climb by thousands, where the limit on |q|^2 is at an end of its range. "no bound":
+    squares of the keys overflow and those of the queries come to 0. Tolerance as in
+    test_rows_with_and_without_a_running_maximum."""
+    lengths = np.asarray(lengths, np.int32)
+    scale, q_size, k_size = {"no bound": (0.0, 1e-23, 4e27)}[end]
+    q, k, v = _case(lengths, hq, hkv, d, seed=d + hq)
+    pos = torch.cat([torch.arange(int(l)) / int(l) for l in lengths]).view(-1, 1)
+    q, k = q.float() * 0.01, k.float() * 0.01
+    q[:, :, d // 2 - 1] += 1
+    k[:, :, d // 2 - 1] += 0.05 + pos
+    q, k = (q * q_size).to(torch.bfloat16), (k * k_size).to(torch.bfloat16)
+    three, fused = (PrefillBatch(lengths, hq, hkv, d, 10000.0, softmax_scale=scale) for _ in range(2))
+    for b, call in ((three, three.run), (fused, fused.run_fused)):
+        _assert_schedule(b, hq, hkv, 0, 0 if (hq // hkv) % 2 == 0 else 1)
+        b.load(q, k, v)
+        call()
+        torch.cuda.synchronize()
+        assert b.device_status() == 0
+    ref = _float64_attention(three.rotated_tokens(), v, lengths, scale or d ** -0.5)
+    for b in (three, fused):
+        err = (b.o_tokens().double() - ref).abs().max().item()
+        assert err <= 2.0 ** -7 * float(v.abs().max()), err
