@@ -44,6 +44,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <cfloat>
 #include <cmath>
 #include <cstdlib>
 #include <type_traits>
@@ -1447,7 +1448,8 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       float q2_limit = 0.f;
       if (args.k_norm2 && lazy_log2 == kLazyLog2) {
         const float k2 = __uint_as_float(__ldg(args.k_norm2 + kv_head));
-        if (k2 < INFINITY) q2_limit = args.bound2 / fmaxf(k2, 1e-30f);      // (a NaN among the keys bounds nothing)
+        // (a NaN among the keys bounds nothing; the limit is finite, for a |q|^2 that overflows is beyond any)
+        if (k2 < INFINITY) q2_limit = fminf(args.bound2 / fmaxf(k2, 1e-30f), FLT_MAX);
       }
       bool bounded = false;
       // Fused path: Q arrives raw and is rotated in shared memory. Each half of a row is held to half
@@ -1771,7 +1773,7 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.total_work = (int32_t)total;
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 1.0f / sqrtf((float)D);
   a.scale_log2 = scale * 1.4426950408889634f;
-  a.bound2 = (kBoundLog2 / a.scale_log2) * (kBoundLog2 / a.scale_log2);
+  a.bound2 = fminf((kBoundLog2 / a.scale_log2) * (kBoundLog2 / a.scale_log2), FLT_MAX);
   const bool norms = have_norms && tracks_ranges(p, L);
   a.k_norm2 = norms ? reinterpret_cast<const uint32_t*>(d_table + L.norms) : nullptr;
   a.q_norm2 = norms && !rope_table ? a.k_norm2 + p.n_kv_heads : nullptr;

@@ -380,14 +380,14 @@ def test_large_values_where_scores_climb(lengths, hq, hkv, d, climb, v_scale):
             assert torch.equal(x, y), name
 
 
-@pytest.mark.parametrize("end", ["no bound"])
+@pytest.mark.parametrize("end", ["no bound", "infinite"])
 @pytest.mark.parametrize("lengths,hq,hkv,d", [([2432, 640], 2, 2, 128), ([3000, 1500, 700], 4, 1, 64)])
 def test_bound_on_the_scores_at_its_ends(lengths, hq, hkv, d, end):
     """Shared-stream mode, scores that climb by thousands, where the limit on |q|^2 is at an end of its range. "no bound":
-    squares of the keys overflow and those of the queries come to 0. Tolerance as in
-    test_rows_with_and_without_a_running_maximum."""
+    squares of the keys overflow and those of the queries come to 0; "infinite": the scale is so small that the
+    limit itself overflows. Tolerance as in test_rows_with_and_without_a_running_maximum."""
     lengths = np.asarray(lengths, np.int32)
-    scale, q_size, k_size = {"no bound": (0.0, 1e-23, 4e27)}[end]
+    scale, q_size, k_size = {"no bound": (0.0, 1e-23, 4e27), "infinite": (1e-20, 1e12, 3.5e11)}[end]
     q, k, v = _case(lengths, hq, hkv, d, seed=d + hq)
     pos = torch.cat([torch.arange(int(l)) / int(l) for l in lengths]).view(-1, 1)
     q, k = q.float() * 0.01, k.float() * 0.01
