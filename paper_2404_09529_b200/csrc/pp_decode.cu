@@ -171,17 +171,28 @@ __device__ __forceinline__ void softmax_step(Softmax<D>& s, float (&c)[4], float
   }
 }
 
+// (a, b) cut to bf16, a in the low half.
+__device__ __forceinline__ uint32_t truncate_bf16x2(float a, float b) {
+  uint32_t y;
+  asm("cvt.rz.bf16x2.f32 %0, %1, %2;" : "=r"(y) : "f"(b), "f"(a));
+  return y;
+}
+
 // O^T += V^T P. Product j: row g is d = 8g + j, row g + 8 is d = 64 + 8g + j (D = 128) or 8g + 4 + j (D = 64).
 template <int D>
 __device__ __forceinline__ void pv(Softmax<D>& s, const StepV<D>& f, const float (&p)[4]) {
+  // P in three parts of 8 bits, cut and not rounded, so that none is negative, and none is 0: an infinite value (also in the
+  // row that stands in for those past the chunk) then gives an infinity and not a NaN, a finite one 2^-126 of itself.
+  const __nv_bfloat162 least = __halves2bfloat162(__ushort_as_bfloat16(0x0080), __ushort_as_bfloat16(0x0080));
   uint32_t b[3][2];
   float r[4] = {p[0], p[1], p[2], p[3]};
 #pragma unroll
   for (int part = 0; part < 3; ++part)
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
-      const __nv_bfloat162 v = __floats2bfloat162_rn(r[2 * x], r[2 * x + 1]);
-      b[part][x] = transpose8x8(*reinterpret_cast<const uint32_t*>(&v));
+      const uint32_t cut = truncate_bf16x2(r[2 * x], r[2 * x + 1]);
+      const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&cut), w = __hmax2_nan(v, least);
+      b[part][x] = transpose8x8(*reinterpret_cast<const uint32_t*>(&w));
       const float2 back = __bfloat1622float2(v);
       r[2 * x] -= back.x;
       r[2 * x + 1] -= back.y;

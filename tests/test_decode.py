@@ -112,3 +112,38 @@ def test_decode_chunks_and_tables(lengths, hq, hkv, d):
             assert torch.equal(now[:, :l], was[:, :l]) and torch.equal(now[:, l + 1:], was[:, l + 1:])
     e = np.concatenate(errs)
     assert e.max() <= MAX_ABS_TOL and e.mean() <= MEAN_ABS_TOL, (e.max(), e.mean())
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(2, 2, 128), (8, 1, 128), (6, 2, 64)])
+def test_decode_with_infinite_values(hq, hkv, d):
+    """An infinity among the cached values, or in the new token's, makes that element of O infinite (with both signs, or a
+    NaN, not a number) and no other: the first, a middle and the last key of a step, in one chunk and in several."""
+    from paper_2404_09529_b200.runner import DecodeBatch
+    lengths = np.array([1, 16, 17, 50, 64, 65, 200, 700], np.int32)
+    dec = DecodeBatch(lengths, hq, hkv, d, 10000.0, room=2)
+    g = torch.Generator().manual_seed(hq + d)
+    for pool in (dec.k_cache, dec.v_cache):
+        pool.copy_(torch.randn(pool.shape, generator=g).to(torch.bfloat16))
+    qn, kn, vn = (torch.randn(dec.k, h, d, generator=g).to(torch.bfloat16) for h in (hq, hkv, hkv))
+    inf = float("inf")
+    for i, l in enumerate(int(x) for x in lengths):
+        cv = dec.caches(i)[1]
+        cv[0, 0, 1] = inf
+        cv[hkv - 1, l - 1, d - 1] = -inf
+        cv[0, l // 2, d // 2 + 3] = inf
+        cv[0, l - 1, 8] = float("nan")
+        vn[i, 0, 5] = -inf if i % 2 else inf
+        cv[0, l // 3, 6] = inf
+        vn[i, 0, 6] = -inf
+        cv[0, l:] = inf                        # spare rows are not read
+        dec.caches(i)[0][0, l:] = float("nan")
+    before = [tuple(to64(c[:, :int(l)]) for c in dec.caches(i)) for i, l in enumerate(lengths)]
+    got = to64(dec.step(qn.cuda(), kn.cuda(), vn.cuda()))
+    for i in range(dec.k):
+        with np.errstate(invalid="ignore"):
+            ref = orc.decode_step(to64(qn[i]), to64(kn[i]), to64(vn[i]), *before[i], 10000.0)[0]
+        assert np.isinf(ref).any() and np.isnan(ref).any()
+        finite = np.isfinite(ref)
+        assert np.array_equal(np.isnan(got[i]), np.isnan(ref)), i
+        assert np.array_equal(got[i][np.isinf(ref)], ref[np.isinf(ref)]), i
+        assert np.isfinite(got[i][finite]).all() and np.abs(got[i] - ref)[finite].max() <= MAX_ABS_TOL, i
