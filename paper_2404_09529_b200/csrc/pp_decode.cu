@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cfloat>
 #include <cmath>
 
 #include "pp_internal.h"
@@ -122,9 +123,12 @@ __device__ __forceinline__ void load_v(StepV<D>& f, const __nv_bfloat16* base, i
   }
 }
 
+// A maximum over nothing. Finite, so that a score of -inf (a key with an infinite element) weighs nothing beside it.
+constexpr float kNoScore = -FLT_MAX;
+
 template <int D>
 struct Softmax {
-  float m[2] = {-INFINITY, -INFINITY};    // running maximum of query heads 2t and 2t + 1 (all lanes of equal t agree)
+  float m[2] = {kNoScore, kNoScore};      // running maximum of query heads 2t and 2t + 1 (all lanes of equal t agree)
   float l[2] = {0.f, 0.f};                // this thread's keys' share of the running sum
   float acc[D / 16][4];                   // O^T: product j, rows d (see pv), columns = heads 2t, 2t + 1
 };
@@ -155,7 +159,7 @@ __device__ __forceinline__ void softmax_step(Softmax<D>& s, float (&c)[4], float
   if (__any_sync(0xffffffffu, mx[0] > s.m[0] || mx[1] > s.m[1])) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const float m_new = fmaxf(s.m[h], mx[h]);          // every step has a real key: finite
+      const float m_new = fmaxf(s.m[h], mx[h]);
       const float alpha = ex2(s.m[h] - m_new);           // 0 on the first step
       s.m[h] = m_new;
       s.l[h] *= alpha;
@@ -334,7 +338,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Deco
       *reinterpret_cast<uint4*>(a.v_cache + row + 8 * lane) = __ldg(reinterpret_cast<const uint4*>(vn + 8 * lane));
     }
   }
-  // merge the four warps (one without keys has m = -inf, l = 0)
+  // merge the four warps (one without keys has m = kNoScore, l = 0)
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     float l = s.l[h];
@@ -383,12 +387,12 @@ decode_combine_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
   const int c0 = chunk_ptr_at(a, in, i), c1 = chunk_ptr_at(a, in, i + 1);
   if (c1 - c0 < 2 || head >= a.n_q_heads) return;
   pdl_wait();                           // the partial results come from the kernel before this one
-  float mm = -INFINITY, ll = 0.f, oo[E];
+  float mm = kNoScore, ll = 0.f, oo[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) oo[e] = 0.f;
   for (int base = c0; base < c1; base += 32) {           // 32 chunks at a time: one (m, l) per lane
     const int n = min(32, c1 - base);
-    const float2 ml = lane < n ? a.part_ml[(int64_t)(base + lane) * a.n_q_heads + head] : make_float2(-INFINITY, 0.f);
+    const float2 ml = lane < n ? a.part_ml[(int64_t)(base + lane) * a.n_q_heads + head] : make_float2(kNoScore, 0.f);
     float m_new = ml.x;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m_new = fmaxf(m_new, __shfl_xor_sync(0xffffffffu, m_new, o));

@@ -147,3 +147,28 @@ def test_decode_with_infinite_values(hq, hkv, d):
         assert np.array_equal(np.isnan(got[i]), np.isnan(ref)), i
         assert np.array_equal(got[i][np.isinf(ref)], ref[np.isinf(ref)]), i
         assert np.isfinite(got[i][finite]).all() and np.abs(got[i] - ref)[finite].max() <= MAX_ABS_TOL, i
+
+
+@pytest.mark.parametrize("lengths", [[40], [64, 65, 200], [700]])
+def test_decode_with_scores_of_minus_infinity(lengths):
+    """Keys with an infinite element whose score is -inf weigh nothing, whether they are some of a 16-key step, all of it or
+    a whole chunk."""
+    from paper_2404_09529_b200.runner import DecodeBatch
+    lengths = np.asarray(lengths, np.int32)
+    h, d, base = 2, 128, 10000.0
+    dec = DecodeBatch(lengths, h, h, d, base, room=2)
+    g = torch.Generator().manual_seed(5)
+    for pool in (dec.k_cache, dec.v_cache):
+        pool.copy_(torch.randn(pool.shape, generator=g).to(torch.bfloat16))
+    qn, kn, vn = (torch.randn(dec.k, h, d, generator=g).to(torch.bfloat16) for _ in range(3))
+    for i, l in enumerate(int(x) for x in lengths):
+        q_rot = orc.rope_rotate(to64(qn[i])[None], np.array([l]), base)[0]
+        for key in list(range(18)) + [l // 2] + list(range(64, min(l, 128))) + list(range(320, min(l, 640))):
+            for head in range(h):
+                dec.caches(i)[0][head, key, 7] = -float("inf") * float(np.sign(q_rot[head, 7]))
+    before = [tuple(to64(c[:, :int(l)]) for c in dec.caches(i)) for i, l in enumerate(lengths)]
+    got = to64(dec.step(qn.cuda(), kn.cuda(), vn.cuda()))
+    for i in range(dec.k):
+        ref = orc.decode_step(to64(qn[i]), to64(kn[i]), to64(vn[i]), *before[i], base)[0]
+        assert np.isfinite(ref).all() and np.isfinite(got[i]).all(), i
+        assert np.abs(got[i] - ref).max() <= MAX_ABS_TOL, i
