@@ -96,6 +96,7 @@ template <bool kToPacked, class Table>
 __global__ void __launch_bounds__(kTzThreads)
 host_rows_kernel(HostRows h, RowTable m, int32_t q_vec, int32_t kv_vec, const __grid_constant__ Table tab) {
   __shared__ int64_t s_tok[kTzTokens];           // token of each packed row, -1 for padding
+  if (!kToPacked && Table::kUploaded) pdl_wait();
   const int64_t row0 = (int64_t)blockIdx.x * m.rows_per_block;
   if (threadIdx.x < m.rows_per_block) {
     const int64_t row = row0 + threadIdx.x;
