@@ -225,8 +225,10 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Deco
   __shared__ float s_o[kDecodeWarps][kMaxGroup][D];
   const int chunk = blockIdx.x, kvh = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, t = lane & 3;
+  // An uploaded table is not read before the work in front is done; nor by the combine kernel, which looks at it before its own
+  // wait and therefore must not start earlier.
+  if constexpr (N == 0) pdl_wait();
   pdl_launch_dependents();              // the combine kernel may set up while this one runs
-  if constexpr (N == 0) pdl_wait();     // an uploaded table is not read before the work in front is done
   int lo = 0, hi = a.n_prompts - 1;     // last prompt whose first chunk is <= chunk
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
@@ -385,7 +387,6 @@ __global__ void __launch_bounds__(kDecodeThreads)
 decode_combine_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ DecodeInline<N> in) {
   constexpr int E = D / 32;             // consecutive elements per lane
   const int i = blockIdx.x, head = blockIdx.y * kDecodeWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-  if constexpr (N == 0) pdl_wait();
   const int c0 = chunk_ptr_at(a, in, i), c1 = chunk_ptr_at(a, in, i + 1);
   if (c1 - c0 < 2 || head >= a.n_q_heads) return;
   pdl_wait();                           // the partial results come from the kernel before this one
