@@ -1444,10 +1444,11 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           lo = seg_start_at(tab, args.off_seg_start, seg_first_t + 1, seg_end, i_row, i_row - lane + 31, lo, lane);
         if (i_row < bin_used) { key_lo = lo; key_hi = i_row; }
       }
-      // |q|^2 up to which every score of a row stays below the bound (0 if nothing is known about the keys)
+      // |q|^2 up to which every score of a row stays below the bound (0 if nothing is known about the keys). The norms grew
+      // while this kernel was starting, beside table words that the rotation kernel reads through L1: not from there.
       float q2_limit = 0.f;
       if (args.k_norm2 && lazy_log2 == kLazyLog2) {
-        const float k2 = __uint_as_float(__ldg(args.k_norm2 + kv_head));
+        const float k2 = __uint_as_float(__ldcg(args.k_norm2 + kv_head));
         // (a NaN among the keys bounds nothing; the limit is finite, for a |q|^2 that overflows is beyond any)
         if (k2 < INFINITY) q2_limit = fminf(args.bound2 / fmaxf(k2, 1e-30f), FLT_MAX);
       }
@@ -1458,7 +1459,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         ok = rotate_q(used ? key_hi - key_lo : -1, 0.5f * q2_limit, it_n & 1u);
         if (!ok) break;
       } else if (args.q_norm2) {
-        bounded = q2_limit > 0.f && __uint_as_float(__ldg(args.q_norm2 + head_t)) <= q2_limit;
+        bounded = q2_limit > 0.f && __uint_as_float(__ldcg(args.q_norm2 + head_t)) <= q2_limit;
       }
       float m_run = -INFINITY;      // running maximum of the whole row, in scaled log2 units
       uint64_t sum_a = 0ull, sum_b = 0ull;   // this thread's share of the running sum of exp2(s * c - m_run), in four parts

@@ -85,9 +85,11 @@ __device__ __forceinline__ uint32_t transpose8x8(uint32_t x) {
   asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
   return y;
 }
-__device__ __forceinline__ uint4 load16(const __nv_bfloat16* p) {      // read once: do not keep in L1
+// Read once, so not kept in L1. And, like all tensors here, not through the read-only path: this kernel may have started before
+// the one in front of it has written them (the rows it appends to the caches, the new token).
+__device__ __forceinline__ uint4 load16(const __nv_bfloat16* p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
 __device__ __forceinline__ float ex2(float x) {
@@ -266,8 +268,8 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Deco
     if (u < kRotUnits && (h < a.group || (h == kMaxGroup && last_chunk))) {
       const __nv_bfloat16* src = h == kMaxGroup ? a.k_new + ((int64_t)i * a.n_kv_heads + kvh) * D
                                                 : a.q_new + ((int64_t)i * a.n_q_heads + kvh * a.group + h) * D;
-      lo2[x] = __ldg(reinterpret_cast<const uint2*>(src + j));
-      hi2[x] = __ldg(reinterpret_cast<const uint2*>(src + j + kHalf));
+      lo2[x] = *reinterpret_cast<const uint2*>(src + j);
+      hi2[x] = *reinterpret_cast<const uint2*>(src + j + kHalf);
     }
   }
   StepK<D> fk;
@@ -330,7 +332,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Deco
     for (int x = 0; x < 4; ++x)
 #pragma unroll
       for (int y = 0; y < D / 64; ++y)
-        fv.r[x][y] = x == 0 && t == 0 ? __ldg(reinterpret_cast<const uint4*>(vn + 8 * g + 64 * y)) : make_uint4(0u, 0u, 0u, 0u);
+        fv.r[x][y] = x == 0 && t == 0 ? *reinterpret_cast<const uint4*>(vn + 8 * g + 64 * y) : make_uint4(0u, 0u, 0u, 0u);
     scores<D>(c, fk, q);
     softmax_step<D>(s, c, a.scale_log2, 1, g);
     pv<D>(s, fv, c);
@@ -338,7 +340,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Deco
     const int64_t row = base + (int64_t)pr.length * D;
     if (lane < D / 8) {
       *reinterpret_cast<uint4*>(a.k_cache + row + 8 * lane) = *reinterpret_cast<const uint4*>(&s_q[kMaxGroup][8 * lane]);
-      *reinterpret_cast<uint4*>(a.v_cache + row + 8 * lane) = __ldg(reinterpret_cast<const uint4*>(vn + 8 * lane));
+      *reinterpret_cast<uint4*>(a.v_cache + row + 8 * lane) = *reinterpret_cast<const uint4*>(vn + 8 * lane);
     }
   }
   // merge the four warps (one without keys has m = kNoScore, l = 0)
