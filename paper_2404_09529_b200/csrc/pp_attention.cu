@@ -1262,7 +1262,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
                 for (int uu = 0; uu < 2; ++uu)
 #pragma unroll
                   for (int i = 0; i < 4; ++i)
-                    cs[uu][i] = __ldg(tab + (size_t)((u0 + uu) * 4 + i) * (size_t)args.capacity);
+                    cs[uu][i] = tab[(size_t)((u0 + uu) * 4 + i) * (size_t)args.capacity];
 #pragma unroll
                 for (int uu = 0; uu < 2; ++uu) {
                   const int u = u0 + uu;                 // pairs (8u .. 8u+7, + D/2)
@@ -1386,7 +1386,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         for (int uu = 0; uu < kUnits / 2; ++uu)
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            cs[uu][i] = __ldg(tab + (size_t)((h * (kUnits / 2) + uu) * 4 + i) * (size_t)args.capacity);
+            cs[uu][i] = tab[(size_t)((h * (kUnits / 2) + uu) * 4 + i) * (size_t)args.capacity];
 #pragma unroll
         for (int uu = 0; uu < kUnits / 2; ++uu) {
           const int u = h * (kUnits / 2) + uu;         // pairs (8u .. 8u+7, + D/2)

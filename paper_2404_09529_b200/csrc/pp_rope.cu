@@ -93,7 +93,7 @@ __device__ __forceinline__ void publish_ranges(const uint32_t* s_max, int n, uin
 // counter: null, or the work counter to reset for the attention kernel.
 template <int D, bool kRange, class Table>
 __global__ void __launch_bounds__(kRopeThreads)
-rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, uint32_t* norms,
+rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, const __nv_bfloat16* v, uint32_t* norms,
             uint32_t* v_max, int32_t* counter,
             const __grid_constant__ Table tab, int32_t off_bin_seg_ptr, int32_t off_bin_used,
             int32_t off_seg_start, int32_t n_bins, int32_t capacity, int32_t n_q_heads,
@@ -189,7 +189,7 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, const 
 #pragma unroll
         for (int i = 0; i < kAtOnce; ++i) {
           const int u = u0 + i * kRopeThreads, r = u / vecs;
-          val[i] = u < kRopeRows * vecs && s_pos[r] >= 0 ? __ldg(reinterpret_cast<const uint4*>(v) + row0 * vecs + u) : make_uint4(0u, 0u, 0u, 0u);
+          val[i] = u < kRopeRows * vecs && s_pos[r] >= 0 ? reinterpret_cast<const uint4*>(v)[row0 * vecs + u] : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
         for (int i = 0; i < kAtOnce; ++i) m = max_abs(m, val[i]);
@@ -221,6 +221,9 @@ rope_table_kernel(float2* __restrict__ table, int32_t capacity, int32_t half,
   table[((size_t)(j >> 1) * capacity + pos) * 2 + (j & 1)] = make_float2(cs, sn);
 }
 
+// (The kernels here read what a kernel in front may still be writing when they start, q, k, v and the cos/sin table, through
+// ordinary loads, not through the read-only path.)
+//
 // Fused K rotation + UNPACK (Algorithm 1 (RESTART-PE to UNPACK) in one pass over K and V): every real packed
 // row of K is rotated (cos/sin from the table), written back to the packed tensor (the attention
 // kernel reads it there) and into its prompt's K cache; the V row is copied into the V cache.
@@ -240,10 +243,10 @@ constexpr int kRuK = 2;      // (lower, upper) K pairs in flight per thread
 // kRange: the norms and the largest |v| are wanted (shared-stream mode).
 template <int D, int kRuRows, bool kRange, class Table>
 __global__ void __launch_bounds__(kRopeThreads)
-rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, uint32_t* norms,
+rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* v, uint32_t* norms,
                    uint32_t* v_max, int32_t* counter, __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
                    const __grid_constant__ Table tab, int32_t off_bin_seg_ptr, int32_t off_bin_used,
-                   int32_t off_seg_start, SegExt ext, const float2* __restrict__ rope_table,
+                   int32_t off_seg_start, SegExt ext, const float2* rope_table,
                    int32_t n_bins, int32_t capacity, int32_t n_kv_heads) {
   constexpr int kHalf = D / 2;
   constexpr int kPairUnits = kHalf / 8;             // (lower, upper) 16-byte pairs per head
@@ -292,7 +295,7 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
   for (int u = tid; u < kRuRows * (D / 4); u += kRopeThreads) {
     const int r = u / (D / 4), g = u - r * (D / 4);
     const int32_t pos = s_pos[r];
-    if (pos > 0) s_tab[r][g] = __ldg(reinterpret_cast<const float4*>(rope_table) + (size_t)g * (size_t)capacity + pos);
+    if (pos > 0) s_tab[r][g] = reinterpret_cast<const float4*>(rope_table)[(size_t)g * (size_t)capacity + pos];
   }
 
   // V rows first: plain 16-byte copies, kRuV in flight per thread (rows that are attended to but not cached are
@@ -310,7 +313,7 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
         const int r = u / units_v, w = u - r * units_v;
         if (s_dst[r] >= 0 || (kRange && s_pos[r] >= 0)) {
           const int head = w / kVecs, c = w - head * kVecs;
-          val[i] = __ldg(reinterpret_cast<const uint4*>(v + ((row0 + r) * n_kv_heads + head) * D + c * 8));
+          val[i] = *reinterpret_cast<const uint4*>(v + ((row0 + r) * n_kv_heads + head) * D + c * 8);
           dsts[i] = !kRange || s_dst[r] >= 0 ? s_dst[r] + head * s_head_stride[r] + c * 8 : -2;
         }
       }
@@ -378,7 +381,7 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restric
 // grid = (bins, slices of a bin).
 constexpr int kRangeVecs = 8;      // 16-byte loads in flight per thread
 __global__ void __launch_bounds__(kRopeThreads)
-value_range_kernel(const uint4* __restrict__ v, const TableInMemory tab, int32_t off_bin_used, int32_t capacity, int32_t vec_per_row,
+value_range_kernel(const uint4* v, const TableInMemory tab, int32_t off_bin_used, int32_t capacity, int32_t vec_per_row,
                    uint32_t* v_max) {
   __shared__ uint32_t s_max;
   if (threadIdx.x == 0) s_max = 0u;
@@ -392,7 +395,7 @@ value_range_kernel(const uint4* __restrict__ v, const TableInMemory tab, int32_t
   for (int64_t at = (int64_t)blockIdx.y * kRopeThreads + threadIdx.x; at < n; at += kRangeVecs * stride) {
     uint4 val[kRangeVecs];
 #pragma unroll
-    for (int i = 0; i < kRangeVecs; ++i) val[i] = at + i * stride < n ? __ldg(src + at + i * stride) : make_uint4(0u, 0u, 0u, 0u);
+    for (int i = 0; i < kRangeVecs; ++i) val[i] = at + i * stride < n ? src[at + i * stride] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
     for (int i = 0; i < kRangeVecs; ++i) m = max_abs(m, val[i]);
   }
