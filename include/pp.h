@@ -299,8 +299,8 @@ int pp_decode_step(const pp_attn_params* params, const int32_t* lengths, int32_t
  *                            lengths), laid out [Hkv, lengths[i], D]
  *   arena, arena_bytes       device scratch >= pp_prefill_host_arena_bytes(params, lengths, k),
  *                            256-byte aligned
- * Pinned host buffers give full copy bandwidth (and a small batch in them is read and written by the
- * kernels where it is); pageable ones work too. A batch of 32 MB or more is cut into up to eight groups
+ * Pinned host buffers give full copy bandwidth (and a batch of up to 20 MB of q, k and v in them, or one
+ * prompt of up to 40 MB, is read and written by the kernels where it is); pageable ones work too. A batch of 32 MB or more is cut into up to eight groups
  * of consecutive prompts with about equal token counts. Each
  * group is packed on its own (pp_pack with the batch-wide capacity = longest prompt; n_bins is the
  * sum over the groups) and runs on a stream the library creates once per device and thread, so

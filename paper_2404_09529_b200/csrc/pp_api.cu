@@ -366,6 +366,7 @@ struct HostGroup {
 struct HostPlan {
   int32_t capacity = 0, n_bins = 0;
   int64_t total_tokens = 0;
+  size_t batch_bytes = 0;          // of q, k and v
   std::vector<HostGroup> groups;
   // arena offsets (bytes)
   size_t q = 0, k = 0, v = 0, o = 0, q_tok = 0, k_tok = 0, v_tok = 0, o_tok = 0, kc = 0, vc = 0;
@@ -384,8 +385,8 @@ int plan_host(const pp_attn_params& p, const int32_t* lengths, int32_t k, HostPl
   h.capacity = m;
   const size_t q_row = (size_t)p.n_q_heads * p.head_dim * 2, kv_row = (size_t)p.n_kv_heads * p.head_dim * 2;
   // pipelining pays once the transfers are tens of megabytes; small batches stay in one group
-  const size_t batch_bytes = (size_t)h.total_tokens * (q_row + 2 * kv_row);
-  int n_groups = batch_bytes >= (size_t(32) << 20) ? kHostGroupsDefault : 1;
+  h.batch_bytes = (size_t)h.total_tokens * (q_row + 2 * kv_row);
+  int n_groups = h.batch_bytes >= (size_t(32) << 20) ? kHostGroupsDefault : 1;
   if (g_host_groups > 0) n_groups = g_host_groups;
   n_groups = std::min<int>(n_groups, k);
   h.groups.resize(n_groups);
@@ -491,14 +492,21 @@ int host_pipe(HostPipe** out) {
   return PP_OK;
 }
 
-// pp_prefill_host for one group whose six tensors are mapped: the kernels read and write them where they are, on the
+// pp_prefill_host for one small group whose six tensors are mapped: the kernels read and write them where they are, on the
 // caller's stream: six launches at most instead of nineteen copies, kernels and events, which took a small batch
-// longer than its bytes on the bus (1.1 MB both ways 132 -> 70 us, 3.9 MB 177 -> 125, 11 MB 312 -> 269, 39 MB 941
-// -> 881). Sets *done if it took the call.
+// longer than its bytes on the bus. The kernels have 51 and 52 GB/s of the bus where the copy engines have 55 and 53, so
+// from a size on the copies are faster again. Copies -> in place (us) by the bytes of q, k and v, on 32 / 32, 32 / 8 and
+// 32 / 4 heads of 128, 4 / 4 and 8 / 8 of 64: 0.5 MB 110-137 -> 60-73, 2 MB 166-223 -> 114-140, 8 MB 393-695 -> 355-439,
+// 16 MB 713-1061 -> 682-885, 20 MB 854-1270 -> 842-1080, never slower so far; 24 MB, 8 prompts on 8 / 8 heads 1053 -> 1070;
+// 31 MB, 64 prompts 1298 -> 1346 there, 1295 -> 1295 on 32 / 32. One prompt, whose kernels take longest: 31 MB 1327 -> 1299 on
+// 32 / 32 heads, 1626 -> 1565 on 8 / 8; 40 MB 1682 -> 1665, 1788 -> 1793 on 32 / 8; 48 MB 2011 -> 2057, 192 MB 8147 -> 8398.
+// Sets *done if it took the call.
+constexpr size_t kMappedBytes = size_t(20) << 20, kMappedBytesOnePrompt = size_t(40) << 20;
 int prefill_host_mapped(const pp_attn_params& p, const HostPlan& h, const int32_t* lengths, int32_t k, const void* q_host,
                         const void* k_host, const void* v_host, void* o_host, void* k_cache_host, void* v_cache_host, char* base,
                         HostPipe* pipe, cudaStream_t s, bool* done) {
   *done = false;
+  if (h.batch_bytes > (k == 1 ? kMappedBytesOnePrompt : kMappedBytes)) return PP_OK;
   const size_t q_bytes = (size_t)h.total_tokens * p.n_q_heads * p.head_dim * 2;
   const size_t kv_bytes = (size_t)h.total_tokens * p.n_kv_heads * p.head_dim * 2;
   HostRows r;

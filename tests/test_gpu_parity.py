@@ -332,3 +332,35 @@ def test_host_entry_point_one_group_mapped_or_copied(lengths, hq, hkv, d, pinned
         for got, want in zip(bufs[3:], (ref.o_tokens(), ref.k_cache, ref.v_cache)):
             assert torch.equal(got[:-16], want.cpu().flatten()) and bool((got[-16:] == -7.0).all())
             got[:-16].zero_()
+
+
+@pytest.mark.parametrize("tokens,prompts,in_place", [
+    (1300, 3, True), (1700, 3, True), (1800, 3, False),      # 20 MB of q, k and v: 1706 tokens
+    (3400, 1, True), (3500, 1, False),                       # one prompt, 40 MB: 3413 tokens
+])
+def test_host_entry_point_large_batches_are_copied(tokens, prompts, in_place):
+    """One group in pinned memory: in place up to the size where copies are faster. Which way a batch went shows in the arena:
+    only the copies leave token-major q there, behind the packed q, k, v and o."""
+    import paper_2404_09529_b200 as pp
+    hq, hkv, d = 16, 16, 128
+    lengths = np.full(prompts, tokens // prompts, np.int32)
+    lengths[0] += tokens - int(lengths.sum())
+    q, k, v = _random_case(lengths, hq, hkv, d, seed=tokens)
+    ref = run_cuda(lengths, q, k, v, hq, hkv, d, 10000.0)
+    params = pp.AttnParams(hq, hkv, d, 10000.0, 0.0, 0, 0, 0)
+    before = pp.pp_prefill_host_groups(1)
+    try:
+        nbytes = pp.pp_prefill_host_arena_bytes(params, lengths)
+        arena = torch.full((nbytes,), 255, dtype=torch.uint8, device="cuda")
+        outs = [torch.zeros(x.numel(), dtype=torch.bfloat16).pin_memory() for x in (q, k, v)]
+        pp.pp_prefill_host(params, lengths, *(x.contiguous().pin_memory() for x in (q, k, v)), *outs, arena, nbytes,
+                           torch.cuda.current_stream().cuda_stream)
+    finally:
+        pp.pp_prefill_host_groups(before)
+    for got, want in zip(outs, (ref.o_tokens(), ref.k_cache, ref.v_cache)):
+        assert torch.equal(got, want.cpu().flatten())
+    up256 = lambda x: (x + 255) // 256 * 256
+    rows = params.n_bins * params.capacity
+    q_tok = sum(up256(rows * h * d * 2) for h in (hq, hkv, hkv, hq))
+    held = arena[q_tok:q_tok + q.numel() * 2].cpu()
+    assert bool((held == 255).all()) if in_place else torch.equal(held, q.contiguous().flatten().view(torch.uint8))
