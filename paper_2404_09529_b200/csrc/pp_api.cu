@@ -518,7 +518,7 @@ int prefill_host_mapped(const pp_attn_params& p, const HostPlan& h, const int32_
   const HostGroup& G = h.groups[0];
   const FusedLayout f = fused_layout(p, k);
   void* stage = nullptr;
-  int st = host_staging(pipe, 0, 256 + f.total_bytes, &stage);
+  int st = host_staging(pipe, 0, 256 + sizeof(int32_t) * f.upload_ints, &stage);
   if (st != PP_OK) return st;
   r.status = reinterpret_cast<int32_t*>(base + h.status);
   r.host_status = static_cast<int32_t*>(stage);
@@ -634,9 +634,9 @@ extern "C" int pp_prefill_host(pp_attn_params* params, const int32_t* lengths, i
       gp.n_bins = G.n_bins;
       const size_t map_ints64 = 2 * (size_t)kg + 1 + (size_t)G.n_bins;
       const size_t map_bytes = pp::up256(sizeof(int64_t) * map_ints64);
-      const size_t tab_bytes = pp::up256(pp::fused_layout(gp, kg).total_bytes);
+      const pp::FusedLayout gl = pp::fused_layout(gp, kg);
       void* stage = nullptr;
-      if ((st = pp::host_staging(pipe, g, map_bytes + tab_bytes, &stage)) != PP_OK) return bail(st);
+      if ((st = pp::host_staging(pipe, g, map_bytes + sizeof(int32_t) * gl.upload_ints, &stage)) != PP_OK) return bail(st);
       int64_t* map = static_cast<int64_t*>(stage);
       int64_t* used = map + 2 * (size_t)kg + 1;
       g_cache_off.resize(kg);
@@ -663,7 +663,7 @@ extern "C" int pp_prefill_host(pp_attn_params* params, const int32_t* lengths, i
       pp::TableLayout g_layout;
       st = pp::prefill_fused_impl(&gp, G.bin_seg_ptr.data(), G.seg_start.data(), G.seg_len.data(), G.seg_prompt.data(),
                                   kg, lengths + G.i0, gq, gk, gv, go, base + h.kc, base + h.vc, g_cache_off.data(),
-                                  lengths + G.i0, gws, gstage, tab_bytes, d_status, sg, pp::TableStep::kUploadOnly, &g_layout);
+                                  lengths + G.i0, gws, gstage, gl.total_bytes, d_status, sg, pp::TableStep::kUploadOnly, &g_layout);
       if (st != PP_OK) return bail(st);
       PP_TRY(cudaMemcpyAsync(base + h.q_tok + tok0 * q_row, (const char*)q_host + tok0 * q_row, ntok * q_row,
                              cudaMemcpyHostToDevice, sg), "H2D q");
@@ -679,7 +679,7 @@ extern "C" int pp_prefill_host(pp_attn_params* params, const int32_t* lengths, i
       if ((st = pp::launch_tensorize(true, gv, base + h.v_tok + tok0 * kv_row, d_map, kg, (int64_t)ntok, (int32_t)kv_row, sg)) != PP_OK) return bail(st);
       st = pp::prefill_fused_impl(&gp, G.bin_seg_ptr.data(), G.seg_start.data(), G.seg_len.data(), G.seg_prompt.data(),
                                   kg, lengths + G.i0, gq, gk, gv, go, base + h.kc, base + h.vc, g_cache_off.data(),
-                                  lengths + G.i0, gws, gstage, tab_bytes, d_status, sg, pp::TableStep::kLaunchOnly, &g_layout);
+                                  lengths + G.i0, gws, gstage, gl.total_bytes, d_status, sg, pp::TableStep::kLaunchOnly, &g_layout);
       if (st != PP_OK) return bail(st);
       // O and the caches are final once the attention has run
       if ((st = pp::launch_tensorize(false, go, base + h.o_tok + tok0 * q_row, d_map, kg, (int64_t)ntok, (int32_t)q_row, sg)) != PP_OK) return bail(st);
