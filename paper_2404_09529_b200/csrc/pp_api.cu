@@ -1,5 +1,7 @@
 // C-ABI entry points that touch the device: argument validation, table upload, kernel launches.
 // Algorithm 1 (TENSORIZE to UNPACK) of the prepacking paper; see include/pp.h for the contracts.
+#include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -60,20 +62,31 @@ int check_device() {
 }
 
 // Device address of `bytes` of pinned host memory at p that kernels can work on in 16-byte pieces; null if it is
-// anything else (pageable memory, an odd address).
+// anything else (pageable memory, an odd address). All of it has to lie in one allocation or registration: of a buffer that
+// only begins and ends in pinned memory the part between is none of the device's.
 void* mapped(const void* p, size_t bytes) {
-  if (!aligned16(p)) return nullptr;
-  void* dev[2];
-  for (int end = 0; end < 2; ++end) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, static_cast<const char*>(p) + (end ? bytes - 1 : 0)) != cudaSuccess) {
-      (void)cudaGetLastError();
-      return nullptr;
-    }
-    if (a.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
-    dev[end] = a.devicePointer;
+  static const PFN_cuPointerGetAttributes query = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &fn, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess)
+      fn = nullptr;
+    return reinterpret_cast<PFN_cuPointerGetAttributes>(fn);
+  }();
+  if (!query || !aligned16(p)) return nullptr;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return nullptr;
   }
-  return static_cast<char*>(dev[1]) - static_cast<char*>(dev[0]) == (std::ptrdiff_t)(bytes - 1) ? dev[0] : nullptr;
+  if (a.type != cudaMemoryTypeHost || !a.devicePointer) return nullptr;
+  // the range lies at device addresses, which the host addresses need not equal
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  CUpointer_attribute what[2] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* out[2] = {&start, &size};
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(a.devicePointer);
+  if (query(2, what, out, at) != CUDA_SUCCESS || at < start || at - start > size || size - (at - start) < bytes) return nullptr;
+  return a.devicePointer;
 }
 
 // A table from the host staging buffer to the workspace, in stream order. From pinned memory a small kernel reads it:

@@ -334,6 +334,16 @@ def test_host_entry_point_one_group_mapped_or_copied(lengths, hq, hkv, d, pinned
             got[:-16].zero_()
 
 
+def _went_in_place(arena, params, q):
+    up256 = lambda x: (x + 255) // 256 * 256
+    rows, heads = params.n_bins * params.capacity, (params.n_q_heads, params.n_kv_heads, params.n_kv_heads, params.n_q_heads)
+    q_tok = sum(up256(rows * h * params.head_dim * 2) for h in heads)
+    held = arena[q_tok:q_tok + q.numel() * 2].cpu()
+    in_place = bool((held == 255).all())
+    assert in_place or torch.equal(held, q.contiguous().flatten().view(torch.uint8))
+    return in_place
+
+
 @pytest.mark.parametrize("tokens,prompts,in_place", [
     (1300, 3, True), (1700, 3, True), (1800, 3, False),      # 20 MB of q, k and v: 1706 tokens
     (3400, 1, True), (3500, 1, False),                       # one prompt, 40 MB: 3413 tokens
@@ -359,8 +369,43 @@ def test_host_entry_point_large_batches_are_copied(tokens, prompts, in_place):
         pp.pp_prefill_host_groups(before)
     for got, want in zip(outs, (ref.o_tokens(), ref.k_cache, ref.v_cache)):
         assert torch.equal(got, want.cpu().flatten())
-    up256 = lambda x: (x + 255) // 256 * 256
-    rows = params.n_bins * params.capacity
-    q_tok = sum(up256(rows * h * d * 2) for h in (hq, hkv, hkv, hq))
-    held = arena[q_tok:q_tok + q.numel() * 2].cpu()
-    assert bool((held == 255).all()) if in_place else torch.equal(held, q.contiguous().flatten().view(torch.uint8))
+    assert _went_in_place(arena, params, q) == in_place
+
+
+@pytest.mark.parametrize("memory,in_place", [("one allocation", True), ("one registration", True), ("odd address", False),
+                                             ("pageable", False), ("outputs only", False)])
+def test_host_entry_point_in_place_in_one_pinned_range_only(memory, in_place):
+    """A batch is worked on in place where each tensor lies whole in one pinned range, also in the middle of it."""
+    import paper_2404_09529_b200 as pp
+    hq, hkv, d = 4, 2, 64
+    lengths = np.array([70, 3, 64, 1, 33], np.int32)
+    q, k, v = _random_case(lengths, hq, hkv, d, seed=9)
+    ref = run_cuda(lengths, q, k, v, hq, hkv, d, 10000.0)
+    params = pp.AttnParams(hq, hkv, d, 10000.0, 0.0, 0, 0, 0)
+    nbytes = pp.pp_prefill_host_arena_bytes(params, lengths)
+    arena = torch.full((nbytes,), 255, dtype=torch.uint8, device="cuda")
+    sizes = [x.numel() for x in (q, k, v, q, k, v)]
+    whole = torch.zeros(sum(sizes) + 6 * 64 + 4096, dtype=torch.bfloat16)
+    if memory in ("one allocation", "odd address"):
+        whole = whole.pin_memory()
+    rt, page = torch.cuda.cudart(), 4096
+    first = (whole.data_ptr() + page - 1) // page * page
+    if memory == "one registration":
+        assert int(rt.cudaHostRegister(first, (whole.numel() * 2 - page) // page * page, 0)) == 0
+    at = (first - whole.data_ptr()) // 2 + 64 + (4 if memory == "odd address" else 0)
+    bufs = []
+    for n, src in zip(sizes, (q, k, v, None, None, None)):
+        bufs.append(whole[at:at + n])
+        if src is not None:
+            bufs[-1].copy_(src.contiguous().flatten())
+        at += (n + 63) // 64 * 64
+    if memory == "outputs only":
+        bufs[3:] = [x.pin_memory() for x in bufs[3:]]
+    try:
+        pp.pp_prefill_host(params, lengths, *bufs, arena, nbytes, torch.cuda.current_stream().cuda_stream)
+    finally:
+        if memory == "one registration":
+            assert int(rt.cudaHostUnregister(first)) == 0
+    for got, want in zip(bufs[3:], (ref.o_tokens(), ref.k_cache, ref.v_cache)):
+        assert torch.equal(got, want.cpu().flatten())
+    assert _went_in_place(arena, params, q) == in_place
