@@ -152,13 +152,13 @@ struct WaitCtx {
   unsigned long long limit_ns;
 };
 __device__ __forceinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, const WaitCtx& w, int code) {
-  // The clock is read only every 32 failed polls (each poll may park the thread in hardware for a
+  // The clock is read only every 8 failed polls (each poll may park the thread in hardware for a
   // while), so a short wait costs nothing but the polls; the limit counts from the first reading.
   unsigned long long t0 = 0;
   uint32_t spins = 0;
   while (true) {
     if (mbar_try_wait(bar, parity)) return true;
-    if ((++spins & 31u) == 0) {
+    if ((++spins & 7u) == 0) {
       if (*w.abort_flag) return false;
       const unsigned long long now = global_ns();
       if (t0 == 0) t0 = now;
@@ -180,7 +180,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, co
   unsigned long long t0 = 0;
   uint32_t spins = 0;
   while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
-    if ((++spins & 31u) == 0) {
+    if ((++spins & 7u) == 0) {
       bool give_up = *w.abort_flag != 0;
       const unsigned long long now = global_ns();
       if (t0 == 0) t0 = now;

@@ -409,3 +409,35 @@ def test_host_entry_point_in_place_in_one_pinned_range_only(memory, in_place):
     for got, want in zip(bufs[3:], (ref.o_tokens(), ref.k_cache, ref.v_cache)):
         assert torch.equal(got, want.cpu().flatten())
     assert _went_in_place(arena, params, q) == in_place
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(2, 2, 128), (2, 2, 64), (4, 1, 128)])
+def test_independent_mode_gives_up_cleanly_when_its_waits_expire(hq, hkv, d, monkeypatch):
+    """The same on the fused route in the independent mode; the first shape is one where the attention kernel fills the V caches,
+    so that its cache writers are among the warps that have to find their way out. An item of the long prompt keeps the
+    threads that wait for its end waiting for a hundred times the limit."""
+    import paper_2404_09529_b200 as pp
+    from paper_2404_09529_b200.runner import PrefillBatch
+    lengths = np.array([8000] + [50] * 1500, np.int32)
+    q, k, v = _random_case(lengths, hq, hkv, d, seed=d)
+    b = PrefillBatch(lengths, hq, hkv, d, 10000.0)
+    assert pp.pp_prefill_schedule_info(b.params, b.pack)["mode"] == 1
+    b.load(q, k, v)
+    b.run_fused()
+    torch.cuda.synchronize()
+    want = [x.clone() for x in (b.o_tokens(), b.k_cache, b.v_cache)]
+    b.load(q, k, v)
+    monkeypatch.setenv("PP_WAIT_LIMIT_US", "1")
+    b.run_fused()
+    torch.cuda.synchronize()
+    assert 1 <= b.device_status() <= 20
+    monkeypatch.delenv("PP_WAIT_LIMIT_US")
+    b.ws.status.zero_()
+    b.load(q, k, v)
+    for x in (b.o, b.k_cache, b.v_cache):
+        x.zero_()
+    b.run_fused()
+    torch.cuda.synchronize()
+    assert b.device_status() == 0
+    for x, y in zip(want, (b.o_tokens(), b.k_cache, b.v_cache)):
+        assert torch.equal(x, y)
