@@ -152,8 +152,9 @@ size_t pp_prefill_workspace_bytes(const pp_attn_params* params, int32_t k);
  *   workspace       device, >= pp_prefill_workspace_bytes, 16-byte aligned; holds the segment
  *                   table and the tile work list for the duration of the enqueued work
  *   host_workspace  host, same size (pinned memory keeps the call asynchronous); the library
- *                   builds the tables here and copies them with one async H2D on `stream`; it
- *                   must stay untouched until that copy has run
+ *                   builds the tables here, and from here they reach the device on `stream` (by a
+ *                   kernel that reads them in place, a copy, or as kernel parameters); it must
+ *                   stay untouched until the call's work on `stream` is done
  *   device_status   device int32 or NULL; set non-zero by the kernel if a bounded wait inside
  *                   it gave up (then outputs are invalid). The caller zeroes and reads it. Every
  *                   wait in the kernel is limited to 2 s; the environment variables
@@ -187,8 +188,8 @@ int pp_prefill_attention(const pp_attn_params* params,
  *   workspace    device, >= pp_prefill_fused_workspace_bytes, 256-byte aligned (tables and a
  *                cos/sin table of capacity * D/2 pairs); host_workspace: host staging of at least
  *                pp_prefill_fused_host_bytes (the tables, which are what is uploaded; the cos/sin
- *                table is built on the device), pinned memory keeps the call asynchronous
- *                (and is read in place by a kernel of the call's)
+ *                table is built on the device), pinned memory keeps the call asynchronous;
+ *                to be left alone as in pp_prefill_attention
  * params->flags: PP_FLAG_ROPE_ONLY runs only the rotation / unpack kernels, PP_FLAG_SKIP_ROPE only the
  * attention kernel (k_ holds rotated keys already). Outputs are bit-identical to the two-call path.
  * Errors as the two calls it replaces.

@@ -408,19 +408,17 @@ __host__ __device__ constexpr uint32_t instr_desc(uint32_t n, bool b_mn_major) {
 
 struct AttnArgs {
   int32_t* counter;              // global work counter (a header word of the table)
-  int32_t off_bin_seg_ptr, off_bin_used, off_seg_start, off_items;
+  int32_t off_seg_start, off_items;
   int32_t n_items;               // geometry entries in the work list
   int32_t subs;                  // work indices per (KV head, geometry entry)
   int32_t pair_heads;            // 1: slots are two query heads; 0: two row tiles of one head
   int32_t group;                 // query heads per KV head
   int32_t fold;                  // independent mode: query heads folded into a query tile (tile row m is
   int32_t fold_shift;            //   bin row q_row0 + (m >> fold_shift) of head head[0] + (m & (fold - 1)))
-  int32_t n_q_heads;
   int32_t capacity;              // rows per bin
   int32_t total_work;            // n_kv_heads * n_items * subs
   float scale_log2;              // softmax scale * log2(e)
   float bound2;                  // (kBoundLog2 / scale_log2)^2: |q|^2 |k|^2 up to which scores are bounded
-  __nv_bfloat16* o;
   const float2* rope_table;      // [D/4][capacity][2] (cos, sin) pairs, or null: Q arrives already rotated
   const uint32_t* k_norm2;       // shared-stream mode: [Hkv] largest |k|^2 (float bits); null: no bound on the scores
   const uint32_t* q_norm2;       // [Hq] largest |q|^2; used when Q arrives already rotated
@@ -510,16 +508,17 @@ __device__ __forceinline__ int seg_start_at(const Table& tab, int starts, int se
   return lo;
 }
 
-// kIndep = false: the two slots of a CTA work on one item and share its K/V stream (long
-//   sequences, GQA head pairs). kIndep = true: every slot draws its own single-tile items and loads
-//   its own K/V tiles (64 rows each), so neither slot ever waits for the other (short prompts, where
-//   pairing two row tiles of different length would leave one slot idle for a tile per item).
 // Independent mode: place in the slot's K / V ring sequence K0 K1 V0 K2 V1 K3 V2 ... of the k-th key tile of the slot.
 // With three stages K(k+3) then follows V(k) and V(k+2) follows K(k+2) in a stage: either load has more than a
 // tile's time (in the sequence K0 V0 K1 V1 ..., K(k+3) followed V(k+1), and its load was waited for every time).
 __device__ __forceinline__ uint32_t kv_index_k(uint32_t k) { return k ? 2u * k - 1u : 0u; }
 __device__ __forceinline__ uint32_t kv_index_v(uint32_t k) { return 2u * k + 2u; }
 
+// kIndep = false: the two slots of a CTA work on one item and share its K/V stream (long
+//   sequences, GQA head pairs). kIndep = true: every slot draws its own single-tile items and loads
+//   its own K/V tiles (64 rows each), so neither slot ever waits for the other (short prompts, where
+//   pairing two row tiles of different length would leave one slot idle for a tile per item).
+// kFill (independent mode): two more warps write the V rows to the caches.
 template <int D, bool kIndep, bool kFill, class Table>
 __global__ void __launch_bounds__(kFill ? kAttnThreadsFill : kAttnThreads, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
@@ -1421,18 +1420,16 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       return true;
     };
     while (true) {
-      // in independent mode slot t has its own ring, and an item describes one tile (its slot-0 fields)
-      const uint32_t ring = it_n % kRing;
-      const int f = t;                                 // which slot fields of the entry to read
+      const uint32_t ring = it_n % kRing;              // both slots read the one ring, each its own fields of an entry
       ok = __all_sync(0xffffffffu, mbar_wait(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull));
       if (!ok) break;
       const volatile int* e = s_ring + ring * kRingInts;
       const int w = e[0];
       const int item_bin = e[1], item_kv_row0 = e[2];
-      const int jb_t = f ? e[6] : 0, je_t = f ? e[8] : e[7];
-      const int q_row0_t = e[4 + f], head_t = e[9 + f], kv_head = e[11];
-      const int bin_used = e[12], seg_end = e[13], key_lo_t = e[14 + f], seg_first_t = e[16 + f];
-      const int single_seg = e[18] >> f;
+      const int jb_t = t ? e[6] : 0, je_t = t ? e[8] : e[7];
+      const int q_row0_t = e[4 + t], head_t = e[9 + t], kv_head = e[11];
+      const int bin_used = e[12], seg_end = e[13], key_lo_t = e[14 + t], seg_first_t = e[16 + t];
+      const int single_seg = e[18] >> t;
       mbar_arrive(bar_item_empty + 8 * ring);
       if (w < 0) break;
       const bool used = jb_t < je_t;
@@ -1724,6 +1721,17 @@ unsigned long long wait_limit_ns() {
   return 2000000000ull;   // 2 s
 }
 
+int sm_count() {
+  static thread_local int cached_dev = -1, cached = 0;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (dev != cached_dev) {
+    if (cudaDeviceGetAttribute(&cached, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    cached_dev = dev;
+  }
+  return cached;
+}
+
 template <int D, bool kIndep, bool kFill, class Table>
 int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& L, const Table& tab, const void* q,
                        const void* k, const void* v, void* o, const void* rope_table, bool have_norms,
@@ -1757,8 +1765,6 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.off_true_len = caches ? caches->off_true_len : 0;
   a.off_cap = caches ? caches->off_cap : 0;
   a.off_cache_off = caches ? caches->off_cache_off : 0;
-  a.off_bin_seg_ptr = L.bin_seg_ptr;
-  a.off_bin_used = L.bin_used;
   a.off_seg_start = L.seg_start;
   a.off_items = L.items;
   a.n_items = L.n_items;
@@ -1767,7 +1773,6 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.fold = fold;
   a.fold_shift = fold_shift;
   a.subs = a.pair_heads ? a.group / 2 : a.group / fold;
-  a.n_q_heads = p.n_q_heads;
   a.capacity = p.capacity;
   const int64_t total = (int64_t)p.n_kv_heads * L.n_items * a.subs;
   if (total > INT32_MAX) return PP_ERR_UNSUPPORTED;
@@ -1780,7 +1785,6 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.q_norm2 = norms && !rope_table ? a.k_norm2 + p.n_kv_heads : nullptr;
   a.v_max = tracks_ranges(p, L) ? reinterpret_cast<const uint32_t*>(d_table + kHeaderValueMax) : nullptr;
   a.v_room = ldexpf(1.f, kValueRoomLog2) / (float)p.capacity;
-  a.o = static_cast<__nv_bfloat16*>(o);
   a.rope_table = static_cast<const float2*>(rope_table);
   a.status = device_status;
   a.wait_limit_ns = wait_limit_ns();
@@ -1792,17 +1796,6 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
 }
 
 }  // namespace
-
-int sm_count() {
-  static thread_local int cached_dev = -1, cached = 0;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (dev != cached_dev) {
-    if (cudaDeviceGetAttribute(&cached, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    cached_dev = dev;
-  }
-  return cached;
-}
 
 int launch_bounded_wait_selftest(int32_t* device_status, uint64_t limit_ns, void* stream) {
   bounded_wait_selftest_kernel<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(device_status, limit_ns);

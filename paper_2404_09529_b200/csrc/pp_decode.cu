@@ -438,11 +438,11 @@ decode_combine_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
   else *reinterpret_cast<uint32_t*>(dst) = r[0];
 }
 
-// Keys per chunk. Enough (chunk, KV head) CTAs for about four rounds of the 3 x 148 that run at once, so that
+// Keys per chunk. Enough (chunk, KV head) CTAs for about four rounds of the three per SM that run at once, so that
 // the last round is a small part of the whole; at least one 16-key step for each of the four warps, at most
 // 512 keys (a CTA's set-up is then a few per cent of its loads), and more only where a very long prompt would
 // otherwise be cut into more pieces than one warp merges quickly.
-constexpr int64_t kChunkCtasWanted = 148 * 3 * 4;
+constexpr int64_t kChunkCtasWanted = kSms * 3 * 4;
 constexpr int kMostChunksPerPrompt = 64;
 
 struct DecodeLayout {

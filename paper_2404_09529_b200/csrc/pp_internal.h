@@ -17,6 +17,8 @@ constexpr int kHeaderSegments = 4;   // header word with the number of segments
 constexpr int kHeaderCounter = 10;   // header word the persistent CTAs draw work indices from
 constexpr int kHeaderValueMax = 11;  // header word with the largest |v| (bf16 bits), shared-stream mode; zero in the uploaded table
 constexpr int kItemInts = 16;
+constexpr int kSms = 148;        // multiprocessors of a B200, for rules that split work (and size workspaces) on the host alike
+                                 // whether or not a device is there; the persistent kernel asks the device
 constexpr int kMaxFold = 8;      // most query heads of one KV head folded into the rows of a query tile
 constexpr int kMaxNormHeads = 512;   // Hq + Hkv up to which the rotation kernels track the norms (shared memory)
 
@@ -62,8 +64,6 @@ int32_t max_fold(int32_t group);   // largest power of two <= kMaxFold that divi
 int build_prefill_tables(int32_t n_bins, int32_t capacity, const int32_t* bin_seg_ptr,
                          const int32_t* seg_start, const int32_t* seg_len, int32_t k, int32_t n_q_heads,
                          int32_t n_kv_heads, int32_t* out, size_t out_ints, TableLayout* layout);
-
-int sm_count();     // multiprocessors of the current device; 0 if it cannot be asked
 
 // Records a failed CUDA call for pp_last_cuda_error(); returns PP_ERR_CUDA.
 int note_cuda_error(int cuda_error, const char* what);
@@ -138,8 +138,12 @@ size_t unpack_table_bytes(int32_t k);
 // A table of at most this many ints is not uploaded but handed to the kernels as a parameter (independent mode:
 // the shared-stream mode wants words of it zeroed in memory). Without the copy, the gap behind it and the wait
 // for it a step of 8 prompts on 4 heads takes 13.5 us instead of 16.9, one of 16 prompts on 32 heads 54 instead
-// of 65 (the rotation kernel's look-ups then run under the end of the kernel before). Larger tables would
-// slow every launch down.
+// of 65 (the rotation kernel's look-ups then run under the end of the kernel before). But the block is copied whole at every
+// launch of a call that uses it. Steps of n prompts of 16 to 128 tokens on 4 / 4 heads of 64 with a block of 448, 896,
+// 1792, 3584 and 7168 ints (us): n = 8 (140 ints) 14.0, 14.2, 14.9, 16.7, 20.5; n = 32 (584) 16.8, 15.4, 16.2, 17.8, 21.5;
+// n = 64 (1088) 17.8, 18.0, 17.0, 18.8, 23.9; n = 160 (2628) 26.1, 26.1, 26.1, 23.2, 26.1.
+// On 32 / 32 heads of 128, where the kernels are longer than the host: n = 24 (492) 34.0, 31.9, 32.0, 32.0, 32.8; n = 64 (1144)
+// 74.1, 73.5, 71.4, 71.4, 71.5.
 constexpr int kInlineInts = 896;
 
 #ifdef __CUDACC__

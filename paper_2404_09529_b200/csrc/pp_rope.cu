@@ -237,7 +237,7 @@ constexpr int kRuRowsWide = 8, kRuRowsNarrow = 32;
 constexpr int kRuNarrowRowElems = 1024;   // n_kv_heads * D up to which a row counts as narrow
 // ... and only where that still gives every SM a few blocks: a few hundred rows in blocks of 32 leave most of the chip
 // idle (448 rows of 4 heads, D = 64: 14 blocks; with 56 blocks of 8 rows and the table as a parameter 5.8 -> 3.3 us).
-constexpr int64_t kRuNarrowRows = 32 * 148 * 4;
+constexpr int64_t kRuNarrowRows = 32 * kSms * 4;
 constexpr int kRuV = 8;      // 16-byte V copies in flight per thread
 constexpr int kRuK = 2;      // (lower, upper) K pairs in flight per thread
 // kRange: the norms and the largest |v| are wanted (shared-stream mode).
@@ -480,7 +480,7 @@ int launch_value_range(const pp_attn_params& p, int32_t* d_table, const TableLay
   const int32_t vec_per_row = p.n_kv_heads * p.head_dim / 8;
   // about four blocks per SM, but no slice of a bin shorter than one pass of a block
   const int64_t per_bin = ((int64_t)p.capacity * vec_per_row + kRopeThreads * kRangeVecs - 1) / (kRopeThreads * kRangeVecs);
-  const int64_t wanted = (4 * (int64_t)std::max(sm_count(), 1) + p.n_bins - 1) / p.n_bins;
+  const int64_t wanted = (4 * kSms + (int64_t)p.n_bins - 1) / p.n_bins;
   const unsigned slices = (unsigned)std::min<int64_t>(std::min(per_bin, wanted), 65535);
   const cudaError_t e = launch_dependent(value_range_kernel, dim3((unsigned)p.n_bins, slices), dim3(kRopeThreads), 0,
                                          static_cast<cudaStream_t>(stream), static_cast<const uint4*>(v), TableInMemory{d_table},

@@ -186,7 +186,7 @@ int launch_host_rows(bool to_packed, const pp_attn_params& p, int32_t* d_table, 
   RowTable m{L.bin_seg_ptr, L.bin_used, L.seg_start, off_cache_off, p.capacity, p.n_kv_heads * p.head_dim, 1,
              (int64_t)p.n_bins * p.capacity};
   // a bus read takes 1 to 2 us, so few rows are spread over as many blocks as there are
-  while (m.rows_per_block < kTzTokens && m.n_rows > (int64_t)m.rows_per_block * 148 * 2) m.rows_per_block *= 2;
+  while (m.rows_per_block < kTzTokens && m.n_rows > (int64_t)m.rows_per_block * kSms * 2) m.rows_per_block *= 2;
   const dim3 grid((unsigned)((m.n_rows + m.rows_per_block - 1) / m.rows_per_block)), block(kTzThreads);
   const int32_t q_vec = p.n_q_heads * p.head_dim / 8, kv_vec = m.kv_elems / 8;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
