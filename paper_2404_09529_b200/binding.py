@@ -16,6 +16,8 @@ _lib = None
 PP_FLAG_SKIP_ROPE = 1
 PP_FLAG_ROPE_ONLY = 2
 PP_FLAG_KEEP_ROPE_TABLE = 4
+# Tables of at most this many int32 words travel as kernel parameters in the independent mode (kInlineInts of the library).
+PARAMETER_TABLE_INTS = 896
 
 
 class PrepackError(RuntimeError):

@@ -135,3 +135,29 @@ def compare_sampled(batch, lengths, q_tok, k_tok, v_tok, base, prompts, kv_heads
     e_o.check("O"); e_k.check("K cache"); e_v.check("V cache")
     assert e_v.max_abs == 0.0
     return e_o, e_k, e_v
+
+
+def table_ints(params, pack):
+    """(int32 words of pp_prefill_attention's table, of pp_prefill_fused's) for a packing, and whether either may travel as a
+    kernel parameter at all (independent mode)."""
+    import paper_2404_09529_b200 as pp
+    up4 = lambda x: (x + 3) // 4 * 4
+    info = pp.pp_prefill_schedule_info(params, pack)
+    three = (16 + up4(params.n_q_heads + params.n_kv_heads) + up4(pack.n_bins + 1) + up4(pack.n_bins) + up4(pack.k) +
+             16 * info["entries"])
+    return three, pp.pp_prefill_fused_host_bytes(params, pack.k) // 4, info["mode"] == 1
+
+
+def decode_chunks(params, lengths):
+    """Chunks that pp_decode_step cuts the prompts into, from the size of its workspace: table of 16 bytes per prompt and a
+    prefix, then 8 bytes and head_dim floats per chunk and query head, each block on a 256-byte boundary."""
+    import paper_2404_09529_b200 as pp
+    up = lambda x: (x + 255) // 256 * 256
+    need, k = pp.pp_decode_workspace_bytes(params, lengths), len(lengths)
+    hq, d = params.n_q_heads, params.head_dim
+    size = lambda n: up(up(16 * k + 4 * (k + 1)) + 8 * n * hq) + 4 * n * hq * d
+    n = need // (hq * (4 * d + 8))
+    while size(n) > need:
+        n -= 1
+    assert size(n) == need
+    return n

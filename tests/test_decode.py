@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from oracle import prepack_oracle as orc
-from parity_utils import MAX_ABS_TOL, MEAN_ABS_TOL, to64
+from parity_utils import MAX_ABS_TOL, MEAN_ABS_TOL, decode_chunks, to64
 from workloads import split_by_prompt
 
 pytestmark = pytest.mark.gpu
@@ -21,7 +21,7 @@ def _case(lengths, hq, hkv, d, seed):
     (np.array([1, 1, 1, 1000, 1, 1, 1, 1, 1, 1], np.int32), 8, 8, 128, 10000.0),   # the paper's toy mix
     (np.array([300, 17, 255, 256, 257, 64], np.int32), 8, 2, 128, 500000.0),
     (np.array([40, 9, 513], np.int32), 4, 4, 64, 10000.0),
-    # enough (chunk, KV head) pairs for the 256-key chunks (smaller batches run 64-key chunks)
+    # many prompts at the edges of chunks of 256 keys (the batches above run chunks of 64)
     (np.array([255, 256, 257, 511, 512, 513, 767, 768, 300, 64, 1000, 129] * 4, np.int32), 16, 16, 64, 10000.0),
 ])
 def test_decode_steps_match_oracle(lengths, hq, hkv, d, base):
@@ -79,20 +79,23 @@ def test_decode_argument_checks():
                           ws, host, 16)
 
 
-@pytest.mark.parametrize("lengths,hq,hkv,d", [
+@pytest.mark.parametrize("lengths,hq,hkv,d,chunk_keys", [
     # every remainder of a 16-key step and of a 64-key chunk, in one chunk and in several; group 8
-    (np.array([1, 2, 15, 16, 17, 31, 32, 33, 47, 48, 49, 63, 64, 65, 127, 128, 129, 191, 192, 193], np.int32), 16, 2, 128),
-    (np.array([1, 15, 16, 17, 63, 64, 65, 129, 255, 257], np.int32), 6, 2, 64),          # group 3: absent head columns
-    (np.array([5000, 3], np.int32), 2, 1, 128),                                          # most chunks per prompt
-    (np.arange(600, dtype=np.int32) % 37 + 1, 2, 2, 64),                                 # table uploaded, not in the parameters
-    (np.array([70] * 40 + [200], np.int32), 4, 1, 128),                                  # the larger parameter block
-    (np.array([3000] * 3 + [512, 513], np.int32), 128, 32, 64),                          # chunks of 512 keys
+    (np.array([1, 2, 15, 16, 17, 31, 32, 33, 47, 48, 49, 63, 64, 65, 127, 128, 129, 191, 192, 193], np.int32), 16, 2, 128, 64),
+    (np.array([1, 15, 16, 17, 63, 64, 65, 129, 255, 257], np.int32), 6, 2, 64, 64),      # group 3: absent head columns
+    (np.array([4096, 3], np.int32), 2, 1, 128, 64),                                      # 64 chunks, the most of a prompt
+    (np.array([4097, 3], np.int32), 2, 1, 128, 128),                                     # one key more: larger chunks
+    (np.arange(600, dtype=np.int32) % 37 + 1, 2, 2, 64, 64),                             # table uploaded, not in the parameters
+    (np.array([70] * 40 + [200], np.int32), 4, 1, 128, 64),                              # the larger parameter block
+    (np.array([3000] * 3 + [512, 513], np.int32), 128, 32, 64, 192),                     # between the smallest and the largest
+    (np.array([9000] * 3 + [1536, 512, 513], np.int32), 64, 32, 64, 512),                # the largest
 ])
-def test_decode_chunks_and_tables(lengths, hq, hkv, d):
+def test_decode_chunks_and_tables(lengths, hq, hkv, d, chunk_keys):
     """The generation step on caches of random contents at the edges of its steps, chunks and table forms,
     spare rows untouched."""
     from paper_2404_09529_b200.runner import DecodeBatch
     dec = DecodeBatch(lengths, hq, hkv, d, 10000.0, room=2)
+    assert decode_chunks(dec.params, lengths) == sum(-(-int(l) // chunk_keys) for l in lengths)
     g = torch.Generator().manual_seed(int(lengths.sum()))
     for pool in (dec.k_cache, dec.v_cache):
         pool.copy_(torch.randn(pool.shape, generator=g).to(torch.bfloat16))

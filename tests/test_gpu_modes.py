@@ -22,7 +22,7 @@ import pytest
 import torch
 
 import paper_2404_09529_b200 as pp
-from parity_utils import compare_with_refs, expected_schedule, oracle_refs, run_cuda
+from parity_utils import compare_with_refs, expected_schedule, oracle_refs, run_cuda, table_ints
 from paper_2404_09529_b200.runner import DecodeBatch, PrefillBatch
 from workloads import split_by_prompt
 
@@ -194,9 +194,14 @@ def test_keep_rope_table_flag_gives_identical_results():
         assert torch.equal(a, c)
 
 
-@pytest.mark.parametrize("k", [1, 30, 45])        # small tables travel as kernel parameters (1, 30), larger ones are uploaded
-@pytest.mark.parametrize("hq,hkv,d", [(4, 4, 64), (4, 2, 128)])
-def test_table_as_parameter_or_uploaded(k, hq, hkv, d):
+# whether the fused and the three-call table travel as kernel parameters: the sizes next to the line, without and with heads
+# folded into the query tiles
+@pytest.mark.parametrize("hq,hkv,d,k,fused_as_parameter,three_as_parameter", [
+    (4, 4, 64, 1, True, True), (4, 4, 64, 37, True, True), (4, 4, 64, 38, False, True), (4, 4, 64, 45, False, True),
+    (4, 4, 64, 46, False, False),
+    (4, 2, 128, 1, True, True), (4, 2, 128, 22, True, True), (4, 2, 128, 23, False, True), (4, 2, 128, 24, False, True),
+    (4, 2, 128, 25, False, False)])
+def test_table_as_parameter_or_uploaded(hq, hkv, d, k, fused_as_parameter, three_as_parameter):
     """Both forms of the prefill table give the oracle's results, on the first and on a repeated call on the
     same workspace (the work counter starts anew), and whole or split by flags."""
     lengths = np.asarray([100 - 3 * (i % 7) for i in range(k)], np.int32)
@@ -205,6 +210,9 @@ def test_table_as_parameter_or_uploaded(k, hq, hkv, d):
     refs = oracle_refs(lengths, q, kk, v, base)
     fused = PrefillBatch(lengths, hq, hkv, d, base, guard=True)
     three = PrefillBatch(lengths, hq, hkv, d, base, guard=True)
+    three_ints, fused_ints, may = table_ints(fused.params, fused.pack)
+    line = pp.binding.PARAMETER_TABLE_INTS
+    assert (may and fused_ints <= line, may and three_ints <= line) == (fused_as_parameter, three_as_parameter)
     for _ in range(2):
         for b, call in ((fused, fused.run_fused), (three, three.run)):
             b.load(q, kk, v)
@@ -222,9 +230,10 @@ def test_table_as_parameter_or_uploaded(k, hq, hkv, d):
     assert fused.device_status() == 0 and torch.equal(fused.o_tokens(), o.view(-1, hq, d)[fused.token_rows])
 
 
-@pytest.mark.parametrize("k", [31, 45, 333])
+# prompts: only the unpack table is uploaded (31, 45), the fused table too (70), all three (120, 333)
+@pytest.mark.parametrize("k,uploaded", [(31, (False, False)), (45, (False, False)), (70, (False, True)), (120, (True, True)), (333, (True, True))])
 @pytest.mark.parametrize("staging", ["pinned", "pinned + 16", "pinned + 8", "pageable"])
-def test_tables_from_any_staging_memory(k, staging):
+def test_tables_from_any_staging_memory(k, uploaded, staging):
     """Tables are read by a kernel from aligned pinned memory and copied from any other, several calls in a row
     through the ring of staging buffers."""
     lengths = np.asarray([60 - 7 * (i % 9) for i in range(k)], np.int32)
@@ -233,6 +242,7 @@ def test_tables_from_any_staging_memory(k, staging):
     at = int(staging.split("+")[1]) if "+" in staging else 0
     fused = PrefillBatch(lengths, 2, 1, 64, 10000.0, guard=True)
     three = PrefillBatch(lengths, 2, 1, 64, 10000.0, guard=True)
+    assert tuple(n > pp.binding.PARAMETER_TABLE_INTS for n in table_ints(three.params, three.pack)[:2]) == uploaded
 
     def buffer(like):
         t = torch.empty(like.numel() + at, dtype=torch.uint8)

@@ -218,3 +218,9 @@ def test_per_device_once_guard(tmp_path):
     subprocess.run([gxx, "-std=c++17", "-O1", "-pthread", "-I", inc, str(src), "-o", str(exe)], check=True)
     out = subprocess.run([str(exe)], capture_output=True, text=True)
     assert out.returncode == 0 and out.stdout.strip() == "ok", (out.returncode, out.stdout, out.stderr)
+
+
+def test_binding_knows_the_size_of_parameter_tables():
+    """binding.PARAMETER_TABLE_INTS (from which the benchmark counts launches) is the library's kInlineInts."""
+    with open(os.path.join(ROOT, "paper_2404_09529_b200", "csrc", "pp_internal.h")) as f:
+        assert int(re.search(r"kInlineInts = (\d+);", f.read()).group(1)) == pp.binding.PARAMETER_TABLE_INTS
