@@ -31,11 +31,9 @@ METRIC = "useful_prefill_tokens_per_s"
 UNIT = "tokens/s"
 DEFAULT_WORKLOAD = "llama2_7b"
 
-# DRAM traffic of one attention-kernel launch (dram__bytes_read.sum + dram__bytes_write.sum) from
-# the ncu captures summarised in profiles/attention_<workload>.md (fused-route launches; long_mix: a
-# launch of the three-call route, which reads and writes the same tensors); None where no capture
-# exists for the workload.
-NCU_ATTENTION_TRAFFIC_BYTES = {"llama2_7b": 562.4e6, "many_short": 424.2e6, "long_mix": 3.82e9}
+# DRAM traffic of a fused step's kernels (dram__bytes_read.sum + dram__bytes_write.sum, each kernel from a cold L2)
+# from the ncu captures in profiles/launches_<workload>.md; None where no capture exists for the workload.
+NCU_STEP_TRAFFIC_BYTES = {}
 
 
 def load_peaks():
@@ -125,7 +123,8 @@ def workload_counts(cfg, lengths):
         useful_flops=4 * hq * d * pairs,                       # QK^T and PV, 2*D flops each per visible pair
         attn_bytes=2 * total * d * (2 * hq + 2 * hkv),         # read Q', K', V once, write O once
         rope_bytes=4 * total * d * (hq + hkv),                 # read + write Q and K
-        unpack_bytes=8 * total * d * hkv)                      # read K', V; write both caches
+        unpack_bytes=8 * total * d * hkv,                      # read K', V; write both caches
+        step_bytes=2 * total * d * (2 * hq + 5 * hkv))         # fused step: read Q, K, V; write O, K' and both caches
 
 
 def max_over_ranks(ms: float, dist=None, device="cpu") -> float:
@@ -412,26 +411,29 @@ def main():
         "unpack": {"ms": ms_unpack, "gbs": counts["unpack_bytes"] / ms_unpack * 1e-6,
                    "frac_hbm": counts["unpack_bytes"] / ms_unpack * 1e-6 / peaks["hbm_gbs"]},
     }
-    # the attention kernel dominates; which roofline binds it depends on the workload's FLOP/byte
-    intensity = counts["useful_flops"] / counts["attn_bytes"]
+    # The roofline is that of the headline step's kernels as the step launches them, one behind the other (device time of
+    # queued steps that do not pack anew). Launched alone by a flag, as above, they are not the same: the attention kernel then
+    # fills no V caches, and has no bound on the scores.
+    schedule = pp.pp_prefill_schedule_info(batch.params, batch.pack)
+    fills = (schedule["mode"] == 1 and cfg.head_dim == 128 and cfg.n_q_heads == cfg.n_kv_heads and T >= 32 * len(lengths))
+    ms_kernels = time_loop(lambda: batch.run_fused(), n_it)
+    step_tflops, step_gbs = counts["useful_flops"] / ms_kernels * 1e-9, counts["step_bytes"] / ms_kernels * 1e-6
+    kernels["step_fused"] = {"ms": ms_kernels, "tflops": step_tflops, "gbs": step_gbs, "v_caches_by": "attention_kernel" if fills else "rope_unpack_kernel"}
+    kernels["note"] = "rope_unpack_fused and attention_fused are launched alone by flags, not as the step launches them"
+    intensity = counts["useful_flops"] / counts["step_bytes"]
     ridge = peaks["bf16_tflops"] * 1e3 / peaks["hbm_gbs"]
-    traffic = NCU_ATTENTION_TRAFFIC_BYTES.get(args.workload)
-    # the attention kernel as launched in the headline route
-    dom = kernels["attention_fused"] if path == "fused" else kernels["attention"]
+    traffic = NCU_STEP_TRAFFIC_BYTES.get(args.workload)
+    dom = kernels["attention_fused"]
+    roofline = {"kernel": "rope_unpack_kernel + attention_kernel", "traffic": traffic, "flop_per_byte": intensity, "ridge_flop_per_byte": ridge}
     if intensity < ridge:
-        roofline = {"kernel": "attention", "bound": "hbm", "achieved": dom["gbs"],
-                    "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": dom["frac_hbm"],
-                    "traffic": traffic, "peak_source": peaks["source"] + " (burst copy)",
-                    "flop_per_byte": intensity, "ridge_flop_per_byte": ridge}
+        roofline.update(bound="hbm", achieved=step_gbs, peak=peaks["hbm_gbs"], unit="GB/s", frac=step_gbs / peaks["hbm_gbs"],
+                        peak_source=peaks["source"] + " (burst copy)")
     else:
-        # the burst peak is the stricter denominator; the loop that times the kernel runs long enough
+        # the burst peak is the stricter denominator; the loop that times the kernels runs long enough
         # to sit at the power cap like the sustained cuBLAS measurement, so that fraction is given too
-        roofline = {"kernel": "attention", "bound": "tensor", "achieved": dom["tflops"],
-                    "peak": peaks["bf16_tflops"], "unit": "TFLOP/s", "frac": dom["frac_bf16_peak"],
-                    "traffic": traffic, "peak_source": peaks["source"] + " (burst, kernel timed alone)",
-                    "peak_sustained": peaks["bf16_tflops_sustained"],
-                    "frac_of_sustained_peak": dom["tflops"] / peaks["bf16_tflops_sustained"],
-                    "flop_per_byte": intensity, "ridge_flop_per_byte": ridge}
+        roofline.update(bound="tensor", achieved=step_tflops, peak=peaks["bf16_tflops"], unit="TFLOP/s", frac=step_tflops / peaks["bf16_tflops"],
+                        peak_source=peaks["source"] + " (burst, kernels timed alone)", peak_sustained=peaks["bf16_tflops_sustained"],
+                        frac_of_sustained_peak=step_tflops / peaks["bf16_tflops_sustained"])
 
     # ---------------------------------------------------------------- padded-batch mode of the same kernels
     padded = None
@@ -498,7 +500,9 @@ def main():
     d2h = (ho.numel() + hkc.numel() + hvc.numel()) * 2
     e2e = {"value": whole_job_tokens_per_s(world, T, ms_e2e / e2e_steps), "unit": UNIT, "h2d_bytes_per_step": h2d,
            "d2h_bytes_per_step": d2h, "steps": e2e_steps, "ms_per_step": ms_e2e / e2e_steps,
-           "api": "pp_prefill_host (pinned host buffers, contiguous copies, groups of prompts pipelined over streams)"}
+           "api": "pp_prefill_host (pinned host buffers; " +
+                  ("contiguous copies, groups of prompts pipelined over streams)" if h2d >= 32 << 20 else
+                   "one group: read and written in place by the kernels up to 20 MB, one prompt 40 MB, else copied)")}
 
     # ---------------------------------------------------------------- CPU baseline: the oracle as it stands
     cpu_baseline = None
@@ -508,10 +512,10 @@ def main():
                         "sample": f"first {n_done} of {len(lengths)} prompts in original order ({tok} tokens), "
                                   f"all heads, numpy float64, {sec:.1f} s"}
 
-    # tables of up to 896 ints of the independent mode are kernel parameters
-    small_tables = (batch.ws.fused_host(0).numel() <= 4 * 896 and
-                    pp.pp_prefill_schedule_info(batch.params, batch.pack)["mode"] == 1)
-    launches_per_step = 2 if small_tables else 3
+    # the tables are kernel parameters (small ones of the independent mode), read by a kernel (up to 1 MB), or copied
+    table_bytes = pp.pp_prefill_fused_host_bytes(batch.params, batch.pack.k)
+    as_parameters = table_bytes <= 4 * pp.binding.PARAMETER_TABLE_INTS and schedule["mode"] == 1
+    launches_per_step = 2 if as_parameters or table_bytes > 1 << 20 else 3
     if rank == 0:
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -520,7 +524,7 @@ def main():
             "config": config,
             "clocks": clocks, "e2e": e2e, "gpu_launches": launches_per_step * args.steps, "roofline": roofline,
             "launches_note": "fused route: rope_unpack_kernel + attention_kernel per step, and upload_kernel where the "
-                             "tables are too large for the kernels' parameters; the cos/sin table kernel "
+                             "tables are too large for the kernels' parameters and at most 1 MB; the cos/sin table kernel "
                              "runs once (first warm-up step) and is kept while the bin capacity stays the same",
             "cpu_baseline": cpu_baseline, "host": host, "kernels": kernels, "padded": padded,
             "routes": {"three_call": {"tokens_per_s": whole_job_tokens_per_s(world, T, route_ms["three_call"]),
@@ -530,7 +534,7 @@ def main():
                                  "ms_per_step": route_ms["fused"], "api": "pp_pack + pp_prefill_fused"}},
             "attention": {"useful_tflops": dom["tflops"],
                           "frac_bf16_peak_measured": dom["frac_bf16_peak"],
-                          "frac_bf16_peak_datasheet": dom["frac_bf16_datasheet"]},
+                          "frac_bf16_peak_datasheet": dom["frac_bf16_datasheet"], "launched": "alone, by a flag"},
             "peaks": peaks,
         }
         print(json.dumps(line))
