@@ -33,7 +33,7 @@ DEFAULT_WORKLOAD = "llama2_7b"
 
 # DRAM traffic of a fused step's kernels (dram__bytes_read.sum + dram__bytes_write.sum, each kernel from a cold L2)
 # from the ncu captures in profiles/launches_<workload>.md; None where no capture exists for the workload.
-NCU_STEP_TRAFFIC_BYTES = {}
+NCU_STEP_TRAFFIC_BYTES = {"llama2_7b": 1070.2e6, "many_short": 585.4e6}
 
 
 def load_peaks():
