@@ -128,6 +128,17 @@ __device__ __forceinline__ void load_v(StepV<D>& f, const __nv_bfloat16* base, i
 // A maximum over nothing. Finite, so that a score of -inf (a key with an infinite element) weighs nothing beside it.
 constexpr float kNoScore = -FLT_MAX;
 
+// The rows past the last real one are copies of it, whose weight is 0: no part of O, not as 0 times an infinity either.
+template <int D>
+__device__ __forceinline__ void clear_past(StepV<D>& f, int n_real, int t) {
+#pragma unroll
+  for (int x = 0; x < 4; ++x)
+    if (2 * t + (x & 1) + 8 * (x >> 1) >= n_real) {
+#pragma unroll
+      for (int i = 0; i < D / 64; ++i) f.r[x][i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+}
+
 template <int D>
 struct Softmax {
   float m[2] = {kNoScore, kNoScore};      // running maximum of query heads 2t and 2t + 1 (all lanes of equal t agree)
@@ -187,17 +198,20 @@ __device__ __forceinline__ uint32_t truncate_bf16x2(float a, float b) {
 // O^T += V^T P. Product j: row g is d = 8g + j, row g + 8 is d = 64 + 8g + j (D = 128) or 8g + 4 + j (D = 64).
 template <int D>
 __device__ __forceinline__ void pv(Softmax<D>& s, const StepV<D>& f, const float (&p)[4]) {
-  // P in three parts of 8 bits, cut and not rounded, so that none is negative, and none is 0: an infinite value (also in the
-  // row that stands in for those past the chunk) then gives an infinity and not a NaN, a finite one 2^-126 of itself.
-  const __nv_bfloat162 least = __halves2bfloat162(__ushort_as_bfloat16(0x0080), __ushort_as_bfloat16(0x0080));
+  // P in three parts of 8 bits, cut and not rounded, so that none is negative, and none of a weight above 0 (which is at least
+  // 2^-126) is 0: an infinite value then gives an infinity and not a NaN, a finite one up to 2^-125 of itself too much.
   uint32_t b[3][2];
   float r[4] = {p[0], p[1], p[2], p[3]};
+  uint32_t least[2];
+#pragma unroll
+  for (int x = 0; x < 2; ++x) least[x] = (p[2 * x] > 0.f ? 0x0080u : 0u) | (p[2 * x + 1] > 0.f ? 0x00800000u : 0u);
 #pragma unroll
   for (int part = 0; part < 3; ++part)
 #pragma unroll
     for (int x = 0; x < 2; ++x) {
       const uint32_t cut = truncate_bf16x2(r[2 * x], r[2 * x + 1]);
-      const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&cut), w = __hmax2_nan(v, least);
+      const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&cut);
+      const __nv_bfloat162 w = part == 0 ? v : __hmax2_nan(v, *reinterpret_cast<const __nv_bfloat162*>(&least[x]));
       b[part][x] = transpose8x8(*reinterpret_cast<const uint32_t*>(&w));
       const float2 back = __bfloat1622float2(v);
       r[2 * x] -= back.x;
@@ -317,6 +331,7 @@ decode_kernel(const __grid_constant__ DecodeArgs a, const __grid_constant__ Deco
     const int next = key + kTileKeys * kDecodeWarps;
     if (next < key_end) load_k<D>(fk, kb, next, key_end - 1, g, t);
     softmax_step<D>(s, c, a.scale_log2, key_end - key, g);
+    if (key_end - key < kTileKeys) clear_past<D>(fv, key_end - key, t);
     pv<D>(s, fv, c);
     if (next < key_end) load_v<D>(fv, vb, next, key_end - 1, g, t);
     key = next;

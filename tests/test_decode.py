@@ -175,3 +175,30 @@ def test_decode_with_scores_of_minus_infinity(lengths):
         ref = orc.decode_step(to64(qn[i]), to64(kn[i]), to64(vn[i]), *before[i], base)[0]
         assert np.isfinite(ref).all() and np.isfinite(got[i]).all(), i
         assert np.abs(got[i] - ref).max() <= MAX_ABS_TOL, i
+
+
+@pytest.mark.parametrize("hq,hkv,d", [(2, 2, 128), (6, 2, 64)])
+def test_decode_with_huge_values_of_no_weight(hq, hkv, d):
+    """The largest finite bf16 among the values of keys whose weight underflows to 0 adds nothing: in the middle of a chunk and
+    in the last row, of which the rows past the end are copies."""
+    from paper_2404_09529_b200.runner import DecodeBatch
+    lengths = np.array([1, 16, 17, 50, 64, 65, 200, 700], np.int32)
+    dec = DecodeBatch(lengths, hq, hkv, d, 10000.0, room=2)
+    g = torch.Generator().manual_seed(hq + d)
+    for pool in (dec.k_cache, dec.v_cache):
+        pool.copy_(torch.randn(pool.shape, generator=g).to(torch.bfloat16))
+    qn, kn, vn = (torch.randn(dec.k, h, d, generator=g).to(torch.bfloat16) for h in (hq, hkv, hkv))
+    qn[:, :, d // 2 - 1] = 20                     # slowly turning: hardly rotated, positive at every position here
+    qn[:, :, d - 1] = 0
+    for i, l in enumerate(int(x) for x in lengths):
+        ck, cv = dec.caches(i)
+        for key in {l // 3, l // 2, l - 1}:
+            ck[:, key, d // 2 - 1] = -100         # weight exp(-170) or less
+            cv[:, key] = 3.3e38
+    before = [tuple(to64(c[:, :int(l)]) for c in dec.caches(i)) for i, l in enumerate(lengths)]
+    got = to64(dec.step(qn.cuda(), kn.cuda(), vn.cuda()))
+    for i in range(dec.k):
+        kc, vc = before[i]
+        vc = np.where(vc > 1e38, 0.0, vc)         # (their part of O is below 1e-30, but not of an fp64 sum of 1e38 exp(-170))
+        ref = orc.decode_step(to64(qn[i]), to64(kn[i]), to64(vn[i]), kc, vc, 10000.0)[0]
+        assert np.abs(got[i] - ref).max() <= MAX_ABS_TOL, (i, np.abs(got[i] - ref).max())
