@@ -16,6 +16,7 @@ constexpr int kHeaderInts = 16;  // table header, see build_prefill_tables
 constexpr int kHeaderSegments = 4;   // header word with the number of segments
 constexpr int kHeaderCounter = 10;   // header word the persistent CTAs draw work indices from
 constexpr int kHeaderValueMax = 11;  // header word with the largest |v| (bf16 bits), shared-stream mode; zero in the uploaded table
+constexpr int kValueFromNorms = kHeaderValueMax - kHeaderInts;   // that word seen from the norms, which follow the header
 constexpr int kItemInts = 16;
 constexpr int kSms = 148;        // multiprocessors of a B200, for rules that split work (and size workspaces) on the host alike
                                  // whether or not a device is there; the persistent kernel asks the device

@@ -87,16 +87,20 @@ __device__ __forceinline__ void publish_ranges(const uint32_t* s_max, int n, uin
   }
 }
 
-// kRange (shared-stream mode): norms, [Hkv] then [Hq] words, receive the largest |k|^2 / |q|^2 of each head, v_max the
-// largest |v| of the real rows of v (null: not wanted). Reading V here costs its bytes (four prompts of 3000 to 4096
+// Where a kernel finds the segment tables in the prefill table. (One parameter instead of three: each costs a launch about 0.1 us of
+// host time, which is what a small batch takes.)
+struct SegTables {
+  int32_t bin_seg_ptr, bin_used, seg_start;
+};
+
+// kRange (shared-stream mode): norms, [Hkv] then [Hq] words, receive the largest |k|^2 / |q|^2 of each head, and the
+// word kValueFromNorms before them the largest |v| of the real rows of v (null: not wanted). Reading V here costs its bytes (four prompts of 3000 to 4096
 // tokens on 32 / 32 heads of 128, three calls: 638 -> 655 us; as a kernel of its own 633 -> 664).
 // counter: null, or the work counter to reset for the attention kernel.
 template <int D, bool kRange, class Table>
-__global__ void __launch_bounds__(kRopeThreads)
+__global__ void __launch_bounds__(kRopeThreads, 6)
 rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, const __nv_bfloat16* v, uint32_t* norms,
-            uint32_t* v_max, int32_t* counter,
-            const __grid_constant__ Table tab, int32_t off_bin_seg_ptr, int32_t off_bin_used,
-            int32_t off_seg_start, int32_t n_bins, int32_t capacity, int32_t n_q_heads,
+            int32_t* counter, const __grid_constant__ Table tab, SegTables seg, int32_t n_bins, int32_t capacity, int32_t n_q_heads,
             int32_t n_kv_heads, const __grid_constant__ RopeFreq freq) {
   constexpr int kHalf = D / 2;
   constexpr int kUnitsPerHead = kHalf / 8;          // 16-byte vector pairs per head
@@ -120,14 +124,14 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, const 
     if (row < n_rows) {
       const int32_t b = (int32_t)(row / capacity);
       const int32_t t = (int32_t)(row - (int64_t)b * capacity);
-      if (t < tab.i32(off_bin_used + b)) {
+      if (t < tab.i32(seg.bin_used + b)) {
         // last segment of bin b whose start row is <= t
-        int32_t lo = tab.i32(off_bin_seg_ptr + b), hi = tab.i32(off_bin_seg_ptr + b + 1) - 1;
+        int32_t lo = tab.i32(seg.bin_seg_ptr + b), hi = tab.i32(seg.bin_seg_ptr + b + 1) - 1;
         while (lo < hi) {
           const int32_t mid = (lo + hi + 1) >> 1;
-          if (tab.i32(off_seg_start + mid) <= t) lo = mid; else hi = mid - 1;
+          if (tab.i32(seg.seg_start + mid) <= t) lo = mid; else hi = mid - 1;
         }
-        pos = t - tab.i32(off_seg_start + lo);
+        pos = t - tab.i32(seg.seg_start + lo);
       }
     }
     s_pos[tid] = pos;
@@ -196,7 +200,7 @@ rope_kernel(__nv_bfloat16* __restrict__ q, __nv_bfloat16* __restrict__ k, const 
       }
       note_max_abs(m, s_norm + n_heads);
     }
-    publish_ranges(s_norm, n_heads, norms, v_max);
+    publish_ranges(s_norm, n_heads, norms, norms + kValueFromNorms);
   }
 }
 
@@ -244,9 +248,8 @@ constexpr int kRuK = 2;      // (lower, upper) K pairs in flight per thread
 template <int D, int kRuRows, bool kRange, class Table>
 __global__ void __launch_bounds__(kRopeThreads)
 rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* v, uint32_t* norms,
-                   uint32_t* v_max, int32_t* counter, __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
-                   const __grid_constant__ Table tab, int32_t off_bin_seg_ptr, int32_t off_bin_used,
-                   int32_t off_seg_start, SegExt ext, const float2* rope_table,
+                   int32_t* counter, __nv_bfloat16* __restrict__ k_cache, __nv_bfloat16* __restrict__ v_cache,
+                   const __grid_constant__ Table tab, SegTables seg, SegExt ext, const float2* rope_table,
                    int32_t n_bins, int32_t capacity, int32_t n_kv_heads) {
   constexpr int kHalf = D / 2;
   constexpr int kPairUnits = kHalf / 8;             // (lower, upper) 16-byte pairs per head
@@ -271,13 +274,13 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* v, uint32
     if (row < n_rows) {
       const int32_t b = (int32_t)(row / capacity);
       const int32_t t = (int32_t)(row - (int64_t)b * capacity);
-      if (t < tab.i32(off_bin_used + b)) {
-        int32_t lo = tab.i32(off_bin_seg_ptr + b), hi = tab.i32(off_bin_seg_ptr + b + 1) - 1;
+      if (t < tab.i32(seg.bin_used + b)) {
+        int32_t lo = tab.i32(seg.bin_seg_ptr + b), hi = tab.i32(seg.bin_seg_ptr + b + 1) - 1;
         while (lo < hi) {
           const int32_t mid = (lo + hi + 1) >> 1;
-          if (tab.i32(off_seg_start + mid) <= t) lo = mid; else hi = mid - 1;
+          if (tab.i32(seg.seg_start + mid) <= t) lo = mid; else hi = mid - 1;
         }
-        pos = t - tab.i32(off_seg_start + lo);
+        pos = t - tab.i32(seg.seg_start + lo);
         if (pos < tab.i32(ext.off_true_len + lo)) {   // rows past the prompt's true length are not cached
           stride = (int64_t)tab.i32(ext.off_cap + lo) * D;
           dst = tab.i64(ext.off_cache_off, lo) + (int64_t)pos * D;
@@ -373,7 +376,7 @@ rope_unpack_kernel(__nv_bfloat16* __restrict__ k, const __nv_bfloat16* v, uint32
   }
   if (kRange) {
     note_max_abs(my_v_max, s_norm + n_kv_heads);
-    publish_ranges(s_norm, n_kv_heads, norms, v_max);
+    publish_ranges(s_norm, n_kv_heads, norms, norms + kValueFromNorms);
   }
 }
 
@@ -407,9 +410,6 @@ value_range_kernel(const uint4* v, const TableInMemory tab, int32_t off_bin_used
 uint32_t* norm_words(const pp_attn_params& p, int32_t* d_table, const TableLayout& L) {
   return tracks_ranges(p, L) ? reinterpret_cast<uint32_t*>(d_table + L.norms) : nullptr;
 }
-uint32_t* value_word(const pp_attn_params& p, int32_t* d_table, const TableLayout& L) {
-  return tracks_ranges(p, L) ? reinterpret_cast<uint32_t*>(d_table + kHeaderValueMax) : nullptr;
-}
 
 RopeFreq make_freq(const pp_attn_params& p) {
   RopeFreq freq;
@@ -429,8 +429,8 @@ int launch_rope_unpack_t(const pp_attn_params& p, int32_t* d_table, const TableL
   const unsigned grid = (unsigned)((n_rows + rows - 1) / rows);
   auto launch = [&](auto kernel) {
     return launch_dependent(kernel, dim3(grid), dim3(kRopeThreads), 0, s, (__nv_bfloat16*)k, (const __nv_bfloat16*)v,
-                            norm_words(p, d_table, L), value_word(p, d_table, L), counter, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, tab,
-                            L.bin_seg_ptr, L.bin_used, L.seg_start, ext, (const float2*)rope_table, p.n_bins, p.capacity,
+                            norm_words(p, d_table, L), counter, (__nv_bfloat16*)k_cache, (__nv_bfloat16*)v_cache, tab,
+                            SegTables{L.bin_seg_ptr, L.bin_used, L.seg_start}, ext, (const float2*)rope_table, p.n_bins, p.capacity,
                             p.n_kv_heads);
   };
   cudaError_t e;
@@ -455,7 +455,7 @@ int launch_rope_t(const pp_attn_params& p, int32_t* d_table, const TableLayout& 
   const unsigned grid = (unsigned)((n_rows + kRopeRows - 1) / kRopeRows);
   auto launch = [&](auto kernel) {
     return launch_dependent(kernel, dim3(grid), dim3(kRopeThreads), 0, s, (__nv_bfloat16*)q, (__nv_bfloat16*)k, (const __nv_bfloat16*)v,
-                            norm_words(p, d_table, L), value_word(p, d_table, L), counter, tab, L.bin_seg_ptr, L.bin_used, L.seg_start, p.n_bins,
+                            norm_words(p, d_table, L), counter, tab, SegTables{L.bin_seg_ptr, L.bin_used, L.seg_start}, p.n_bins,
                             p.capacity, p.n_q_heads, p.n_kv_heads, freq);
   };
   const auto launch_d = [&](auto range) {
@@ -484,7 +484,7 @@ int launch_value_range(const pp_attn_params& p, int32_t* d_table, const TableLay
   const unsigned slices = (unsigned)std::min<int64_t>(std::min(per_bin, wanted), 65535);
   const cudaError_t e = launch_dependent(value_range_kernel, dim3((unsigned)p.n_bins, slices), dim3(kRopeThreads), 0,
                                          static_cast<cudaStream_t>(stream), static_cast<const uint4*>(v), TableInMemory{d_table},
-                                         L.bin_used, p.capacity, vec_per_row, value_word(p, d_table, L));
+                                         L.bin_used, p.capacity, vec_per_row, norm_words(p, d_table, L) + kValueFromNorms);
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "value range kernel launch");
 }
 
