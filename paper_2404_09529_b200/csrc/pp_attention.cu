@@ -135,61 +135,52 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 }
 // A value that is the same in all lanes, said so to the compiler (all 32 lanes call).
 __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
 
 // Every wait in the kernel goes through here: it gives up after `limit`, leaving why in the CTA-wide abort word, so
 // that all roles leave their loops; the code goes to the device status word at the end of the kernel. A kernel of this
-// file has some forty waits, inlined, and its roles share one instruction cache per scheduler: with a 64-bit clock,
-// a global atomic and a poll counter in each wait, 1.1 of the 6 warps of a scheduler stood without an instruction at any
-// time where the V caches are filled (0.3 in the smaller kernel without rotation and caches), now 0.55. So what a wait
-// does when its first poll has failed is kept to a dozen instructions: one 32-bit clock, no global memory. Whole steps:
-// 64 prompts on a 7B layer 264 -> 241 us, 2048 short ones, 32 / 8 heads of 64, 199 -> 178, 34 bins of a stream 1030 -> 970,
-// 16 prompts 49.7 -> 48.8. (As calls of one function the waits do not fit the softmax threads' registers.)
+// file has some forty waits, inlined, and the warps of a scheduler run three to five roles: what they execute has to fit
+// its instruction cache (a straight line of code takes 1.0 cycles an instruction up to 32 KB, 3.1 to 128 KB, 6 beyond,
+// one scheduler at work). With a 64-bit clock, a global atomic and a poll counter in each wait, 1.1 of the 6 warps of a
+// scheduler stood without an instruction at any time where the V caches are filled; in this form, and with each load
+// of the producer loop at one place, 0.18. Attention of 64 prompts on a 7B layer 195 -> 168 us under ncu; whole
+// steps 264 -> 236 us, 2048 short prompts, 32 / 8 heads of 64, 199 -> 171, 34 bins of a stream 1040 -> 990, 16 prompts
+// 49.7 -> 48.8. (As calls of one function the waits do not fit the softmax threads' registers.)
 struct WaitCtx {
   uint32_t abort;               // address in shared memory, 0: go on
   uint32_t limit;               // in units of 1024 ns
 };
-__device__ __forceinline__ uint32_t clock_1024ns() { return (uint32_t)(global_ns() >> 10); }
-__device__ __forceinline__ int abort_code(const WaitCtx& w) {
-  int x;
-  asm volatile("ld.volatile.shared.b32 %0, [%1];" : "=r"(x) : "r"(w.abort));
-  return x;
+// (A poll parks the thread for about 20 us, so the clock, which starts at the first failed one, is read seldom.)
+template <int kCode>
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx& w) {
+  uint32_t ok;
+  asm volatile(
+      "{\n.reg .pred p;\n.reg .b32 t0, t1, x;\n.reg .b64 g;\n"
+      "mov.b32 t0, 0;\n"
+      "AGAIN_%=:\n"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "@p bra DONE_%=;\n"
+      "ld.volatile.shared.b32 x, [%3];\n"
+      "setp.ne.b32 p, x, 0;\n"
+      "@p bra DONE_%=;\n"
+      "mov.u64 g, %%globaltimer;\n"
+      "shr.u64 g, g, 10;\n"
+      "cvt.u32.u64 t1, g;\n"
+      "or.b32 t1, t1, 1;\n"
+      "setp.eq.b32 p, t0, 0;\n"
+      "selp.b32 t0, t1, t0, p;\n"
+      "sub.u32 t1, t1, t0;\n"
+      "setp.le.u32 p, t1, %4;\n"
+      "@p bra AGAIN_%=;\n"
+      "st.volatile.shared.b32 [%3], %5;\n"
+      "DONE_%=:\n}"
+      : "=r"(ok) : "r"(bar), "r"(parity), "r"(w.abort), "r"(w.limit), "n"(kCode) : "memory");
+  return ok != 0;
 }
-__device__ __forceinline__ void set_abort(const WaitCtx& w, int code) {
-  asm volatile("st.volatile.shared.b32 [%0], %1;" ::"r"(w.abort), "r"(code) : "memory");
-}
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx& w, int code) {
-  if (mbar_try_wait(bar, parity)) return true;
-  // (a poll parks the thread for about 20 us, so the clock is read seldom)
-  const uint32_t t0 = clock_1024ns();
-#pragma unroll 1
-  do {
-    if (mbar_try_wait(bar, parity)) return true;
-    if (abort_code(w)) return false;
-  } while (clock_1024ns() - t0 <= w.limit);
-  set_abort(w, code);
-  return false;
-}
-
 // The same for a whole warp in uniform control flow: every lane polls, the vote decides.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtx& w, int code) {
-  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-  const uint32_t t0 = clock_1024ns();
-#pragma unroll 1
-  do {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    if (__any_sync(0xffffffffu, abort_code(w))) return false;
-  } while (__all_sync(0xffffffffu, clock_1024ns() - t0 <= w.limit));
-  set_abort(w, code);
-  return false;
+template <int kCode>
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, const WaitCtx& w) {
+  return __all_sync(0xffffffffu, mbar_wait<kCode>(bar, parity, w));
 }
 
 // The warps that issue TMA loads and MMAs run in uniform control flow: all 32 lanes execute the loop, the waits
@@ -444,7 +435,9 @@ __device__ __forceinline__ void decode_work(const AttnArgs& a, const Table& tab,
   wk.bin = x.x; wk.kv_row0 = x.y; wk.n = x.z; wk.q_row0[0] = x.w; wk.q_row0[1] = y.x;
   wk.jb[0] = 0; wk.je[0] = y.z;
   wk.jb[1] = y.y; wk.je[1] = (y.x >= 0) ? x.z : y.y;       // unused slot: empty range
-  wk.bin_used = 0;
+  const int4 r = tab.i128(at + 8), z = tab.i128(at + 12);    // what the softmax threads need to place their rows
+  wk.bin_used = r.x; wk.seg_end = r.y; wk.key_lo[0] = r.z; wk.key_lo[1] = r.w;
+  wk.seg_first[0] = z.x; wk.seg_first[1] = z.y; wk.single_seg = z.z;
   if (a.pair_heads) {
     wk.head[0] = wk.kv_head * a.group + 2 * sub;
     wk.head[1] = wk.head[0] + 1;
@@ -460,16 +453,6 @@ __device__ __forceinline__ int draw_work(const AttnArgs& a, int lane, int drawer
   if (lane == 0) w = drawers + atomicAdd(a.counter, 1);
   w = __shfl_sync(0xffffffffu, w, 0);
   return w < a.total_work ? w : -1;
-}
-
-// Second half of a work-list entry: what the softmax threads need to place their rows.
-template <class Table>
-__device__ __forceinline__ void decode_rows(const AttnArgs& a, const Table& tab, int w, Work& wk) {
-  const int gi = (w / a.subs) % a.n_items;
-  const int at = a.off_items + kItemInts * gi;
-  const int4 x = tab.i128(at + 8), y = tab.i128(at + 12);
-  wk.bin_used = x.x; wk.seg_end = x.y; wk.key_lo[0] = x.z; wk.key_lo[1] = x.w;
-  wk.seg_first[0] = y.x; wk.seg_first[1] = y.y; wk.single_seg = y.z;
 }
 
 // The fetching thread decodes an item once and publishes it in shared memory; every other role
@@ -648,12 +631,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t ring_bar = 8 * (uint32_t)t * kRing;
         volatile int* ring_base = s_ring + t * (int)kRing * kRingInts;
         auto announce = [&](const uint32_t it, const int w, Work& wk) -> bool {      // w < 0: there is no item `it`
-          if (w >= 0) {
-            decode_work(args, tab, w, wk);
-            decode_rows(args, tab, w, wk);
-          }
+          if (w >= 0) decode_work(args, tab, w, wk);
           const uint32_t ring = it % kRing;
-          if (!mbar_wait_warp(bar_item_empty + ring_bar + 8 * ring, ((it / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) return false;
+          if (!mbar_wait_warp<kWaitItemEmpty>(bar_item_empty + ring_bar + 8 * ring, ((it / kRing) & 1u) ^ 1u, wctx)) return false;
           if (issue) {
             if (w >= 0) ring_write(ring_base + ring * kRingInts, w, wk);
             else ring_base[ring * kRingInts] = -1;
@@ -665,16 +645,16 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           // O of the item before the previous one must have left this Q tile (or, where O is staged
           // elsewhere, its last scores must have been computed)
           const uint32_t qb = 2u * (uint32_t)t + (it & 1u);
-          if (!mbar_wait_warp(bar_q_empty + 8 * qb, ((it >> 1) & 1u) ^ 1u, wctx, kWaitQEmpty)) return false;
+          if (!mbar_wait_warp<kWaitQEmpty>(bar_q_empty + 8 * qb, ((it >> 1) & 1u) ^ 1u, wctx)) return false;
           mbar_expect_tx(bar_q_full + 8 * qb, Cfg::kQBytes, issue);
           tma_load(s_q + qb * Cfg::kQBytes, &map_q, bar_q_full + 8 * qb, wk.head[0], wk.q_row0[0], wk.bin, issue);
           return true;
         };
-        auto load_kv = [&](const CUtensorMap* map, const uint32_t idx, const Work& wk, const int j) -> bool {
+        auto load_kv = [&](const CUtensorMap* map, const uint32_t idx, const int head, const int row, const int bin) -> bool {
           const uint32_t st = idx % NS, bar = 8 * (4u * (uint32_t)t + st);
-          if (!mbar_wait_warp(bar_kv_empty + bar, ((idx / NS) & 1u) ^ 1u, wctx, kWaitKEmpty)) return false;
+          if (!mbar_wait_warp<kWaitKEmpty>(bar_kv_empty + bar, ((idx / NS) & 1u) ^ 1u, wctx)) return false;
           mbar_expect_tx(bar_kv_full + bar, Cfg::kKVBytes, issue);
-          tma_load(s_kv + ((uint32_t)t * NS + st) * Cfg::kKVBytes, map, bar_kv_full + bar, wk.kv_head, wk.kv_row0 + j * BN, wk.bin, issue);
+          tma_load(s_kv + ((uint32_t)t * NS + st) * Cfg::kKVBytes, map, bar_kv_full + bar, head, row, bin, issue);
           return true;
         };
         const int drawers = 2 * (int)gridDim.x;
@@ -682,15 +662,17 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (w >= args.total_work) w = -1;
         Work wk, wk_next;
         bool ok = announce(0, w, wk);
-        if (ok && w >= 0) ok = load_q(0, wk) && load_kv(&map_k, kv_index_k(0), wk, 0);
+        if (ok && w >= 0) ok = load_q(0, wk) && load_kv(&map_k, kv_index_k(0), wk.kv_head, wk.kv_row0, wk.bin);
         uint32_t kc = 0;                      // key tiles of the slot's stream whose V has been loaded
         for (uint32_t it_n = 0; ok && w >= 0; ++it_n) {
           const int w_next = draw_work(args, lane, drawers);
           if (!(ok = announce(it_n + 1u, w_next, wk_next))) break;
           for (int j = 0; ok && j < wk.n; ++j, ++kc) {
-            if (j + 1 < wk.n) ok = load_kv(&map_k, kv_index_k(kc + 1), wk, j + 1);
-            else if (w_next >= 0) ok = load_kv(&map_k, kv_index_k(kc + 1), wk_next, 0);
-            if (ok) ok = load_kv(&map_v, kv_index_v(kc), wk, j);
+            const bool here = j + 1 < wk.n;             // K of this item, or the first of the next
+            if (here || w_next >= 0)
+              ok = load_kv(&map_k, kv_index_k(kc + 1), here ? wk.kv_head : wk_next.kv_head,
+                           here ? wk.kv_row0 + (j + 1) * BN : wk_next.kv_row0, here ? wk.bin : wk_next.bin);
+            if (ok) ok = load_kv(&map_v, kv_index_v(kc), wk.kv_head, wk.kv_row0 + j * BN, wk.bin);
             if (ok && j == min(1, wk.n - 1) && w_next >= 0) ok = load_q(it_n + 1u, wk_next);
           }
           w = w_next;
@@ -725,7 +707,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // S(kq) = Q_t K(kq)^T into buffer kq & 1, for the slot's item `item`
         auto issue_qk = [&](const uint32_t kq, const uint32_t item, const bool last_of_item) -> bool {
           const uint32_t idx = kv_index_k(kq), st = idx % NS;
-          if (!mbar_wait_warp(b_kv_full + 8 * st, (idx / NS) & 1u, wctx, kWaitKFull)) return false;
+          if (!mbar_wait_warp<kWaitKFull>(b_kv_full + 8 * st, (idx / NS) & 1u, wctx)) return false;
           tc_fence_after();
           const uint32_t d = tm_s + 64u * (kq & 1u);
           const uint32_t a_lo = q_lo + (item & 1u) * (Cfg::kQBytes >> 4);
@@ -747,43 +729,43 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // next item (its Q has been loaded and rotated under this item).
         int w = -1, n = 0, j = 0;
         {
-          if (!mbar_wait_warp(b_item_full, 0u, wctx, kWaitItemFull)) ok = false;
+          if (!mbar_wait_warp<kWaitItemFull>(b_item_full, 0u, wctx)) ok = false;
           if (ok) {
             const volatile int* e = s_ring + (t * (int)kRing) * kRingInts;
             w = uniform(e[0]); n = uniform(e[3]);
             if (issue) mbar_arrive(b_item_empty);
           }
         }
-        if (ok && w >= 0) ok = mbar_wait_warp(b_q_ready, 0u, wctx, kWaitQFull) && issue_qk(kc, 0u, n == 1);
+        if (ok && w >= 0) ok = mbar_wait_warp<kWaitQFull>(b_q_ready, 0u, wctx) && issue_qk(kc, 0u, n == 1);
         while (ok && w >= 0) {
           const bool last_tile = (j + 1 == n);
           int w_next = w, n_next = n;
           // With one tile per item the next item's scores would be issued before the previous item's
           // epilogue has read O_t; the softmax threads must not get that far ahead of it.
-          if (j == 0 && last_tile && !(ok = mbar_wait_warp(b_o_empty, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
+          if (j == 0 && last_tile && !(ok = mbar_wait_warp<kWaitOEmpty>(b_o_empty, (it_n & 1u) ^ 1u, wctx))) break;
           const uint32_t item = it_n + (last_tile ? 1u : 0u);         // whose tile comes next
           if (last_tile) {
             const uint32_t ring = item % kRing;
-            if (!(ok = mbar_wait_warp(b_item_full + 8 * ring, (item / kRing) & 1u, wctx, kWaitItemFull))) break;
+            if (!(ok = mbar_wait_warp<kWaitItemFull>(b_item_full + 8 * ring, (item / kRing) & 1u, wctx))) break;
             const volatile int* e = s_ring + (t * (int)kRing + (int)ring) * kRingInts;
             w_next = uniform(e[0]); n_next = uniform(e[3]);
             if (issue) mbar_arrive(b_item_empty + 8 * ring);
-            if (w_next >= 0 && !(ok = mbar_wait_warp(b_q_ready + 8 * (item & 1u), (item >> 1) & 1u, wctx, kWaitQFull))) break;
+            if (w_next >= 0 && !(ok = mbar_wait_warp<kWaitQFull>(b_q_ready + 8 * (item & 1u), (item >> 1) & 1u, wctx))) break;
           }
           if (w_next >= 0 && !(ok = issue_qk(kc + 1, item, last_tile ? n_next == 1 : j + 2 == n))) break;
           // the previous item's epilogue must have read O_t before it is overwritten
-          if (j == 0 && !last_tile && !(ok = mbar_wait_warp(b_o_empty, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
+          if (j == 0 && !last_tile && !(ok = mbar_wait_warp<kWaitOEmpty>(b_o_empty, (it_n & 1u) ^ 1u, wctx))) break;
           const uint32_t idx = kv_index_v(kc), st = idx % NS;
-          if (!(ok = mbar_wait_warp(b_kv_full + 8 * st, (idx / NS) & 1u, wctx, kWaitVFull))) break;
+          if (!(ok = mbar_wait_warp<kWaitVFull>(b_kv_full + 8 * st, (idx / NS) & 1u, wctx))) break;
           if constexpr (kFill) {
             // The cache writer must have seen V(kc - 2), whose barrier this is again, before V(kc) is announced. K(kc + 1)
             // could not have been loaded otherwise (three stages; with four, V(kc)); the slot's last tile has none.
             const uint32_t before = kv_index_v(kc - 2u);
             if (last_tile && w_next < 0 && kc >= 2u &&
-                !(ok = mbar_wait_warp(b_kv_empty + 8 * (before % NS), (before / NS) & 1u, wctx, kWaitVEmpty))) break;
+                !(ok = mbar_wait_warp<kWaitVEmpty>(b_kv_empty + 8 * (before % NS), (before / NS) & 1u, wctx))) break;
             if (issue) mbar_arrive((t ? bar_v_seen1 : bar_v_seen0) + 8 * (kc & 1u));
           }
-          if (!(ok = mbar_wait_warp(b_p_full + 8 * (kc & 1u), (kc >> 1) & 1u, wctx, kWaitP))) break;
+          if (!(ok = mbar_wait_warp<kWaitP>(b_p_full + 8 * (kc & 1u), (kc >> 1) & 1u, wctx))) break;
           tc_fence_after();            // O_t (+)= P(k) V(k)
           const uint32_t a = tm_s + 64u * (kc & 1u);
           const uint32_t vb = v_lo + st * (Cfg::kKVBytes >> 4);
@@ -811,12 +793,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       Work wk;
       while (true) {
         const int w = it_n == 0 ? (int)blockIdx.x : draw_work(args, lane, (int)gridDim.x);   // (at most one CTA per index)
-        if (w >= 0) {
-          decode_work(args, tab, w, wk);
-          decode_rows(args, tab, w, wk);
-        }
+        if (w >= 0) decode_work(args, tab, w, wk);
         const uint32_t ring = it_n % kRing;
-        if (!mbar_wait_warp(bar_item_empty + 8 * ring, ((it_n / kRing) & 1u) ^ 1u, wctx, kWaitItemEmpty)) break;
+        if (!mbar_wait_warp<kWaitItemEmpty>(bar_item_empty + 8 * ring, ((it_n / kRing) & 1u) ^ 1u, wctx)) break;
         if (issue) {
           if (w >= 0) ring_write(s_ring + ring * kRingInts, w, wk);
           else s_ring[ring * kRingInts] = -1;
@@ -827,12 +806,12 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         for (int j = 0; ok && j < wk.n; ++j, ++kc) {
           const int kv0 = wk.kv_row0 + j * BN;
           uint32_t s = kc % NK;
-          ok = mbar_wait_warp(bar_k_empty + 8 * s, ((kc / NK) & 1u) ^ 1u, wctx, kWaitKEmpty);
+          ok = mbar_wait_warp<kWaitKEmpty>(bar_k_empty + 8 * s, ((kc / NK) & 1u) ^ 1u, wctx);
           if (!ok) break;
           mbar_expect_tx(bar_k_full + 8 * s, Cfg::kKVBytes, issue);
           tma_load(s_k + s * Cfg::kKVBytes, &map_k, bar_k_full + 8 * s, wk.kv_head, kv0, wk.bin, issue);
           s = kc % NV;
-          ok = mbar_wait_warp(bar_v_empty + 8 * s, ((kc / NV) & 1u) ^ 1u, wctx, kWaitVEmpty);
+          ok = mbar_wait_warp<kWaitVEmpty>(bar_v_empty + 8 * s, ((kc / NV) & 1u) ^ 1u, wctx);
           if (!ok) break;
           mbar_expect_tx(bar_v_full + 8 * s, Cfg::kKVBytes, issue);
           tma_load(s_v + s * Cfg::kKVBytes, &map_v, bar_v_full + 8 * s, wk.kv_head, kv0, wk.bin, issue);
@@ -847,7 +826,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       uint32_t it_n = 0;
       while (true) {
         const uint32_t ring = it_n % kRing;
-        if (!mbar_wait_warp(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull)) break;
+        if (!mbar_wait_warp<kWaitItemFull>(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx)) break;
         const volatile int* e = s_ring + ring * kRingInts;
         const int w = uniform(e[0]), bin = uniform(e[1]);
         const int q_row0 = uniform(e[4 + t]), head = uniform(e[9 + t]);
@@ -855,7 +834,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (issue) mbar_arrive(bar_item_empty + 8 * ring);
         if (w < 0) break;
         // the slot's last Q.K^T of the previous item must have finished reading the buffer
-        if (!mbar_wait_warp(bar_q_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitQEmpty)) break;
+        if (!mbar_wait_warp<kWaitQEmpty>(bar_q_empty + 8 * t, (it_n & 1u) ^ 1u, wctx)) break;
         if (used) {
           mbar_expect_tx(bar_q_full + 8 * t, Cfg::kQBytes, issue);
           tma_load(s_q + t * Cfg::kQBytes, &map_q, bar_q_full + 8 * t, head, q_row0, bin, issue);
@@ -878,7 +857,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       bool ok = true;
       auto wait_k = [&](const int j) -> bool {
         const uint32_t kc = kc0 + (uint32_t)j, s = kc % NK;
-        return mbar_wait_warp(bar_k_full + 8 * s, (kc / NK) & 1u, wctx, kWaitKFull);
+        return mbar_wait_warp<kWaitKFull>(bar_k_full + 8 * s, (kc / NK) & 1u, wctx);
       };
       // S_t = Q_t K_j^T (K_j has been waited for); the K stage is released after the last slot that reads it
       auto issue_qk = [&](const int t, const int j) {
@@ -905,11 +884,11 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (j >= jb && j < je) {
           const bool first = (j == jb);
           // the previous item's epilogue must have read O_t before it is overwritten
-          if (first && !mbar_wait_warp(bar_o_empty + 8 * t, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty)) return false;
+          if (first && !mbar_wait_warp<kWaitOEmpty>(bar_o_empty + 8 * t, (it_n & 1u) ^ 1u, wctx)) return false;
           const uint32_t vc = vc0 + (uint32_t)j, s = vc % NV;
-          if (!mbar_wait_warp(bar_v_full + 8 * s, (vc / NV) & 1u, wctx, kWaitVFull)) return false;
+          if (!mbar_wait_warp<kWaitVFull>(bar_v_full + 8 * s, (vc / NV) & 1u, wctx)) return false;
           if (j + 1 < je && !wait_k(j + 1)) return false;
-          if (!mbar_wait_warp(bar_p_full + 16 * t, tcount & 1u, wctx, kWaitP)) return false;
+          if (!mbar_wait_warp<kWaitP>(bar_p_full + 16 * t, tcount & 1u, wctx)) return false;
           tc_fence_after();
           const uint32_t a = tmem_base + Cfg::kTmemS + 128u * t;
           const uint32_t d = tmem_base + Cfg::kTmemO + (uint32_t)D * t;
@@ -932,15 +911,15 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       };
       while (ok) {
         const uint32_t ring = it_n % kRing;
-        if (!mbar_wait_warp(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull)) break;
+        if (!mbar_wait_warp<kWaitItemFull>(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx)) break;
         const volatile int* e = s_ring + ring * kRingInts;
         const int w = uniform(e[0]);
         n = uniform(e[3]); jb1 = uniform(e[6]); je0 = uniform(e[7]); je1 = uniform(e[8]);
         if (issue) mbar_arrive(bar_item_empty + 8 * ring);
         if (w < 0) break;
         const uint32_t bar_q_ready = args.rope_table ? bar_q_rot : bar_q_full;
-        ok = mbar_wait_warp(bar_q_ready + 0, it_n & 1u, wctx, kWaitQFull) &&
-             mbar_wait_warp(bar_q_ready + 8, it_n & 1u, wctx, kWaitQFull);
+        ok = mbar_wait_warp<kWaitQFull>(bar_q_ready + 0, it_n & 1u, wctx) &&
+             mbar_wait_warp<kWaitQFull>(bar_q_ready + 8, it_n & 1u, wctx);
         if (!ok) break;
         if (!(ok = wait_k(0))) break;                     // every item has a first tile
         if (je0 > 0) issue_qk(0, 0);
@@ -954,11 +933,11 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         // before every softmax thread has seen the first, so wait until all of them are past the
         // previous item's o_full (they signal that on o_empty).
         if (je0 <= 0) {
-          if (!(ok = mbar_wait_warp(bar_o_empty + 0, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
+          if (!(ok = mbar_wait_warp<kWaitOEmpty>(bar_o_empty + 0, (it_n & 1u) ^ 1u, wctx))) break;
           if (issue) { mbar_arrive(bar_q_empty + 0); mbar_arrive(bar_o_full + 0); }
         }
         if (jb1 >= je1) {
-          if (!(ok = mbar_wait_warp(bar_o_empty + 8, (it_n & 1u) ^ 1u, wctx, kWaitOEmpty))) break;
+          if (!(ok = mbar_wait_warp<kWaitOEmpty>(bar_o_empty + 8, (it_n & 1u) ^ 1u, wctx))) break;
           if (issue) { mbar_arrive(bar_q_empty + 8); mbar_arrive(bar_o_full + 8); }
         }
         kc0 += (uint32_t)n;
@@ -988,7 +967,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       bool ok = true;
       for (uint32_t it_n = 0; ok; ++it_n) {
         const uint32_t ring = (uint32_t)t * kRing + it_n % kRing;
-        if (!mbar_wait_warp(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull)) break;
+        if (!mbar_wait_warp<kWaitItemFull>(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx)) break;
         const volatile int* e = s_ring + ring * kRingInts;
         const int w = uniform(e[0]), kv_row0 = e[2], n = uniform(e[3]), q_row0 = e[4], kv_head = e[11];
         const int bin_used = e[12], seg_end = e[13], seg_first = e[16];
@@ -1011,7 +990,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           const int r0 = kv_row0 + j * BN;
           const int lo = max(r0, q_row0), hi = min(r0 + BN, own_end);
           const uint32_t st = kv_index_v(kc) % NS;
-          ok = mbar_wait_warp(bar_v_seen + 8 * (kc & 1u), (kc >> 1) & 1u, wctx, kWaitVFull);
+          ok = mbar_wait_warp<kWaitVFull>(bar_v_seen + 8 * (kc & 1u), (kc >> 1) & 1u, wctx);
           if (!ok) break;
           const uint32_t tile = s_kv + ((uint32_t)t * NS + st) * Cfg::kKVBytes + (uint32_t)(piece >> 3) * (BN * 128);
           __nv_bfloat16* cache = args.v_cache + 8 * piece;
@@ -1081,85 +1060,55 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         uint32_t it_n = 0, tcount = 0;
         while (true) {
           const uint32_t ring = ring0 + it_n % kRing;
-          ok = __all_sync(0xffffffffu, mbar_wait(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull));
+          ok = mbar_wait_warp<kWaitItemFull>(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx);
           if (!ok) break;
           const volatile int* e = s_ring + ring * kRingInts;
           const int w = e[0], item_kv_row0 = e[2], n_tiles = e[3];
           const int i_row = e[4] + (row >> fs), bin_used = e[12];
           mbar_arrive(bar_item_empty + 8 * ring);
           if (w < 0) break;
-          ok = mbar_wait_warp(bar_q_rot + 8 * (2 * t + (it_n & 1u)), (it_n >> 1) & 1u, wctx, kWaitQFull);
+          ok = mbar_wait_warp<kWaitQFull>(bar_q_rot + 8 * (2 * t + (it_n & 1u)), (it_n >> 1) & 1u, wctx);
           if (!ok) break;
           const int key_lo = __float_as_int(x_l[256 * (it_n & 1u)]);
           const int key_hi = i_row < bin_used ? i_row : 0;       // padding rows: key_lo = 1, an empty range
           float m_run = -INFINITY;      // running maximum of the row, in scaled log2 units
           float l_run = 0.f;            // running sum of exp2(s * c - m_run)
           for (int j = 0; j < n_tiles; ++j) {
-            constexpr int EPT = BN;                              // scores per thread and tile
-            constexpr int NCH = EPT / 32;                        // 32-column TMEM round trips
+            static_assert(BN == 64, "a row's scores of a tile are one 64-bit mask");
             const int kv0 = item_kv_row0 + j * BN;
             const int c_lo = max(key_lo - kv0, 0);
-            const int c_hi = min(key_hi - kv0, EPT - 1);         // visible columns [c_lo, c_hi]
-            // one warp reduction for all the per-warp flags of the tile: which 32-column chunks
-            // somebody can see, and whether any row's interval ends or begins inside the tile
-            static_assert(NCH == 2, "flag bits below are laid out for two chunks");
+            const int c_hi = min(key_hi - kv0, BN - 1);          // visible columns [c_lo, c_hi]
             const uint64_t vis = visible_mask64(c_lo, c_hi);     // bit i: column i is visible to this row
-            const uint32_t vis_lo = (uint32_t)vis, vis_hi = (uint32_t)(vis >> 32);
-            const uint32_t lane_flags = (uint32_t)(vis_lo != 0u) | ((uint32_t)(vis_hi != 0u) << 1) |
-                                        ((uint32_t)(~vis != 0ull) << 2);
-            const uint32_t warp_flags = __reduce_or_sync(0xffffffffu, lane_flags);
-            const bool need[NCH] = {(warp_flags & 1u) != 0, (warp_flags & 2u) != 0};
-            const bool cut = (warp_flags & 4u) != 0;
+            const bool cut = __any_sync(0xffffffffu, ~vis != 0ull);   // some row's interval ends or begins inside the tile
             const uint32_t sbuf = tcount & 1u;                   // tile k of the stream lives in S buffer k & 1
             const uint32_t tmem_sb = tmem_s + 64u * sbuf;
-            ok = mbar_wait_warp(bar_s_full + 8 * (2 * t + sbuf), (tcount >> 1) & 1u, wctx, kWaitS);
+            ok = mbar_wait_warp<kWaitS>(bar_s_full + 8 * (2 * t + sbuf), (tcount >> 1) & 1u, wctx);
             if (!ok) break;
             tc_fence_after();
-            uint32_t v[EPT];
+            // Both halves of the tile, also one that no row of the warp can see: leaving it out costs more in code than
+            // it saves (64 prompts on a 7B layer 239 -> 236 us a step).
+            uint32_t v[BN];
 #pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) {
-              if (need[ch]) {
-                tmem_ld32(tmem_sb + 32 * ch, *reinterpret_cast<uint32_t(*)[32]>(&v[32 * ch]));
-              } else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) v[32 * ch + i] = 0xff800000u;        // -inf
-              }
-            }
+            for (int ch = 0; ch < BN / 32; ++ch) tmem_ld32(tmem_sb + 32 * ch, *reinterpret_cast<uint32_t(*)[32]>(&v[32 * ch]));
             tc_wait_ld();
             // masked tiles (the causal diagonal, the first tile of a prompt): one select per score,
             // steered by the bits of the row's visibility mask
             if (cut) {
+              const uint32_t vis_lo = (uint32_t)vis, vis_hi = (uint32_t)(vis >> 32);
 #pragma unroll
               for (int i = 0; i < 32; ++i) v[i] = (vis_lo & (1u << i)) ? v[i] : 0xff800000u;
 #pragma unroll
               for (int i = 0; i < 32; ++i) v[32 + i] = (vis_hi & (1u << i)) ? v[32 + i] : 0xff800000u;
             }
-            float mx;
-            {
-              float m0 = fmax3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
-              float m1 = fmax3(__uint_as_float(v[3]), __uint_as_float(v[4]), __uint_as_float(v[5]));
-              float m2 = fmax3(__uint_as_float(v[6]), __uint_as_float(v[7]), __uint_as_float(v[8]));
-              float m3 = fmax3(__uint_as_float(v[9]), __uint_as_float(v[10]), __uint_as_float(v[11]));
-#pragma unroll
-              for (int i = 12; i + 7 < EPT; i += 8) {
-                m0 = fmax3(m0, __uint_as_float(v[i]), __uint_as_float(v[i + 1]));
-                m1 = fmax3(m1, __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
-                m2 = fmax3(m2, __uint_as_float(v[i + 4]), __uint_as_float(v[i + 5]));
-                m3 = fmax3(m3, __uint_as_float(v[i + 6]), __uint_as_float(v[i + 7]));
-              }
-              m0 = fmax3(m0, __uint_as_float(v[EPT - 4]), __uint_as_float(v[EPT - 3]));
-              m1 = fmax3(m1, __uint_as_float(v[EPT - 2]), __uint_as_float(v[EPT - 1]));
-              mx = fmaxf(fmax3(m0, m1, m2), m3);
-            }
             // lazy running-maximum update: keep the stale maximum while the new one is < 2^8 above it
-            const float m_tile = mx * c_scale;
+            const float m_tile = max64(v) * c_scale;
             float m_new = m_run;
             if (m_tile > m_run + 8.f) m_new = m_tile;
             const bool rescale = (m_new != m_run) && (m_run != -INFINITY);
             const float alpha = rescale ? fast_exp2(m_run - m_new) : 1.f;
             if (j > 0 && __any_sync(0xffffffffu, rescale)) {
               // S(k) is computed ahead of P(k-1) V(k-1): O_t is stable only once that product is there
-              ok = mbar_wait_warp(bar_pv_done + 8 * t, (tcount - 1u) & 1u, wctx, kWaitVEmpty);
+              ok = mbar_wait_warp<kWaitVEmpty>(bar_pv_done + 8 * t, (tcount - 1u) & 1u, wctx);
               if (!ok) break;
               tc_fence_after();
 #pragma unroll 1
@@ -1180,31 +1129,12 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const uint64_t negm2 = pack_f2(__float_as_uint(neg_m), __float_as_uint(neg_m));
             uint64_t sum_a = 0ull, sum_b = 0ull;
 #pragma unroll
-            for (int ch = 0; ch < NCH; ++ch) {
+            for (int ch = 0; ch < BN / 32; ++ch) {
               uint32_t pk[16];
-              if (need[ch]) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 4) {
-                  float p0, p1, p2, p3;
-                  unpack_f2(fma_f2(pack_f2(v[ch * 32 + i], v[ch * 32 + i + 1]), c2, negm2), p0, p1);
-                  unpack_f2(fma_f2(pack_f2(v[ch * 32 + i + 2], v[ch * 32 + i + 3]), c2, negm2), p2, p3);
-                  p0 = fast_exp2(p0); p1 = fast_exp2(p1); p2 = fast_exp2(p2); p3 = fast_exp2(p3);
-                  sum_a = add_f2(sum_a, pack_f2(__float_as_uint(p0), __float_as_uint(p1)));
-                  sum_b = add_f2(sum_b, pack_f2(__float_as_uint(p2), __float_as_uint(p3)));
-                  pk[i >> 1] = pack_bf16(p0, p1);
-                  pk[(i >> 1) + 1] = pack_bf16(p2, p3);
-                }
-              } else {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) pk[i] = 0u;
-              }
-              // S(k) was read completely above, so P(k) may overwrite its first columns
-              tmem_st16(tmem_sb + ch * 16, pk);
+              exp_chunk(&v[32 * ch], c2, negm2, sum_a, sum_b, pk);
+              tmem_st16(tmem_sb + ch * 16, pk);              // S(k) was read completely above
             }
-            float sum0, sum1, sum2, sum3;
-            unpack_f2(sum_a, sum0, sum1);
-            unpack_f2(sum_b, sum2, sum3);
-            l_run += (sum0 + sum2) + (sum1 + sum3);
+            l_run += sum_f2x2(sum_a, sum_b);
             tc_wait_st();
             tc_fence_before();
             mbar_arrive(bar_p_full + 8 * (2 * t + sbuf));
@@ -1225,7 +1155,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         int p_q_row0 = 0, p_head = 0, p_bin = 0;         // coordinates of the previous item (its epilogue is due)
         while (true) {
           const uint32_t ring = ring0 + it_n % kRing;
-          ok = __all_sync(0xffffffffu, mbar_wait(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull));
+          ok = mbar_wait_warp<kWaitItemFull>(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx);
           if (!ok) break;
           const volatile int* e = s_ring + ring * kRingInts;
           const int w = e[0], c_bin = e[1], c_q_row0 = e[4], c_head = e[9];
@@ -1243,7 +1173,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             // the same fp32 arithmetic and rounding as the stand-alone kernel, leave the row's first key
             // where its row sum will be (this thread has read that of the item before the previous one
             // from there), then report Q_t ready
-            ok = mbar_wait_warp(bar_q_full + 8 * qb, (it_n >> 1) & 1u, wctx, kWaitQFull);
+            ok = mbar_wait_warp<kWaitQFull>(bar_q_full + 8 * qb, (it_n >> 1) & 1u, wctx);
             if (!ok) break;
             const int pos = key_hi - key_lo;             // < 0 for padding rows
             if (args.rope_table && pos > 0) {
@@ -1290,9 +1220,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           if (it_n > 0) {
             // epilogue of the previous item: O_t / l -> bf16 -> shared memory (128-byte swizzle) -> TMA store
             const uint32_t pi = it_n - 1u;
-            ok = mbar_wait_warp(bar_o_full + 8 * t, pi & 1u, wctx, kWaitOFull);
+            ok = mbar_wait_warp<kWaitOFull>(bar_o_full + 8 * t, pi & 1u, wctx);
             if (!ok) break;
-            ok = mbar_wait_warp(bar_l_ready + 16 * t + 8 * (pi & 1u), (pi >> 1) & 1u, wctx, kWaitRowSum);
+            ok = mbar_wait_warp<kWaitRowSum>(bar_l_ready + 16 * t + 8 * (pi & 1u), (pi >> 1) & 1u, wctx);
             if (!ok) break;
             tc_fence_after();
             const float l_row = x_l[256 * (pi & 1u)];
@@ -1351,9 +1281,9 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // that a warp whose partner gave up on a wait cannot be left waiting for it.
     const uint32_t bar_pair = bar_pair0 + 8 * (uint32_t)(t * 4 + quad);
     uint32_t pair_ph = 0;
-    auto rendezvous = [&](const uint32_t bar, uint32_t& ph, const int code) -> bool {
+    auto rendezvous = [&](const uint32_t bar, uint32_t& ph) -> bool {
       mbar_arrive(bar);
-      const bool r = __all_sync(0xffffffffu, mbar_wait(bar, ph, wctx, code));
+      const bool r = __all_sync(0xffffffffu, mbar_wait<kWaitPair>(bar, ph, wctx));
       ph ^= 1u;
       return r;
     };
@@ -1370,7 +1300,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     volatile uint8_t* const bounded_mine = s_bounded + (t * 4 + quad) * 2 + h;
     volatile uint8_t* const bounded_other = s_bounded + (t * 4 + quad) * 2 + (h ^ 1);
     auto rotate_q = [&](const int pos, const float limit, const uint32_t parity) -> bool {
-      if (!__all_sync(0xffffffffu, mbar_wait(bar_q_full + 8 * t, parity, wctx, kWaitQFull))) return false;
+      if (!__all_sync(0xffffffffu, mbar_wait<kWaitQFull>(bar_q_full + 8 * t, parity, wctx))) return false;
       uint64_t n2a = 0ull, n2b = 0ull;
       if (pos >= 0) {
         constexpr int kUnits = D / 16;                 // 16-byte units per half of a row
@@ -1418,7 +1348,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     };
     while (true) {
       const uint32_t ring = it_n % kRing;              // both slots read the one ring, each its own fields of an entry
-      ok = __all_sync(0xffffffffu, mbar_wait(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx, kWaitItemFull));
+      ok = mbar_wait_warp<kWaitItemFull>(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx);
       if (!ok) break;
       const volatile int* e = s_ring + ring * kRingInts;
       const int w = e[0];
@@ -1473,7 +1403,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (fast && j >= clean_jb && j < clean_je) {
           // The common tile: nothing to mask, no maximum to find. The scores of the second chunk are
           // loaded while the exponentials of the first are computed.
-          ok = mbar_wait_warp(bar_s_full + 16 * t, tcount & 1u, wctx, kWaitS);
+          ok = mbar_wait_warp<kWaitS>(bar_s_full + 16 * t, tcount & 1u, wctx);
           if (!ok) break;                                    // warp-uniform
           tc_fence_after();
           const uint64_t negm2 = pack_f2(__float_as_uint(neg_m), __float_as_uint(neg_m));
@@ -1505,7 +1435,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         const uint32_t warp_flags = __reduce_or_sync(0xffffffffu, lane_flags);
         const bool need[NCH] = {(warp_flags & 1u) != 0, (warp_flags & 2u) != 0};
         const bool cut = (warp_flags & 4u) != 0;
-        ok = mbar_wait_warp(bar_s_full + 16 * t, tcount & 1u, wctx, kWaitS);
+        ok = mbar_wait_warp<kWaitS>(bar_s_full + 16 * t, tcount & 1u, wctx);
         if (!ok) break;                                      // warp-uniform
         tc_fence_after();
         uint32_t v[EPT];
@@ -1532,7 +1462,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           // have announced their P of this tile.)
           float mx = max64(v);
           *x_mine = mx;
-          if (!(ok = rendezvous(bar_pair, pair_ph, kWaitPair))) break;
+          if (!(ok = rendezvous(bar_pair, pair_ph))) break;
           mx = fmaxf(mx, *x_other);
           if (j == jb_t && args.rope_table) bounded = (*bounded_mine & *bounded_other) != 0;
           const float m_tile = mx * c_scale;
@@ -1583,15 +1513,15 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       const float l_run = sum_f2x2(sum_a, sum_b);
 
       // epilogue: O_t / l -> bf16 -> shared memory (128-byte swizzle) -> TMA store
-      ok = __all_sync(0xffffffffu, mbar_wait(bar_o_full + 8 * t, it_n & 1u, wctx, kWaitOFull));
+      ok = __all_sync(0xffffffffu, mbar_wait<kWaitOFull>(bar_o_full + 8 * t, it_n & 1u, wctx));
       if (!ok) break;
       if (used) {
         // the half-1 threads hand their share of the row sum to the half-0 threads, which run the
         // epilogue; the second barrier keeps the exchange slot from being reused too early
         if (h == 1) *x_mine = l_run;
-        if (!(ok = rendezvous(bar_pair, pair_ph, kWaitPair))) break;
+        if (!(ok = rendezvous(bar_pair, pair_ph))) break;
         const float l_row = (h == 0) ? l_run + *x_other : 0.f;
-        if (!(ok = rendezvous(bar_pair, pair_ph, kWaitPair))) break;
+        if (!(ok = rendezvous(bar_pair, pair_ph))) break;
         if (h == 1) mbar_arrive(bar_o_empty + 8 * t);      // this thread is past o_full and never reads O_t
         if (h == 0) {
           tc_fence_after();
@@ -1669,7 +1599,7 @@ __global__ void bounded_wait_selftest_kernel(int32_t* status, unsigned long long
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  if (threadIdx.x == 0) mbar_wait(smem_u32(&bar), 0, wctx, 77);
+  if (threadIdx.x == 0) mbar_wait<77>(smem_u32(&bar), 0, wctx);
   __syncthreads();
   if (threadIdx.x == 0 && abort_flag) atomicCAS(status, 0, abort_flag);
 }
