@@ -4,7 +4,7 @@
 // row carries the key range [start row of its prompt, its own row], and the host work list
 // restricts each query tile to the key tiles that can intersect such a range.
 //
-// Persistent kernel, one CTA per SM, 640 threads (768 with kFill), two 128-row query-tile slots per CTA. CTAs draw
+// Persistent kernel, one CTA per SM, 640 threads (768 in the independent mode), two 128-row query-tile slots per CTA. CTAs draw
 // work from a global counter (items are listed KV-head-major, longest first). Two modes, chosen on
 // the host from the mean number of key tiles per query tile:
 //
@@ -26,13 +26,14 @@
 // group), loaded and stored as one TMA box over (row, head). One stream of key tiles then serves
 // the f heads, a short prompt fills a tile with heads instead of empty rows, and an item's key
 // tiles start at the first row of the first prompt it touches rather than at a tile boundary.
-//   warps 0-1    issue the tcgen05.mma of slot 0 / slot 1
+//   warps 0-1    issue the tcgen05.mma of the scores of slot 0 / slot 1
 //   warps 2-3    draw items and TMA-load Q (two tiles: the next item's is there early), K, V of slot 0 / slot 1
 //   warps 4-7    softmax threads of slot 0, one per query row; they never leave the tile loop
 //   warps 8-11   helper threads of slot 0, one per row: find the first key of each row of the next item,
 //                rotate its Q in shared memory (fused path) and run the previous item's epilogue
 //   warps 12-19  the same for slot 1
 //   warps 20-21  (kFill) write the V rows of the slots' own query tiles from shared memory to the caches
+//   warps 22-23  issue the tcgen05.mma of the products P V of slot 0 / slot 1
 // Softmax: tcgen05.ld the thread's scores, mask to the row's key range, lazy running maximum (O is
 // rescaled only when the maximum grows by more than 2^8, or 2^90 in the shared-stream mode, where rows
 // whose scores are bounded drop the maximum altogether), exp2, P written as bf16 over the S
@@ -58,16 +59,14 @@ namespace {
 
 constexpr int BM = kTileM;
 constexpr int kAttnThreads = 640;
-constexpr int kAttnThreadsFill = 768;      // one warpgroup more, two of its warps fill the V caches
+constexpr int kAttnThreadsIndep = 768;     // independent mode: one warpgroup more
 constexpr int kSoftmaxThreads = 256;       // per slot: two threads per query row
 constexpr uint32_t kTmemCols = 512;
-constexpr int kRegsSoftmax = 104;          // setmaxnreg budgets: 640 threads start with 96 registers each;
-constexpr int kRegsSoftmaxIndep = 120;     // independent mode: 256 softmax threads at 120, 256 helper threads at 88
-constexpr int kRegsHelper = 88;
-constexpr int kRegsOther = 64;              // warps 0-3 give back 32 each, the 512 softmax threads take 8 each
-constexpr int kRegsSoftmaxFill = 112;      // with cache writers: 768 threads start with 80 registers each; the 256 softmax
-constexpr int kRegsOtherFill = 56;         //   threads take 32 each from warps 0-3 (24 each) and the cache writers'
-constexpr int kRegsWriter = 40;            //   warpgroup (40 each); the 256 helper threads keep their 80
+constexpr int kRegsSoftmax = 104;          // setmaxnreg budgets, shared-stream mode: 640 threads start with 96 registers
+constexpr int kRegsOther = 64;             //   each; warps 0-3 give back 32 each, the 512 softmax threads take 8 each
+constexpr int kRegsSoftmaxIndep = 112;     // independent mode: 768 threads start with 80 each; the 256 softmax threads take
+constexpr int kRegsOtherIndep = 56;        //   32 each from warps 0-3 (24 each) and 20-23 (40 each); the 256 helper
+constexpr int kRegsLast = 40;              //   threads keep their 80
 // Shared-stream mode, when a row needs no maximum any more. Its running maximum is lazy: it stays at the
 // maximum of the row's first visible tile until a score exceeds it by more than kLazyLog2 (log2 units).
 // Probabilities, sums and O have 8 exponent bits, so a common factor of up to 2^90 costs no precision, and
@@ -500,7 +499,7 @@ __device__ __forceinline__ uint32_t kv_index_v(uint32_t k) { return 2u * k + 2u;
 //   pairing two row tiles of different length would leave one slot idle for a tile per item).
 // kFill (independent mode): two more warps write the V rows to the caches.
 template <int D, bool kIndep, bool kFill, class Table>
-__global__ void __launch_bounds__(kFill ? kAttnThreadsFill : kAttnThreads, 1)
+__global__ void __launch_bounds__(kIndep ? kAttnThreadsIndep : kAttnThreads, 1)
 attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                  const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
                  const __grid_constant__ AttnArgs args, const __grid_constant__ Table tab) {
@@ -531,19 +530,18 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   const uint32_t bar_q_empty = s_misc + (kIndep ? 128 : 144);   // [2]; independent mode: [2 slots][2 Q tiles]
   const uint32_t bar_s_full = s_misc + 160;      // [2 slots][2 S buffers]; shared mode uses [t][0]
   const uint32_t bar_p_full = s_misc + 192;      // [2 slots][2 S buffers]
-  const uint32_t bar_o_full = s_misc + 224;      // [2]
-  const uint32_t bar_o_empty = s_misc + 240;     // [2]
+  const uint32_t bar_o_full = s_misc + (kIndep ? 384 : 224);    // [2]
+  const uint32_t bar_o_empty = s_misc + (kIndep ? 224 : 240);   // [2]; independent mode: [2 slots][item & 1]
   const uint32_t bar_k_full = s_misc + 256;      // [4]
   const uint32_t bar_k_empty = s_misc + 288;     // [4]
-  const uint32_t bar_v_full = s_misc + 320;      // [4]
+  const uint32_t bar_v_full = s_misc + (kIndep ? 288 : 320);    // [4]; independent mode: bar_k_full, bar_v_full [2 slots][k & 1]
   const uint32_t bar_v_empty = s_misc + 352;     // [4]
-  const uint32_t bar_kv_full = s_misc + 256;     // independent mode, in their place: [2 slots][4 stages]
-  const uint32_t bar_kv_empty = s_misc + 320;    // [2 slots][4 stages]
+  const uint32_t bar_pv_done = s_misc + 320;     // [2 slots][2] independent mode: P(k) V(k) has been computed ([k & 1])
+  const uint32_t bar_v_read = s_misc + 352;      // [2 slots][2] and the rows of V(k) have been read for the caches
   const uint32_t bar_q_rot = s_misc + (kIndep ? 928 : 384);     // [2] Q_t has been rotated in place (fused path);
                                                  // independent mode: [2 slots][2 Q tiles], its rows' first keys are there too
-  const uint32_t bar_pv_done = s_misc + 384;     // [2] independent mode: P(k) V(k) has been computed
   const uint32_t bar_pair0 = s_misc + 896;       // [2 slots][4 quadrants] shared-stream mode: rendezvous of the two warps that share rows
-  const uint32_t bar_v_seen0 = s_misc + 960, bar_v_seen1 = s_misc + 1008;   // [2] each, independent mode: the slot's MMA warp has seen V(k)
+  const uint32_t bar_v_seen0 = s_misc + 960, bar_v_seen1 = s_misc + 1008;   // [2] each, independent mode: V(k) is there, said the slot's warp 22 / 23
   const uint32_t bar_l_ready = s_misc + 976;     // [2][2] independent mode: the slot's row sums of item i are in shared memory ([slot][i & 1])
   uint32_t* s_tmem_base = reinterpret_cast<uint32_t*>(misc + 400);
   volatile int* s_abort = reinterpret_cast<volatile int*>(misc + 404);
@@ -560,10 +558,10 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2 * (int)kRing; ++i) {
       mbar_init(bar_item_full + 8 * i, 1);
-      // readers of a ring entry: the MMA thread and the softmax threads of the slot(s) it feeds;
+      // readers of a ring entry: the MMA warp(s) and the softmax threads of the slot(s) it feeds;
       // in shared mode also the two Q loaders
       // (and in independent mode the slot's cache writer, where caches are filled)
-      mbar_init(bar_item_empty + 8 * i, kIndep ? 1 + kSoftmaxThreads + (kFill ? 1 : 0) : 1 + 2 + 2 * kSoftmaxThreads);
+      mbar_init(bar_item_empty + 8 * i, kIndep ? 2 + kSoftmaxThreads + (kFill ? 1 : 0) : 1 + 2 + 2 * kSoftmaxThreads);
     }
     for (int i = 0; i < 2; ++i) {
       for (int b = 0; b < 2; ++b) {
@@ -573,6 +571,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
       mbar_init(bar_o_full + 8 * i, 1);
       mbar_init(bar_o_empty + 8 * i, kIndep ? kSoftmaxThreads / 2 : kSoftmaxThreads);
+      if (kIndep) mbar_init(bar_o_empty + 16 + 8 * i, kSoftmaxThreads / 2);
     }
     if constexpr (kIndep) {
       for (int i = 0; i < 4; ++i) {
@@ -580,9 +579,13 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         mbar_init(bar_q_empty + 8 * i, Cfg::kStageInQ ? 4 : 1);   // one lane of each helper warp, or a commit
         mbar_init(bar_q_rot + 8 * i, kSoftmaxThreads / 2);
       }
-      // a stage is free when its product has been computed and, where caches are filled, its rows have been read
-      for (int i = 0; i < 8; ++i) { mbar_init(bar_kv_full + 8 * i, 1); mbar_init(bar_kv_empty + 8 * i, kFill ? 2 : 1); }
-      for (int i = 0; i < 2; ++i) { mbar_init(bar_pv_done + 8 * i, 1); if (kFill) { mbar_init(bar_v_seen0 + 8 * i, 1); mbar_init(bar_v_seen1 + 8 * i, 1); } }
+      for (int i = 0; i < 4; ++i) {
+        mbar_init(bar_k_full + 8 * i, 1);
+        mbar_init(bar_v_full + 8 * i, 1);
+        mbar_init(bar_pv_done + 8 * i, 1);
+        mbar_init(bar_v_read + 8 * i, 1);
+      }
+      for (int i = 0; i < 2; ++i) if (kFill) { mbar_init(bar_v_seen0 + 8 * i, 1); mbar_init(bar_v_seen1 + 8 * i, 1); }
     } else {
       for (int i = 0; i < 2; ++i) {
         mbar_init(bar_q_full + 8 * i, 1);
@@ -615,7 +618,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
   if (Table::kUploaded) pdl_launch_dependents();
 
   if (warp < 4) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kFill ? kRegsOtherFill : kRegsOther));
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kIndep ? kRegsOtherIndep : kRegsOther));
     if constexpr (kIndep) {
       if (warp >= 2) {
         // -------------------------------------------------------------- producer of slot t:
@@ -650,11 +653,34 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           tma_load(s_q + qb * Cfg::kQBytes, &map_q, bar_q_full + 8 * qb, wk.head[0], wk.q_row0[0], wk.bin, issue);
           return true;
         };
-        auto load_kv = [&](const CUtensorMap* map, const uint32_t idx, const int head, const int row, const int bin) -> bool {
-          const uint32_t st = idx % NS, bar = 8 * (4u * (uint32_t)t + st);
-          if (!mbar_wait_warp<kWaitKEmpty>(bar_kv_empty + bar, ((idx / NS) & 1u) ^ 1u, wctx)) return false;
-          mbar_expect_tx(bar_kv_full + bar, Cfg::kKVBytes, issue);
-          tma_load(s_kv + ((uint32_t)t * NS + st) * Cfg::kKVBytes, map, bar_kv_full + bar, head, row, bin, issue);
+        // A stage is free when what it held has been used: K(k) when S(k) is there, V(k) when P(k) V(k) is, and, where
+        // caches are filled, its rows have been read. These are barriers that others wait on anyway: a commit
+        // of its own behind each group of MMAs takes the issuing warp ~140 cycles. None can complete the next phase
+        // before this warp has seen the one it waits for: that takes K(k) where K(k) waits (S(k), or P(k - 1) V(k - 1), whose
+        // V comes after it), V(k) or K(k + 2) where V(k) waits.
+        static_assert(NS == 3 || NS == 4, "which tile a stage held is worked out for these");
+        auto wait_s = [&](const uint32_t k) -> bool {
+          return mbar_wait_warp<kWaitKEmpty>(bar_s_full + 8 * (2u * (uint32_t)t + (k & 1u)), (k >> 1) & 1u, wctx);
+        };
+        auto wait_pv = [&](const uint32_t k) -> bool {
+          const uint32_t bar = 8 * (2u * (uint32_t)t + (k & 1u));
+          return mbar_wait_warp<kWaitVEmpty>(bar_pv_done + bar, (k >> 1) & 1u, wctx) &&
+                 (!kFill || mbar_wait_warp<kWaitVEmpty>(bar_v_read + bar, (k >> 1) & 1u, wctx));
+        };
+        auto load_kv = [&](const CUtensorMap* map, const uint32_t idx, const uint32_t bar, const int head, const int row, const int bin) {
+          mbar_expect_tx(bar, Cfg::kKVBytes, issue);
+          tma_load(s_kv + ((uint32_t)t * NS + idx % NS) * Cfg::kKVBytes, map, bar, head, row, bin, issue);
+        };
+        // K(k): of four stages, after K(k - 2), whose barrier this is again too; of three, after V(k - 3), or K(0) where k = 2
+        auto load_k = [&](const uint32_t k, const int head, const int row, const int bin) -> bool {
+          if (NS == 4 ? k >= 2u && !wait_s(k - 2u) : k >= 3u ? !wait_pv(k - 3u) : k == 2u && !wait_s(0u)) return false;
+          load_kv(&map_k, kv_index_k(k), bar_k_full + 8 * (2u * (uint32_t)t + (k & 1u)), head, row, bin);
+          return true;
+        };
+        // V(k): of four stages, after V(k - 2), or K(0) where k = 1 (S(1) comes after S(0)); of three, after K(k)
+        auto load_v = [&](const uint32_t k, const int head, const int row, const int bin) -> bool {
+          if (NS == 4 ? (k >= 2u ? !wait_pv(k - 2u) : k == 1u && !wait_s(1u)) : k >= 1u && !wait_s(k)) return false;
+          load_kv(&map_v, kv_index_v(k), bar_v_full + 8 * (2u * (uint32_t)t + (k & 1u)), head, row, bin);
           return true;
         };
         const int drawers = 2 * (int)gridDim.x;
@@ -662,7 +688,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         if (w >= args.total_work) w = -1;
         Work wk, wk_next;
         bool ok = announce(0, w, wk);
-        if (ok && w >= 0) ok = load_q(0, wk) && load_kv(&map_k, kv_index_k(0), wk.kv_head, wk.kv_row0, wk.bin);
+        if (ok && w >= 0) ok = load_q(0, wk) && load_k(0u, wk.kv_head, wk.kv_row0, wk.bin);
         uint32_t kc = 0;                      // key tiles of the slot's stream whose V has been loaded
         for (uint32_t it_n = 0; ok && w >= 0; ++it_n) {
           const int w_next = draw_work(args, lane, drawers);
@@ -670,118 +696,58 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           for (int j = 0; ok && j < wk.n; ++j, ++kc) {
             const bool here = j + 1 < wk.n;             // K of this item, or the first of the next
             if (here || w_next >= 0)
-              ok = load_kv(&map_k, kv_index_k(kc + 1), here ? wk.kv_head : wk_next.kv_head,
-                           here ? wk.kv_row0 + (j + 1) * BN : wk_next.kv_row0, here ? wk.bin : wk_next.bin);
-            if (ok) ok = load_kv(&map_v, kv_index_v(kc), wk.kv_head, wk.kv_row0 + j * BN, wk.bin);
+              ok = load_k(kc + 1u, here ? wk.kv_head : wk_next.kv_head, here ? wk.kv_row0 + (j + 1) * BN : wk_next.kv_row0,
+                          here ? wk.bin : wk_next.bin);
+            if (ok) ok = load_v(kc, wk.kv_head, wk.kv_row0 + j * BN, wk.bin);
             if (ok && j == min(1, wk.n - 1) && w_next >= 0) ok = load_q(it_n + 1u, wk_next);
           }
           w = w_next;
           wk = wk_next;
         }
       } else if (warp < 2) {
-        // -------------------------------------------------------------- MMA issuer of slot t
-        // One issuing warp per slot (warps 0 and 1 sit on different schedulers), plain blocking
-        // waits. S_t has two 64-column buffers, tile k of the slot's stream uses buffer k & 1, and
-        // P(k) is written over S(k). The issue order  S(k+1), then P(k) V(k)  lets the tensor pipe
-        // compute the next scores while the softmax threads work on tile k, and P(k) V(k) while they
-        // work on tile k+1; the pipe runs one thread's MMAs in order, so S(k+2) cannot overwrite
-        // P(k) before P(k) V(k) has read it.
+        // -------------------------------------------------------------- scores of slot t: S(k) = Q K(k)^T
+        // The slot's tiles form one stream across items; tile k uses S buffer k & 1. S(k) is issued as soon as its
+        // K tile is there and P(k - 2) V(k - 2), which reads the same buffer, is done: while the softmax
+        // threads work on tile k - 1, also when tile k opens the slot's next item (its Q has been loaded and rotated
+        // under this one). The products P V have a warp of their own (22, 23): one warp that issued both took 1400 cycles
+        // of its own per tile, besides the ~1200 it waited (2048 short prompts on 32 / 8 heads of 64 174 -> 167 us a step, 64
+        // prompts on a 7B layer 237.3 -> 235.6, 34 bins of a stream 896 -> 889).
         const int t = warp;
         const uint32_t issue = elect_one();
         constexpr uint32_t idesc_qk = instr_desc(BN, false);
-        constexpr uint32_t idesc_pv = instr_desc(D, true);
         constexpr int NS = Cfg::kKVStages;
         const uint32_t q_lo = desc_lo(s_q, 0) + 2u * (uint32_t)t * (Cfg::kQBytes >> 4);
         const uint32_t k_lo = desc_lo(s_kv, 0) + (uint32_t)(t * NS) * (Cfg::kKVBytes >> 4);
-        const uint32_t v_lo = desc_lo(s_kv, BN * 128) + (uint32_t)(t * NS) * (Cfg::kKVBytes >> 4);
         const uint32_t tm_s = tmem_base + Cfg::kTmemS + 128u * (uint32_t)t;
-        const uint32_t tm_o = tmem_base + Cfg::kTmemO + (uint32_t)D * (uint32_t)t;
-        const uint32_t b_q_ready = bar_q_rot + 16 * t;         // [Q tile]
-        const uint32_t b_item_full = bar_item_full + 8 * (uint32_t)t * kRing;
-        const uint32_t b_item_empty = bar_item_empty + 8 * (uint32_t)t * kRing;
-        const uint32_t b_kv_full = bar_kv_full + 32 * t, b_kv_empty = bar_kv_empty + 32 * t;   // [stage]
-        const uint32_t b_s_full = bar_s_full + 16 * t, b_p_full = bar_p_full + 16 * t;     // [buffer]
-        const uint32_t b_o_full = bar_o_full + 8 * t, b_o_empty = bar_o_empty + 8 * t;
-        uint32_t it_n = 0, kc = 0;       // items and key tiles consumed
+        uint32_t kc = 0;
         bool ok = true;
-        // S(kq) = Q_t K(kq)^T into buffer kq & 1, for the slot's item `item`
-        auto issue_qk = [&](const uint32_t kq, const uint32_t item, const bool last_of_item) -> bool {
-          const uint32_t idx = kv_index_k(kq), st = idx % NS;
-          if (!mbar_wait_warp<kWaitKFull>(b_kv_full + 8 * st, (idx / NS) & 1u, wctx)) return false;
-          tc_fence_after();
-          const uint32_t d = tm_s + 64u * (kq & 1u);
-          const uint32_t a_lo = q_lo + (item & 1u) * (Cfg::kQBytes >> 4);
-          const uint32_t kb = k_lo + st * (Cfg::kKVBytes >> 4);
+        for (uint32_t it_n = 0; ok; ++it_n) {
+          const uint32_t ring = (uint32_t)t * kRing + it_n % kRing, it2 = 2u * (uint32_t)t + (it_n & 1u);
+          if (!mbar_wait_warp<kWaitItemFull>(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx)) break;
+          const volatile int* e = s_ring + ring * kRingInts;
+          const int w = uniform(e[0]), n = uniform(e[3]);
+          if (issue) mbar_arrive(bar_item_empty + 8 * ring);
+          if (w < 0) break;
+          // The epilogue of the item before the previous one has read O_t, and the row sums: the softmax threads must not
+          // get further ahead of it, also where every item is one tile.
+          if (it_n >= 2u && !mbar_wait_warp<kWaitOEmpty>(bar_o_empty + 8 * it2, ((it_n - 2u) >> 1) & 1u, wctx)) break;
+          if (!mbar_wait_warp<kWaitQFull>(bar_q_rot + 8 * it2, (it_n >> 1) & 1u, wctx)) break;
+          const uint32_t a_lo = q_lo + (it_n & 1u) * (Cfg::kQBytes >> 4);
+          for (int j = 0; j < n; ++j, ++kc) {
+            const uint32_t st = kv_index_k(kc) % NS, buf = 2u * (uint32_t)t + (kc & 1u);
+            if (kc >= 2u && !(ok = mbar_wait_warp<kWaitVEmpty>(bar_pv_done + 8 * buf, ((kc - 2u) >> 1) & 1u, wctx))) break;
+            if (!(ok = mbar_wait_warp<kWaitKFull>(bar_k_full + 8 * buf, (kc >> 1) & 1u, wctx))) break;
+            tc_fence_after();
+            const uint32_t d = tm_s + 64u * (kc & 1u);
+            const uint32_t kb = k_lo + st * (Cfg::kKVBytes >> 4);
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            constexpr uint32_t kChunkQ = (BM * 128) >> 4, kChunkK = (BN * 128) >> 4;
-            mma_ss(d, a_lo + (uint32_t)(kk >> 2) * kChunkQ + (uint32_t)(kk & 3) * 2,
-                   kb + (uint32_t)(kk >> 2) * kChunkK + (uint32_t)(kk & 3) * 2, idesc_qk, kk > 0 ? 1u : 0u, issue);
-          }
-          tc_commit(b_kv_empty + 8 * st, issue);
-          if (kFill && issue) mbar_arrive(b_kv_empty + 8 * st);      // (no row of a K tile is written to a cache)
-          tc_commit(b_s_full + 8 * (kq & 1u), issue);
-          if (!Cfg::kStageInQ && last_of_item) tc_commit(bar_q_empty + 16 * t + 8 * (item & 1u), issue);   // last read of Q
-          return true;
-        };
-        // The slot's tiles form one stream across items: while the softmax threads work on tile k,
-        // the scores of the stream's next tile are computed, also when that tile opens the slot's
-        // next item (its Q has been loaded and rotated under this item).
-        int w = -1, n = 0, j = 0;
-        {
-          if (!mbar_wait_warp<kWaitItemFull>(b_item_full, 0u, wctx)) ok = false;
-          if (ok) {
-            const volatile int* e = s_ring + (t * (int)kRing) * kRingInts;
-            w = uniform(e[0]); n = uniform(e[3]);
-            if (issue) mbar_arrive(b_item_empty);
-          }
-        }
-        if (ok && w >= 0) ok = mbar_wait_warp<kWaitQFull>(b_q_ready, 0u, wctx) && issue_qk(kc, 0u, n == 1);
-        while (ok && w >= 0) {
-          const bool last_tile = (j + 1 == n);
-          int w_next = w, n_next = n;
-          // With one tile per item the next item's scores would be issued before the previous item's
-          // epilogue has read O_t; the softmax threads must not get that far ahead of it.
-          if (j == 0 && last_tile && !(ok = mbar_wait_warp<kWaitOEmpty>(b_o_empty, (it_n & 1u) ^ 1u, wctx))) break;
-          const uint32_t item = it_n + (last_tile ? 1u : 0u);         // whose tile comes next
-          if (last_tile) {
-            const uint32_t ring = item % kRing;
-            if (!(ok = mbar_wait_warp<kWaitItemFull>(b_item_full + 8 * ring, (item / kRing) & 1u, wctx))) break;
-            const volatile int* e = s_ring + (t * (int)kRing + (int)ring) * kRingInts;
-            w_next = uniform(e[0]); n_next = uniform(e[3]);
-            if (issue) mbar_arrive(b_item_empty + 8 * ring);
-            if (w_next >= 0 && !(ok = mbar_wait_warp<kWaitQFull>(b_q_ready + 8 * (item & 1u), (item >> 1) & 1u, wctx))) break;
-          }
-          if (w_next >= 0 && !(ok = issue_qk(kc + 1, item, last_tile ? n_next == 1 : j + 2 == n))) break;
-          // the previous item's epilogue must have read O_t before it is overwritten
-          if (j == 0 && !last_tile && !(ok = mbar_wait_warp<kWaitOEmpty>(b_o_empty, (it_n & 1u) ^ 1u, wctx))) break;
-          const uint32_t idx = kv_index_v(kc), st = idx % NS;
-          if (!(ok = mbar_wait_warp<kWaitVFull>(b_kv_full + 8 * st, (idx / NS) & 1u, wctx))) break;
-          if constexpr (kFill) {
-            // The cache writer must have seen V(kc - 2), whose barrier this is again, before V(kc) is announced. K(kc + 1)
-            // could not have been loaded otherwise (three stages; with four, V(kc)); the slot's last tile has none.
-            const uint32_t before = kv_index_v(kc - 2u);
-            if (last_tile && w_next < 0 && kc >= 2u &&
-                !(ok = mbar_wait_warp<kWaitVEmpty>(b_kv_empty + 8 * (before % NS), (before / NS) & 1u, wctx))) break;
-            if (issue) mbar_arrive((t ? bar_v_seen1 : bar_v_seen0) + 8 * (kc & 1u));
-          }
-          if (!(ok = mbar_wait_warp<kWaitP>(b_p_full + 8 * (kc & 1u), (kc >> 1) & 1u, wctx))) break;
-          tc_fence_after();            // O_t (+)= P(k) V(k)
-          const uint32_t a = tm_s + 64u * (kc & 1u);
-          const uint32_t vb = v_lo + st * (Cfg::kKVBytes >> 4);
-          mma_ts(tm_o, a, vb, idesc_pv, j == 0 ? 0u : 1u, issue);
-#pragma unroll
-          for (int kk = 1; kk < BN / 16; ++kk)
-            mma_ts(tm_o, a + kk * 8, vb + (uint32_t)kk * ((16 * 128) >> 4), idesc_pv, 1u, issue);
-          tc_commit(b_kv_empty + 8 * st, issue);
-          tc_commit(bar_pv_done + 8 * t, issue);
-          ++kc;
-          if (last_tile) {
-            tc_commit(b_o_full, issue);
-            ++it_n;
-            w = w_next; n = n_next; j = 0;
-          } else {
-            ++j;
+            for (int kk = 0; kk < D / 16; ++kk) {
+              constexpr uint32_t kChunkQ = (BM * 128) >> 4, kChunkK = (BN * 128) >> 4;
+              mma_ss(d, a_lo + (uint32_t)(kk >> 2) * kChunkQ + (uint32_t)(kk & 3) * 2,
+                     kb + (uint32_t)(kk >> 2) * kChunkK + (uint32_t)(kk & 3) * 2, idesc_qk, kk > 0 ? 1u : 0u, issue);
+            }
+            tc_commit(bar_s_full + 8 * buf, issue);
+            if (!Cfg::kStageInQ && j + 1 == n) tc_commit(bar_q_empty + 8 * it2, issue);   // last read of Q
           }
         }
       }
@@ -946,7 +912,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
       }
     }
     }   // shared-stream roles
-  } else if (kFill && warp >= 20) {
+  } else if (kIndep && warp >= 20) {
     // ------------------------------------------------------------------ cache writer of slot t (warps 20, 21)
     // UNPACK of V: every row of V passes through shared memory here anyway, so the warp writes it to its prompt's
     // cache from there while the slot's other warps compute, and the kernel in front of this one reads and writes K
@@ -955,8 +921,49 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
     // heads of 128, rotation kernel 121 -> 77 us, this one 194 -> 210 (they overlap), both 299 -> 292.
     // (K' written the same way made this kernel 58 us longer, as much as the rotation kernel got shorter: a K stage
     // is wanted back as soon as the scores are there, a V stage is held for the softmax's time in any case.)
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsWriter));
-    if (warp < 22) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLast));
+    if (warp >= 22) {
+      // ---------------------------------------------------------------- products of slot t: O (+)= P(k) V(k)
+      const int t = warp - 22;
+      const uint32_t issue = elect_one();
+      constexpr uint32_t idesc_pv = instr_desc(D, true);
+      constexpr int NS = Cfg::kKVStages;
+      const uint32_t v_lo = desc_lo(s_kv, BN * 128) + (uint32_t)(t * NS) * (Cfg::kKVBytes >> 4);
+      const uint32_t tm_s = tmem_base + Cfg::kTmemS + 128u * (uint32_t)t;
+      const uint32_t tm_o = tmem_base + Cfg::kTmemO + (uint32_t)D * (uint32_t)t;
+      uint32_t kc = 0;
+      bool ok = true;
+      for (uint32_t it_n = 0; ok; ++it_n) {
+        const uint32_t ring = (uint32_t)t * kRing + it_n % kRing;
+        if (!mbar_wait_warp<kWaitItemFull>(bar_item_full + 8 * ring, (it_n / kRing) & 1u, wctx)) break;
+        const volatile int* e = s_ring + ring * kRingInts;
+        const int w = uniform(e[0]), n = uniform(e[3]);
+        if (issue) mbar_arrive(bar_item_empty + 8 * ring);
+        if (w < 0) break;
+        for (int j = 0; j < n; ++j, ++kc) {            // (no item is without tiles)
+          const uint32_t st = kv_index_v(kc) % NS, buf = 2u * (uint32_t)t + (kc & 1u);
+          // the previous item's epilogue must have read O_t before it is overwritten
+          if (j == 0 && it_n > 0u &&
+              !(ok = mbar_wait_warp<kWaitOEmpty>(bar_o_empty + 8 * (2u * (uint32_t)t + ((it_n - 1u) & 1u)), ((it_n - 1u) >> 1) & 1u, wctx))) break;
+          if (!(ok = mbar_wait_warp<kWaitVFull>(bar_v_full + 8 * buf, (kc >> 1) & 1u, wctx))) break;
+          if constexpr (kFill) {
+            // the cache writer must have seen V(k - 2), whose barrier this is again, before V(k) is announced
+            if (kc >= 2u && !(ok = mbar_wait_warp<kWaitVEmpty>(bar_v_read + 8 * buf, ((kc - 2u) >> 1) & 1u, wctx))) break;
+            if (issue) mbar_arrive((t ? bar_v_seen1 : bar_v_seen0) + 8 * (kc & 1u));
+          }
+          if (!(ok = mbar_wait_warp<kWaitP>(bar_p_full + 8 * buf, (kc >> 1) & 1u, wctx))) break;
+          tc_fence_after();
+          const uint32_t a = tm_s + 64u * (kc & 1u);
+          const uint32_t vb = v_lo + st * (Cfg::kKVBytes >> 4);
+          mma_ts(tm_o, a, vb, idesc_pv, j == 0 ? 0u : 1u, issue);
+#pragma unroll
+          for (int kk = 1; kk < BN / 16; ++kk)
+            mma_ts(tm_o, a + kk * 8, vb + (uint32_t)kk * ((16 * 128) >> 4), idesc_pv, 1u, issue);
+          tc_commit(bar_pv_done + 8 * buf, issue);
+          if (j + 1 == n) tc_commit(bar_o_full + 8 * t, issue);
+        }
+      }
+    } else if (kFill) {
       const int t = warp - 20;
       const uint32_t bar_v_seen = t ? bar_v_seen1 : bar_v_seen0;
       constexpr int NS = Cfg::kKVStages;
@@ -1017,7 +1024,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             row = stop;
           }
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar_kv_empty + 8 * (4 * t + st));
+          if (lane == 0) mbar_arrive(bar_v_read + 8 * (2u * (uint32_t)t + (kc & 1u)));
         }
       }
     }
@@ -1056,7 +1063,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
         key_hi = real ? i_row : 0;
       };
       if (h == 0) {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kFill ? kRegsSoftmaxFill : kRegsSoftmaxIndep));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmaxIndep));
         uint32_t it_n = 0, tcount = 0;
         while (true) {
           const uint32_t ring = ring0 + it_n % kRing;
@@ -1108,7 +1115,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
             const float alpha = rescale ? fast_exp2(m_run - m_new) : 1.f;
             if (j > 0 && __any_sync(0xffffffffu, rescale)) {
               // S(k) is computed ahead of P(k-1) V(k-1): O_t is stable only once that product is there
-              ok = mbar_wait_warp<kWaitVEmpty>(bar_pv_done + 8 * t, (tcount - 1u) & 1u, wctx);
+              ok = mbar_wait_warp<kWaitVEmpty>(bar_pv_done + 16 * t + 8 * (sbuf ^ 1u), ((tcount - 1u) >> 1) & 1u, wctx);
               if (!ok) break;
               tc_fence_after();
 #pragma unroll 1
@@ -1150,7 +1157,6 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
           ++it_n;
         }
       } else {
-        if (!kFill) asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsHelper));
         uint32_t it_n = 0;
         int p_q_row0 = 0, p_head = 0, p_bin = 0;         // coordinates of the previous item (its epilogue is due)
         while (true) {
@@ -1245,7 +1251,7 @@ attention_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constan
               tc_wait_ld();
               if (hh == D / 64 - 1) {
                 tc_fence_before();
-                mbar_arrive(bar_o_empty + 8 * t);        // O_t may be overwritten by the next item now
+                mbar_arrive(bar_o_empty + 16 * t + 8 * (pi & 1u));   // O_t may be overwritten by the next item now
               }
 #pragma unroll
               for (int c16 = 0; c16 < 8; ++c16) {
@@ -1718,7 +1724,7 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.status = device_status;
   a.wait_limit = (uint32_t)std::min<unsigned long long>(wait_limit_ns() >> 10, 0x7fffffffu);
   const unsigned grid = (unsigned)(total < sms ? total : sms);
-  const cudaError_t launch_err = launch_dependent(attention_kernel<D, kIndep, kFill, Table>, dim3(grid), dim3(kFill ? kAttnThreadsFill : kAttnThreads),
+  const cudaError_t launch_err = launch_dependent(attention_kernel<D, kIndep, kFill, Table>, dim3(grid), dim3(kIndep ? kAttnThreadsIndep : kAttnThreads),
                                                   (size_t)Cfg::kSmemBytes, stream, mq, mk, mv, mo, a, tab);
   const cudaError_t e = launch_err != cudaSuccess ? launch_err : cudaGetLastError();
   return e == cudaSuccess ? PP_OK : note_cuda_error((int)e, "attention kernel launch");
