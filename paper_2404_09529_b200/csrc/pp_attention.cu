@@ -404,6 +404,8 @@ struct AttnArgs {
   int32_t fold_shift;            //   bin row q_row0 + (m >> fold_shift) of head head[0] + (m & (fold - 1)))
   int32_t capacity;              // rows per bin
   int32_t total_work;            // n_kv_heads * n_items * subs
+  int32_t tail_head0;            // KV heads from here on are drawn together (launch_attention_t says why):
+  int32_t tail_start, tail_cols; //   work indices from tail_start on, tail_cols of them per geometry entry
   float scale_log2;              // softmax scale * log2(e)
   float bound2;                  // (kBoundLog2 / scale_log2)^2: |q|^2 |k|^2 up to which scores are bounded
   const float2* rope_table;      // [D/4][capacity][2] (cos, sin) pairs, or null: Q arrives already rotated
@@ -425,10 +427,14 @@ struct Work {
 
 template <class Table>
 __device__ __forceinline__ void decode_work(const AttnArgs& a, const Table& tab, int w, Work& wk) {
-  const int sub = w % a.subs;
-  const int rest = w / a.subs;
-  const int gi = rest % a.n_items;
-  wk.kv_head = rest / a.n_items;
+  // KV head, entry, sub (outermost first); in the tail entry, KV head, sub
+  const bool tail = w >= a.tail_start;
+  const uint32_t wr = (uint32_t)(tail ? w - a.tail_start : w), cols = (uint32_t)(tail ? a.tail_cols : a.subs);
+  const uint32_t q = wr / cols, c = wr - q * cols;
+  const uint32_t num = tail ? c : q, den = (uint32_t)(tail ? a.subs : a.n_items);
+  const uint32_t d = num / den, m = num - d * den;
+  const int gi = (int)(tail ? q : m), sub = (int)(tail ? m : c);
+  wk.kv_head = (int)d + (tail ? a.tail_head0 : 0);
   const int at = a.off_items + kItemInts * gi;
   const int4 x = tab.i128(at), y = tab.i128(at + 4);
   wk.bin = x.x; wk.kv_row0 = x.y; wk.n = x.z; wk.q_row0[0] = x.w; wk.q_row0[1] = y.x;
@@ -1723,6 +1729,19 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.rope_table = static_cast<const float2*>(rope_table);
   a.status = device_status;
   a.wait_limit = (uint32_t)std::min<unsigned long long>(wait_limit_ns() >> 10, 0x7fffffffu);
+  // The order of the work: KV heads one after another, so that those at work at a time find their K and V in L2, each
+  // head's entries longest first. How evenly the CTAs finish is then left to the last head alone; in the independent
+  // mode the last heads are drawn together, the longest entries of all of them first: two heads, or as many as make two
+  // entries for every slot. (Longest finish / mean, replayed: 16 prompts on 32 heads 1.41 -> 1.17, 64 of them 1.09 -> 1.03,
+  // 2048 short ones on 8 heads 1.05 -> 1.01. Measured, whole steps: 48.8 -> 46.1 us, 235 -> 231.5, 170 -> 168; with four entries
+  // per slot 46.7, 232.5, 169; with one 48.2, 234, 169.) The shared-stream mode's long lists end evenly by themselves, and two
+  // heads at a time cost it L2 hits (256 prompts on 32 / 8 heads 6330 -> 6400): its heads are drawn together only where one
+  // has less than two entries for every CTA.
+  const int64_t per_head = (int64_t)L.n_items * a.subs, drawers = (int64_t)(kIndep ? 2 : 1) * sms;
+  const int64_t together = std::min<int64_t>(p.n_kv_heads, std::max<int64_t>(kIndep ? 2 : 1, (2 * drawers + per_head - 1) / per_head));
+  a.tail_head0 = p.n_kv_heads - (int32_t)together;
+  a.tail_start = (int32_t)(a.tail_head0 * per_head);
+  a.tail_cols = (int32_t)(together * a.subs);
   const unsigned grid = (unsigned)(total < sms ? total : sms);
   const cudaError_t launch_err = launch_dependent(attention_kernel<D, kIndep, kFill, Table>, dim3(grid), dim3(kIndep ? kAttnThreadsIndep : kAttnThreads),
                                                   (size_t)Cfg::kSmemBytes, stream, mq, mk, mv, mo, a, tab);

@@ -103,6 +103,22 @@ def test_head_folding_variants_full_parity(lengths, hq, hkv, d, fold):
             compare_with_refs(b, lengths, refs)
 
 
+# KV heads that are drawn one after another and those drawn together at the end of the work list: all of them together (one
+# head, several), two of four, two of three with three query heads each that are not folded, two of three in the shared-stream mode
+@pytest.mark.parametrize("lengths,hq,hkv,d,mode,entries_per_head", [
+    ([50, 20, 300], 1, 1, 64, 1, 4), ([50, 20, 300], 5, 5, 128, 1, 4), ([130] * 300, 4, 4, 64, 1, 600),
+    ([130] * 100, 9, 3, 64, 1, 600), ([4000, 3000, 2600], 12, 3, 64, 0, 154)])
+def test_every_head_is_drawn_once(lengths, hq, hkv, d, mode, entries_per_head):
+    lengths = np.asarray(lengths, np.int32)
+    q, k, v = _case(lengths, hq, hkv, d, seed=len(lengths) + hq)
+    b = run_cuda(lengths, q, k, v, hq, hkv, d, 10000.0, "packed", fused=True, guard=True)
+    info = pp.pp_prefill_schedule_info(b.params, b.pack)
+    assert info["mode"] == mode
+    heads_per_entry = info["heads_folded"] if mode == 1 else 2
+    assert info["entries"] * (hq // hkv) // heads_per_entry == entries_per_head
+    compare_with_refs(b, lengths, oracle_refs(lengths, q, k, v, 10000.0))
+
+
 @pytest.mark.parametrize("room", [1, 7, 64])
 @pytest.mark.parametrize("lengths,hq,hkv,d", [
     ([112, 87, 73, 46, 50, 20, 24, 17], 4, 4, 64),          # several prompts per bin, independent mode
