@@ -455,14 +455,16 @@ decode_combine_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
 
 // Keys per chunk. Enough (chunk, KV head) CTAs for about four rounds of the three per SM that run at once, so that
 // the last round is a small part of the whole; at least one 16-key step for each of the four warps, at most
-// 512 keys (a CTA's set-up is then a few per cent of its loads), and more only where a very long prompt would
+// 512 keys (a CTA's set-up is then a few per cent of its loads), 1024 where those make the four rounds too (256
+// prompts, 240 k cached tokens, 32 / 8 heads: 512 keys 165.6 us a step, 768 161.0, 1024 160.9, 1536 163.0, 2048 167.4),
+// and more only where a very long prompt would
 // otherwise be cut into more pieces than one warp merges quickly.
 constexpr int64_t kChunkCtasWanted = kSms * 3 * 4;
 constexpr int kMostChunksPerPrompt = 64;
 
 struct DecodeLayout {
   size_t chunk_ptr_off, table_bytes;    // table: prompts, chunk_ptr (uploaded where they do not fit the parameters)
-  size_t ml_off, o_off, total_bytes;
+  size_t ml_off, o_off, total_bytes, sized_bytes;
   int64_t n_chunks;
   int32_t chunk_keys;
 };
@@ -475,17 +477,27 @@ DecodeLayout decode_layout(const pp_attn_params& p, const int32_t* lengths, int3
     longest = std::max(longest, lengths[i]);
   }
   const int64_t unit = kTileKeys * kDecodeWarps;
-  int64_t keys = std::min<int64_t>(std::max<int64_t>(total * p.n_kv_heads / kChunkCtasWanted, 1), 512);
+  const int64_t even = total * p.n_kv_heads / kChunkCtasWanted;
+  int64_t keys = even >= 1024 ? 1024 : std::min<int64_t>(std::max<int64_t>(even, 1), 512);
   keys = std::max<int64_t>(keys, ((int64_t)longest + kMostChunksPerPrompt - 1) / kMostChunksPerPrompt);
   L.chunk_keys = (int32_t)((keys + unit - 1) / unit * unit);
+  // What pp_decode_workspace_bytes says leaves room for chunks half as long, where these may be: the same prompts a few
+  // tokens shorter then fit a workspace that was sized for the longer ones.
+  const int32_t sized_for = L.chunk_keys == 1024 ? 512 : L.chunk_keys;
   L.n_chunks = 0;
-  for (int32_t i = 0; i < k; ++i) L.n_chunks += ((int64_t)lengths[i] + L.chunk_keys - 1) / L.chunk_keys;
+  int64_t chunks_sized_for = 0;
+  for (int32_t i = 0; i < k; ++i) {
+    L.n_chunks += ((int64_t)lengths[i] + L.chunk_keys - 1) / L.chunk_keys;
+    chunks_sized_for += ((int64_t)lengths[i] + sized_for - 1) / sized_for;
+  }
   auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
   L.chunk_ptr_off = (size_t)k * sizeof(DecodePrompt);
   L.table_bytes = L.chunk_ptr_off + ((size_t)k + 1) * sizeof(int32_t);
   L.ml_off = up(L.table_bytes);
   L.o_off = up(L.ml_off + (size_t)L.n_chunks * p.n_q_heads * sizeof(float2));
-  L.total_bytes = L.o_off + (size_t)L.n_chunks * p.n_q_heads * p.head_dim * sizeof(float);
+  const size_t row = (size_t)p.n_q_heads * p.head_dim * sizeof(float);
+  L.total_bytes = L.o_off + (size_t)L.n_chunks * row;
+  L.sized_bytes = up(L.ml_off + (size_t)chunks_sized_for * p.n_q_heads * sizeof(float2)) + (size_t)chunks_sized_for * row;
   return L;
 }
 
@@ -538,7 +550,7 @@ extern "C" size_t pp_decode_workspace_bytes(const pp_attn_params* params, const 
   if (pp::check_decode_params(params) != PP_OK || !lengths || k < 1) return 0;
   for (int32_t i = 0; i < k; ++i)
     if (lengths[i] < 1) return 0;
-  return pp::decode_layout(*params, lengths, k).total_bytes;
+  return pp::decode_layout(*params, lengths, k).sized_bytes;
 }
 
 extern "C" int pp_decode_step(const pp_attn_params* params, const int32_t* lengths, int32_t k,

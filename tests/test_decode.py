@@ -89,6 +89,7 @@ def test_decode_argument_checks():
     (np.array([70] * 40 + [200], np.int32), 4, 1, 128, 64),                              # the larger parameter block
     (np.array([3000] * 3 + [512, 513], np.int32), 128, 32, 64, 192),                     # between the smallest and the largest
     (np.array([9000] * 3 + [1536, 512, 513], np.int32), 64, 32, 64, 512),                # the largest
+    (np.array([18955] * 3 + [1], np.int32), 32, 32, 64, 512),                            # chunks of 1024, room for those of 512
 ])
 def test_decode_chunks_and_tables(lengths, hq, hkv, d, chunk_keys):
     """The generation step on caches of random contents at the edges of its steps, chunks and table forms,
