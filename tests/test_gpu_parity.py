@@ -441,3 +441,36 @@ def test_independent_mode_gives_up_cleanly_when_its_waits_expire(hq, hkv, d, mon
     assert b.device_status() == 0
     for x, y in zip(want, (b.o_tokens(), b.k_cache, b.v_cache)):
         assert torch.equal(x, y)
+
+
+# two heads over the same rows; two row tiles of one head
+@pytest.mark.parametrize("hq,hkv,d", [(8, 4, 64), (3, 1, 128)])
+def test_shared_stream_mode_gives_up_cleanly_when_its_waits_expire(hq, hkv, d, monkeypatch):
+    """The same on the fused route in the shared-stream mode, whose loading and issuing warps wait in a form of their own: a
+    warp that has loaded the Q of the next item waits for the whole of the present one."""
+    import paper_2404_09529_b200 as pp
+    from paper_2404_09529_b200.runner import PrefillBatch
+    lengths = np.array([16000, 16000], np.int32)
+    q, k, v = _random_case(lengths, hq, hkv, d, seed=d)
+    b = PrefillBatch(lengths, hq, hkv, d, 10000.0)
+    assert pp.pp_prefill_schedule_info(b.params, b.pack)["mode"] == 0
+    b.load(q, k, v)
+    b.run_fused()
+    torch.cuda.synchronize()
+    assert b.device_status() == 0
+    want = [x.clone() for x in (b.o_tokens(), b.k_cache, b.v_cache)]
+    b.load(q, k, v)
+    monkeypatch.setenv("PP_WAIT_LIMIT_US", "1")
+    b.run_fused()
+    torch.cuda.synchronize()
+    assert 1 <= b.device_status() <= 20
+    monkeypatch.delenv("PP_WAIT_LIMIT_US")
+    b.ws.status.zero_()
+    b.load(q, k, v)
+    for x in (b.o, b.k_cache, b.v_cache):
+        x.zero_()
+    b.run_fused()
+    torch.cuda.synchronize()
+    assert b.device_status() == 0
+    for x, y in zip(want, (b.o_tokens(), b.k_cache, b.v_cache)):
+        assert torch.equal(x, y)
