@@ -464,12 +464,11 @@ constexpr int kMostChunksPerPrompt = 64;
 
 struct DecodeLayout {
   size_t chunk_ptr_off, table_bytes;    // table: prompts, chunk_ptr (uploaded where they do not fit the parameters)
-  size_t ml_off, o_off, total_bytes, sized_bytes;
+  size_t ml_off, o_off, total_bytes;
   int64_t n_chunks;
   int32_t chunk_keys;
 };
-DecodeLayout decode_layout(const pp_attn_params& p, const int32_t* lengths, int32_t k) {
-  DecodeLayout L;
+int32_t decode_chunk_keys(const pp_attn_params& p, const int32_t* lengths, int32_t k) {
   int64_t total = 0;
   int32_t longest = 0;
   for (int32_t i = 0; i < k; ++i) {
@@ -480,24 +479,19 @@ DecodeLayout decode_layout(const pp_attn_params& p, const int32_t* lengths, int3
   const int64_t even = total * p.n_kv_heads / kChunkCtasWanted;
   int64_t keys = even >= 1024 ? 1024 : std::min<int64_t>(std::max<int64_t>(even, 1), 512);
   keys = std::max<int64_t>(keys, ((int64_t)longest + kMostChunksPerPrompt - 1) / kMostChunksPerPrompt);
-  L.chunk_keys = (int32_t)((keys + unit - 1) / unit * unit);
-  // What pp_decode_workspace_bytes says leaves room for chunks half as long, where these may be: the same prompts a few
-  // tokens shorter then fit a workspace that was sized for the longer ones.
-  const int32_t sized_for = L.chunk_keys == 1024 ? 512 : L.chunk_keys;
+  return (int32_t)((keys + unit - 1) / unit * unit);
+}
+DecodeLayout decode_layout(const pp_attn_params& p, const int32_t* lengths, int32_t k, int32_t chunk_keys) {
+  DecodeLayout L;
+  L.chunk_keys = chunk_keys;
   L.n_chunks = 0;
-  int64_t chunks_sized_for = 0;
-  for (int32_t i = 0; i < k; ++i) {
-    L.n_chunks += ((int64_t)lengths[i] + L.chunk_keys - 1) / L.chunk_keys;
-    chunks_sized_for += ((int64_t)lengths[i] + sized_for - 1) / sized_for;
-  }
+  for (int32_t i = 0; i < k; ++i) L.n_chunks += ((int64_t)lengths[i] + chunk_keys - 1) / chunk_keys;
   auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
   L.chunk_ptr_off = (size_t)k * sizeof(DecodePrompt);
   L.table_bytes = L.chunk_ptr_off + ((size_t)k + 1) * sizeof(int32_t);
   L.ml_off = up(L.table_bytes);
   L.o_off = up(L.ml_off + (size_t)L.n_chunks * p.n_q_heads * sizeof(float2));
-  const size_t row = (size_t)p.n_q_heads * p.head_dim * sizeof(float);
-  L.total_bytes = L.o_off + (size_t)L.n_chunks * row;
-  L.sized_bytes = up(L.ml_off + (size_t)chunks_sized_for * p.n_q_heads * sizeof(float2)) + (size_t)chunks_sized_for * row;
+  L.total_bytes = L.o_off + (size_t)L.n_chunks * p.n_q_heads * p.head_dim * sizeof(float);
   return L;
 }
 
@@ -550,7 +544,11 @@ extern "C" size_t pp_decode_workspace_bytes(const pp_attn_params* params, const 
   if (pp::check_decode_params(params) != PP_OK || !lengths || k < 1) return 0;
   for (int32_t i = 0; i < k; ++i)
     if (lengths[i] < 1) return 0;
-  return pp::decode_layout(*params, lengths, k).sized_bytes;
+  // Where a step takes chunks of 1024 keys there is room for chunks of 512: the same prompts a few tokens shorter, across
+  // the line between the two, then fit a workspace that was sized for the longer ones. (Not across the smaller steps of
+  // the chunks below 512.)
+  const int32_t keys = pp::decode_chunk_keys(*params, lengths, k);
+  return pp::decode_layout(*params, lengths, k, keys == 1024 ? 512 : keys).total_bytes;
 }
 
 extern "C" int pp_decode_step(const pp_attn_params* params, const int32_t* lengths, int32_t k,
@@ -571,7 +569,7 @@ extern "C" int pp_decode_step(const pp_attn_params* params, const int32_t* lengt
     if (cache_off[i] < 0) return PP_ERR_INVALID_ARG;
     if (cache_off[i] % 8 != 0) return PP_ERR_ALIGNMENT;
   }
-  const pp::DecodeLayout L = pp::decode_layout(*params, lengths, k);
+  const pp::DecodeLayout L = pp::decode_layout(*params, lengths, k, pp::decode_chunk_keys(*params, lengths, k));
   if (L.n_chunks > INT32_MAX / 4) return PP_ERR_UNSUPPORTED;
   if (workspace_bytes < L.total_bytes) return PP_ERR_BUFFER_TOO_SMALL;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
