@@ -148,16 +148,10 @@ def table_ints(params, pack):
     return three, pp.pp_prefill_fused_host_bytes(params, pack.k) // 4, info["mode"] == 1
 
 
-def decode_chunks(params, lengths):
-    """Chunks that pp_decode_step cuts the prompts into, from the size of its workspace: table of 16 bytes per prompt and a
-    prefix, then 8 bytes and head_dim floats per chunk and query head, each block on a 256-byte boundary."""
-    import paper_2404_09529_b200 as pp
+def decode_bytes(params, lengths, chunk_keys):
+    """Workspace that a step of pp_decode_step takes if it cuts the prompts into chunks of chunk_keys: a table of 16 bytes per
+    prompt and a prefix, then 8 bytes and head_dim floats per chunk and query head, each block on a 256-byte boundary."""
     up = lambda x: (x + 255) // 256 * 256
-    need, k = pp.pp_decode_workspace_bytes(params, lengths), len(lengths)
+    k, n = len(lengths), sum(-(-int(l) // chunk_keys) for l in lengths)
     hq, d = params.n_q_heads, params.head_dim
-    size = lambda n: up(up(16 * k + 4 * (k + 1)) + 8 * n * hq) + 4 * n * hq * d
-    n = need // (hq * (4 * d + 8))
-    while size(n) > need:
-        n -= 1
-    assert size(n) == need
-    return n
+    return up(up(16 * k + 4 * (k + 1)) + 8 * n * hq) + 4 * n * hq * d

@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from oracle import prepack_oracle as orc
-from parity_utils import MAX_ABS_TOL, MEAN_ABS_TOL, decode_chunks, to64
+from parity_utils import MAX_ABS_TOL, MEAN_ABS_TOL, decode_bytes, to64
 from workloads import split_by_prompt
 
 pytestmark = pytest.mark.gpu
@@ -89,20 +89,29 @@ def test_decode_argument_checks():
     (np.array([70] * 40 + [200], np.int32), 4, 1, 128, 64),                              # the larger parameter block
     (np.array([3000] * 3 + [512, 513], np.int32), 128, 32, 64, 192),                     # between the smallest and the largest
     (np.array([9000] * 3 + [1536, 512, 513], np.int32), 64, 32, 64, 512),                # the largest
-    (np.array([18955] * 3 + [1], np.int32), 32, 32, 64, 512),                            # chunks of 1024, room for those of 512
+    (np.array([18943] * 3 + [1], np.int32), 32, 32, 64, 512),                            # the last before the line
+    (np.array([18944] * 3 + [1], np.int32), 32, 32, 64, 1024),                           # and past it
 ])
 def test_decode_chunks_and_tables(lengths, hq, hkv, d, chunk_keys):
     """The generation step on caches of random contents at the edges of its steps, chunks and table forms,
-    spare rows untouched."""
+    spare rows untouched. The chunks are those that the step takes: it runs in the workspace that they need and in no less."""
+    import paper_2404_09529_b200 as pp
     from paper_2404_09529_b200.runner import DecodeBatch
     dec = DecodeBatch(lengths, hq, hkv, d, 10000.0, room=2)
-    assert decode_chunks(dec.params, lengths) == sum(-(-int(l) // chunk_keys) for l in lengths)
+    need = decode_bytes(dec.params, lengths, chunk_keys)
+    assert pp.pp_decode_workspace_bytes(dec.params, lengths) == decode_bytes(dec.params, lengths, min(chunk_keys, 512))
     g = torch.Generator().manual_seed(int(lengths.sum()))
     for pool in (dec.k_cache, dec.v_cache):
         pool.copy_(torch.randn(pool.shape, generator=g).to(torch.bfloat16))
     before = [tuple(c.clone() for c in dec.caches(i)) for i in range(dec.k)]
     qn, kn, vn = (torch.randn(dec.k, h, d, generator=g).to(torch.bfloat16) for h in (hq, hkv, hkv))
-    got = to64(dec.step(qn.cuda(), kn.cuda(), vn.cuda()))
+    ws, host = torch.empty(need, dtype=torch.uint8, device="cuda"), torch.empty(need, dtype=torch.uint8).pin_memory()
+    step = lambda nbytes: pp.pp_decode_step(dec.params, lengths, qn.cuda(), kn.cuda(), vn.cuda(), dec.o, dec.k_cache, dec.v_cache,
+                                            dec.cache_off, dec.cache_cap, ws, host, nbytes)
+    with pytest.raises(pp.PrepackError):
+        step(need - 1)
+    step(need)
+    got = to64(dec.o)
     errs = []
     for i in range(dec.k):
         l = int(lengths[i])
@@ -116,6 +125,30 @@ def test_decode_chunks_and_tables(lengths, hq, hkv, d, chunk_keys):
             assert torch.equal(now[:, :l], was[:, :l]) and torch.equal(now[:, l + 1:], was[:, l + 1:])
     e = np.concatenate(errs)
     assert e.max() <= MAX_ABS_TOL and e.mean() <= MEAN_ABS_TOL, (e.max(), e.mean())
+
+
+@pytest.mark.parametrize("sized,used,keys", [
+    ([18955] * 3, [18900] * 3, 512),         # sized where a step takes chunks of 1024, used where it takes 512
+    ([18900] * 3, [18955] * 3, 1024),        # the other way round
+])
+def test_decode_workspace_on_the_other_side_of_the_line(sized, used, keys):
+    """A workspace that was sized on one side of the line between chunks of 512 and of 1024 keys holds a step on the other side;
+    the step gives what it gives in a workspace of its own."""
+    import paper_2404_09529_b200 as pp
+    from paper_2404_09529_b200.runner import DecodeBatch
+    sized, used = np.array(sized, np.int32), np.array(used, np.int32)
+    h, d = 32, 64
+    dec = DecodeBatch(used, h, h, d, 10000.0, room=2)
+    nbytes = pp.pp_decode_workspace_bytes(dec.params, sized)
+    assert decode_bytes(dec.params, used, keys) <= nbytes
+    g = torch.Generator(device="cuda").manual_seed(7)
+    for pool in (dec.k_cache, dec.v_cache):
+        pool.copy_(torch.randn(pool.shape, generator=g, device="cuda"))
+    new = [torch.randn(dec.k, h, d, generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)]
+    ws, host = torch.empty(nbytes, dtype=torch.uint8, device="cuda"), torch.empty(nbytes, dtype=torch.uint8).pin_memory()
+    o = torch.zeros_like(dec.o)
+    pp.pp_decode_step(dec.params, used, *new, o, dec.k_cache, dec.v_cache, dec.cache_off, dec.cache_cap, ws, host, nbytes)
+    assert torch.equal(o, dec.step(*new))
 
 
 @pytest.mark.parametrize("hq,hkv,d", [(2, 2, 128), (8, 1, 128), (6, 2, 64)])
