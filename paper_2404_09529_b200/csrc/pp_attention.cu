@@ -135,15 +135,15 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // A value that is the same in all lanes, said so to the compiler (all 32 lanes call).
 __device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
 
-// Every wait in the kernel goes through here or through the two forms for a warp below: it gives up after `limit`, leaving why in the CTA-wide abort word, so
-// that all roles leave their loops; the code goes to the device status word at the end of the kernel. A kernel of this
-// file has some forty waits, inlined, and the warps of a scheduler run three to five roles: what they execute has to fit
-// its instruction cache (a straight line of code takes 1.0 cycles an instruction up to 32 KB, 3.1 to 128 KB, 6 beyond,
-// one scheduler at work). With a 64-bit clock, a global atomic and a poll counter in each wait, 1.1 of the 6 warps of a
-// scheduler stood without an instruction at any time where the V caches are filled; in this form, and with each load
-// of the producer loop at one place, 0.18. Attention of 64 prompts on a 7B layer 195 -> 168 us under ncu; whole
-// steps 264 -> 236 us, 2048 short prompts, 32 / 8 heads of 64, 199 -> 171, 34 bins of a stream 1040 -> 990, 16 prompts
-// 49.7 -> 48.8. (As calls of one function the waits do not fit the softmax threads' registers.)
+// Every wait in the kernel goes through here or through the two forms for a warp below: it gives up after `limit`, leaving
+// why in the CTA-wide abort word, so that all roles leave their loops; the code goes to the device status word at the end
+// of the kernel at the latest. A kernel of this file has some forty waits, inlined, and the warps of a scheduler run three
+// to five roles: what they execute has to fit its instruction cache (a straight line of code takes 1.0 cycles an
+// instruction up to 32 KB, 3.1 to 128 KB, 6 beyond, one scheduler at work). In the independent mode, with a 64-bit clock,
+// a global atomic and a poll counter in each wait 1.1 of the 6 warps of a scheduler stood without an instruction at any
+// time; in this form, and with each load of the producer loop at one place, 0.18 (64 prompts on a 7B layer: attention
+// 194 -> 158 us under ncu with the changes around them, whole steps 285 -> 258). (As calls of one function the waits do not
+// fit the softmax threads' registers.)
 struct WaitCtx {
   uint32_t abort;               // address in shared memory, 0: go on
   uint32_t limit;               // in units of 1024 ns
@@ -1759,13 +1759,16 @@ int launch_attention_t(const pp_attn_params& p, int32_t* d_table, const TableLay
   a.status = device_status;
   a.wait_limit = (uint32_t)std::min<unsigned long long>(wait_limit_ns() >> 10, 0x7fffffffu);
   // The order of the work: KV heads one after another, so that those at work at a time find their K and V in L2, each
-  // head's entries longest first. How evenly the CTAs finish is then left to the last head alone; in the independent
-  // mode the last heads are drawn together, the longest entries of all of them first: two heads, or as many as make two
-  // entries for every slot. (Longest finish / mean, replayed: 16 prompts on 32 heads 1.41 -> 1.17, 64 of them 1.09 -> 1.03,
-  // 2048 short ones on 8 heads 1.05 -> 1.01. Measured, whole steps: 48.8 -> 46.1 us, 235 -> 231.5, 170 -> 168; with four entries
-  // per slot 46.7, 232.5, 169; with one 48.2, 234, 169.) The shared-stream mode's long lists end evenly by themselves, and two
-  // heads at a time cost it L2 hits (256 prompts on 32 / 8 heads 6330 -> 6400): its heads are drawn together only where one
-  // has less than two entries for every CTA.
+  // head's entries longest first. How evenly the CTAs finish is then left to the last head alone, so the last heads are
+  // drawn together, the longest entries of all of them first.
+  // Independent mode: two heads, or as many as make two entries for every slot (16 prompts on 32 heads, longest finish /
+  // mean as replayed 1.41 -> 1.17, whole step 48.8 -> 46.1 us, with four entries per slot 46.7, with one 48.2; 64 prompts
+  // 235 -> 231.5, 232.5, 234).
+  // Shared-stream mode: as many as make two entries for every CTA, where one head has less (one after another -> together:
+  // one prompt of 4000 tokens on 32 heads of 128 192 -> 163 us, of 12 800 1295 -> 1219, two of 12 800 2474 -> 2410, one of 6400 on
+  // 32 / 8 heads 342 -> 317, of 3000 on 32 / 8 heads of 64 97 -> 75; 0.998 to 1.01 close to the line). From there on one:
+  // two made 0.994 to 1.006 of it on seven batches of up to 1.5 times as many entries, and cost 256 prompts on 32 / 8
+  // heads L2 hits (6330 -> 6400).
   const int64_t per_head = (int64_t)L.n_items * a.subs, drawers = (int64_t)(kIndep ? 2 : 1) * sms;
   const int64_t together = std::min<int64_t>(p.n_kv_heads, std::max<int64_t>(kIndep ? 2 : 1, (2 * drawers + per_head - 1) / per_head));
   a.tail_head0 = p.n_kv_heads - (int32_t)together;

@@ -16,9 +16,9 @@
 // both operands use the same, so a thread's 16-byte piece of a K row serves two products, and its 16-byte
 // pieces of four V rows (paired with byte permutes) serve eight. P is split into three bf16 numbers (24 bits
 // of it), so P V is as exact as with P in fp32.
-// Measured, whole step (D = 128): 256 prompts, 240 k cached tokens, 32 / 8 heads 568 -> 167 us (decode_kernel 159 us,
-// 6.2 TB/s, 96 % of the copy peak); 64 prompts, 17.5 k tokens, 32 / 32 heads 76 -> 57.5 us (54 us); ten prompts, 1009
-// tokens 38.5 -> 12.6 us, where the latencies in front of the first product count: the search for the prompt and
+// Measured, whole step (D = 128): 256 prompts, 240 k cached tokens, 32 / 8 heads 568 -> 165-172 us (decode_kernel 157 us,
+// 6.3 TB/s, 97 % of the copy peak); 64 prompts, 17.5 k tokens, 32 / 32 heads 76 -> 59 us (57.5 us); ten prompts, 1009
+// tokens 38.5 -> 12.7 us, where the latencies in front of the first product count: the search for the prompt and
 // the angles run while the kernel before is finishing (programmatic dependent launch), and the loads of q, k
 // and the first keys and values are all issued before any is waited for (16.0 us without the two).
 #include <cuda_bf16.h>
@@ -454,11 +454,13 @@ decode_combine_kernel(const __grid_constant__ DecodeArgs a, const __grid_constan
 }
 
 // Keys per chunk. Enough (chunk, KV head) CTAs for about four rounds of the three per SM that run at once, so that
-// the last round is a small part of the whole; at least one 16-key step for each of the four warps, at most
-// 512 keys (a CTA's set-up is then a few per cent of its loads), 1024 where those make the four rounds too (256
-// prompts, 240 k cached tokens, 32 / 8 heads: 512 keys 165.6 us a step, 768 161.0, 1024 160.9, 1536 163.0, 2048 167.4),
-// and more only where a very long prompt would
-// otherwise be cut into more pieces than one warp merges quickly.
+// the last round is a small part of the whole; at least one 16-key step for each of the four warps, at most 512 keys (a
+// CTA's set-up is then a few per cent of its loads), or 1024 where those make the four rounds too; and more only where a
+// very long prompt would otherwise be cut into more pieces than one warp merges quickly. 1024 against 512, whole steps:
+// 256 prompts, 240 k cached tokens, 32 / 8 heads 176 -> 169 us, of 893 tokens each 165 -> 156, 32 / 4 heads, 256 of 1786 180 ->
+// 165, 16 heads of 64, 256 of 867 168 -> 152; 0.90 to 1.007 on ten more (768 keys as 1024, 1536 and 2048 1 to 4 % longer). Below
+// that line even chunks of 513 to 1023 keys made 0.92 to 1.005 of the time of 512 on 25 batches and 1.02 on one (100 prompts of
+// 777 tokens on 16 heads of 64): not the same way everywhere, so those batches keep 512.
 constexpr int64_t kChunkCtasWanted = kSms * 3 * 4;
 constexpr int kMostChunksPerPrompt = 64;
 
